@@ -123,12 +123,13 @@ typedef struct rp_options {
                              Z <= 2048 FP32, 1024 FP64, deterministic 0-2,
                              rp_yields, rp_yields_batch and the converged
                              entries; elsewhere kernel 5 selects as 0 */
-  int gram;               /* time integral (Eqs. 20, 22) of each macro-step: 0 choose
-                             (2 where it applies); 1 CUDA cores (any precision);
-                             2 tensor cores (FP32 single systems with the
-                             per-term kernels: tcgen05.mma
-                             kind::tf32 on hi/lo-split values, FP32 partial
-                             sums, FP64 contraction; otherwise falls back to 1) */
+  int gram;               /* time integral (Eqs. 20, 22) of each macro-step: 0 or 1
+                             the low-rank factor of its weights on the CUDA cores (any
+                             precision and kernel); 2 the Gram matrix of the singlet
+                             slices on the tensor cores (FP32 with the per-term and
+                             cluster kernels: tcgen05.mma kind::tf32 on hi/lo-split
+                             values, FP32 partial sums, FP64 contraction; otherwise as
+                             1), which does three times the products and is slower */
   int graph;              /* 1: capture each macro-step's launches (Chebyshev terms
                              and time integral) in a CUDA graph and replay it; the
                              kernels then read the macro-step index from a device

@@ -256,12 +256,12 @@ class YieldEngine {
     const int nf = (int)plans.size();
     d_fdev_ = ar_.get<rp::FieldDev<T>>(nf);
     d_coef_ = ar_.get<T>((size_t)nf * n_c_ * 4);
-    d_W_ = ar_.get<double>((size_t)nf * n_c_ * n_c_ * 2);
+    d_iin_ = ar_.get<rp::IntegralIn>(nf);
+    iin_.resize(nf);
     std::vector<rp::FieldDev<T>> fdev(nf);
     // per field: c_n (re, im) in T, then the remainder c_n - fl(c_n) (FP32
     // only: the kernels add it, so the coefficients act with FP64 accuracy)
     std::vector<T> coef((size_t)nf * n_c_ * 4, T(0));
-    std::vector<double> W((size_t)nf * n_c_ * n_c_ * 2);
     for (int f = 0; f < nf; ++f) {
       const rp::FieldPlan& P = plans[f];
       fdev[f].omega = (T)P.omega;
@@ -278,15 +278,12 @@ class YieldEngine {
           cf[2 * n_c_ + 2 * n + 1] = (T)(P.coef[n].imag() - (double)im);
         }
       }
-      for (size_t i = 0; i < (size_t)n_c_ * n_c_; ++i) {
-        W[((size_t)f * n_c_ * n_c_ + i) * 2] = P.W[i].real();
-        W[((size_t)f * n_c_ * n_c_ + i) * 2 + 1] = P.W[i].imag();
-      }
+      iin_[f] = rp::IntegralIn{P.dE, P.h, P.kbar};
     }
     ck(cudaMemcpyAsync(d_fdev_, fdev.data(), fdev.size() * sizeof(fdev[0]), cudaMemcpyHostToDevice, st_), "h2d fields");
     ck(cudaMemcpyAsync(d_coef_, coef.data(), coef.size() * sizeof(T), cudaMemcpyHostToDevice, st_), "h2d coef");
-    ck(cudaMemcpyAsync(d_W_, W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice, st_), "h2d W");
-    h2d += (long long)(fdev.size() * sizeof(fdev[0]) + coef.size() * sizeof(T) + W.size() * sizeof(double));
+    ck(cudaMemcpyAsync(d_iin_, iin_.data(), nf * sizeof(iin_[0]), cudaMemcpyHostToDevice, st_), "h2d integral");
+    h2d += (long long)(fdev.size() * sizeof(fdev[0]) + coef.size() * sizeof(T) + nf * sizeof(iin_[0]));
   }
 
   static size_t row_bytes(long long Z, int n_c) {
@@ -312,6 +309,7 @@ class YieldEngine {
       pctas_ = rp::persistent_ctas<T>(Zslot_, n_c_, aniso_);
       if (pctas_ <= 0) throw CudaFail{RP_ECUDA, "persistent kernel: no device"};
       Xp_ = ar_.get<T>((size_t)pctas_ * n_c_ * Zslot_ * 2);
+      plan_integral(false);
       d_counter_ = ar_.get<int>(1);
       S_ = rp::SysTab<T>{d_ham_, d_lay_, d_kS_, nullptr, Zslot_, o_.pair_id, d_pair_, d_err_,
                          sec_rank_, sec_scale_};
@@ -336,20 +334,24 @@ class YieldEngine {
                                  : rp::macro_cluster_default(hf)) &&
                  rp::macro_cluster_max_active(hf) > 0;
     }
-    // tensor-core time integral: FP32 with the per-term kernels (each row's
-    // integral covers its own system's Z; the step kernel keeps the padding of
-    // the last 16-configuration chunk at zero)
-    tc_gram_ = sizeof(T) == 4 && !small_ && o_.gram != 1 && rp::gram_tc_supported(n_c_);
-    const size_t x_row = std::max<size_t>((size_t)n_c_ * Zslot_ * 2,
-                                          rp::xblk_floats_per_row(Zslot_, n_c_));
+    // tensor-core Gram integral on request: FP32 with the per-term and cluster
+    // kernels (each row's integral covers its own system's Z; the step kernel
+    // keeps the padding of the last 16-configuration chunk at zero).  The
+    // low-rank integral is the default: 5.3k multiply-adds per configuration
+    // and macro-step against 16k, no hi/lo split
+    tc_gram_ = sizeof(T) == 4 && !small_ && o_.gram == 2 && rp::gram_tc_supported(n_c_);
+    if (!d_trace_) plan_integral(tc_gram_);
+    const size_t x_row = tc_gram_ ? std::max<size_t>((size_t)n_c_ * Zslot_ * 2,
+                                                     rp::xblk_floats_per_row(Zslot_, n_c_))
+                                  : (size_t)n_c_ * Zslot_ * 2;
     X_ = ar_.get<T>((size_t)R * x_row);
     // cluster macro-steps leave SMs idle (clusters fill whole GPC pairs of 8):
     // the time integral of macro-step k runs on a second stream, reading its own
     // copy of the singlet slices, while macro-step k + 1 propagates
-    overlap_ = cluster_ && tc_gram_ && !o_.graph && !d_trace_;
+    overlap_ = cluster_ && !o_.graph && !d_trace_;
     if (overlap_) {
       X2_ = ar_.get<T>((size_t)R * x_row);
-      ck(cudaMemsetAsync(X2_, 0, (size_t)R * x_row * sizeof(T), st_), "cudaMemsetAsync");
+      if (tc_gram_) ck(cudaMemsetAsync(X2_, 0, (size_t)R * x_row * sizeof(T), st_), "cudaMemsetAsync");
       if (!side_st_) ck(cudaStreamCreateWithFlags(&side_st_, cudaStreamNonBlocking), "cudaStreamCreate");
       for (int i = 0; i < 2; ++i) {
         if (!ev_step_[i]) ck(cudaEventCreateWithFlags(&ev_step_[i], cudaEventDisableTiming), "cudaEventCreate");
@@ -371,6 +373,21 @@ class YieldEngine {
     rows_.flag = ar_.get<int>(R);
     rows_.integral = ar_.get<double>(2 * (size_t)R);
     rows_.survival = rows_.integral + R;
+  }
+
+  // The weights of the time integral of every field, formed on the device: their
+  // low-rank factor, or (Gram kernels) the weights themselves.
+  void plan_integral(bool weights) {
+    const int nf = (int)iin_.size();
+    if (weights) {
+      d_W_ = ar_.get<double>((size_t)nf * n_c_ * n_c_ * 2);
+    } else {
+      d_L_ = ar_.get<T>((size_t)nf * n_c_ * rp::integral_ldk(n_c_));
+      d_meta_ = ar_.get<int2>(nf);
+    }
+    launched(rp::launch_plan_integral<T>(d_iin_, iin_.data(), nf, n_c_, weights ? nullptr : d_L_,
+                                         d_meta_, weights ? d_W_ : nullptr, st_),
+             "integral planning kernel");
   }
 
   // All items in one launch of k_persistent_small: CTAs take items from a
@@ -410,7 +427,7 @@ class YieldEngine {
       pev.push_back(e1);
       ck(cudaEventRecord(e0, st_), "cudaEventRecord");
     }
-    launched(rp::launch_persistent_small<T>(S_, aniso_, d_fdev_, d_coef_, d_W_, d_items, (int)n,
+    launched(rp::launch_persistent_small<T>(S_, aniso_, d_fdev_, d_coef_, d_L_, d_meta_, d_items, (int)n,
                                             d_counter_, n_c_, o_.deterministic, seed_, Xp_, pctas_,
                                             d_ps, st_),
              "persistent kernel");
@@ -502,7 +519,7 @@ class YieldEngine {
       int n_step = 0;
       if (!o_.graph || d_trace_) {
         n_step = issue(k, st_, nullptr, ev_end);
-        launches += n_step + 1;
+        launches += n_step + (d_trace_ ? 0 : 1);
       } else if (k < 2) {
         // the first macro-step of each parity runs eagerly (kernel attributes get set)
         n_step = issue(k, st_, d_macro_, ev_end);
@@ -644,27 +661,26 @@ class YieldEngine {
       ++n_step;
     }
     if (ev_steps) ck(cudaEventRecord(ev_steps, s), "cudaEventRecord");
+    cudaStream_t si = s;  // stream of the time integral
     if (overlap_) {
       ck(cudaEventRecord(ev_step_[k & 1], s), "cudaEventRecord");
       ck(cudaStreamWaitEvent(side_st_, ev_step_[k & 1], 0), "cudaStreamWaitEvent");
+      si = side_st_;
+    }
+    if (d_trace_) {
+      // a time trace reports no yields: nothing to integrate
+    } else if (tc_gram_)
       ck(rp::launch_gram_tc(reinterpret_cast<const float*>(Xk), d_W_, rows_.field, rows_.win, k,
                             mdev, R_, n_c_, Zslot_,
                             reinterpret_cast<const rp::HamDev<float>*>(d_ham_),
                             sys_.size() == 1 ? nullptr : row_sys_, n_sm_, rows_.integral, d_err_,
-                            side_st_),
-         "tensor-core time-integral kernel");
-      ck(cudaEventRecord(ev_int_[k & 1], side_st_), "cudaEventRecord");
-    } else if (tc_gram_)
-      ck(rp::launch_gram_tc(reinterpret_cast<const float*>(X_), d_W_, rows_.field, rows_.win, k,
-                            mdev, R_, n_c_, Zslot_,
-                            reinterpret_cast<const rp::HamDev<float>*>(d_ham_),
-                            sys_.size() == 1 ? nullptr : row_sys_, n_sm_, rows_.integral, d_err_,
-                            s),
+                            si),
          "tensor-core time-integral kernel");
     else
-      ck(rp::launch_gram_integrate<T>(S_, X_, d_W_, rows_.field, rows_.win, k, mdev, R_, n_c_,
-                                      rows_.integral, s),
-         "gram-integral kernel");
+      ck(rp::launch_project<T>(S_, Xk, d_L_, d_meta_, rows_.field, rows_.win, k, mdev, R_, n_c_,
+                               rows_.integral, si),
+         "time-integral kernel");
+    if (overlap_) ck(cudaEventRecord(ev_int_[k & 1], side_st_), "cudaEventRecord");
     if (mdev) ck(rp::launch_tick(mdev, s), "tick kernel");
     return n_step;
   }
@@ -735,6 +751,10 @@ class YieldEngine {
   rp::FieldDev<T>* d_fdev_ = nullptr;
   T* d_coef_ = nullptr;
   double* d_W_ = nullptr;
+  T* d_L_ = nullptr;
+  int2* d_meta_ = nullptr;
+  rp::IntegralIn* d_iin_ = nullptr;
+  std::vector<rp::IntegralIn> iin_;
   T *S0_ = nullptr, *S1_ = nullptr, *F1_ = nullptr, *F2_ = nullptr, *X_ = nullptr;
   double* amps_ = nullptr;
   rp::RowsDev rows_{};
@@ -788,7 +808,7 @@ rp_status plan_all(const rp::HostSystem& hs, int n_fields, const double* fields,
                    int n_c, double tol, std::vector<rp::FieldPlan>& plans) {
   plans.resize(n_fields);
   for (int f = 0; f < n_fields; ++f) {
-    std::string e = rp::plan_field(hs, fields[f], t_max, n_c, tol, true, &plans[f]);
+    std::string e = rp::plan_field(hs, fields[f], t_max, n_c, tol, true, &plans[f], false);
     if (!e.empty()) return fail(RP_ENOTCONV, "field " + std::to_string(f) + ": " + e);
     if (plans[f].n_macro > 2000000000LL) return fail(RP_ENOTCONV, "too many macro-steps");
   }
@@ -1678,7 +1698,7 @@ rp_status rp_plan_field(const rp_system* s, double B, double t_max, int precisio
   const int n_c = n_cheb > 0 ? n_cheb : default_ncheb(precision);
   const double tl = tol > 0 ? tol : default_tol(precision);
   rp::FieldPlan P;
-  std::string e = rp::plan_field(s->hs, B, t_max, n_c, tl, coef || W, &P);
+  std::string e = rp::plan_field(s->hs, B, t_max, n_c, tl, coef || W, &P, W != nullptr);
   if (!e.empty()) return fail(RP_ENOTCONV, e);
   plan->E_min = P.E_min;
   plan->E_max = P.E_max;

@@ -7,6 +7,8 @@
 
 #include "rp_kernels.cuh"
 #include "rp_device.cuh"
+#include "rp_project.cuh"
+#include "rp_sample.cuh"
 
 namespace rp {
 
@@ -1486,141 +1488,6 @@ __global__ void __launch_bounds__(ClusterCfg<KPT>::kNT, 1) k_macro_cluster(
   }
 }
 
-// Exact time integral of one macro-step (Eq. 20 / Eq. 22 over [t, t + h]):
-//   integral[r] += sum_nm W_nm G_nm,  G_nm = sum_z conj(x_n(z)) x_m(z),
-// where x_n = <S|phi_n> are the singlet slices stored by the step kernel.
-// Each CTA forms the partial Gram of a slice of z for 4x4 tiles (n, m), n <= m
-// (chunks of z staged z-major in shared memory; `groups` thread groups split
-// each chunk), contracts it with W of the row's field in FP64 (factor 2 for
-// n < m: W and G are Hermitian) and adds one scalar to integral[r].  Sums run
-// in T within a chunk and in a second T accumulator across chunks.
-constexpr int kGramThreads = 256;
-
-template <typename T>
-__global__ void __launch_bounds__(kGramThreads) k_gram_integrate(
-    const SysTab<T> S, const T* __restrict__ X, const double* __restrict__ W,
-    const int* __restrict__ row_field, const int2* __restrict__ row_win, int macro_arg,
-    const int* __restrict__ macro_dev, int n_c, int tiles, int groups, int zc,
-    long long z_per_cta, double* __restrict__ integral) {
-  const int r = blockIdx.y;
-  const int macro = macro_dev ? *macro_dev : macro_arg;
-  {
-    const int2 w = row_win[r];
-    if (macro < w.x || macro >= w.y) return;
-  }
-  const long long Z = S.ham[S.row_sys ? S.row_sys[r] : 0].Z;
-  const long long Zs = S.Zslot;
-  const long long z0 = (long long)blockIdx.x * z_per_cta;
-  const long long z1 = min(Z, z0 + z_per_cta);
-  if (z0 >= z1) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ldn = n_c + 2;  // row stride of the z-major tile (16-byte multiple)
-  Cx<T>* sx = reinterpret_cast<Cx<T>*>(smem_raw);  // [zc][ldn]
-  const int tid = threadIdx.x;
-  const int g = tid / tiles, t = tid % tiles;
-  const bool active = g < groups;
-  int ti = 0, tj = 0;
-  {
-    const int nt = n_c / 4;
-    int k = t;
-    for (int i = 0; i < nt; ++i) {
-      const int cnt = nt - i;
-      if (k < cnt) {
-        ti = i;
-        tj = i + k;
-        break;
-      }
-      k -= cnt;
-    }
-  }
-  T a2r[4][4], a2i[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) a2r[i][j] = a2i[i][j] = T(0);
-  const T* Xr = X + (size_t)r * n_c * Zs * 2;
-  for (long long c0 = z0; c0 < z1; c0 += zc) {
-    __syncthreads();
-    for (int idx = tid; idx < n_c * zc; idx += blockDim.x) {
-      const int nn = idx / zc, zz = idx - nn * zc;
-      const long long z = c0 + zz;
-      Cx<T> v = {T(0), T(0)};
-      if (z < z1) {
-        v.re = Xr[((size_t)nn * Zs + z) * 2];
-        v.im = Xr[((size_t)nn * Zs + z) * 2 + 1];
-      }
-      sx[zz * ldn + nn] = v;
-    }
-    __syncthreads();
-    if (active) {
-      T pr[4][4], pi[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) pr[i][j] = pi[i][j] = T(0);
-      for (int zz = g; zz < zc; zz += groups) {
-        const Cx<T>* row = sx + zz * ldn;
-        Cx<T> xi[4], xj[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          xi[i] = row[4 * ti + i];
-          xj[i] = row[4 * tj + i];
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            pr[i][j] = fma(xi[i].re, xj[j].re, fma(xi[i].im, xj[j].im, pr[i][j]));
-            pi[i][j] = fma(xi[i].re, xj[j].im, fma(-xi[i].im, xj[j].re, pi[i][j]));
-          }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          a2r[i][j] += pr[i][j];
-          a2i[i][j] += pi[i][j];
-        }
-    }
-  }
-  // combine the thread groups of each tile through shared memory
-  __syncthreads();
-  T* red = reinterpret_cast<T*>(smem_raw);  // [groups][tiles][32]
-  if (active && groups > 1) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        red[((size_t)g * tiles + t) * 32 + 2 * (4 * i + j)] = a2r[i][j];
-        red[((size_t)g * tiles + t) * 32 + 2 * (4 * i + j) + 1] = a2i[i][j];
-      }
-  }
-  __syncthreads();
-  double s = 0.0;
-  if (active && g == 0) {
-    const double* Wf = W + (size_t)row_field[r] * n_c * n_c * 2;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int nn = 4 * ti + i, mm = 4 * tj + j;
-        if (nn > mm) continue;
-        double gr = (double)a2r[i][j], gi = (double)a2i[i][j];
-        for (int q = 1; q < groups; ++q) {
-          gr += (double)red[((size_t)q * tiles + t) * 32 + 2 * (4 * i + j)];
-          gi += (double)red[((size_t)q * tiles + t) * 32 + 2 * (4 * i + j) + 1];
-        }
-        const size_t w = ((size_t)nn * n_c + mm) * 2;
-        const double v = Wf[w] * gr - Wf[w + 1] * gi;
-        s += (nn == mm) ? v : 2.0 * v;
-      }
-  }
-  __syncthreads();
-  double* sh = reinterpret_cast<double*>(smem_raw);
-  const double tot = block_sum<kGramThreads>(s, sh);
-  if (tid == 0) atomicAdd(integral + r, tot);
-}
-
 // Time-resolved observables (Eq. 18 for A = P_S, A = 1 and an electron
 // operator A_e): after macro-step k, every row active in it holds psi(t_i),
 // i = k + 1 - start, in Q; adds |<S|psi>|^2 (P_S = |S><S| on the electrons,
@@ -1795,60 +1662,6 @@ __global__ void __launch_bounds__(256) k_stats_weighted(const double* __restrict
   }
 }
 
-// ---- Philox4x32-10 (Salmon et al., SC'11) and coherent states (Eq. 15) ----
-
-__device__ __forceinline__ void philox4x32_10(uint32_t (&c)[4], uint32_t k0, uint32_t k1) {
-  const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
-  const uint32_t W0 = 0x9E3779B9u, W1 = 0xBB67AE85u;
-#pragma unroll
-  for (int r = 0; r < 10; ++r) {
-    if (r > 0) {
-      k0 += W0;
-      k1 += W1;
-    }
-    const uint32_t lo0 = M0 * c[0], hi0 = __umulhi(M0, c[0]);
-    const uint32_t lo1 = M1 * c[2], hi1 = __umulhi(M1, c[2]);
-    const uint32_t n0 = hi1 ^ c[1] ^ k0, n2 = hi0 ^ c[3] ^ k1;
-    c[0] = n0;
-    c[1] = lo1;
-    c[2] = n2;
-    c[3] = lo0;
-  }
-}
-
-__device__ __forceinline__ double u53(uint32_t hi, uint32_t lo) {
-  return ((double)(hi >> 5) * 67108864.0 + (double)(lo >> 6)) * (1.0 / 9007199254740992.0);
-}
-
-// Components c_j (o[2 j], o[2 j + 1], j = 0 .. 2I) of the coherent state of the
-// nucleus at layout position p for sample s: Philox draw of the direction
-// (counter (input index, s_lo, s_hi, pair), key seed; cos theta = 1 - 2 u1,
-// phi = 2 pi u2, Eq. 17) and c_j = sqrt(C(2I, j)) cos^{2I-j}(theta/2)
-// sin^j(theta/2) e^{i j phi} (Eq. 15); u receives (u1, u2).
-__device__ __forceinline__ void coherent_amp(const LayoutDev& L, int p, uint32_t pair,
-                                             unsigned long long s, uint64_t seed, double* o,
-                                             double* u) {
-  const int k = L.input_index[p];
-  uint32_t c[4] = {(uint32_t)k, (uint32_t)(s & 0xFFFFFFFFull), (uint32_t)(s >> 32), pair};
-  philox4x32_10(c, (uint32_t)(seed & 0xFFFFFFFFull), (uint32_t)(seed >> 32));
-  const double u1 = u53(c[0], c[1]), u2 = u53(c[2], c[3]);
-  u[0] = u1;
-  u[1] = u2;
-  const double ch = sqrt(1.0 - u1), sh = sqrt(u1);  // cos(theta/2), sin(theta/2)
-  const int d = L.d[p], twoI = d - 1;
-  double binom = 1.0;  // C(2I, j)
-  for (int j = 0; j < d; ++j) {
-    if (j > 0) binom = binom * (double)(twoI - j + 1) / (double)j;
-    double mag = sqrt(binom);
-    for (int i = 0; i < twoI - j; ++i) mag *= ch;
-    for (int i = 0; i < j; ++i) mag *= sh;
-    double sn, cs;
-    sincospi(2.0 * (double)j * u2, &sn, &cs);
-    o[2 * j] = mag * cs;
-    o[2 * j + 1] = mag * sn;
-  }
-}
-
 // One thread per (row, nucleus position): Philox draw of the direction
 // (cos theta = 1 - 2 u1, phi = 2 pi u2; uniform on the sphere, Eq. 17) and the
 // coherent-state components c_j = sqrt(C(2I, j)) cos^{2I-j}(theta/2)
@@ -1938,18 +1751,19 @@ __global__ void __launch_bounds__(256) k_init_state(const SysTab<T> S,
 // phi_S = k_S integral, phi_T = 1 - survival - phi_S into the per-sample
 // output.  Items are independent, so no CTA waits for another.
 constexpr int kPersistThreads = 256;
-constexpr int kPersistGramZc = 32;  // configurations per staged Gram chunk
 
 template <typename T>
 size_t persist_smem_bytes(long long Zs, int n_c) {
-  const int zc = sizeof(T) == 4 ? kPersistGramZc : kPersistGramZc / 2;
-  return (size_t)3 * 4 * Zs * sizeof(Cx<T>) + (size_t)zc * (n_c + 2) * sizeof(Cx<T>);
+  // the ring of the integral shares the phi_n buffer where that is large enough
+  const size_t ring = proj_ring_bytes<T>(kPersistThreads, 1), buf = (size_t)4 * Zs * sizeof(Cx<T>);
+  return 3 * buf + (size_t)n_c * ProjCfg<T>::kB * sizeof(T) + (buf >= ring ? 0 : ring);
 }
 
 template <typename T, bool ANISO>
 __global__ void __launch_bounds__(kPersistThreads) k_persistent_small(
     const SysTab<T> S, const FieldDev<T>* __restrict__ fields, const T* __restrict__ coef,
-    const double* __restrict__ W, const PItem* __restrict__ items, int n_items,
+    const T* __restrict__ L, int ldk, const int2* __restrict__ meta,
+    const PItem* __restrict__ items, int n_items,
     int* __restrict__ counter, int n_c, int deterministic, uint64_t seed,
     T* __restrict__ Xscratch, double* __restrict__ per_sample) {
   extern __shared__ __align__(16) unsigned char psmem[];
@@ -1958,32 +1772,15 @@ __global__ void __launch_bounds__(kPersistThreads) k_persistent_small(
   __shared__ double red[kPersistThreads];
   __shared__ int s_item;
   const int Zs = (int)S.Zslot;
-  const int zc = sizeof(T) == 4 ? kPersistGramZc : kPersistGramZc / 2;
-  const int ldn = n_c + 2;
   Cx<T>* buf0 = reinterpret_cast<Cx<T>*>(psmem);
   Cx<T>* buf1 = buf0 + (size_t)4 * Zs;
   Cx<T>* buf2 = buf1 + (size_t)4 * Zs;
-  Cx<T>* sx = buf2 + (size_t)4 * Zs;  // Gram staging [zc][ldn]
+  T* sl = reinterpret_cast<T*>(buf2 + (size_t)4 * Zs);  // integral factor [n_c][KB]
+  const bool own_ring = (size_t)4 * Zs * sizeof(Cx<T>) < proj_ring_bytes<T>(kPersistThreads, 1);
+  auto* ring = (own_ring ? reinterpret_cast<typename SliceVal<T>::type*>(sl + (size_t)n_c * ProjCfg<T>::kB)
+                         : reinterpret_cast<typename SliceVal<T>::type*>(buf1)) + threadIdx.x;
   T* xr = Xscratch + (size_t)blockIdx.x * n_c * Zs * 2;
   const int tid = threadIdx.x;
-  // the 4 x 4 tile (ti, tj), ti <= tj, of the Gram this thread sums
-  const int nt = n_c / 4, tiles = nt * (nt + 1) / 2;
-  int ti = 0, tj = 0;
-  {
-    int q = tid % (tiles > 0 ? tiles : 1);
-    for (int i = 0; i < nt; ++i) {
-      const int cnt = nt - i;
-      if (q < cnt) {
-        ti = i;
-        tj = i + q;
-        break;
-      }
-      q -= cnt;
-    }
-  }
-  const int groups = tiles >= kPersistThreads ? 1 : kPersistThreads / tiles;
-  const int g = tid / (tiles > 0 ? tiles : 1);
-  const bool tile_on = tid < tiles * groups;
   for (;;) {
     if (tid == 0) s_item = atomicAdd(counter, 1);
     __syncthreads();
@@ -1995,11 +1792,11 @@ __global__ void __launch_bounds__(kPersistThreads) k_persistent_small(
       int4* dst = reinterpret_cast<int4*>(&Hs);
       for (int i = tid; i < (int)(sizeof(HamDev<T>) / 16); i += blockDim.x) dst[i] = src[i];
     }
-    const LayoutDev& L = S.lay[I.sys];
-    if (!deterministic && tid < L.n_nuc) {
+    const LayoutDev& Ly = S.lay[I.sys];
+    if (!deterministic && tid < Ly.n_nuc) {
       double u[2];
       const uint32_t pair = S.pair_of ? S.pair_of[I.sys] : S.pair_base + (uint32_t)I.sys;
-      coherent_amp(L, tid, pair, (unsigned long long)I.sample, seed, amps + tid * 20, u);
+      coherent_amp(Ly, tid, pair, (unsigned long long)I.sample, seed, amps + tid * 20, u);
     }
     __syncthreads();
     const int Z = (int)Hs.Z;
@@ -2013,8 +1810,8 @@ __global__ void __launch_bounds__(kPersistThreads) k_persistent_small(
         pr = (m == I.sample) ? 1.0 : 0.0;
       } else {
         int q = m;
-        for (int p = 0; p < L.n_nuc; ++p) {
-          const int d = L.d[p];
+        for (int p = 0; p < Ly.n_nuc; ++p) {
+          const int d = Ly.d[p];
           const int j = q % d;
           q /= d;
           const double ar = amps[(p * 10 + j) * 2], ai = amps[(p * 10 + j) * 2 + 1];
@@ -2035,8 +1832,10 @@ __global__ void __launch_bounds__(kPersistThreads) k_persistent_small(
     const FieldDev<T> F = fields[I.field];
     const T* cf = coef + (size_t)I.field * n_c * 4;
     const T* cl = cf + 2 * n_c;
-    const double* Wf = W + (size_t)I.field * n_c * n_c * 2;
-    double integral = 0.0;  // thread 0
+    const T* Lf = L + (size_t)I.field * n_c * ldk;
+    const int2 mt = meta[I.field];  // rank, terms
+    const int n_e = (mt.y + 1) & ~1;
+    double integral = 0.0;  // this thread's configurations
     for (int km = 0; km < I.n_macro; ++km) {
       // ---- one macro-step: psi(t) in P, psi(t + h) into A, phi_n in P / B ----
       {
@@ -2089,74 +1888,17 @@ __global__ void __launch_bounds__(kPersistThreads) k_persistent_small(
           __syncthreads();
         }
       }
-      // ---- exact time integral of the step: Re sum_nm W_nm G_nm ----
-      {
-        // sums in T within a chunk (pr_, pi_) and in a second T accumulator
-        // across chunks (ar_, ai_), as in k_gram_integrate
-        T ar_[4][4], ai_[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) ar_[i][j] = ai_[i][j] = T(0);
-        for (int c0 = 0; c0 < Z; c0 += zc) {
-          for (int idx = tid; idx < n_c * zc; idx += blockDim.x) {
-            const int nn = idx / zc, zz = idx - nn * zc;
-            const int z = c0 + zz;
-            Cx<T> v = {T(0), T(0)};
-            if (z < Z) {
-              v.re = xr[((size_t)nn * Zs + z) * 2];
-              v.im = xr[((size_t)nn * Zs + z) * 2 + 1];
-            }
-            sx[zz * ldn + nn] = v;
-          }
-          __syncthreads();
-          if (tile_on) {
-            T pr_[4][4], pi_[4][4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) pr_[i][j] = pi_[i][j] = T(0);
-            for (int zz = g; zz < zc; zz += groups) {
-              const Cx<T>* row = sx + zz * ldn;
-              Cx<T> xi[4], xj[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                xi[i] = row[4 * ti + i];
-                xj[i] = row[4 * tj + i];
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  pr_[i][j] = fma(xi[i].re, xj[j].re, fma(xi[i].im, xj[j].im, pr_[i][j]));
-                  pi_[i][j] = fma(xi[i].re, xj[j].im, fma(-xi[i].im, xj[j].re, pi_[i][j]));
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                ar_[i][j] += pr_[i][j];
-                ai_[i][j] += pi_[i][j];
-              }
-          }
-          __syncthreads();
+      // ---- exact time integral of the step (see rp_integral.cu) ----
+      for (int k0 = 0; k0 < mt.x; k0 += ProjCfg<T>::kB) {
+        stage_factor<T>(sl, Lf, ldk, n_e, k0, tid, kPersistThreads);
+        __syncthreads();
+        for (int m = tid; m < Z; m += blockDim.x) {
+          typename ProjAcc<T>::type yr[1][16], yi[1][16];
+          const T* const p[1] = {xr + (size_t)m * 2};
+          project_block<T, 1>(yr, yi, p, (size_t)Zs * 2, sl, ProjCfg<T>::kB, n_e, ring,
+                              kPersistThreads);
+          integral += proj_norm(yr[0], yi[0]);
         }
-        double sum = 0.0;
-        if (tile_on) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int nn = 4 * ti + i, mm = 4 * tj + j;
-              if (nn > mm) continue;
-              const size_t w = ((size_t)nn * n_c + mm) * 2;
-              const double v = Wf[w] * (double)ar_[i][j] - Wf[w + 1] * (double)ai_[i][j];
-              sum += (nn == mm) ? v : 2.0 * v;
-            }
-        }
-        const double tot = block_sum<kPersistThreads>(sum, red);
-        if (tid == 0) integral += tot;
         __syncthreads();
       }
       // psi(t + h) is phi_0 of the next step
@@ -2173,8 +1915,10 @@ __global__ void __launch_bounds__(kPersistThreads) k_persistent_small(
         nn += (double)a[e].re * (double)a[e].re + (double)a[e].im * (double)a[e].im;
     }
     const double surv = block_sum<kPersistThreads>(nn, red);
+    __syncthreads();
+    const double tot = block_sum<kPersistThreads>(integral, red);
     if (tid == 0) {
-      const double phS = S.k_S[I.sys] * integral;
+      const double phS = S.k_S[I.sys] * tot;
       per_sample[I.out * 3] = phS;
       per_sample[I.out * 3 + 1] = 1.0 - surv - phS;
       per_sample[I.out * 3 + 2] = surv;
@@ -2512,45 +2256,17 @@ int persistent_ctas(long long Zs, int n_c, int aniso) {
 
 template <typename T>
 cudaError_t launch_persistent_small(const SysTab<T>& S, int aniso, const FieldDev<T>* fields,
-                                    const T* coef, const double* W, const PItem* items,
-                                    int n_items, int* counter, int n_c, int deterministic,
+                                    const T* coef, const T* L, const int2* meta,
+                                    const PItem* items, int n_items, int* counter, int n_c, int deterministic,
                                     uint64_t seed, T* Xscratch, int ctas, double* per_sample,
                                     cudaStream_t st) {
   if (n_items == 0 || ctas == 0) return cudaSuccess;
   if (S.Zslot > SmallCfg<T>::kMax) return cudaErrorInvalidValue;
-  if (n_c % 4 != 0 || n_c > 88) return cudaErrorInvalidValue;  // <= 253 Gram tiles
   const size_t smem = persist_smem_bytes<T>(S.Zslot, n_c);
   auto kf = aniso ? k_persistent_small<T, true> : k_persistent_small<T, false>;
   // the shared-memory attribute was set by persistent_ctas, which gave `ctas`
-  kf<<<ctas, kPersistThreads, smem, st>>>(S, fields, coef, W, items, n_items, counter, n_c,
+  kf<<<ctas, kPersistThreads, smem, st>>>(S, fields, coef, L, integral_ldk(n_c), meta, items, n_items, counter, n_c,
                                           deterministic, seed, Xscratch, per_sample);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_gram_integrate(const SysTab<T>& S, const T* X, const double* W,
-                                  const int* row_field, const int2* row_win, int macro,
-                                  const int* macro_dev, int rows, int n_c, double* integral,
-                                  cudaStream_t st) {
-  if (rows == 0) return cudaSuccess;
-  const int nt = n_c / 4;
-  const int tiles = nt * (nt + 1) / 2;
-  const int groups = tiles >= kGramThreads ? 1 : kGramThreads / tiles;
-  const int zc = sizeof(T) == 4 ? 32 : 16;
-  const long long z_per_cta = 1024;
-  const size_t tile_b = (size_t)zc * (n_c + 2) * sizeof(Cx<T>);
-  const size_t red_b = (size_t)groups * tiles * 32 * sizeof(T);
-  size_t smem = tile_b > red_b ? tile_b : red_b;
-  if (smem < kGramThreads * sizeof(double)) smem = kGramThreads * sizeof(double);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_gram_integrate<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  dim3 grid((unsigned)((S.Zslot + z_per_cta - 1) / z_per_cta), rows);
-  k_gram_integrate<T><<<grid, kGramThreads, smem, st>>>(S, X, W, row_field, row_win, macro,
-                                                        macro_dev, n_c, tiles, groups, zc,
-                                                        z_per_cta, integral);
   return cudaGetLastError();
 }
 
@@ -2619,14 +2335,11 @@ template cudaError_t launch_step<float>(const SysTab<float>&, const HamDev<float
                                         const FieldDev<float>*, const int*, const int2*, int,
                                         const int*, int, const float*, const float*, float*, float*, float*,
                                         const float*, int, int, int, int, cudaStream_t);
-template cudaError_t launch_gram_integrate<float>(const SysTab<float>&, const float*, const double*,
-                                                  const int*, const int2*, int, const int*, int,
-                                                  int, double*, cudaStream_t);
 template int small_max_configs<float>();
 template size_t persistent_smem<float>(long long, int);
 template int persistent_ctas<float>(long long, int, int);
 template cudaError_t launch_persistent_small<float>(const SysTab<float>&, int, const FieldDev<float>*,
-                                                    const float*, const double*, const PItem*, int,
+                                                    const float*, const float*, const int2*, const PItem*, int,
                                                     int*, int, int, uint64_t, float*, int, double*,
                                                     cudaStream_t);
 template cudaError_t launch_macro_small<float>(const SysTab<float>&, const HamDev<float>*, int,
@@ -2648,14 +2361,11 @@ template cudaError_t launch_step<double>(const SysTab<double>&, const HamDev<dou
                                         const FieldDev<double>*, const int*, const int2*, int,
                                         const int*, int, const double*, const double*, double*, double*, double*,
                                         const double*, int, int, int, int, cudaStream_t);
-template cudaError_t launch_gram_integrate<double>(const SysTab<double>&, const double*, const double*,
-                                                  const int*, const int2*, int, const int*, int,
-                                                  int, double*, cudaStream_t);
 template int small_max_configs<double>();
 template size_t persistent_smem<double>(long long, int);
 template int persistent_ctas<double>(long long, int, int);
 template cudaError_t launch_persistent_small<double>(const SysTab<double>&, int, const FieldDev<double>*,
-                                                     const double*, const double*, const PItem*, int,
+                                                     const double*, const double*, const int2*, const PItem*, int,
                                                      int*, int, int, uint64_t, double*, int, double*,
                                                      cudaStream_t);
 template cudaError_t launch_macro_small<double>(const SysTab<double>&, const HamDev<double>*, int,

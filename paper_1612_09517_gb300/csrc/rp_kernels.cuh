@@ -158,8 +158,8 @@ template <typename T>
 int persistent_ctas(long long Zs, int n_c, int aniso);
 template <typename T>
 cudaError_t launch_persistent_small(const SysTab<T>& S, int aniso, const FieldDev<T>* fields,
-                                    const T* coef, const double* W, const PItem* items,
-                                    int n_items, int* counter, int n_c, int deterministic,
+                                    const T* coef, const T* L, const int2* meta,
+                                    const PItem* items, int n_items, int* counter, int n_c, int deterministic,
                                     uint64_t seed, T* Xscratch, int ctas, double* per_sample,
                                     cudaStream_t st);
 
@@ -189,13 +189,29 @@ cudaError_t launch_macro_cluster(const HamDev<float>& H, const FieldDev<float>* 
                                  float* X, const float* coef, int n_c, long long Zslot, int xblk,
                                  cudaStream_t st);
 
-// integral[r] += sum_nm W_nm <x_n|x_m> for the macro-step just finished
-// (x_n = singlet slices X[r][n], W per field); one FP64 atomic per CTA.
+// One field's time integral: Chebyshev half-width and macro-step length, and
+// the decay rate (k_S + k_T)/2 factored out of the propagator.
+struct IntegralIn {
+  double dE, h, kbar;
+};
+
+// Low-rank factor of the time-integral weights of every field (see
+// k_plan_integral): L[f][n][k], n < n_c, k < integral_ldk(n_c) (zero past the
+// rank), meta[f] = (rank, leading terms that count), and, if W is not NULL, the
+// complex weights W[f][n][m] themselves (L may be NULL then).  host_in: the
+// same records on the host (they size the launch).
+int integral_ldk(int n_c);
 template <typename T>
-cudaError_t launch_gram_integrate(const SysTab<T>& S, const T* X, const double* W,
-                                  const int* row_field, const int2* row_win, int macro,
-                                  const int* macro_dev, int rows, int n_c, double* integral,
-                                  cudaStream_t st);
+cudaError_t launch_plan_integral(const IntegralIn* in, const IntegralIn* host_in, int n_fields,
+                                 int n_c, T* L, int2* meta, double* W, cudaStream_t st);
+
+// integral[r] += sum_z sum_k |sum_n L_nk (-i)^n x_n(z)|^2 for the macro-step
+// just finished (x_n = singlet slices X[r][n]); one FP64 atomic per CTA.
+template <typename T>
+cudaError_t launch_project(const SysTab<T>& S, const T* X, const T* L, const int2* meta,
+                           const int* row_field, const int2* row_win, int macro,
+                           const int* macro_dev, int rows, int n_c, double* integral,
+                           cudaStream_t st);
 
 // The same time integral on the tensor cores (FP32 singlet slices written by
 // launch_step with xblk = 1; tcgen05.mma kind::tf32 with a hi/lo split of

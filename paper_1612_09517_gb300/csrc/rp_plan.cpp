@@ -18,7 +18,7 @@ void bessel_jn(double x, int nmax, double* out) {
   const int big = std::max(nmax, static_cast<int>(x));
   int m = big + 32 + static_cast<int>(std::sqrt(40.0 * (big + 1)));
   m += (m & 1);  // start from an even order
-  std::vector<double> v(nmax + 1, 0.0);
+  double* v = out;
   double jp1 = 0.0;  // J_{n+1}
   double jn = 1e-30; // J_n, arbitrary seed at n = m
   double norm = 2.0 * jn;  // m is even and > 0
@@ -37,7 +37,7 @@ void bessel_jn(double x, int nmax, double* out) {
       for (int i = k; i <= nmax; ++i) v[i] *= 1e-200;
     }
   }
-  for (int k = 0; k <= nmax; ++k) out[k] = v[k] / norm;
+  for (int k = 0; k <= nmax; ++k) out[k] /= norm;
 }
 
 void gauss_legendre(int q, double* x, double* w) {
@@ -222,9 +222,9 @@ double ellipse_rho(double delta) {
 }
 
 double tail_bound(double x, int n_c, double rho, double crouzeix) {
-  const int extra = 120;
-  std::vector<double> J(n_c + extra + 1);
-  bessel_jn(x, n_c + extra, J.data());
+  constexpr int extra = 120;
+  double J[256 + extra + 1];
+  bessel_jn(x, n_c + extra, J);
   double t = 0.0, rp = std::pow(rho, n_c);
   for (int n = n_c; n <= n_c + extra; ++n) {
     t += 2.0 * std::fabs(J[n]) * rp;
@@ -233,10 +233,51 @@ double tail_bound(double x, int n_c, double rho, double crouzeix) {
   return crouzeix * t;
 }
 
+// Largest x = dE h with tail_bound <= tol.  log(tail) is close to linear in
+// log(x) near the bound, so a bracketing secant (Illinois) ends in about ten
+// evaluations; a bisection to the last bit took a hundred (0.17 ms per field).
+double largest_x(int n_c, double rho, double crz, double tol) {
+  auto g = [&](double x) {
+    return std::log(std::max(tail_bound(x, n_c, rho, crz), 1e-300) / tol);
+  };
+  double lo = 1.0, hi = static_cast<double>(n_c);
+  double glo = g(lo), ghi = g(hi);
+  if (ghi <= 0.0) return hi;
+  if (!(glo <= 0.0)) {  // a loose step: the bound is met only below x = 1
+    for (int it = 0; it < 200 && !(glo <= 0.0); ++it) {
+      hi = lo;
+      ghi = glo;
+      lo *= 0.5;
+      glo = g(lo);
+    }
+  }
+  int side = 0;
+  for (int it = 0; it < 100; ++it) {
+    if (hi - lo <= 4e-16 * hi) break;
+    double x = lo * std::pow(hi / lo, glo / (glo - ghi));
+    if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
+    if (!(x > lo && x < hi)) break;
+    const double gx = g(x);
+    if (gx <= 0.0) {
+      if (hi - x <= 1e-14 * hi || -gx < 1e-12) return x;
+      lo = x;
+      glo = gx;
+      if (side == -1) ghi *= 0.5;
+      side = -1;
+    } else {
+      hi = x;
+      ghi = gx;
+      if (side == 1) glo *= 0.5;
+      side = 1;
+    }
+  }
+  return lo;
+}
+
 }  // namespace
 
 std::string plan_field(const HostSystem& s, double B_mT, double t_max, int n_c, double tol,
-                       bool want_coef, FieldPlan* out) {
+                       bool want_coef, FieldPlan* out, bool want_W) {
   if (n_c < 8 || n_c > 256) return "n_cheb must be in [8, 256]";
   if (!(tol > 0.0 && tol < 1e-2)) return "tol must be in (0, 1e-2)";
   if (!(t_max > 0.0) || !std::isfinite(t_max)) return "t_max must be positive and finite";
@@ -264,13 +305,8 @@ std::string plan_field(const HostSystem& s, double B_mT, double t_max, int n_c, 
   const double rho = ellipse_rho(delta);
   const double crz = delta > 0.0 ? 1.0 + std::sqrt(2.0) : 1.0;  // Crouzeix's constant
   // largest x = dE h with the truncation bound below tol
-  double xl = 0.0, xh = static_cast<double>(n_c);
   if (tail_bound(1e-6, n_c, rho, crz) > tol) return "tolerance unreachable with this n_cheb";
-  for (int it = 0; it < 100; ++it) {
-    const double xm = 0.5 * (xl + xh);
-    if (tail_bound(xm, n_c, rho, crz) <= tol) xl = xm;
-    else xh = xm;
-  }
+  const double xl = largest_x(n_c, rho, crz, tol);
   const double h_max = xl / P.dE;
   const double nm = std::ceil(t_max / h_max);
   if (!(nm >= 1.0) || nm > 4e9) return "too many macro-steps for t_max";
@@ -290,6 +326,7 @@ std::string plan_field(const HostSystem& s, double B_mT, double t_max, int n_c, 
     P.coef[n] = phase * ipow * ((n == 0 ? 1.0 : 2.0) * J[n]);
     ipow *= mi;
   }
+  if (!want_W) return "";
   // W_nm = eps_n eps_m i^(n-m) int_0^h exp(-kbar tau) J_n(dE tau) J_m(dE tau) dtau
   const int q = n_c + static_cast<int>(std::ceil(x)) + 48;
   std::vector<double> gx(q), gw(q), Jq((size_t)q * (n_c + 1));

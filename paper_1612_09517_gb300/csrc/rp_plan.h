@@ -69,8 +69,10 @@ struct FieldPlan {
 std::string finish_system(HostSystem& s);
 
 // Plan one field.  Returns an empty string on success or an error message.
+// want_coef fills coef; want_W also fills W (the entry points that integrate on
+// the device leave it out: launch_plan_integral forms the weights there).
 std::string plan_field(const HostSystem& s, double B_mT, double t_max, int n_cheb, double tol,
-                       bool want_coef, FieldPlan* out);
+                       bool want_coef, FieldPlan* out, bool want_W = true);
 
 // Nuclear basis index of sample `sample` for basis-state sampling (Eq. 14
 // sampled instead of summed): Philox4x32-10 (Salmon et al., SC'11) with

@@ -165,7 +165,7 @@ rp_status run_static(const rp::HostSystem& hs, int n_fields, const double* field
   const long long Z = hs.Z;
   std::vector<rp::FieldPlan> plans(n_fields);
   for (int f = 0; f < n_fields; ++f) {
-    std::string e = rp::plan_field(hs, fields[f], t_max, n_c, tol, true, &plans[f]);
+    std::string e = rp::plan_field(hs, fields[f], t_max, n_c, tol, true, &plans[f], false);
     if (!e.empty()) return sfail(RP_ENOTCONV, "field " + std::to_string(f) + ": " + e);
   }
   std::vector<int> forder(n_fields);
@@ -201,7 +201,12 @@ rp_status run_static(const rp::HostSystem& hs, int n_fields, const double* field
   long long* d_offcnt = b.get<long long>(2 * (size_t)n_fields);
   auto* d_fdev = b.get<rp::FieldDev<T>>(n_fields);
   T* d_coef = b.get<T>((size_t)n_fields * n_c * 4);
-  double* d_W = b.get<double>((size_t)n_fields * n_c * n_c * 2);
+  // factor of the integral weights: inside the n_c x n_c complex weights that
+  // the budget above counts
+  unsigned char* d_wts = b.get<unsigned char>((size_t)n_fields * n_c * n_c * 2 * sizeof(double));
+  T* d_L = reinterpret_cast<T*>(d_wts);
+  auto* d_iin = reinterpret_cast<rp::IntegralIn*>(d_L + (size_t)n_fields * n_c * rp::integral_ldk(n_c));
+  auto* d_meta = reinterpret_cast<int2*>(d_iin + n_fields);
   T* S0 = b.get<T>(R * vec);
   T* S1 = b.get<T>(R * vec);
   T* F1 = b.get<T>(R * vec);
@@ -217,7 +222,7 @@ rp_status run_static(const rp::HostSystem& hs, int n_fields, const double* field
 
   std::vector<rp::FieldDev<T>> fdev(n_fields);
   std::vector<T> coef((size_t)n_fields * n_c * 4, T(0));  // c_n, then (FP32) c_n - fl(c_n)
-  std::vector<double> W((size_t)n_fields * n_c * n_c * 2);
+  std::vector<rp::IntegralIn> iin(n_fields);
   for (int f = 0; f < n_fields; ++f) {
     const rp::FieldPlan& P = plans[f];
     fdev[f].omega = (T)P.omega;
@@ -234,10 +239,7 @@ rp_status run_static(const rp::HostSystem& hs, int n_fields, const double* field
         cf[2 * n_c + 2 * n + 1] = (T)(P.coef[n].imag() - (double)im);
       }
     }
-    for (size_t i = 0; i < (size_t)n_c * n_c; ++i) {
-      W[((size_t)f * n_c * n_c + i) * 2] = P.W[i].real();
-      W[((size_t)f * n_c * n_c + i) * 2 + 1] = P.W[i].imag();
-    }
+    iin[f] = rp::IntegralIn{P.dE, P.h, P.kbar};
   }
   long long launches = 0, steps = 0, row_terms = 0, h2d = 0, d2h = 0;
   auto L1 = [&](cudaError_t e, const char* w) {
@@ -246,8 +248,10 @@ rp_status run_static(const rp::HostSystem& hs, int n_fields, const double* field
   };
   sck(cudaMemcpyAsync(d_fdev, fdev.data(), fdev.size() * sizeof(fdev[0]), cudaMemcpyHostToDevice, st), "h2d");
   sck(cudaMemcpyAsync(d_coef, coef.data(), coef.size() * sizeof(T), cudaMemcpyHostToDevice, st), "h2d");
-  sck(cudaMemcpyAsync(d_W, W.data(), W.size() * sizeof(double), cudaMemcpyHostToDevice, st), "h2d");
-  h2d += (long long)(fdev.size() * sizeof(fdev[0]) + coef.size() * sizeof(T) + W.size() * sizeof(double));
+  sck(cudaMemcpyAsync(d_iin, iin.data(), iin.size() * sizeof(iin[0]), cudaMemcpyHostToDevice, st), "h2d");
+  h2d += (long long)(fdev.size() * sizeof(fdev[0]) + coef.size() * sizeof(T) + iin.size() * sizeof(iin[0]));
+  L1(rp::launch_plan_integral<T>(d_iin, iin.data(), n_fields, n_c, d_L, d_meta, nullptr, st),
+     "integral planning kernel");
 
   const rp::HamDev<T> H = ham_of<T>(hs);
   const rp::LayoutDev L = layout_of(hs);
@@ -306,9 +310,9 @@ rp_status run_static(const rp::HostSystem& hs, int n_fields, const double* field
         steps++;
       }
       row_terms += act * n_c;
-      L1(rp::launch_gram_integrate<T>(SYS, X, d_W, d_field, d_win, (int)k, nullptr, rows, n_c,
-                                      d_int, st),
-         "gram-integral kernel");
+      L1(rp::launch_project<T>(SYS, X, d_L, d_meta, d_field, d_win, (int)k, nullptr, rows, n_c,
+                               d_int, st),
+         "time-integral kernel");
     }
     L1(rp::launch_norm<T>(SYS, S0, S1, d_win, nullptr, rows, d_surv, st), "norm kernel");
     rp::RowsDev RD{d_field, d_win, d_sample, d_out, nullptr, d_int, d_surv};
