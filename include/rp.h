@@ -147,7 +147,8 @@ typedef struct rp_stats {
   double step_ms;               /* CUDA-event time of the timed step launches (profile=1) */
   long long step_launches_timed;/* step launches inside the timed intervals */
   double device_ms;             /* CUDA-event time of the whole call on its stream */
-  int rows;                     /* concurrent propagations used */
+  int rows;                     /* concurrent propagations used (kernel 5: CTAs in flight,
+                                   each of one or more propagations of one field) */
   int n_cheb;                   /* Chebyshev terms per macro-step used */
   long long h2d_bytes;          /* host-to-device bytes copied by the call */
   long long d2h_bytes;          /* device-to-host bytes copied by the call */

@@ -166,7 +166,8 @@ int default_kernel_fp32(const HostSystem& hs, bool* cluster_ok) {
   const HamDev<float> hf = make_ham<float>(hs);
   const bool ok = macro_cluster_plan(hf, nullptr);
   if (cluster_ok) *cluster_ok = ok;
-  if (hs.Z <= small_max_configs<float>()) return persistent_default(hs.Z, 1) ? 5 : 2;
+  if (hs.Z <= small_max_configs<float>())
+    return persistent_default(hs.Z, 1) || !hs.aniso ? 5 : 2;
   return macro_cluster_default(hf) ? 4 : 1;
 }
 
@@ -207,12 +208,16 @@ class YieldEngine {
       : sys_(systems), o_(o), n_c_(n_c), st_(st), ar_(ar) {
     const int ns = (int)systems.size();
     std::vector<rp::HamDev<T>> ham(ns);
+    std::vector<rp::HamDev<double>> hamd(ns);
     std::vector<rp::LayoutDev> lay(ns);
     std::vector<double> kS(ns);
     Zslot_ = 1;
     ham1_ = make_ham<T>(*systems[0]);
     for (int i = 0; i < ns; ++i) {
       ham[i] = make_ham<T>(*systems[i]);
+      hamd[i] = make_ham<double>(*systems[i]);
+      min_half_ = std::min(min_half_, systems[i]->n_half);
+      max_nuc_ = std::max(max_nuc_, systems[i]->n_nuc);
       lay[i] = make_layout(*systems[i]);
       kS[i] = systems[i]->k_S;
       Zslot_ = std::max<long long>(Zslot_, systems[i]->Z);
@@ -221,10 +226,12 @@ class YieldEngine {
     d_ham_ = ar_.get<rp::HamDev<T>>(ns);
     d_lay_ = ar_.get<rp::LayoutDev>(ns);
     d_kS_ = ar_.get<double>(ns);
+    d_hamd_ = ar_.get<rp::HamDev<double>>(ns);
     ck(cudaMemcpyAsync(d_ham_, ham.data(), ns * sizeof(ham[0]), cudaMemcpyHostToDevice, st_), "h2d systems");
+    ck(cudaMemcpyAsync(d_hamd_, hamd.data(), ns * sizeof(hamd[0]), cudaMemcpyHostToDevice, st_), "h2d systems");
     ck(cudaMemcpyAsync(d_lay_, lay.data(), ns * sizeof(lay[0]), cudaMemcpyHostToDevice, st_), "h2d systems");
     ck(cudaMemcpyAsync(d_kS_, kS.data(), ns * sizeof(double), cudaMemcpyHostToDevice, st_), "h2d systems");
-    h2d += (long long)(ns * (sizeof(ham[0]) + sizeof(lay[0]) + sizeof(double)));
+    h2d += (long long)(ns * (sizeof(ham[0]) + sizeof(hamd[0]) + sizeof(lay[0]) + sizeof(double)));
     if (pairs) {
       d_pair_ = ar_.get<uint32_t>(ns);
       ck(cudaMemcpyAsync(d_pair_, pairs->data(), ns * sizeof(uint32_t), cudaMemcpyHostToDevice, st_), "h2d pairs");
@@ -256,14 +263,24 @@ class YieldEngine {
     const int nf = (int)plans.size();
     d_fdev_ = ar_.get<rp::FieldDev<T>>(nf);
     d_coef_ = ar_.get<T>((size_t)nf * n_c_ * 4);
+    d_fd_ = ar_.get<rp::FieldDev<double>>(nf);
+    d_rcoef_ = ar_.get<T>((size_t)nf * n_c_ * 2);
     d_iin_ = ar_.get<rp::IntegralIn>(nf);
     iin_.resize(nf);
     std::vector<rp::FieldDev<T>> fdev(nf);
+    std::vector<rp::FieldDev<double>> fd(nf);
+    std::vector<T> rcoef((size_t)nf * n_c_ * 2);  // r_n with the sign of (-i)^n, then r_n - fl(r_n)
     // per field: c_n (re, im) in T, then the remainder c_n - fl(c_n) (FP32
     // only: the kernels add it, so the coefficients act with FP64 accuracy)
     std::vector<T> coef((size_t)nf * n_c_ * 4, T(0));
     for (int f = 0; f < nf; ++f) {
       const rp::FieldPlan& P = plans[f];
+      fd[f] = rp::FieldDev<double>{P.omega, 1.0 / P.dE, P.E_c / P.dE, 0.0};
+      for (int n = 0; n < n_c_; ++n) {
+        const double rn = (n & 2) ? -P.rcoef[n] : P.rcoef[n];
+        rcoef[(size_t)f * n_c_ * 2 + n] = (T)rn;
+        rcoef[(size_t)f * n_c_ * 2 + n_c_ + n] = (T)(rn - (double)(T)rn);
+      }
       fdev[f].omega = (T)P.omega;
       fdev[f].s = (T)(1.0 / P.dE);
       fdev[f].sh_re = (T)(P.E_c / P.dE);
@@ -282,8 +299,11 @@ class YieldEngine {
     }
     ck(cudaMemcpyAsync(d_fdev_, fdev.data(), fdev.size() * sizeof(fdev[0]), cudaMemcpyHostToDevice, st_), "h2d fields");
     ck(cudaMemcpyAsync(d_coef_, coef.data(), coef.size() * sizeof(T), cudaMemcpyHostToDevice, st_), "h2d coef");
+    ck(cudaMemcpyAsync(d_fd_, fd.data(), nf * sizeof(fd[0]), cudaMemcpyHostToDevice, st_), "h2d fields");
+    ck(cudaMemcpyAsync(d_rcoef_, rcoef.data(), rcoef.size() * sizeof(T), cudaMemcpyHostToDevice, st_), "h2d coef");
     ck(cudaMemcpyAsync(d_iin_, iin_.data(), nf * sizeof(iin_[0]), cudaMemcpyHostToDevice, st_), "h2d integral");
-    h2d += (long long)(fdev.size() * sizeof(fdev[0]) + coef.size() * sizeof(T) + nf * sizeof(iin_[0]));
+    h2d += (long long)(nf * (sizeof(fdev[0]) + sizeof(fd[0]) + sizeof(iin_[0])) +
+                       (coef.size() + rcoef.size()) * sizeof(T));
   }
 
   static size_t row_bytes(long long Z, int n_c) {
@@ -295,16 +315,31 @@ class YieldEngine {
 
   void alloc_rows(int R) {
     R_ = R;
-    // one persistent launch over all items (kernel = 5) where every system
-    // fits one CTA's shared memory; kernel = 5 elsewhere selects as 0.
-    // kernel = 0 (without graph replay, which asks for macro-step launches)
-    // takes it where it measured faster than one launch per macro-step:
-    // 128 <= Z <= 1024, and batches of several systems
-    const bool fits = Zslot_ <= rp::small_max_configs<T>() && o_.deterministic != 3 && !d_trace_;
-    persist_ = fits && (o_.kernel == 5 || (o_.kernel == 0 && !o_.graph &&
-                                           rp::persistent_default(Zslot_, (int)sys_.size())));
+    // Isotropic systems that fit one CTA run their whole horizon on chip in one
+    // launch over all items (kernel = 5, and kernel = 0 without graph replay,
+    // which asks for macro-step launches): rp_chip.cu.  Anisotropic ones, and
+    // shapes beyond its thread limits, take the generic persistent kernel where
+    // that measured faster than one launch per macro-step (128 <= Z <= 1024, and
+    // batches of several systems).
+    const bool fits = Zslot_ <= rp::small_max_configs<T>();
+    chip_ = fits && !aniso_ && rp::chip_plan<T>(Zslot_, min_half_, max_nuc_, (long long)R * Zslot_,
+                                                R, n_c_, d_trace_ != nullptr, &cplan_);
+    persist_ = o_.kernel == 5 || (o_.kernel == 0 && !o_.graph &&
+                                  (chip_ || rp::persistent_default(Zslot_, (int)sys_.size())));
+    if (!fits || (!chip_ && (o_.deterministic == 3 || d_trace_))) persist_ = false;
     d_err_ = ar_.get<int>(1);
     ck(cudaMemsetAsync(d_err_, 0, sizeof(int), st_), "cudaMemsetAsync");
+    if (persist_ && chip_) {
+      pctas_ = rp::chip_ctas<T>(cplan_);
+      if (pctas_ <= 0) throw CudaFail{RP_ECUDA, "on-chip kernel: no device"};
+      pctas_ = std::min(pctas_, (R + cplan_.rpc - 1) / cplan_.rpc);
+      d_counter_ = ar_.get<int>(1);
+      if (!d_trace_) {
+        if (!cplan_.split) Xp_ = ar_.get<T>((size_t)pctas_ * n_c_ * ((size_t)cplan_.slots << cplan_.lk) * 2);
+        plan_integral(false);
+      }
+      return;
+    }
     if (persist_) {
       pctas_ = rp::persistent_ctas<T>(Zslot_, n_c_, aniso_);
       if (pctas_ <= 0) throw CudaFail{RP_ECUDA, "persistent kernel: no device"};
@@ -375,6 +410,12 @@ class YieldEngine {
     rows_.survival = rows_.integral + R;
   }
 
+  rp::ChipArgs<T> chip_args() const {
+    return rp::ChipArgs<T>{d_hamd_, d_lay_, d_kS_, d_fd_, d_rcoef_, d_L_, rp::integral_ldk(n_c_),
+                           d_meta_, o_.pair_id, d_pair_, n_c_, max_nuc_, o_.deterministic, seed_,
+                           sec_rank_, sec_scale_};
+  }
+
   // The weights of the time integral of every field, formed on the device: their
   // low-rank factor, or (Gram kernels) the weights themselves.
   void plan_integral(bool weights) {
@@ -427,7 +468,25 @@ class YieldEngine {
       pev.push_back(e1);
       ck(cudaEventRecord(e0, st_), "cudaEventRecord");
     }
-    launched(rp::launch_persistent_small<T>(S_, aniso_, d_fdev_, d_coef_, d_L_, d_meta_, d_items, (int)n,
+    if (chip_) {
+      // groups of items of one field (the rows of a CTA)
+      std::vector<int2> groups;
+      for (size_t i = 0; i < h.size(); ++i) {
+        if (!groups.empty() && groups.back().y < cplan_.rpc &&
+            h[(size_t)groups.back().x].field == h[i].field)
+          groups.back().y++;
+        else
+          groups.push_back(make_int2((int)i, 1));
+      }
+      int2* d_groups = ar_.get<int2>(groups.size());
+      ck(cudaMemcpyAsync(d_groups, groups.data(), groups.size() * sizeof(int2), cudaMemcpyHostToDevice, st_),
+         "h2d groups");
+      h2d += (long long)(groups.size() * sizeof(int2));
+      launched(rp::launch_chip_items<T>(chip_args(), cplan_, d_items, d_groups, (int)groups.size(),
+                                        d_counter_, Xp_, pctas_, d_ps, d_trace_, trace_op_, st_),
+               "on-chip kernel");
+    } else
+      launched(rp::launch_persistent_small<T>(S_, aniso_, d_fdev_, d_coef_, d_L_, d_meta_, d_items, (int)n,
                                             d_counter_, n_c_, o_.deterministic, seed_, Xp_, pctas_,
                                             d_ps, st_),
              "persistent kernel");
@@ -631,7 +690,12 @@ class YieldEngine {
     T* phi[3] = {P, F1_, F2_};
     const rp::HamDev<T>* one = sys_.size() == 1 ? &ham1_ : nullptr;
     int n_step = 0;
-    if (small_) {
+    if (small_ && chip_) {
+      ck(rp::launch_chip_macro<T>(chip_args(), cplan_, sys_.size() == 1 ? nullptr : row_sys_,
+                                  rows_.field, rows_.win, k, mdev, R_, P, Q, X_, Zslot_, s),
+         "macro-step kernel");
+      n_step = 1;
+    } else if (small_) {
       ck(rp::launch_macro_small<T>(S_, one, aniso_, d_fdev_, rows_.field, rows_.win, k, mdev, R_,
                                    P, Q, X_, d_coef_, n_c_, s),
          "macro-step kernel");
@@ -734,6 +798,12 @@ class YieldEngine {
   bool cluster_ = false;
   bool overlap_ = false;
   bool persist_ = false;
+  bool chip_ = false;
+  rp::ChipPlan cplan_{};
+  int min_half_ = 1 << 30, max_nuc_ = 0;
+  rp::HamDev<double>* d_hamd_ = nullptr;
+  rp::FieldDev<double>* d_fd_ = nullptr;
+  T* d_rcoef_ = nullptr;
   int pctas_ = 0;
   T* Xp_ = nullptr;
   int* d_counter_ = nullptr;

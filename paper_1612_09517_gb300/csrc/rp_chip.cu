@@ -1,0 +1,1124 @@
+// Whole propagations on chip for isotropic systems that fit one SM.
+//
+// One CTA holds the Chebyshev vectors of its rows for a whole horizon
+// (k_chip_items: items from a device counter) or one macro-step
+// (k_chip_macro).  A thread owns KPT = 2^LK nuclear configurations that differ
+// in the LK innermost spin-1/2 nuclei:
+//   * phi_{n-1} and the accumulator psi(h) of its own configurations stay in
+//     registers; shared memory holds phi_{n-1} (read by the partners) and
+//     phi_{n-2} in the buffer that receives phi_n, one block barrier per term;
+//   * flip-flops of the in-thread nuclei are register to register;
+//   * digits, directions and addresses of the other nuclei are found once per
+//     nucleus and serve the KPT configurations, whose partners' components lie
+//     side by side (one 16-byte access per two FP32 values).
+// Arithmetic per configuration and term, in this order for every LK:
+//   u = (D + J-, kappa- and flip-flop terms) phi_{n-1},  phi_n = u - phi_{n-2}
+// with the factor 2/dE of the recurrence folded into the constants (formed in
+// FP64, rounded once).  FP32 subtracts phi_{n-2} last: summing into it rounds
+// every product at the size of phi (norm errors twice as large); FP64 starts
+// from it, which costs no operation.  An isotropic H is real, so a product is
+// one packed fma.rn.f32x2 on (re, im); only kappa mixes re and im.  The global
+// phase exp(-i E_c h) of the propagator is left out (no yield, survival or
+// expectation value depends on it), which makes the coefficients of the sum
+// real: c_n = r_n (-i)^n; cf holds r_n with the sign of (-i)^n for n mod 4 >= 2.
+#include <algorithm>
+#include <cstring>
+
+#include "rp_device.cuh"
+#include "rp_iso.cuh"
+#include "rp_kernels.cuh"
+#include "rp_project.cuh"
+#include "rp_sample.cuh"
+
+namespace rp {
+
+namespace {
+
+// Partner "up" (nuclear quantum number one lower: S_- I_+ brings it here) adds
+// its components (u0, u1) to targets (t0, t1), "down" the reverse:
+//   radical 0: 0 -> 2, 1 -> 3;  radical 1: 0 -> 1, 2 -> 3.
+// One component at a time, so that only KPT values are in flight.
+// Flip-flop of a spin-1/2 nucleus from a slot that holds the partner above (down
+// = false) or below: FP32 multiplies both directions (one by zero); FP64, whose
+// products cost 16 times as much as a select, picks the target first.
+template <int KPT>
+__device__ __forceinline__ void add_either(Cx<float> (&y)[KPT][4], int tu, int td, bool down,
+                                           float gu, float gd, const Cx<float> (&q)[KPT]) {
+#pragma unroll
+  for (int c = 0; c < KPT; ++c) {
+    madd(y[c][tu], gu, q[c]);
+    madd(y[c][td], gd, q[c]);
+  }
+}
+template <int KPT>
+__device__ __forceinline__ void add_either(Cx<double> (&y)[KPT][4], int tu, int td, bool down,
+                                           double gu, double gd, const Cx<double> (&q)[KPT]) {
+  const double g = down ? gd : gu;
+#pragma unroll
+  for (int c = 0; c < KPT; ++c) {
+    Cx<double> t = down ? y[c][td] : y[c][tu];
+    madd(t, g, q[c]);
+    if (down) y[c][td] = t;
+    else y[c][tu] = t;
+  }
+}
+template <typename T, int LK>
+__device__ __forceinline__ void flip_either(Cx<T> (&y)[1 << LK][4], int rr, bool down, T g,
+                                            const Cx<T>* cur, int S, int sl) {
+  constexpr int KPT = 1 << LK;
+  const T gu = down ? T(0) : g, gd = down ? g : T(0);
+  Cx<T> q[KPT];
+  if (rr == 0) {
+    Vec<T, LK>::get(cur, S, down ? 2 : 0, sl, q);
+    add_either<KPT>(y, 2, 0, down, gu, gd, q);
+    Vec<T, LK>::get(cur, S, down ? 3 : 1, sl, q);
+    add_either<KPT>(y, 3, 1, down, gu, gd, q);
+  } else {
+    Vec<T, LK>::get(cur, S, down ? 1 : 0, sl, q);
+    add_either<KPT>(y, 1, 0, down, gu, gd, q);
+    Vec<T, LK>::get(cur, S, down ? 3 : 2, sl, q);
+    add_either<KPT>(y, 3, 2, down, gu, gd, q);
+  }
+}
+template <typename T, int LK, bool UP>
+__device__ __forceinline__ void flip_one(Cx<T> (&y)[1 << LK][4], int rr, T g, const Cx<T>* cur,
+                                         int S, int sl) {
+  constexpr int KPT = 1 << LK;
+  Cx<T> q[KPT];
+  if (rr == 0) {
+    Vec<T, LK>::get(cur, S, UP ? 0 : 2, sl, q);
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) madd(y[c][UP ? 2 : 0], g, q[c]);
+    Vec<T, LK>::get(cur, S, UP ? 1 : 3, sl, q);
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) madd(y[c][UP ? 3 : 1], g, q[c]);
+  } else {
+    Vec<T, LK>::get(cur, S, UP ? 0 : 1, sl, q);
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) madd(y[c][UP ? 1 : 0], g, q[c]);
+    Vec<T, LK>::get(cur, S, UP ? 2 : 3, sl, q);
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) madd(y[c][UP ? 3 : 2], g, q[c]);
+  }
+}
+
+// Diagonal 2 (H_mm - E_c) / dE of the four electron states of configuration m.
+template <typename T>
+__device__ __forceinline__ void chip_diag(const HamDev<double>& H, const FieldDev<double>& F,
+                                          unsigned m, T (&d)[4]) {
+  double b[2] = {0.0, 0.0};
+  unsigned q = m;
+  for (int p = 0; p < H.n_nuc; ++p) {
+    const unsigned dd = (unsigned)H.d[p], j = q % dd;
+    q /= dd;
+    const double v = (0.5 * (double)(dd - 1) - (double)j) * H.v[p][2];
+    if (H.rad[p] == 0) b[0] += v;
+    else b[1] += v;
+  }
+  const double sp = 0.5 * (b[0] + b[1]), sm = 0.5 * (b[0] - b[1]), hJ = 0.5 * H.Je;
+  d[0] = (T)(2.0 * (F.s * (F.omega + hJ + sp) - F.sh_re));
+  d[1] = (T)(2.0 * (F.s * (-hJ + sm) - F.sh_re));
+  d[2] = (T)(2.0 * (F.s * (-hJ - sm) - F.sh_re));
+  d[3] = (T)(2.0 * (F.s * (-F.omega + hJ - sp) - F.sh_re));
+}
+
+// Constants of a CTA's rows (one system, one field) in shared memory.
+template <typename T>
+struct alignas(16) ChipConst {
+  T g[kMaxNucDev];  // 2 (a/2) / dE (x sqrt 2 for spin 1)
+  T J, kappa;       // 2 J / dE, 2 kappa / dE
+  int d[kMaxNucDev], st[kMaxNucDev];  // dimension and stride in slots (spins above 1)
+  unsigned rad;                       // radical of nucleus p in bit p
+  int n_half, n_one, n_nuc;
+};
+
+template <typename T>
+__device__ void chip_const(ChipConst<T>& K, const HamDev<double>& H, const FieldDev<double>& F,
+                           int lk, int tid) {
+  if (tid < H.n_nuc) {
+    const int p = tid;
+    const double g = 2.0 * F.s * H.U[p][4] * (H.d[p] == 3 ? 1.41421356237309504880 : 1.0);
+    K.g[p] = (T)g;
+    K.d[p] = H.d[p];
+    K.st[p] = (int)(H.stride[p] >> lk);
+  }
+  if (tid == 0) {
+    K.J = (T)(2.0 * F.s * H.Je);
+    K.kappa = (T)(2.0 * F.s * H.kappa);
+    K.n_half = H.n_half;
+    K.n_one = H.n_one;
+    K.n_nuc = H.n_nuc;
+    unsigned m = 0;
+    for (int p = 0; p < H.n_nuc; ++p) m |= (unsigned)(H.rad[p] & 1) << p;
+    K.rad = m;
+  }
+}
+
+// The thread's configurations to and from a buffer.
+template <typename T, int LK>
+__device__ __forceinline__ void chip_put(Cx<T>* b, int S, int slot, const Cx<T> (&v)[1 << LK][4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    Cx<T> q[1 << LK];
+#pragma unroll
+    for (int c = 0; c < (1 << LK); ++c) q[c] = v[c][e];
+    Vec<T, LK>::put(b, S, e, slot, q);
+  }
+}
+template <typename T, int LK>
+__device__ __forceinline__ void chip_get(const Cx<T>* b, int S, int slot, Cx<T> (&v)[1 << LK][4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    Cx<T> q[1 << LK];
+    Vec<T, LK>::get(b, S, e, slot, q);
+#pragma unroll
+    for (int c = 0; c < (1 << LK); ++c) v[c][e] = q[c];
+  }
+}
+
+// One term: u = phi_n from phi_{n-1} (own values a, partners in cur) and, unless
+// FIRST, phi_{n-2} (own entries of prev).  dt: diagonals, four per
+// configuration.  t: slot within the row, base: the row's first slot.
+template <typename T, int LK>
+__device__ __forceinline__ void chip_term(const ChipConst<T>& K, Cx<T> (&y)[1 << LK][4],
+                                          const Cx<T> (&a)[1 << LK][4], const T* dt,
+                                          const Cx<T>* cur, const Cx<T>* prev, bool first, int S,
+                                          int base, int t, unsigned dig) {
+  constexpr int KPT = 1 << LK;
+  if constexpr (sizeof(T) == 8) {
+    if (first) {
+#pragma unroll
+      for (int c = 0; c < KPT; ++c)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) y[c][e] = {T(0), T(0)};
+    } else {
+      chip_get<T, LK>(prev, S, base + t, y);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < KPT; ++c) {
+    T d[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) d[e] = dt[((size_t)c * S + base + t) * 4 + e];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (sizeof(T) == 4) y[c][e] = {d[e] * a[c][e].re, d[e] * a[c][e].im};
+      else y[c][e] = {fma(d[e], a[c][e].re, -y[c][e].re), fma(d[e], a[c][e].im, -y[c][e].im)};
+    }
+  }
+  const T J = K.J, kp = K.kappa;
+  if (J != T(0)) {
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) {
+      madd(y[c][1], J, a[c][2]);
+      madd(y[c][2], J, a[c][1]);
+    }
+  }
+  if (kp != T(0)) {  // -i kappa (2 P_S - 1)
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) {
+      madd_i(y[c][0], kp, a[c][0]);
+      madd_i(y[c][1], kp, a[c][2]);
+      madd_i(y[c][2], kp, a[c][1]);
+      madd_i(y[c][3], kp, a[c][3]);
+    }
+  }
+  // in-thread nuclei
+#pragma unroll
+  for (int p = 0; p < LK; ++p) {
+    const T g = K.g[p];
+    if (!((K.rad >> p) & 1u)) {
+#pragma unroll
+      for (int c = 0; c < KPT; ++c) {
+        const int o = c ^ (1 << p), down = (c >> p) & 1;
+        madd(y[c][down ? 0 : 2], g, a[o][down ? 2 : 0]);
+        madd(y[c][down ? 1 : 3], g, a[o][down ? 3 : 1]);
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < KPT; ++c) {
+        const int o = c ^ (1 << p), down = (c >> p) & 1;
+        madd(y[c][down ? 0 : 1], g, a[o][down ? 1 : 0]);
+        madd(y[c][down ? 2 : 3], g, a[o][down ? 3 : 2]);
+      }
+    }
+  }
+  // other spin-1/2 nuclei; above the lane bits the direction is the warp's
+  unsigned rm = K.rad >> LK;
+  const int nh = K.n_half;
+  int bit = 1;
+#pragma unroll 1
+  for (int p = LK; p < nh; ++p, bit <<= 1, rm >>= 1) {
+    const int sl = base + (t ^ bit), rr = (int)(rm & 1u);
+    const bool down = (t & bit) != 0;
+    const T g = K.g[p];
+    if (bit >= 32) {
+      if (down) flip_one<T, LK, false>(y, rr, g, cur, S, sl);
+      else flip_one<T, LK, true>(y, rr, g, cur, S, sl);
+    } else {
+      flip_either<T, LK>(y, rr, down, g, cur, S, sl);
+    }
+  }
+  // spin-1 nuclei: digit j, up from j + 1, down from j - 1 (FP32: a missing
+  // partner reads the own slot with weight zero)
+  const int n1 = nh + K.n_one;
+  int st = bit;
+#pragma unroll 1
+  for (int p = nh; p < n1; ++p, st *= 3, rm >>= 1, dig >>= 2) {
+    const unsigned j = dig & 3u;
+    const int rr = (int)(rm & 1u);
+    const T g = K.g[p];
+    if (sizeof(T) == 4 || j < 2u)
+      flip_one<T, LK, true>(y, rr, j < 2u ? g : T(0), cur, S, base + (j < 2u ? t + st : t));
+    if (sizeof(T) == 4 || j > 0u)
+      flip_one<T, LK, false>(y, rr, j > 0u ? g : T(0), cur, S, base + (j > 0u ? t - st : t));
+  }
+  // any other spin
+  if (n1 < K.n_nuc) {
+    unsigned q = (unsigned)t / (unsigned)K.st[n1];
+#pragma unroll 1
+    for (int p = n1; p < K.n_nuc; ++p) {
+      const unsigned dd = (unsigned)K.d[p], j = q % dd;
+      q /= dd;
+      const int rr = (int)((K.rad >> p) & 1u), so = K.st[p];
+      const T I = T(0.5) * T(dd - 1), M = I - T(j);
+      if (j + 1u < dd)
+        flip_one<T, LK, true>(y, rr, K.g[p] * sqrt(I * (I + 1) - M * (M - 1)), cur, S,
+                              base + t + so);
+      if (j > 0u)
+        flip_one<T, LK, false>(y, rr, K.g[p] * sqrt(I * (I + 1) - M * (M + 1)), cur, S,
+                               base + t - so);
+    }
+  }
+  if (first) {  // phi_1 = H phi_0, half of the recurrence's sum
+#pragma unroll
+    for (int c = 0; c < KPT; ++c)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) y[c][e] = {T(0.5) * y[c][e].re, T(0.5) * y[c][e].im};
+  } else if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      Cx<T> q[KPT];
+      Vec<T, LK>::get(prev, S, e, base + t, q);
+#pragma unroll
+      for (int c = 0; c < KPT; ++c) y[c][e] = {y[c][e].re - q[c].re, y[c][e].im - q[c].im};
+    }
+  }
+}
+
+// psi(h) += r_n (-i)^n phi_n: r phi (n even) or -i r phi (n odd), r with the sign of
+// n mod 4 >= 2; lo = r_n - fl(r_n).
+template <typename T, int KPT, bool ODD>
+__device__ __forceinline__ void chip_accumulate(Cx<T> (&acc)[KPT][4], const Cx<T> (&y)[KPT][4], T r,
+                                                T lo) {
+#pragma unroll
+  for (int c = 0; c < KPT; ++c)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (ODD) {
+        if (sizeof(T) == 4) madd_i(acc[c][e], -lo, y[c][e]);
+        madd_i(acc[c][e], -r, y[c][e]);
+      } else {
+        if (sizeof(T) == 4) madd(acc[c][e], lo, y[c][e]);
+        madd(acc[c][e], r, y[c][e]);
+      }
+    }
+}
+
+// Singlet slice <S|phi_n> = (phi_1 - phi_2) / sqrt 2 of the thread's configurations:
+// entry c * xs of the row's slice n.
+template <typename T, int KPT>
+__device__ __forceinline__ void chip_singlet(T* x, int xs, const Cx<T> (&y)[KPT][4]) {
+  const T r = T(0.70710678118654752440);
+#pragma unroll
+  for (int c = 0; c < KPT; ++c) {
+    typename SliceVal<T>::type v;
+    v.x = (y[c][1].re - y[c][2].re) * r;
+    v.y = (y[c][1].im - y[c][2].im) * r;
+    *reinterpret_cast<typename SliceVal<T>::type*>(x + (size_t)c * xs * 2) = v;
+  }
+}
+
+// A macro-step of the thread's configurations: psi(t) in the thread's entries of
+// buffer 0, on return psi(t + h) there (so nothing of the state is held in
+// registers while the integral runs).  Threads without configurations (on =
+// false) only keep the barriers.  xn: the thread's entry of the row's slices,
+// stride between slices xstride (complex), between the thread's configurations
+// xs.  Not inlined: the caller's live values would spill inside the term loop.
+template <typename T, int LK>
+__device__ __noinline__ void chip_macro(int S, int base, int t, bool on, unsigned dig,
+                                        const T* __restrict__ cf, int n_c, T* xn, size_t xstride,
+                                        int xs, bool store_x) {
+  constexpr int KPT = 1 << LK;
+  extern __shared__ __align__(16) unsigned char chip_smem[];
+  const ChipConst<T>& K = *reinterpret_cast<const ChipConst<T>*>(chip_smem);
+  Cx<T>* b0 = reinterpret_cast<Cx<T>*>(chip_smem + sizeof(ChipConst<T>));
+  Cx<T>* b1 = b0 + (size_t)4 * KPT * S;
+  const T* dt = reinterpret_cast<const T*>(b1 + (size_t)4 * KPT * S);
+  const T* cl = cf + n_c;
+  Cx<T> a[KPT][4], y[KPT][4], acc[KPT][4];
+  if (on) {
+    chip_get<T, LK>(b0, S, base + t, a);
+    if (store_x) chip_singlet<T, KPT>(xn, xs, a);
+#pragma unroll
+    for (int c = 0; c < KPT; ++c)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[c][e] = {T(0), T(0)};
+    chip_accumulate<T, KPT, false>(acc, a, cf[0], cl[0]);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int n = 1; n < n_c; n += 2) {  // n_c is even: n odd, then n + 1 even
+    if (on) {
+      chip_term<T, LK>(K, y, a, dt, b0, b1, n == 1, S, base, t, dig);
+      chip_put<T, LK>(b1, S, base + t, y);
+      if (store_x) chip_singlet<T, KPT>(xn + (size_t)n * xstride * 2, xs, y);
+      chip_accumulate<T, KPT, true>(acc, y, cf[n], cl[n]);
+    }
+    __syncthreads();
+    if (n + 1 < n_c) {
+      if (on) {
+        chip_term<T, LK>(K, a, y, dt, b1, b0, false, S, base, t, dig);
+        chip_put<T, LK>(b0, S, base + t, a);
+        if (store_x) chip_singlet<T, KPT>(xn + (size_t)(n + 1) * xstride * 2, xs, a);
+        chip_accumulate<T, KPT, false>(acc, a, cf[n + 1], cl[n + 1]);
+      }
+      __syncthreads();
+    }
+  }
+  if (on) chip_put<T, LK>(b0, S, base + t, acc);
+}
+
+// Two-bit digits of the spin-1 nuclei of slot t.
+__device__ __forceinline__ unsigned chip_digits(const HamDev<double>& H, int t, int lk) {
+  unsigned q = (unsigned)t >> (H.n_half - lk), dig = 0;
+  for (int i = 0; i < H.n_one; ++i) {
+    dig |= (q % 3u) << (2 * i);
+    q /= 3u;
+  }
+  return dig;
+}
+
+// Most threads of a CTA, which bounds the registers: FP32 128, FP64 255 with
+// several configurations per thread.
+template <typename T>
+__host__ __device__ constexpr int chip_max_threads(int lk) {
+  return sizeof(T) == 4 || lk == 0 ? 512 : 256;
+}
+
+// Survival and time-trace sums of a thread's configurations.
+template <typename T, int KPT>
+__device__ __forceinline__ double chip_norm(const Cx<T> (&a)[KPT][4]) {
+  double s = 0.0;
+#pragma unroll
+  for (int c = 0; c < KPT; ++c)
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      s += (double)a[c][e].re * (double)a[c][e].re + (double)a[c][e].im * (double)a[c][e].im;
+  return s;
+}
+
+// v += (P_S, norm, Re, Im <A_e x 1>) of one configuration (see k_trace).
+template <typename T>
+__device__ __forceinline__ void trace_terms(const Cx<T> (&a)[4], const ElecOp& A, double (&v)[4]) {
+  const double dr = (double)a[1].re - (double)a[2].re, di = (double)a[1].im - (double)a[2].im;
+  v[0] += 0.5 * (dr * dr + di * di);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const double cr = (double)a[e].re, ci = (double)a[e].im;
+    v[1] += cr * cr + ci * ci;
+    if (A.on) {
+      double yr = 0.0, yi = 0.0;
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const double xr = (double)a[f].re, xi = (double)a[f].im;
+        yr += A.re[4 * e + f] * xr - A.im[4 * e + f] * xi;
+        yi += A.re[4 * e + f] * xi + A.im[4 * e + f] * xr;
+      }
+      v[2] += cr * yr + ci * yi;
+      v[3] += cr * yi - ci * yr;
+    }
+  }
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// One launch over all items: CTAs take groups of up to rpc items of one field
+// from a device counter and run their whole horizon.  Shared memory: two
+// buffers of S slots (the second doubles as the integral's ring), the factor L,
+// rows' sums.  The singlet slices of a macro-step
+// go to the CTA's scratch and come back as the thread's own entries for the
+// time integral (rp_integral.cu).
+// MT, MB: most threads of a CTA and CTAs per SM, which bound the registers (two
+// CTAs of 224 threads hold 144 registers each: at 128 the spills of four
+// configurations per thread took 15 % of the instructions and missed L1).
+template <typename T, int LK, int MT, int MB>
+__global__ void __launch_bounds__(MT, MB) k_chip_items(
+    const ChipArgs<T> A, const PItem* __restrict__ items, const int2* __restrict__ groups,
+    int n_groups, int* __restrict__ counter, int rpc, int S, T* __restrict__ Xscratch, double* __restrict__ per_sample, double* __restrict__ trace,
+    const ElecOp op) {
+  constexpr int KPT = 1 << LK, KB = ProjCfg<T>::kB;
+  extern __shared__ __align__(16) unsigned char chip_smem[];
+  __shared__ int s_group;
+  ChipConst<T>& K = *reinterpret_cast<ChipConst<T>*>(chip_smem);
+  Cx<T>* buf = reinterpret_cast<Cx<T>*>(chip_smem + sizeof(ChipConst<T>));
+  T* dt = reinterpret_cast<T*>(buf + (size_t)8 * KPT * S);  // diagonals [KPT][S][4]
+  T* sl = dt + (size_t)4 * KPT * S;
+  double* sums = reinterpret_cast<double*>(sl + (size_t)A.n_c * KB);  // [rpc][2]
+  double* amps = sums + 2 * rpc;                                      // [rpc][max_nuc][20]
+  // the integral's ring: buffer 1, 4 KPT slices per thread
+  auto* ring = reinterpret_cast<typename SliceVal<T>::type*>(buf + (size_t)4 * KPT * S) + threadIdx.x;
+  const int tid = threadIdx.x;
+  T* xc = Xscratch + (size_t)blockIdx.x * A.n_c * KPT * S * 2;
+  for (;;) {
+    if (tid == 0) s_group = atomicAdd(counter, 1);
+    __syncthreads();
+    const int gi = s_group;
+    if (gi >= n_groups) break;  // the same for the whole CTA
+    const int2 grp = groups[gi];
+    const PItem I0 = items[grp.x];
+    const HamDev<double>& H = A.ham[I0.sys];
+    const FieldDev<double> F = A.fields[I0.field];
+    const int Sr = (int)(H.Z >> LK);
+    const int row = tid / Sr, t = tid - row * Sr, base = row * Sr;
+    const bool on = row < grp.y;
+    chip_const<T>(K, H, F, LK, tid);
+    if (tid < 2 * rpc) sums[tid] = 0.0;
+    const LayoutDev& Ly = A.lay[I0.sys];
+    if (!A.deterministic)
+      for (int q = tid; q < grp.y * Ly.n_nuc; q += blockDim.x) {
+        const int r = q / Ly.n_nuc, p = q % Ly.n_nuc;
+        double u[2];
+        const uint32_t pair = A.pair_of ? A.pair_of[I0.sys] : A.pair_base + (uint32_t)I0.sys;
+        coherent_amp(Ly, p, pair, (unsigned long long)items[grp.x + r].sample, A.seed,
+                     amps + ((size_t)r * A.max_nuc + p) * 20, u);
+      }
+    __syncthreads();
+    unsigned dig = 0;
+    if (on) {
+      Cx<T> a[KPT][4];
+      dig = chip_digits(H, t, LK);
+      const long long sample = items[grp.x + row].sample;
+#pragma unroll
+      for (int c = 0; c < KPT; ++c) {
+        const unsigned m = ((unsigned)t << LK) | (unsigned)c;
+        T d[4];
+        chip_diag<T>(H, F, m, d);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) dt[((size_t)c * S + base + t) * 4 + e] = d[e];
+        double pr = 1.0, pi = 0.0;
+        if (A.deterministic == 3) {
+          pr = A.sec_rank[m] == sample ? A.sec_scale[sample] : 0.0;
+        } else if (A.deterministic) {
+          pr = (long long)m == sample ? 1.0 : 0.0;
+        } else {
+          unsigned q = m;
+          const double* am = amps + (size_t)row * A.max_nuc * 20;
+          for (int p = 0; p < Ly.n_nuc; ++p) {
+            const unsigned dd = (unsigned)Ly.d[p], j = q % dd;
+            q /= dd;
+            const double ar = am[p * 20 + 2 * j], ai = am[p * 20 + 2 * j + 1];
+            const double nr = pr * ar - pi * ai;
+            pi = pr * ai + pi * ar;
+            pr = nr;
+          }
+        }
+        const double s = 0.70710678118654752440;
+        a[c][0] = a[c][3] = {T(0), T(0)};
+        a[c][1] = {(T)(s * pr), (T)(s * pi)};
+        a[c][2] = {(T)(-s * pr), (T)(-s * pi)};
+      }
+      chip_put<T, LK>(buf, S, base + t, a);
+    }
+    const T* cf = A.coef + (size_t)I0.field * 2 * A.n_c;
+    const bool integrate = trace == nullptr;
+    int2 mt = make_int2(0, 0);
+    const T* Lf = nullptr;
+    if (integrate) {
+      mt = A.meta[I0.field];
+      Lf = A.L + (size_t)I0.field * A.n_c * A.ldk;
+      if (mt.x <= KB) stage_factor<T>(sl, Lf, A.ldk, (mt.y + 1) & ~1, 0, tid, blockDim.x);
+    }
+    const int n_e = (mt.y + 1) & ~1;
+    double integral = 0.0;
+    const size_t xrow = (size_t)KPT * S;
+#pragma unroll 1
+    for (int km = 0; km < I0.n_macro; ++km) {
+      chip_macro<T, LK>(S, base, t, on, dig, cf, A.n_c, xc + (size_t)(base + t) * 2,
+                        xrow, S, integrate);
+      if (integrate) {
+        for (int k0 = 0; k0 < mt.x; k0 += KB) {
+          if (mt.x > KB) {  // several blocks of columns: staged in turn
+            __syncthreads();
+            stage_factor<T>(sl, Lf, A.ldk, n_e, k0, tid, blockDim.x);
+            __syncthreads();
+          }
+          if (on) {
+#pragma unroll 1
+            for (int c = 0; c < KPT; ++c) {
+              typename ProjAcc<T>::type yr[1][16], yi[1][16];
+              const T* const p[1] = {xc + ((size_t)c * S + base + t) * 2};
+              project_block<T, 1, 4, KPT>(yr, yi, p, xrow * 2, sl, KB, n_e, ring, S);
+              integral += proj_norm(yr[0], yi[0]);
+            }
+          }
+        }
+      } else {
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        if (on) {
+          Cx<T> a[KPT][4];
+          chip_get<T, LK>(buf, S, base + t, a);
+#pragma unroll
+          for (int c = 0; c < KPT; ++c) trace_terms<T>(a[c], op, v);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (q >= 2 && !op.on) break;
+          const double w = warp_sum(v[q]);
+          if ((tid & 31) == 0 && w != 0.0) atomicAdd(trace + 4 * (km + 1) + q, w);
+        }
+      }
+    }
+    if (on) {
+      Cx<T> a[KPT][4];
+      chip_get<T, LK>(buf, S, base + t, a);
+      atomicAdd(&sums[2 * row], integral);
+      atomicAdd(&sums[2 * row + 1], chip_norm<T, KPT>(a));
+    }
+    __syncthreads();
+    if (tid < grp.y) {
+      const double phS = A.k_S[I0.sys] * sums[2 * tid], surv = sums[2 * tid + 1];
+      double* o = per_sample + items[grp.x + tid].out * 3;
+      o[0] = phS;
+      o[1] = 1.0 - surv - phS;  // Haberkorn: d|psi|^2/dt = -k_S <P_S> - k_T <P_T>
+      o[2] = surv;
+    }
+    __syncthreads();
+  }
+}
+
+// ---- few configurations per SM: one thread per configuration and electron state ----
+//
+// With fewer than about 256 configurations per SM the length of a thread's
+// chain of dependent instructions decides, in FP64 most of all (a warp's FP64
+// instruction holds its scheduler's unit for 64 cycles).  A row then takes 4 Z
+// threads.  A thread's row of H has at most one partner per nucleus (an
+// isotropic coupling brings each electron state either the configuration above
+// or the one below), so offsets and weights of the whole horizon sit in
+// registers and a term is one shared-memory read and one packed multiply-add
+// per nucleus.  The slices of the macro-step stay in shared memory too, and
+// the integral's 32 columns are spread over the four threads of a
+// configuration.  The sums run in chip_term's order: results do not depend on
+// which of the two kernels ran.
+constexpr int kSplitNuc = 8;  // Z <= 256
+template <typename T>
+__host__ __device__ constexpr int split_max_threads() {
+  return sizeof(T) == 4 ? 1024 : 768;
+}
+
+template <typename T>
+struct SplitRow {
+  T w[kSplitNuc];     // couplings (weight zero where there is no partner)
+  int off[kSplitNuc];  // entry of the partner in a buffer
+  T d;                // diagonal (as chip_term forms it)
+  int own;            // entry of state 3 - e of the own configuration
+  int src;            // entry of the state kappa couples to (e for 0 and 3, else own)
+};
+
+// y (phi_{n-2}) becomes phi_n; a = phi_{n-1} of this thread.
+template <typename T>
+__device__ __forceinline__ void split_term(const SplitRow<T>& R, int n_nuc, T J, T kp, bool mid,
+                                           Cx<T>& y, const Cx<T>& a, const Cx<T>* cur) {
+  Cx<T> q[kSplitNuc];
+#pragma unroll
+  for (int p = 0; p < kSplitNuc; ++p)
+    if (p < n_nuc) q[p] = cur[R.off[p]];
+  Cx<T> u;
+  if (sizeof(T) == 4) u = {R.d * a.re, R.d * a.im};
+  else u = {fma(R.d, a.re, -y.re), fma(R.d, a.im, -y.im)};
+  if (J != T(0) && mid) madd_s(u, J, cur[R.own]);
+  if (kp != T(0)) madd_i(u, kp, cur[R.src]);
+#pragma unroll
+  for (int p = 0; p < kSplitNuc; ++p)
+    if (p < n_nuc) madd_s(u, R.w[p], q[p]);
+  if (sizeof(T) == 4) y = {u.re - y.re, u.im - y.im};
+  else y = u;
+}
+
+// MT: most threads of the launch (small CTAs keep more in registers)
+template <typename T, int MT>
+__global__ void __launch_bounds__(MT, 1) k_split_items(
+    const ChipArgs<T> A, const PItem* __restrict__ items, const int2* __restrict__ groups,
+    int n_groups, int* __restrict__ counter, int rpc, int S, double* __restrict__ per_sample,
+    double* __restrict__ trace, const ElecOp op) {
+  extern __shared__ __align__(16) unsigned char chip_smem[];
+  __shared__ int s_group;
+  // two buffers [e][S], slices [n_c][S], factor [n_c][32], sums, amplitudes
+  Cx<T>* buf = reinterpret_cast<Cx<T>*>(chip_smem);
+  Cx<T>* xs = buf + (size_t)8 * S;
+  T* sl = reinterpret_cast<T*>(xs + (trace ? 0 : (size_t)A.n_c * S));
+  double* sums = reinterpret_cast<double*>(sl + (trace ? 0 : (size_t)A.n_c * 32));
+  double* amps = sums + 2 * rpc;
+  const int tid = threadIdx.x;
+  for (;;) {
+    if (tid == 0) s_group = atomicAdd(counter, 1);
+    __syncthreads();
+    const int gi = s_group;
+    if (gi >= n_groups) break;  // the same for the whole CTA
+    const int2 grp = groups[gi];
+    const PItem I0 = items[grp.x];
+    const HamDev<double>& H = A.ham[I0.sys];
+    const FieldDev<double> F = A.fields[I0.field];
+    const int Z = (int)H.Z, n_nuc = H.n_nuc;
+    const int row = tid / (4 * Z), e = (tid - row * 4 * Z) / Z, m = tid % Z;
+    const int slot = row * Z + m;  // 4 Z is a multiple of Z
+    const bool on = row < grp.y;
+    if (tid < 2 * rpc) sums[tid] = 0.0;
+    const LayoutDev& Ly = A.lay[I0.sys];
+    if (!A.deterministic)
+      for (int q = tid; q < grp.y * Ly.n_nuc; q += blockDim.x) {
+        const int r = q / Ly.n_nuc, p = q % Ly.n_nuc;
+        double u[2];
+        const uint32_t pair = A.pair_of ? A.pair_of[I0.sys] : A.pair_base + (uint32_t)I0.sys;
+        coherent_amp(Ly, p, pair, (unsigned long long)items[grp.x + r].sample, A.seed,
+                     amps + ((size_t)r * A.max_nuc + p) * 20, u);
+      }
+    const T* cf = A.coef + (size_t)I0.field * 2 * A.n_c;
+    const T* cl = cf + A.n_c;
+    int2 mt = make_int2(0, 0);
+    const T* Lf = nullptr;
+    if (!trace) {
+      mt = A.meta[I0.field];
+      Lf = A.L + (size_t)I0.field * A.n_c * A.ldk;
+      if (mt.x <= 32) stage_factor<T, 32>(sl, Lf, A.ldk, (mt.y + 1) & ~1, 0, tid, blockDim.x);
+    }
+    const int n_e = (mt.y + 1) & ~1;
+    SplitRow<T> R;
+    const T J = (T)(2.0 * F.s * H.Je), kp = (T)(2.0 * F.s * H.kappa);
+    const bool mid = e == 1 || e == 2;
+    Cx<T> a = {T(0), T(0)};
+    __syncthreads();
+    if (on) {
+      T d4[4];
+      chip_diag<T>(H, F, (unsigned)m, d4);
+      R.d = e == 0 ? d4[0] : e == 1 ? d4[1] : e == 2 ? d4[2] : d4[3];
+      R.own = (3 - e) * S + slot;
+      R.src = mid ? R.own : e * S + slot;
+      unsigned q = (unsigned)m;
+#pragma unroll
+      for (int p = 0; p < kSplitNuc; ++p) {
+        R.w[p] = T(0);
+        R.off[p] = e * S + slot;
+        if (p < n_nuc) {
+          const unsigned dd = (unsigned)H.d[p], j = q % dd;
+          q /= dd;
+          const int flip = H.rad[p] == 0 ? 2 : 1, st = (int)H.stride[p];
+          const bool up = (e & flip) != 0;  // S_- I_+ from j + 1, else S_+ I_- from j - 1
+          if (up ? j + 1u < dd : j > 0u) {
+            double g = 2.0 * F.s * H.U[p][4];
+            if (dd == 3) g *= 1.41421356237309504880;
+            R.w[p] = (T)g;
+            if (dd > 3) {
+              const T I = T(0.5) * T(dd - 1), M = I - T(j);
+              R.w[p] *= up ? sqrt(I * (I + 1) - M * (M - 1)) : sqrt(I * (I + 1) - M * (M + 1));
+            }
+            R.off[p] = (e ^ flip) * S + slot + (up ? st : -st);
+          }
+        }
+      }
+      // psi(0) of this thread's state
+      double pr = 1.0, pi = 0.0;
+      const long long sample = items[grp.x + row].sample;
+      if (A.deterministic == 3) {
+        pr = A.sec_rank[m] == sample ? A.sec_scale[sample] : 0.0;
+      } else if (A.deterministic) {
+        pr = (long long)m == sample ? 1.0 : 0.0;
+      } else {
+        unsigned qq = (unsigned)m;
+        const double* am = amps + (size_t)row * A.max_nuc * 20;
+        for (int p = 0; p < Ly.n_nuc; ++p) {
+          const unsigned dd = (unsigned)Ly.d[p], j = qq % dd;
+          qq /= dd;
+          const double ar = am[p * 20 + 2 * j], ai = am[p * 20 + 2 * j + 1];
+          const double nr = pr * ar - pi * ai;
+          pi = pr * ai + pi * ar;
+          pr = nr;
+        }
+      }
+      const double s = e == 1 ? 0.70710678118654752440 : -0.70710678118654752440;
+      if (mid) a = {(T)(s * pr), (T)(s * pi)};
+    }
+    double integral = 0.0;
+    Cx<T>* b0 = buf + (size_t)e * S + slot;  // this thread's entries
+    Cx<T>* b1 = b0 + (size_t)4 * S;
+    const bool keeps = !trace && on && e == 0;  // stores the slices
+    // slice n from the buffer holding phi_n, by the threads of state 0
+    auto slice = [&](int n, const Cx<T>* b) {
+      const Cx<T> p1 = b[S + slot], p2 = b[2 * S + slot];
+      const T r = T(0.70710678118654752440);
+      xs[(size_t)n * S + slot] = {(p1.re - p2.re) * r, (p1.im - p2.im) * r};
+    };
+#pragma unroll 1
+    for (int km = 0; km < I0.n_macro; ++km) {
+      Cx<T> y = {T(0), T(0)}, acc = {T(0), T(0)};
+      if (on) {
+        *b0 = a;
+        if (sizeof(T) == 4) madd_s(acc, cl[0], a);
+        madd_s(acc, cf[0], a);
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int n = 1; n < A.n_c; n += 2) {
+        if (on) {
+          split_term<T>(R, n_nuc, J, kp, mid, y, a, buf);
+          if (n == 1) {
+            y.re *= T(0.5);
+            y.im *= T(0.5);
+          }
+          *b1 = y;
+          if (keeps) slice(n - 1, buf);
+          if (sizeof(T) == 4) madd_i(acc, -cl[n], y);
+          madd_i(acc, -cf[n], y);
+        }
+        __syncthreads();
+        if (n + 1 < A.n_c) {
+          if (on) {
+            split_term<T>(R, n_nuc, J, kp, mid, a, y, buf + (size_t)4 * S);
+            *b0 = a;
+            if (keeps) slice(n, buf + (size_t)4 * S);
+            if (sizeof(T) == 4) madd_s(acc, cl[n + 1], a);
+            madd_s(acc, cf[n + 1], a);
+          }
+          __syncthreads();
+        }
+      }
+      a = acc;
+      if (!trace) {
+        if (keeps) slice(A.n_c - 1, buf + (size_t)4 * S);  // n_c is even: the last n is odd
+        __syncthreads();
+        for (int k0 = 0; k0 < mt.x; k0 += 32) {
+          if (mt.x > 32) {  // several blocks of columns: staged in turn
+            __syncthreads();
+            stage_factor<T, 32>(sl, Lf, A.ldk, n_e, k0, tid, blockDim.x);
+            __syncthreads();
+          }
+          if (on) {
+            constexpr int N = sizeof(T) == 4 ? 4 : 8;  // eight columns
+            typename ProjAcc<T>::type yr[N], yi[N];
+#pragma unroll
+            for (int k = 0; k < N; ++k) yr[k] = yi[k] = typename ProjAcc<T>::type{};
+            const T* l = sl + 8 * e;
+#pragma unroll 2
+            for (int n = 0; n < n_e; n += 2) {
+              const Cx<T> v = xs[(size_t)n * S + slot], u = xs[(size_t)(n + 1) * S + slot];
+              proj_add(yr, yi, l + n * 32, v.re, v.im);
+              proj_add(yr, yi, l + (n + 1) * 32, u.im, -u.re);
+            }
+            integral += proj_norm8(yr, yi);
+          }
+        }
+      } else {
+        // every state of the configuration for the observables: psi(t + h) once more
+        __syncthreads();
+        if (on) *b0 = a;
+        __syncthreads();
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        if (on && e == 0) {
+          const Cx<T> c4[4] = {buf[slot], buf[S + slot], buf[2 * S + slot], buf[3 * S + slot]};
+          trace_terms<T>(c4, op, v);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (q >= 2 && !op.on) break;
+          const double w = warp_sum(v[q]);
+          if ((tid & 31) == 0 && w != 0.0) atomicAdd(trace + 4 * (km + 1) + q, w);
+        }
+      }
+    }
+    if (on) {
+      atomicAdd(&sums[2 * row], integral);
+      atomicAdd(&sums[2 * row + 1], (double)a.re * (double)a.re + (double)a.im * (double)a.im);
+    }
+    __syncthreads();
+    if (tid < grp.y) {
+      const double phS = A.k_S[I0.sys] * sums[2 * tid], surv = sums[2 * tid + 1];
+      double* o = per_sample + items[grp.x + tid].out * 3;
+      o[0] = phS;
+      o[1] = 1.0 - surv - phS;
+      o[2] = surv;
+    }
+    __syncthreads();
+  }
+}
+
+template <typename T>
+size_t split_smem_bytes(int S, int rpc, int n_c, int max_nuc, bool trace) {
+  return (size_t)(8 + (trace ? 0 : n_c)) * S * sizeof(Cx<T>) +
+         (trace ? 0 : (size_t)n_c * 32 * sizeof(T)) +
+         (size_t)rpc * (2 + max_nuc * 20) * sizeof(double);
+}
+
+// One macro-step of every active row, one CTA per row: psi from P to Q, slices
+// to X (any order within a row: the integral sums over all of it).
+template <typename T, int LK>
+__global__ void __launch_bounds__(chip_max_threads<T>(LK), 1) k_chip_macro(
+    const ChipArgs<T> A, const int* __restrict__ row_sys, const int* __restrict__ row_field,
+    const int2* __restrict__ row_win, int macro_arg, const int* __restrict__ macro_dev,
+    const T* __restrict__ P, T* __restrict__ Q, T* __restrict__ X, long long Zslot) {
+  constexpr int KPT = 1 << LK;
+  extern __shared__ __align__(16) unsigned char chip_smem[];
+  ChipConst<T>& K = *reinterpret_cast<ChipConst<T>*>(chip_smem);
+  const int r = blockIdx.x, tid = threadIdx.x;
+  const int macro = macro_dev ? *macro_dev : macro_arg;
+  const int2 w = row_win[r];
+  if (macro < w.x || macro >= w.y) return;
+  const HamDev<double>& H = A.ham[row_sys ? row_sys[r] : 0];
+  const int f = row_field[r];
+  const FieldDev<double> F = A.fields[f];
+  const int Sr = (int)(H.Z >> LK);
+  const bool on = tid < Sr;
+  chip_const<T>(K, H, F, LK, tid);
+  Cx<T>* buf = reinterpret_cast<Cx<T>*>(chip_smem + sizeof(ChipConst<T>));
+  T* dt = reinterpret_cast<T*>(buf + (size_t)8 * KPT * Sr);
+  unsigned dig = 0;
+  if (on) {
+    Cx<T> a[KPT][4];
+    dig = chip_digits(H, tid, LK);
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) {
+      const unsigned m = ((unsigned)tid << LK) | (unsigned)c;
+      T d[4];
+      chip_diag<T>(H, F, m, d);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) dt[((size_t)c * Sr + tid) * 4 + e] = d[e];
+      const Cx<T>* p = reinterpret_cast<const Cx<T>*>(P) + ((size_t)r * Zslot + m) * 4;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) a[c][e] = p[e];
+    }
+    chip_put<T, LK>(buf, Sr, tid, a);
+  }
+  __syncthreads();
+  chip_macro<T, LK>(Sr, 0, tid, on, dig,
+                    A.coef + (size_t)f * 2 * A.n_c, A.n_c,
+                    X + ((size_t)r * A.n_c * Zslot + tid) * 2, (size_t)Zslot, Sr, true);
+  if (on) {
+    Cx<T> a[KPT][4];
+    chip_get<T, LK>(buf, Sr, tid, a);
+#pragma unroll
+    for (int c = 0; c < KPT; ++c) {
+      Cx<T>* p = reinterpret_cast<Cx<T>*>(Q) +
+                 ((size_t)r * Zslot + (((unsigned)tid << LK) | (unsigned)c)) * 4;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) p[e] = a[c][e];
+    }
+  }
+}
+
+template <typename T, int LK>
+size_t chip_smem_bytes(int S, int rpc, int n_c, int max_nuc) {
+  const size_t buf = (size_t)4 * (1 << LK) * S * sizeof(Cx<T>);
+  return sizeof(ChipConst<T>) + 2 * buf + buf / 2 + (size_t)n_c * ProjCfg<T>::kB * sizeof(T) +
+         (size_t)rpc * (2 + max_nuc * 20) * sizeof(double);
+}
+
+constexpr int kChipSmemMax = 224 * 1024;
+
+}  // namespace
+
+template <typename T>
+bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_items, int n_c,
+               bool trace, ChipPlan* out) {
+  // One SM's share of configurations decides: few, and the length of a term
+  // counts (more threads per configuration); many, and its instructions do.
+  // Measured (GB300): one field of Z = 96, 16 propagations: 2.2 ms split, 4.9 ms
+  // with one configuration per thread; Z = 16 FP64, 704 propagations: 51 and 82
+  // ms; Z = 864, 1024 propagations in FP32: 48 ms with two configurations per
+  // thread, 51 ms with four, which spill.  FP64 gains nothing from in-thread
+  // nuclei (82 -> 143 ms: half the warps), so it takes them only where the
+  // threads would not fit.
+  const long long per_sm = load / 152;
+  out->split = false;
+  if (per_sm <= 256 && max_nuc <= kSplitNuc && 4 * Zmax <= split_max_threads<T>()) {
+    ChipPlan P;
+    P.split = true;
+    P.rpc = std::max<int>(1, (int)(32 / (4 * Zmax)));
+    P.threads = (int)((4 * P.rpc * Zmax + 31) / 32 * 32);
+    P.slots = (int)(P.rpc * Zmax);
+    P.smem = split_smem_bytes<T>(P.slots, P.rpc, n_c, max_nuc, trace);
+    if (P.smem <= (size_t)kChipSmemMax) {
+      // the macro-step launches (graph replay) take one configuration per thread
+      P.lk = Zmax <= chip_max_threads<T>(0) ? 0 : std::min(1, min_half);
+      *out = P;
+      return true;
+    }
+  }
+  const int want = sizeof(T) == 8 || per_sm <= 192 ? 0 : 1;
+  for (int lk = std::min(want, min_half); lk <= std::min(2, min_half); ++lk) {
+    const long long Sr = Zmax >> lk;
+    if (Sr > chip_max_threads<T>(lk)) continue;
+    ChipPlan P;
+    P.lk = lk;
+    // rows per CTA: fill a warp, then up to 128 threads while every SM still
+    // gets a CTA
+    int rpc = std::max<int>(1, (int)(32 / Sr));
+    while (rpc < 32 && (rpc * 2) * Sr <= 128 && n_items / (rpc * 2) >= 152 * 2) rpc *= 2;
+    P.rpc = rpc;
+    P.threads = (int)((rpc * Sr + 31) / 32 * 32);
+    P.slots = (int)(rpc * Sr);
+    P.smem = lk == 0 ? chip_smem_bytes<T, 0>(P.slots, rpc, n_c, max_nuc)
+             : lk == 1 ? chip_smem_bytes<T, 1>(P.slots, rpc, n_c, max_nuc)
+                       : chip_smem_bytes<T, 2>(P.slots, rpc, n_c, max_nuc);
+    if (P.smem > (size_t)kChipSmemMax) continue;
+    *out = P;
+    return true;
+  }
+  return false;
+}
+
+namespace {
+template <typename T, int MT>
+int split_ctas_of(const ChipPlan& P) {
+  static std::atomic<unsigned long long> attr_done;
+  int dev = 0, n_sm = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (smem_attr_once((const void*)k_split_items<T, MT>, kChipSmemMax, attr_done) != cudaSuccess) return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_split_items<T, MT>, P.threads, P.smem) !=
+      cudaSuccess)
+    return 0;
+  return n_sm * std::max(per_sm, 1);
+}
+
+template <typename T, int LK, int MT, int MB>
+int chip_ctas_of(const ChipPlan& P) {
+  static std::atomic<unsigned long long> attr_done;
+  int dev = 0, n_sm = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (smem_attr_once((const void*)k_chip_items<T, LK, MT, MB>, kChipSmemMax, attr_done) !=
+      cudaSuccess)
+    return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_chip_items<T, LK, MT, MB>, P.threads,
+                                                    P.smem) != cudaSuccess)
+    return 0;
+  return n_sm * std::max(per_sm, 1);
+}
+
+// Calls f.operator()<LK, MT, MB>() of the instance of a plan.
+template <typename T, typename F>
+auto chip_instance(const ChipPlan& P, F&& f) {
+  constexpr int M1 = chip_max_threads<T>(1), M2 = chip_max_threads<T>(2);
+  if (P.lk == 0) return f.template operator()<0, chip_max_threads<T>(0), 1>();
+  if (P.lk == 1) return f.template operator()<1, M1, 1>();
+  if constexpr (sizeof(T) == 4) {
+    if (P.threads <= 224) return f.template operator()<2, 224, 2>();
+  }
+  return f.template operator()<2, M2, 1>();
+}
+
+template <typename T>
+struct ChipCtas {
+  const ChipPlan& P;
+  template <int LK, int MT, int MB>
+  int operator()() const {
+    return chip_ctas_of<T, LK, MT, MB>(P);
+  }
+};
+template <typename T>
+struct ChipLaunch {
+  const ChipArgs<T>& A;
+  const ChipPlan& P;
+  const PItem* items;
+  const int2* groups;
+  int n_groups;
+  int* counter;
+  T* X;
+  int grid;
+  double* per_sample;
+  double* trace;
+  const ElecOp& op;
+  cudaStream_t st;
+  template <int LK, int MT, int MB>
+  cudaError_t operator()() const {
+    k_chip_items<T, LK, MT, MB><<<grid, P.threads, P.smem, st>>>(
+        A, items, groups, n_groups, counter, P.rpc, P.slots, X, per_sample,
+        trace, op);
+    return cudaGetLastError();
+  }
+};
+}  // namespace
+
+template <typename T>
+int chip_ctas(const ChipPlan& P) {
+  if (P.split)
+    return P.threads <= 256   ? split_ctas_of<T, 256>(P)
+           : P.threads <= 512 ? split_ctas_of<T, 512>(P)
+                              : split_ctas_of<T, split_max_threads<T>()>(P);
+  return chip_instance<T>(P, ChipCtas<T>{P});
+}
+
+template <typename T>
+cudaError_t launch_chip_items(const ChipArgs<T>& A, const ChipPlan& P, const PItem* items,
+                              const int2* groups, int n_groups, int* counter, T* Xscratch, int ctas,
+                              double* per_sample, double* trace, const ElecOp& op,
+                              cudaStream_t st) {
+  if (n_groups == 0 || ctas == 0) return cudaSuccess;
+  const int g = std::min(ctas, n_groups);
+  if (P.split) {
+    if (P.threads <= 256)
+      k_split_items<T, 256><<<g, P.threads, P.smem, st>>>(A, items, groups, n_groups, counter, P.rpc,
+                                                          P.slots, per_sample, trace, op);
+    else if (P.threads <= 512)
+      k_split_items<T, 512><<<g, P.threads, P.smem, st>>>(A, items, groups, n_groups, counter, P.rpc,
+                                                          P.slots, per_sample, trace, op);
+    else
+      k_split_items<T, split_max_threads<T>()><<<g, P.threads, P.smem, st>>>(
+          A, items, groups, n_groups, counter, P.rpc, P.slots, per_sample, trace, op);
+    return cudaGetLastError();
+  }
+  return chip_instance<T>(P, ChipLaunch<T>{A, P, items, groups, n_groups, counter, Xscratch, g,
+                                           per_sample, trace, op, st});
+}
+
+template <typename T>
+cudaError_t launch_chip_macro(const ChipArgs<T>& A, const ChipPlan& P, const int* row_sys,
+                              const int* row_field, const int2* row_win, int macro,
+                              const int* macro_dev, int rows, const T* psi, T* out, T* X,
+                              long long Zslot, cudaStream_t st) {
+  if (rows == 0) return cudaSuccess;
+  const long long Sr = Zslot >> P.lk;
+  const int threads = (int)((Sr + 31) / 32 * 32);
+  const size_t smem = sizeof(ChipConst<T>) + (size_t)10 * (Sr << P.lk) * sizeof(Cx<T>);
+#define RP_CHIP(LK)                                                                              \
+  {                                                                                              \
+    static std::atomic<unsigned long long> attr_done;                                            \
+    const cudaError_t e = smem_attr_once((const void*)k_chip_macro<T, LK>, kChipSmemMax, attr_done); \
+    if (e != cudaSuccess) return e;                                                              \
+    k_chip_macro<T, LK><<<rows, threads, smem, st>>>(A, row_sys, row_field, row_win, macro,      \
+                                                     macro_dev, psi, out, X, Zslot);             \
+  }
+  if (P.lk == 0) RP_CHIP(0)
+  else if (P.lk == 1) RP_CHIP(1)
+  else RP_CHIP(2)
+#undef RP_CHIP
+  return cudaGetLastError();
+}
+
+#define RP_CHIP_INST(T)                                                                          \
+  template bool chip_plan<T>(long long, int, int, long long, int, int, bool, ChipPlan*);                    \
+  template int chip_ctas<T>(const ChipPlan&);                                                    \
+  template cudaError_t launch_chip_items<T>(const ChipArgs<T>&, const ChipPlan&, const PItem*,   \
+                                            const int2*, int, int*, T*, int, double*, double*,   \
+                                            const ElecOp&, cudaStream_t);                        \
+  template cudaError_t launch_chip_macro<T>(const ChipArgs<T>&, const ChipPlan&, const int*,     \
+                                            const int*, const int2*, int, const int*, int,       \
+                                            const T*, T*, T*, long long, cudaStream_t);
+RP_CHIP_INST(float)
+RP_CHIP_INST(double)
+#undef RP_CHIP_INST
+
+}  // namespace rp

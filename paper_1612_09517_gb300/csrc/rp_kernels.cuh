@@ -163,6 +163,64 @@ cudaError_t launch_persistent_small(const SysTab<T>& S, int aniso, const FieldDe
                                     uint64_t seed, T* Xscratch, int ctas, double* per_sample,
                                     cudaStream_t st);
 
+// ---- whole propagations of isotropic systems that fit one SM (rp_chip.cu) ----
+
+struct ElecOp;
+
+// Tables of a launch: per-system and per-field constants in FP64 (folded and
+// rounded to T in the kernel), real sum coefficients per field r_n then
+// r_n - fl(r_n) (2 n_c values), the time-integral factor.
+template <typename T>
+struct ChipArgs {
+  const HamDev<double>* ham;
+  const LayoutDev* lay;
+  const double* k_S;
+  const FieldDev<double>* fields;
+  const T* coef;
+  const T* L;
+  int ldk;
+  const int2* meta;
+  uint32_t pair_base;
+  const uint32_t* pair_of;
+  int n_c, max_nuc, deterministic;
+  uint64_t seed;
+  const int* sec_rank;
+  const double* sec_scale;
+};
+
+struct ChipPlan {
+  bool split = false;  // one thread per configuration and electron state
+  int lk = 0;        // log2 of the configurations per thread
+  int rpc = 1;       // rows per CTA (items launch)
+  int threads = 0, slots = 0;
+  size_t smem = 0;
+};
+
+// Launch shape for systems of at most Zmax configurations, at least min_half
+// spin-1/2 and at most max_nuc nuclei each, `load` configurations in all over
+// n_items propagations; false if they do not fit one CTA.
+template <typename T>
+bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_items, int n_c,
+               bool trace, ChipPlan* out);
+template <typename T>
+int chip_ctas(const ChipPlan& P);  // CTAs resident at once; before the first launch
+
+// One launch over all groups (groups[i] = first item and count, items of one
+// field); scratch: n_c x slots x 2^lk complex per CTA.  trace != NULL: time-trace sums
+// (as launch_trace) instead of the time integral.
+template <typename T>
+cudaError_t launch_chip_items(const ChipArgs<T>& A, const ChipPlan& P, const PItem* items,
+                              const int2* groups, int n_groups, int* counter, T* Xscratch, int ctas,
+                              double* per_sample, double* trace, const ElecOp& op,
+                              cudaStream_t st);
+// One macro-step of every active row: psi -> out, singlet slices to X (row
+// stride n_c Zslot, any order within a slice).
+template <typename T>
+cudaError_t launch_chip_macro(const ChipArgs<T>& A, const ChipPlan& P, const int* row_sys,
+                              const int* row_field, const int2* row_win, int macro,
+                              const int* macro_dev, int rows, const T* psi, T* out, T* X,
+                              long long Zslot, cudaStream_t st);
+
 // A whole macro-step of every active row of one isotropic FP32 system on a
 // thread-block cluster per row, the row's Chebyshev vectors in distributed
 // shared memory (see k_macro_cluster): reads psi from P, writes the propagated

@@ -319,11 +319,14 @@ std::string plan_field(const HostSystem& s, double B_mT, double t_max, int n_c, 
   std::vector<double> J(n_c + 1);
   bessel_jn(x, n_c, J.data());
   P.coef.resize(n_c);
+  P.rcoef.resize(n_c);
+  const double decay = std::exp(-0.5 * P.kbar * P.h);
   const cplx phase = std::exp(cplx(-0.5 * P.kbar * P.h, -P.E_c * P.h));
   const cplx mi(0.0, -1.0);
   cplx ipow(1.0, 0.0);  // (-i)^n
   for (int n = 0; n < n_c; ++n) {
     P.coef[n] = phase * ipow * ((n == 0 ? 1.0 : 2.0) * J[n]);
+    P.rcoef[n] = decay * ((n == 0 ? 1.0 : 2.0) * J[n]);
     ipow *= mi;
   }
   if (!want_W) return "";

@@ -61,6 +61,7 @@ struct FieldPlan {
   int n_cheb = 0;
   double tail = 0, kbar = 0, kappa = 0, omega = 0;
   std::vector<cplx> coef;  // c_n(h) exp(-kbar h/2), n < n_cheb
+  std::vector<double> rcoef;  // (2 - delta_n0) J_n(dE h) exp(-kbar h/2): c_n = rcoef_n (-i)^n e^{-i E_c h}
   std::vector<cplx> W;     // n_cheb x n_cheb
 };
 

@@ -155,7 +155,7 @@ rp_status rp_tune(rp_system* s, double B, int rows, const rp_options* base, rp_o
   bool cluster_ok = false;
   int default_kernel = o.precision == RP_FP32
                            ? rp::default_kernel_fp32(s->hs, &cluster_ok)
-                           : (Z <= small_max ? (rp::persistent_default(Z, 1) ? 5 : 2) : 1);
+                           : (Z <= small_max ? (rp::persistent_default(Z, 1) || !s->hs.aniso ? 5 : 2) : 1);
   if (default_kernel == 5 && o.graph) default_kernel = 2;  // kernel 0 with graph replay
   for (int nc : ncs)
     for (int g = 0; g <= 1; ++g) {
