@@ -216,12 +216,38 @@ class YieldEngine {
     for (int i = 0; i < ns; ++i) {
       ham[i] = make_ham<T>(*systems[i]);
       hamd[i] = make_ham<double>(*systems[i]);
+      hamd_.push_back(hamd[i]);
       min_half_ = std::min(min_half_, systems[i]->n_half);
       max_nuc_ = std::max(max_nuc_, systems[i]->n_nuc);
       lay[i] = make_layout(*systems[i]);
       kS[i] = systems[i]->k_S;
       Zslot_ = std::max<long long>(Zslot_, systems[i]->Z);
       aniso_ = aniso_ || systems[i]->aniso;
+    }
+    if (aniso_) {
+      // rotated nuclear frames for the per-term kernels: tensors A R and the
+      // matrices that take laboratory amplitudes there
+      std::vector<double> fr((size_t)ns * rp::kMaxNucDev * 200, 0.0);
+      for (int i = 0; i < ns; ++i) {
+        rp::HostSystem h = *systems[i];
+        for (int p = 0; p < h.n_nuc; ++p) {
+          const int k = h.order[p], d = h.two_I[k] + 1;
+          double AR[9];
+          std::vector<rp::cplx> D((size_t)d * d);
+          rp::nuclear_frame(&systems[i]->A[9 * k], h.two_I[k], AR, D.data());
+          for (int q = 0; q < 9; ++q) h.A[9 * k + q] = AR[q];
+          double* o = &fr[((size_t)i * rp::kMaxNucDev + p) * 200];
+          for (int q = 0; q < d * d; ++q) {
+            o[2 * q] = D[q].real();
+            o[2 * q + 1] = D[q].imag();
+          }
+        }
+        hamd_[i] = make_ham<double>(h);
+      }
+      hamd = hamd_;
+      d_frame_ = ar_.get<double>(fr.size());
+      ck(cudaMemcpyAsync(d_frame_, fr.data(), fr.size() * sizeof(double), cudaMemcpyHostToDevice, st_), "h2d frames");
+      h2d += (long long)(fr.size() * sizeof(double));
     }
     d_ham_ = ar_.get<rp::HamDev<T>>(ns);
     d_lay_ = ar_.get<rp::LayoutDev>(ns);
@@ -259,8 +285,13 @@ class YieldEngine {
     }
   }
 
-  void set_fields(const std::vector<rp::FieldPlan>& plans) {
+  // sys_of_field: system of every field (NULL: one system)
+  void set_fields(const std::vector<rp::FieldPlan>& plans,
+                  const std::vector<int>* sys_of_field = nullptr) {
     const int nf = (int)plans.size();
+    plans_ = plans;
+    sys_of_field_.assign(nf, 0);
+    if (sys_of_field) sys_of_field_ = *sys_of_field;
     d_fdev_ = ar_.get<rp::FieldDev<T>>(nf);
     d_coef_ = ar_.get<T>((size_t)nf * n_c_ * 4);
     d_fd_ = ar_.get<rp::FieldDev<double>>(nf);
@@ -351,13 +382,6 @@ class YieldEngine {
       return;
     }
     const int kq = o_.kernel == 5 ? 0 : o_.kernel;
-    const size_t vec = (size_t)Zslot_ * 8;
-    S0_ = ar_.get<T>((size_t)R * vec);
-    S1_ = ar_.get<T>((size_t)R * vec);
-    F1_ = ar_.get<T>((size_t)R * vec);
-    F2_ = ar_.get<T>((size_t)R * vec);
-    amps_ = ar_.get<double>((size_t)R * rp::kMaxNucDev * 10 * 2);
-    row_sys_ = ar_.get<int>(R);
     small_ = (kq == 2 || (kq == 0 && Zslot_ <= rp::small_max_configs<T>())) &&
              Zslot_ <= rp::small_max_configs<T>();
     // a whole macro-step per launch on a thread-block cluster per row (FP32,
@@ -369,6 +393,16 @@ class YieldEngine {
                                  : rp::macro_cluster_default(hf)) &&
                  rp::macro_cluster_max_active(hf) > 0;
     }
+    // the per-term kernels keep the state vectors in planes (rp_term.cu)
+    term_ = !small_ && !cluster_;
+    const long long plane = term_ ? (Zslot_ + 3) & ~3LL : 0;
+    const size_t vec = (size_t)(term_ ? plane : Zslot_) * 8;
+    S0_ = ar_.get<T>((size_t)R * vec);
+    S1_ = ar_.get<T>((size_t)R * vec);
+    F1_ = ar_.get<T>((size_t)R * vec);
+    F2_ = ar_.get<T>((size_t)R * vec);
+    amps_ = ar_.get<double>((size_t)R * rp::kMaxNucDev * 10 * 2);
+    row_sys_ = ar_.get<int>(R);
     // tensor-core Gram integral on request: FP32 with the per-term and cluster
     // kernels (each row's integral covers its own system's Z; the step kernel
     // keeps the padding of the last 16-configuration chunk at zero).  The
@@ -401,8 +435,15 @@ class YieldEngine {
     }
     S_ = rp::SysTab<T>{d_ham_, d_lay_, d_kS_, row_sys_, Zslot_, o_.pair_id, d_pair_, d_err_,
                        sec_rank_, sec_scale_};
+    S_.plane = plane;
+    if (term_) {
+      S_.frame = d_frame_;
+      setup_term(plane);
+    }
     rows_.field = ar_.get<int>(R);
     rows_.win = ar_.get<int2>(R);
+    targs_.row_field = rows_.field;
+    targs_.row_win = rows_.win;
     rows_.sample = ar_.get<long long>(R);
     rows_.out = ar_.get<long long>(R);
     rows_.flag = ar_.get<int>(R);
@@ -531,9 +572,9 @@ class YieldEngine {
       h2d += (long long)R * (3 * sizeof(int) + sizeof(int2) + 2 * sizeof(long long));
     };
     auto init_flagged = [&]() {
-      if (!o_.deterministic)
+      if (!o_.deterministic || (S_.frame && o_.deterministic != 3))
         launched(rp::launch_coherent_amps<T>(S_, rows_.sample, rows_.flag, R, seed_, amps_, nullptr,
-                                             st_), "coherent amplitudes");
+                                             st_, o_.deterministic), "coherent amplitudes");
       launched(rp::launch_init_state<T>(S_, amps_, rows_.sample, rows_.flag, rows_.win, R,
                                         o_.deterministic, S0_, S1_, rows_.integral,
                                         rows_.survival, st_), "initial states");
@@ -715,13 +756,13 @@ class YieldEngine {
          "cluster macro-step kernel");
       n_step = 1;
     }
-    for (int n = 1; n < n_c_ && !small_ && !cluster_; ++n) {
+    for (int n = 1; n < n_c_ && term_; ++n) {
       const int mode = (n == 1) ? rp::MODE_FIRST : (n == n_c_ - 1 ? rp::MODE_LAST : rp::MODE_MID);
-      ck(rp::launch_step<T>(S_, one, aniso_, o_.kernel == 3, d_fdev_, rows_.field, rows_.win, k, mdev, R_,
-                            phi[(n - 1) % 3], n >= 2 ? phi[(n - 2) % 3] : nullptr,
-                            mode == rp::MODE_LAST ? nullptr : phi[n % 3], Q, X_, d_coef_, n_c_, n,
-                            mode, tc_gram_ ? 1 : 0, s),
-         "step kernel");
+      ck(rp::launch_term<T>(targs_, term_lk_, aniso_ != 0, phi[(n - 1) % 3],
+                            n >= 2 ? phi[(n - 2) % 3] : nullptr,
+                            mode == rp::MODE_LAST ? nullptr : phi[n % 3], Q, d_trace_ ? nullptr : X_, k,
+                            mdev, R_, n, mode, s),
+         "term kernel");
       ++n_step;
     }
     if (ev_steps) ck(cudaEventRecord(ev_steps, s), "cudaEventRecord");
@@ -747,6 +788,70 @@ class YieldEngine {
     if (overlap_) ck(cudaEventRecord(ev_int_[k & 1], side_st_), "cudaEventRecord");
     if (mdev) ck(rp::launch_tick(mdev, s), "tick kernel");
     return n_step;
+  }
+
+  // Device tables of the per-term kernels: systems, fields, nuclear fields.
+  void setup_term(long long plane) {
+    const int ns = (int)sys_.size(), nf = (int)plans_.size();
+    term_lk_ = rp::term_lk<T>(aniso_ != 0, min_half_);
+    const int tile = rp::term_tile(term_lk_), nb = aniso_ ? 6 : 2;
+    int lt = 0;
+    while ((1 << lt) < tile) ++lt;
+    std::vector<rp::TermSys<T>> sys(ns);
+    long long tab = 0, tm_max = 1;
+    for (int i = 0; i < ns; ++i) {
+      const rp::HamDev<double>& H = hamd_[i];
+      rp::TermSys<T>& Y = sys[i];
+      std::memset(&Y, 0, sizeof(Y));
+      Y.Z = H.Z;
+      Y.n_half = H.n_half;
+      Y.n_nuc = H.n_nuc;
+      Y.p_in = std::min(H.n_half, lt);
+      // the nuclei whose digit varies within a tile: the innermost lt spin-1/2
+      // nuclei where there are as many, else all (a table of every configuration)
+      const bool whole = H.n_half < lt;
+      Y.tm = whole ? H.Z : tile;
+      Y.p_out = whole ? H.n_nuc : lt;
+      Y.tab = tab;
+      tab += (Y.tm * nb + 3) & ~3LL;
+      tm_max = std::max(tm_max, Y.tm);
+      for (int p = 0; p < H.n_nuc; ++p) {
+        Y.rad |= (unsigned)(H.rad[p] & 1) << p;
+        Y.d[p] = H.d[p];
+        Y.stride[p] = H.stride[p];
+        for (int q = 0; q < 3; ++q) Y.v[p][q] = (T)H.v[p][q];
+      }
+    }
+    std::vector<rp::TermField<T>> tf(nf);
+    for (int f = 0; f < nf; ++f) {
+      const rp::HamDev<double>& H = hamd_[sys_of_field_[f]];
+      const rp::FieldPlan& P = plans_[f];
+      rp::TermField<T>& F = tf[f];
+      std::memset(&F, 0, sizeof(F));
+      const double s2 = 2.0 / P.dE, hJ = 0.5 * H.Je;
+      for (int p = 0; p < H.n_nuc; ++p) {
+        const double c = s2 * (H.d[p] == 3 ? 1.41421356237309504880 : 1.0);
+        F.g[p] = (T)(c * H.U[p][4]);
+        F.ur[p] = (T)(c * H.U[p][2]);
+        F.ui[p] = (T)(c * H.U[p][3]);
+      }
+      F.D[0] = (T)(s2 * (P.omega + hJ - P.E_c));
+      F.D[1] = (T)(s2 * (-hJ - P.E_c));
+      F.D[2] = (T)(s2 * (-P.omega + hJ - P.E_c));
+      F.s2 = (T)s2;
+      F.J = (T)(s2 * H.Je);
+      F.kappa = (T)(s2 * H.kappa);
+    }
+    auto* d_sys = ar_.get<rp::TermSys<T>>(ns);
+    auto* d_tf = ar_.get<rp::TermField<T>>(nf);
+    T* d_tab = ar_.get<T>((size_t)tab);
+    ck(cudaMemcpyAsync(d_sys, sys.data(), ns * sizeof(sys[0]), cudaMemcpyHostToDevice, st_), "h2d systems");
+    ck(cudaMemcpyAsync(d_tf, tf.data(), nf * sizeof(tf[0]), cudaMemcpyHostToDevice, st_), "h2d fields");
+    h2d += (long long)(ns * sizeof(sys[0]) + nf * sizeof(tf[0]));
+    launched(rp::launch_term_table<T>(d_hamd_, d_sys, ns, tm_max, aniso_ != 0, d_tab, st_),
+             "nuclear-field table");
+    targs_ = rp::TermArgs<T>{d_sys, d_tf, d_tab, d_rcoef_, ns == 1 ? nullptr : row_sys_, nullptr, nullptr,
+                             Zslot_, plane, n_c_, tc_gram_ ? 1 : 0};
   }
 
   // Records the launches of a macro-step of parity p (k % 2 == p) into a graph.
@@ -799,6 +904,13 @@ class YieldEngine {
   bool overlap_ = false;
   bool persist_ = false;
   bool chip_ = false;
+  bool term_ = false;
+  int term_lk_ = 0;
+  rp::TermArgs<T> targs_{};
+  std::vector<rp::HamDev<double>> hamd_;  // rotated frames where any system is anisotropic
+  std::vector<rp::FieldPlan> plans_;
+  std::vector<int> sys_of_field_;
+  double* d_frame_ = nullptr;
   rp::ChipPlan cplan_{};
   int min_half_ = 1 << 30, max_nuc_ = 0;
   rp::HamDev<double>* d_hamd_ = nullptr;
@@ -1533,7 +1645,7 @@ rp_status run_batch(int n_sys, rp_system* const* systems, const int* n_fields,
       Arena ar(st);
       YieldEngine<T> eng(group, o, n_c, st, ar, &pairs);
       eng.set_seed(seed);
-      eng.set_fields(gplans);
+      eng.set_fields(gplans, &sys_of_field);
       long long Zmax = 1;
       for (auto* h : group) Zmax = std::max<long long>(Zmax, h->Z);
       rp::HostSystem probe;

@@ -29,6 +29,15 @@ __host__ __device__ __forceinline__ size_t xblk_row_floats(long long Zs, int n_c
   return (size_t)((Zs + kXChunk - 1) / kXChunk) * xrows_pad(n_c) * kXChunk;
 }
 
+// Address of Re x_n(m) (Im is 4 floats further) of row r.
+template <typename T>
+__device__ __forceinline__ T* xblk_addr(T* X, int r, int n, unsigned m, long long Zs, int n_c) {
+  const int row = 2 * n;
+  return X + (size_t)r * xblk_row_floats(Zs, n_c) +
+         (size_t)(m / kXChunk) * xrows_pad(n_c) * kXChunk + (row >> 3) * 128 +
+         ((m % kXChunk) >> 2) * 32 + (row & 7) * 4 + (m & 3);
+}
+
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
   return (unsigned)__cvta_generic_to_shared(p);
 }

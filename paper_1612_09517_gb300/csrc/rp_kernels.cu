@@ -137,15 +137,6 @@ __device__ __forceinline__ void store_singlet(T* x, const Cx<T> (&v)[4]) {
   x[1] = (v[1].im - v[2].im) * r;
 }
 
-// Address of Re x_n(m) (Im is 4 floats further) of row r.
-template <typename T>
-__device__ __forceinline__ T* xblk_addr(T* X, int r, int n, unsigned m, long long Zs, int n_c) {
-  const int row = 2 * n;
-  return X + (size_t)r * xblk_row_floats(Zs, n_c) +
-         (size_t)(m / kXChunk) * xrows_pad(n_c) * kXChunk + (row >> 3) * 128 +
-         ((m % kXChunk) >> 2) * 32 + (row & 7) * 4 + (m & 3);
-}
-
 template <typename T>
 __device__ __forceinline__ void store_singlet_blk(T* x, const Cx<T> (&v)[4]) {
   const T r = T(0.70710678118654752440);
@@ -1488,6 +1479,19 @@ __global__ void __launch_bounds__(ClusterCfg<KPT>::kNT, 1) k_macro_cluster(
   }
 }
 
+// The four electron components of configuration m of row r, in either layout.
+template <typename T>
+__device__ __forceinline__ void load_state(const SysTab<T>& ST, const T* S, int r, long long m,
+                                           Cx<T> (&a)[4]) {
+  if (ST.plane > 0) {
+    const Cx<T>* p = reinterpret_cast<const Cx<T>*>(S) + (size_t)r * 4 * ST.plane + m;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) a[e] = p[(size_t)e * ST.plane];
+  } else {
+    load4(S + ((size_t)r * ST.Zslot + m) * 8, a);
+  }
+}
+
 // Time-resolved observables (Eq. 18 for A = P_S, A = 1 and an electron
 // operator A_e): after macro-step k, every row active in it holds psi(t_i),
 // i = k + 1 - start, in Q; adds |<S|psi>|^2 (P_S = |S><S| on the electrons,
@@ -1504,13 +1508,12 @@ __global__ void __launch_bounds__(256) k_trace(const SysTab<T> ST, const T* __re
   const int2 w = row_win[r];
   if (macro < w.x || macro >= w.y) return;
   const long long Z = ST.ham[ST.row_sys ? ST.row_sys[r] : 0].Z;
-  const T* S = Q + (size_t)r * ST.Zslot * 8;
   const long long z0 = (long long)blockIdx.x * z_per_cta;
   const long long z1 = min(Z, z0 + z_per_cta);
   double ps = 0.0, nn = 0.0, ar = 0.0, ai = 0.0;
   for (long long m = z0 + threadIdx.x; m < z1; m += blockDim.x) {
     Cx<T> a[4];
-    load4(S + m * 8, a);
+    load_state(ST, Q, r, m, a);
     const double dr = (double)a[1].re - (double)a[2].re, di = (double)a[1].im - (double)a[2].im;
     ps += 0.5 * (dr * dr + di * di);
 #pragma unroll
@@ -1561,13 +1564,13 @@ __global__ void __launch_bounds__(256) k_norm(const SysTab<T> ST, const T* __res
   const int r = blockIdx.y;
   if (row_flag && !row_flag[r]) return;
   const long long Z = ST.ham[ST.row_sys ? ST.row_sys[r] : 0].Z;
-  const T* S = ((row_win[r].y & 1) ? S1 : S0) + (size_t)r * ST.Zslot * 8;
+  const T* S = (row_win[r].y & 1) ? S1 : S0;
   const long long z0 = (long long)blockIdx.x * z_per_cta;
   const long long z1 = min(Z, z0 + z_per_cta);
   double s = 0.0;
   for (long long m = z0 + threadIdx.x; m < z1; m += blockDim.x) {
     Cx<T> a[4];
-    load4(S + m * 8, a);
+    load_state(ST, S, r, m, a);
 #pragma unroll
     for (int e = 0; e < 4; ++e)
       s += (double)a[e].re * (double)a[e].re + (double)a[e].im * (double)a[e].im;
@@ -1669,7 +1672,8 @@ __global__ void __launch_bounds__(256) k_stats_weighted(const double* __restrict
 template <typename T>
 __global__ void k_coherent_amps(const SysTab<T> S, const long long* __restrict__ row_sample,
                                 const int* __restrict__ row_flag, int rows, uint64_t seed,
-                                double* __restrict__ amps, double* __restrict__ uv) {
+                                int deterministic, double* __restrict__ amps,
+                                double* __restrict__ uv) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= rows * kMaxNucDev) return;
   const int r = t / kMaxNucDev, p = t % kMaxNucDev;
@@ -1680,7 +1684,28 @@ __global__ void k_coherent_amps(const SysTab<T> S, const long long* __restrict__
   const uint32_t pair = S.pair_of ? S.pair_of[sidx] : S.pair_base + (uint32_t)sidx;
   double* o = amps + ((size_t)r * kMaxNucDev + p) * 10 * 2;
   double u[2];
-  coherent_amp(L, p, pair, (unsigned long long)row_sample[r], seed, o, u);
+  if (deterministic) {  // the basis state's digit (needed in rotated frames only)
+    const int j = (int)((row_sample[r] / L.stride[p]) % L.d[p]);
+    for (int i = 0; i < 2 * L.d[p]; ++i) o[i] = i == 2 * j ? 1.0 : 0.0;
+  } else {
+    coherent_amp(L, p, pair, (unsigned long long)row_sample[r], seed, o, u);
+  }
+  if (S.frame) {
+    const int d = L.d[p];
+    const double* D = S.frame + ((size_t)sidx * kMaxNucDev + p) * 200;
+    double in[20];
+    for (int i = 0; i < 2 * d; ++i) in[i] = o[i];
+    for (int i = 0; i < d; ++i) {
+      double re = 0.0, im = 0.0;
+      for (int j = 0; j < d; ++j) {
+        const double dr = D[2 * (i * d + j)], di = D[2 * (i * d + j) + 1];
+        re += dr * in[2 * j] - di * in[2 * j + 1];
+        im += dr * in[2 * j + 1] + di * in[2 * j];
+      }
+      o[2 * i] = re;
+      o[2 * i + 1] = im;
+    }
+  }
   if (uv) {
     const int k = L.input_index[p];
     uv[((size_t)r * L.n_nuc + k) * 2] = u[0];
@@ -1715,7 +1740,7 @@ __global__ void __launch_bounds__(256) k_init_state(const SysTab<T> S,
     // propagation i carries the i-th state |S, m> of every nuclear-M class
     const long long i = row_sample[r];
     pr = (S.sec_rank[m] == i) ? S.sec_scale[i] : 0.0;
-  } else if (deterministic) {
+  } else if (deterministic && !S.frame) {
     pr = (m == row_sample[r]) ? 1.0 : 0.0;
   } else {
     const double* A = amps + (size_t)r * kMaxNucDev * 10 * 2;
@@ -1736,7 +1761,13 @@ __global__ void __launch_bounds__(256) k_init_state(const SysTab<T> S,
   v[1] = {(T)(s * pr), (T)(s * pi)};
   v[2] = {(T)(-s * pr), (T)(-s * pi)};
   v[3] = {T(0), T(0)};
-  store4(psi + (size_t)r * S.Zslot * 8 + (size_t)m * 8, v);
+  if (S.plane > 0) {
+    Cx<T>* o = reinterpret_cast<Cx<T>*>(psi) + (size_t)r * 4 * S.plane + m;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) o[(size_t)e * S.plane] = v[e];
+  } else {
+    store4(psi + (size_t)r * S.Zslot * 8 + (size_t)m * 8, v);
+  }
 }
 
 // ---- one persistent launch over all work items of small systems ----
@@ -1942,10 +1973,11 @@ inline unsigned grid1(long long n, int b) { return (unsigned)((n + b - 1) / b); 
 template <typename T>
 cudaError_t launch_coherent_amps(const SysTab<T>& S, const long long* row_sample,
                                  const int* row_flag, int rows, uint64_t seed, double* amps,
-                                 double* uv, cudaStream_t st) {
+                                 double* uv, cudaStream_t st, int deterministic) {
   const long long n = (long long)rows * kMaxNucDev;
   if (n == 0) return cudaSuccess;
-  k_coherent_amps<T><<<grid1(n, 128), 128, 0, st>>>(S, row_sample, row_flag, rows, seed, amps, uv);
+  k_coherent_amps<T><<<grid1(n, 128), 128, 0, st>>>(S, row_sample, row_flag, rows, seed,
+                                                      deterministic, amps, uv);
   return cudaGetLastError();
 }
 
@@ -2327,7 +2359,7 @@ cudaError_t launch_zero(double* p, size_t n, cudaStream_t st) {
 }
 
 template cudaError_t launch_coherent_amps<float>(const SysTab<float>&, const long long*, const int*,
-                                                 int, uint64_t, double*, double*, cudaStream_t);
+                                                 int, uint64_t, double*, double*, cudaStream_t, int);
 template cudaError_t launch_init_state<float>(const SysTab<float>&, const double*, const long long*,
                                               const int*, const int2*, int, int, float*, float*, double*,
                                               double*, cudaStream_t);
@@ -2353,7 +2385,7 @@ template cudaError_t launch_trace<float>(const SysTab<float>&, const float*, con
 template cudaError_t launch_finalize<float>(const SysTab<float>&, const RowsDev&, int, double*,
                                             cudaStream_t);
 template cudaError_t launch_coherent_amps<double>(const SysTab<double>&, const long long*, const int*,
-                                                 int, uint64_t, double*, double*, cudaStream_t);
+                                                 int, uint64_t, double*, double*, cudaStream_t, int);
 template cudaError_t launch_init_state<double>(const SysTab<double>&, const double*, const long long*,
                                               const int*, const int2*, int, int, double*, double*, double*,
                                               double*, cudaStream_t);

@@ -87,6 +87,10 @@ struct SysTab {
   // within its nuclear-M class, and 1/sqrt(n_i) of propagation i (n_i states)
   const int* sec_rank = nullptr;
   const double* sec_scale = nullptr;
+  long long plane = 0;  // > 0: state vectors in planes [row][e][plane], else [row][m][e]
+  // rotated nuclear frames (anisotropic systems, or NULL): per system and layout
+  // position the 10 x 10 complex matrix that takes laboratory amplitudes to it
+  const double* frame = nullptr;
 };
 
 // ---- launchers (return cudaGetLastError after the launch) ----
@@ -98,7 +102,7 @@ struct SysTab {
 template <typename T>
 cudaError_t launch_coherent_amps(const SysTab<T>& S, const long long* row_sample,
                                  const int* row_flag, int rows, uint64_t seed, double* amps,
-                                 double* uv, cudaStream_t st);
+                                 double* uv, cudaStream_t st, int deterministic = 0);
 
 template <typename T>
 cudaError_t launch_init_state(const SysTab<T>& S, const double* amps, const long long* row_sample,
@@ -220,6 +224,57 @@ cudaError_t launch_chip_macro(const ChipArgs<T>& A, const ChipPlan& P, const int
                               const int* row_field, const int2* row_win, int macro,
                               const int* macro_dev, int rows, const T* psi, T* out, T* X,
                               long long Zslot, cudaStream_t st);
+
+// ---- one Chebyshev term per launch (rp_term.cu) ----
+
+// Constants of one field, 2/dE folded in: g_p = a_p/2 (isotropic) or the real
+// entry of U_p, (ur, ui) its complex entry (rotated nuclear frame), both x sqrt 2
+// for spin 1; D = the uniform part of the diagonal less the shift; s2 = 2/dE.
+template <typename T>
+struct alignas(16) TermField {
+  T g[kMaxNucDev], ur[kMaxNucDev], ui[kMaxNucDev];
+  T D[3], s2, J, kappa, pad[2];
+};
+
+// One system: p_in = spin-1/2 nuclei whose partner lies in the tile; the table of
+// nuclear fields covers m mod tm (nuclei p < p_out) from entry tab.
+template <typename T>
+struct alignas(16) TermSys {
+  long long Z, tab, tm, pad;
+  int n_half, n_nuc, p_in, p_out;
+  unsigned rad;
+  int pad2[3];
+  int d[kMaxNucDev];
+  long long stride[kMaxNucDev];
+  T v[kMaxNucDev][3];
+};
+
+template <typename T>
+struct TermArgs {
+  const TermSys<T>* sys;
+  const TermField<T>* field;
+  const T* btab;
+  const T* coef;  // r_n with the sign of (-i)^n, then r_n - fl(r_n)
+  const int* row_sys;
+  const int* row_field;
+  const int2* row_win;
+  long long Zslot, plane;  // row slot and plane stride in configurations
+  int n_c;
+  int xblk;  // slices in the tensor-core Gram layout
+};
+
+template <typename T>
+int term_lk(bool aniso, int min_half);
+int term_tile(int lk);  // configurations per block
+template <typename T>
+cudaError_t launch_term_table(const HamDev<double>* ham, const TermSys<T>* sys, int n_sys,
+                              long long tm_max, bool aniso, T* btab, cudaStream_t st);
+// One term over every active row: vectors in planes [row][e][plane], slices to X
+// (may be NULL); modes as k_cheb_step.
+template <typename T>
+cudaError_t launch_term(const TermArgs<T>& A, int lk, bool aniso, const T* cur, const T* prev,
+                        T* next, T* acc, T* X, int macro, const int* macro_dev, int rows, int n,
+                        int mode, cudaStream_t st);
 
 // A whole macro-step of every active row of one isotropic FP32 system on a
 // thread-block cluster per row, the row's Chebyshev vectors in distributed

@@ -149,6 +149,104 @@ void spin_ops(int two_I, std::vector<cplx>& Ix, std::vector<cplx>& Iy, std::vect
 
 }  // namespace
 
+void nuclear_frame(const double* A, int two_I, double* AR, cplx* D) {
+  // columns r_x, r_y, r_z of R: r_z along the z row of A, r_y along what is left
+  // of the y row (unit axes where a row vanishes)
+  auto dot = [](const double* a, const double* b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; };
+  double r[3][3];  // r[c] = column c
+  auto unit = [&](const double* v, double* o, const double* avoid) {
+    double w[3] = {v[0], v[1], v[2]};
+    if (avoid) {
+      const double q = dot(w, avoid);
+      for (int i = 0; i < 3; ++i) w[i] -= q * avoid[i];
+    }
+    const double n = std::sqrt(dot(w, w)), ref = std::sqrt(dot(v, v));
+    if (!(n > 1e-12 * ref) || n == 0.0) return false;
+    for (int i = 0; i < 3; ++i) o[i] = w[i] / n;
+    if (avoid) {  // once more: w may have lost digits
+      const double q = dot(o, avoid);
+      for (int i = 0; i < 3; ++i) o[i] -= q * avoid[i];
+      const double m = std::sqrt(dot(o, o));
+      for (int i = 0; i < 3; ++i) o[i] /= m;
+    }
+    return true;
+  };
+  const double axes[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
+  if (!unit(A + 6, r[2], nullptr))
+    for (int i = 0; i < 3; ++i) r[2][i] = axes[2][i];
+  if (!unit(A + 3, r[1], r[2])) {
+    int k = 0;  // the axis least along r_z
+    for (int i = 1; i < 3; ++i)
+      if (std::fabs(r[2][i]) < std::fabs(r[2][k])) k = i;
+    unit(axes[k], r[1], r[2]);
+  }
+  for (int i = 0; i < 3; ++i)
+    r[0][i] = r[1][(i + 1) % 3] * r[2][(i + 2) % 3] - r[1][(i + 2) % 3] * r[2][(i + 1) % 3];
+  double T[3][3];
+  for (int a = 0; a < 3; ++a)
+    for (int c = 0; c < 3; ++c) T[a][c] = dot(A + 3 * a, r[c]);
+  T[1][0] = T[2][0] = T[2][1] = 0.0;
+  // turn about the new z axis: u -> u e^{i phi}; U_10 = (u_x + i u_y) / 2 real
+  const cplx ux(0.5 * T[0][0], -0.5 * T[0][1]), uy(0.0, -0.5 * T[1][1]), I1(0.0, 1.0);
+  const cplx u10 = 0.5 * (ux + I1 * uy);
+  const double phi = std::abs(u10) > 0.0 ? -std::arg(u10) : 0.0;
+  const double cp = std::cos(phi), sp = std::sin(phi);
+  double q[3][3];  // columns of R
+  for (int i = 0; i < 3; ++i) {
+    q[0][i] = cp * r[0][i] + sp * r[1][i];
+    q[1][i] = -sp * r[0][i] + cp * r[1][i];
+    q[2][i] = r[2][i];
+  }
+  for (int a = 0; a < 3; ++a) {
+    AR[3 * a] = cp * T[a][0] + sp * T[a][1];
+    AR[3 * a + 1] = -sp * T[a][0] + cp * T[a][1];
+    AR[3 * a + 2] = T[a][2];
+  }
+  // V = exp(-i theta n.sigma / 2) of R as a unit quaternion (w, x, y, z):
+  // V = w - i (x sx + y sy + z sz)
+  auto R = [&](int i, int j) { return q[j][i]; };
+  double w4[4] = {1 + R(0, 0) + R(1, 1) + R(2, 2), 1 + R(0, 0) - R(1, 1) - R(2, 2),
+                  1 - R(0, 0) + R(1, 1) - R(2, 2), 1 - R(0, 0) - R(1, 1) + R(2, 2)};
+  int k = 0;
+  for (int i = 1; i < 4; ++i)
+    if (w4[i] > w4[k]) k = i;
+  const double s4 = 0.5 * std::sqrt(w4[k]), f = 0.25 / s4;
+  double Q[4];
+  if (k == 0) {
+    Q[0] = s4; Q[1] = f * (R(2, 1) - R(1, 2)); Q[2] = f * (R(0, 2) - R(2, 0)); Q[3] = f * (R(1, 0) - R(0, 1));
+  } else if (k == 1) {
+    Q[0] = f * (R(2, 1) - R(1, 2)); Q[1] = s4; Q[2] = f * (R(0, 1) + R(1, 0)); Q[3] = f * (R(0, 2) + R(2, 0));
+  } else if (k == 2) {
+    Q[0] = f * (R(0, 2) - R(2, 0)); Q[1] = f * (R(0, 1) + R(1, 0)); Q[2] = s4; Q[3] = f * (R(1, 2) + R(2, 1));
+  } else {
+    Q[0] = f * (R(1, 0) - R(0, 1)); Q[1] = f * (R(0, 2) + R(2, 0)); Q[2] = f * (R(1, 2) + R(2, 1)); Q[3] = s4;
+  }
+  const double qn = std::sqrt(Q[0] * Q[0] + Q[1] * Q[1] + Q[2] * Q[2] + Q[3] * Q[3]);
+  for (double& v : Q) v /= qn;
+  // V^dagger = w + i (x sx + y sy + z sz) on (up, down)
+  const cplx G[2][2] = {{cplx(Q[0], Q[3]), cplx(Q[2], Q[1])}, {cplx(-Q[2], Q[1]), cplx(Q[0], -Q[3])}};
+  // spin I: |I, M = I - j> = u^(2I-j) v^j / sqrt((2I-j)! j!); u, v go to the columns of G
+  const int d = two_I + 1;
+  std::vector<double> fact(d, 1.0);
+  for (int i = 1; i < d; ++i) fact[i] = fact[i - 1] * i;
+  for (int j = 0; j < d; ++j) {
+    std::vector<cplx> pol(d, 0.0);  // coefficient of u^(2I-i) v^i
+    pol[0] = 1.0;
+    int deg = 0;
+    for (int m = 0; m < two_I; ++m) {
+      const cplx a = m < two_I - j ? G[0][0] : G[0][1], b = m < two_I - j ? G[1][0] : G[1][1];
+      for (int i = deg; i >= 0; --i) {
+        const cplx p = pol[i];
+        pol[i] = p * a;
+        pol[i + 1] += p * b;
+      }
+      ++deg;
+    }
+    for (int i = 0; i < d; ++i)
+      D[i * d + j] = pol[i] * std::sqrt(fact[two_I - i] * fact[i] / (fact[two_I - j] * fact[j]));
+  }
+}
+
 std::string finish_system(HostSystem& s) {
   const int n = s.n_nuc;
   s.order.resize(n);

@@ -69,6 +69,14 @@ struct FieldPlan {
 // Returns an empty string on success or an error message.
 std::string finish_system(HostSystem& s);
 
+// Rotated frame of one nucleus: a rotation R with A R upper triangular and the
+// lower-left entry of U = sum_a u_a S_a, u_a = ((A R)_ax - i (A R)_ay) / 2, real
+// and its diagonal zero (S.A.I = S.(A R).I' with I' = R^T I).  A and AR are 3 x 3
+// row-major; D (d x d complex, row-major, d = two_I + 1, basis j = I - M) takes the
+// nucleus's amplitudes to the frame: D = V^dagger for V = exp(-i theta n.I) of R.
+// Electron operators, yields and norms do not depend on the frame.
+void nuclear_frame(const double* A, int two_I, double* AR, cplx* D);
+
 // Plan one field.  Returns an empty string on success or an error message.
 // want_coef fills coef; want_W also fills W (the entry points that integrate on
 // the device leave it out: launch_plan_integral forms the weights there).
