@@ -358,12 +358,27 @@ class YieldEngine {
     persist_ = o_.kernel == 5 || (o_.kernel == 0 && !o_.graph &&
                                   (chip_ || rp::persistent_default(Zslot_, (int)sys_.size())));
     if (!fits || (!chip_ && (o_.deterministic == 3 || d_trace_))) persist_ = false;
+    // larger isotropic FP32 systems: the same on thread-block clusters, eager and
+    // with kernel left to choose (kernel = 4 asks for macro-step launches)
+    // (also where one CTA would need four configurations per thread, which spill)
+    if (sizeof(T) == 4 && !aniso_ && (fits ? persist_ && cplan_.lk == 2
+                                           : (o_.kernel == 0 || o_.kernel == 5) && !o_.graph &&
+                                                 o_.gram != 2)) {
+      bool spin1 = true;
+      for (const auto* h : sys_) spin1 = spin1 && h->n_half + h->n_one == h->n_nuc;
+      rp::ChipPlan q;
+      if (rp::chip_cluster_plan(Zslot_, min_half_, max_nuc_, R, n_c_, spin1, &q) &&
+          rp::chip_ctas<T>(q) > 0) {
+        cplan_ = q;
+        chip_ = persist_ = true;
+      }
+    }
     d_err_ = ar_.get<int>(1);
     ck(cudaMemsetAsync(d_err_, 0, sizeof(int), st_), "cudaMemsetAsync");
     if (persist_ && chip_) {
       pctas_ = rp::chip_ctas<T>(cplan_);
       if (pctas_ <= 0) throw CudaFail{RP_ECUDA, "on-chip kernel: no device"};
-      pctas_ = std::min(pctas_, (R + cplan_.rpc - 1) / cplan_.rpc);
+      pctas_ = std::min(pctas_, ((R + cplan_.rpc - 1) / cplan_.rpc) << cplan_.cb);
       d_counter_ = ar_.get<int>(1);
       if (!d_trace_) {
         if (!cplan_.split) Xp_ = ar_.get<T>((size_t)pctas_ * n_c_ * ((size_t)cplan_.slots << cplan_.lk) * 2);
@@ -700,10 +715,11 @@ class YieldEngine {
   // Kernel path taken (rp_stats.kernel_path): 5 persistent, 4 cluster, 2 one
   // CTA per row, 3 staged per-term, 1 per-term.
   int kernel_path() const {
-    return persist_ ? 5 : cluster_ ? 4 : (small_ ? 2 : (o_.kernel == 3 ? 3 : 1));
+    if (persist_) return Zslot_ <= rp::small_max_configs<T>() ? 5 : 4;
+    return cluster_ ? 4 : (small_ ? 2 : (o_.kernel == 3 ? 3 : 1));
   }
   // Rows propagated at once: CTAs of the persistent launch, else allocated rows.
-  int rows_used() const { return persist_ ? pctas_ : R_; }
+  int rows_used() const { return persist_ ? pctas_ >> cplan_.cb : R_; }
 
   // Time-resolved sums (launch_trace) after every macro-step, 4 doubles per
   // time point, with an optional electron operator; eager launches.
@@ -1007,7 +1023,7 @@ void fill_stats(rp_stats* stats, const YieldEngine<T>& eng, long long items, int
   stats->graph_launches = eng.graph_launches;
   stats->row_terms = eng.row_terms;
   stats->propagations = items;
-  stats->rows = eng.kernel_path() == 5 ? eng.rows_used() : R;
+  stats->rows = eng.rows_used();
   stats->n_cheb = n_c;
   stats->kernel_path = eng.kernel_path();
   float ms = 0.f;

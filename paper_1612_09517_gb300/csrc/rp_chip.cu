@@ -21,6 +21,14 @@
 // phase exp(-i E_c h) of the propagator is left out (no yield, survival or
 // expectation value depends on it), which makes the coefficients of the sum
 // real: c_n = r_n (-i)^n; cf holds r_n with the sign of (-i)^n for n mod 4 >= 2.
+//
+// Rows that exceed one SM (FP32, Z up to 8 x 2048) are split over the 2^cb CTAs of
+// a thread-block cluster by the cb outermost spin-1/2 nuclei (layout positions lb =
+// n_half - cb and up): the local configuration l of CTA `rank` is
+//   m = (l >> lb) << (lb + cb) | rank << lb | l mod 2^lb,
+// the partner under nucleus lb + i is the same slot of CTA rank XOR 2^i (read
+// through distributed shared memory, the direction being the CTA's), and one
+// cluster barrier per term takes the place of the block barrier.
 #include <algorithm>
 #include <cstring>
 
@@ -33,6 +41,55 @@
 namespace rp {
 
 namespace {
+
+__device__ __forceinline__ unsigned chip_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Barrier of the block or, split over a cluster, of the cluster (release /
+// acquire: shared-memory writes before it are seen by every CTA after it).
+template <int CB>
+__device__ __forceinline__ void chip_barrier() {
+  if constexpr (CB > 0)
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  else
+    __syncthreads();
+}
+// The two halves of the cluster's barrier, for work that needs neither.
+template <int CB>
+__device__ __forceinline__ void chip_arrive() {
+  if constexpr (CB > 0) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+template <int CB>
+__device__ __forceinline__ void chip_wait() {
+  if constexpr (CB > 0) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  else __syncthreads();
+}
+// Address in the cluster's shared window of the CTA `rank`.
+__device__ __forceinline__ unsigned chip_peer(unsigned a, unsigned rank) {
+  unsigned ra;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+  return ra;
+}
+// The KPT values of electron state e at a slot of a peer's buffer (base: its
+// shared-cluster address); volatile, so it stays between the barriers.
+template <int LK>
+__device__ __forceinline__ void peer_get(unsigned base, int S, int e, int slot,
+                                         Cx<float> (&q)[1 << LK]) {
+  using V = Vec<float, LK>;
+  const unsigned a = base + (unsigned)(((e * V::G) * S + slot) * (int)sizeof(typename V::Pack));
+#pragma unroll
+  for (int g = 0; g < V::G; ++g) {
+    const unsigned p = a + (unsigned)(g * S * (int)sizeof(typename V::Pack));
+    if constexpr (V::W == 2)
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(q[2 * g].re), "=f"(q[2 * g].im), "=f"(q[2 * g + 1].re), "=f"(q[2 * g + 1].im)
+                   : "r"(p));
+    else
+      asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(q[g].re), "=f"(q[g].im) : "r"(p));
+  }
+}
 
 // Partner "up" (nuclear quantum number one lower: S_- I_+ brings it here) adds
 // its components (u0, u1) to targets (t0, t1), "down" the reverse:
@@ -102,6 +159,58 @@ __device__ __forceinline__ void flip_one(Cx<T> (&y)[1 << LK][4], int rr, T g, co
   }
 }
 
+constexpr int kChipMaxCb = 3;
+
+// Partner values of the nuclei that select the CTA, loaded at the start of a term
+// (a remote load takes far longer than a local one) and used in their turn.
+template <int LK, int CB>
+struct PeerVals {
+  Cx<float> q[CB > 0 ? CB : 1][2][1 << LK];
+};
+template <int LK, int CB>
+__device__ __forceinline__ void peer_load(PeerVals<LK, CB>& v, unsigned own, unsigned rank,
+                                          unsigned rad, int S, int sl) {
+#pragma unroll
+  for (int i = 0; i < CB; ++i) {
+    const unsigned peer = chip_peer(own, rank ^ (1u << i));
+    const bool down = (rank >> i) & 1u, r1 = (rad >> i) & 1u;
+    peer_get<LK>(peer, S, down ? (r1 ? 1 : 2) : 0, sl, v.q[i][0]);
+    peer_get<LK>(peer, S, down ? 3 : (r1 ? 2 : 1), sl, v.q[i][1]);
+  }
+}
+template <int LK, int CB>
+__device__ __forceinline__ void peer_add(Cx<float> (&y)[1 << LK][4], const PeerVals<LK, CB>& v,
+                                         unsigned rank, unsigned rad, const float* g) {
+  constexpr int KPT = 1 << LK;
+#pragma unroll
+  for (int i = 0; i < CB; ++i) {
+    {
+      const bool down = (rank >> i) & 1u, r1 = (rad >> i) & 1u;
+      const float gi = g[i];
+#pragma unroll
+      for (int c = 0; c < KPT; ++c) {
+        if (!r1) {
+          if (down) {
+            madd(y[c][0], gi, v.q[i][0][c]);
+            madd(y[c][1], gi, v.q[i][1][c]);
+          } else {
+            madd(y[c][2], gi, v.q[i][0][c]);
+            madd(y[c][3], gi, v.q[i][1][c]);
+          }
+        } else {
+          if (down) {
+            madd(y[c][0], gi, v.q[i][0][c]);
+            madd(y[c][2], gi, v.q[i][1][c]);
+          } else {
+            madd(y[c][1], gi, v.q[i][0][c]);
+            madd(y[c][3], gi, v.q[i][1][c]);
+          }
+        }
+      }
+    }
+  }
+}
+
 // Diagonal 2 (H_mm - E_c) / dE of the four electron states of configuration m.
 template <typename T>
 __device__ __forceinline__ void chip_diag(const HamDev<double>& H, const FieldDev<double>& F,
@@ -129,23 +238,23 @@ struct alignas(16) ChipConst {
   T J, kappa;       // 2 J / dE, 2 kappa / dE
   int d[kMaxNucDev], st[kMaxNucDev];  // dimension and stride in slots (spins above 1)
   unsigned rad;                       // radical of nucleus p in bit p
-  int n_half, n_one, n_nuc;
+  int n_half, n_one, n_nuc;           // n_half: spin-1/2 nuclei of the CTA's own slots
 };
 
 template <typename T>
 __device__ void chip_const(ChipConst<T>& K, const HamDev<double>& H, const FieldDev<double>& F,
-                           int lk, int tid) {
+                           int lk, int cb, int tid) {
   if (tid < H.n_nuc) {
     const int p = tid;
     const double g = 2.0 * F.s * H.U[p][4] * (H.d[p] == 3 ? 1.41421356237309504880 : 1.0);
     K.g[p] = (T)g;
     K.d[p] = H.d[p];
-    K.st[p] = (int)(H.stride[p] >> lk);
+    K.st[p] = (int)(H.stride[p] >> (lk + cb));
   }
   if (tid == 0) {
     K.J = (T)(2.0 * F.s * H.Je);
     K.kappa = (T)(2.0 * F.s * H.kappa);
-    K.n_half = H.n_half;
+    K.n_half = H.n_half - cb;
     K.n_one = H.n_one;
     K.n_nuc = H.n_nuc;
     unsigned m = 0;
@@ -179,12 +288,18 @@ __device__ __forceinline__ void chip_get(const Cx<T>* b, int S, int slot, Cx<T> 
 // One term: u = phi_n from phi_{n-1} (own values a, partners in cur) and, unless
 // FIRST, phi_{n-2} (own entries of prev).  dt: diagonals, four per
 // configuration.  t: slot within the row, base: the row's first slot.
-template <typename T, int LK>
+template <typename T, int LK, int CB>
 __device__ __forceinline__ void chip_term(const ChipConst<T>& K, Cx<T> (&y)[1 << LK][4],
                                           const Cx<T> (&a)[1 << LK][4], const T* dt,
                                           const Cx<T>* cur, const Cx<T>* prev, bool first, int S,
                                           int base, int t, unsigned dig) {
   constexpr int KPT = 1 << LK;
+  // four configurations per thread have no registers to hold them all term
+  constexpr bool kEarly = CB > 0 && LK == 1;
+  PeerVals<LK, kEarly ? CB : 0> pv;
+  unsigned rank = 0;
+  if constexpr (CB > 0) rank = chip_rank();
+  if constexpr (kEarly) peer_load<LK, CB>(pv, smem_u32(cur), rank, K.rad >> K.n_half, S, base + t);
   if constexpr (sizeof(T) == 8) {
     if (first) {
 #pragma unroll
@@ -247,7 +362,7 @@ __device__ __forceinline__ void chip_term(const ChipConst<T>& K, Cx<T> (&y)[1 <<
   unsigned rm = K.rad >> LK;
   const int nh = K.n_half;
   int bit = 1;
-#pragma unroll 1
+#pragma unroll LK == 1 ? 2 : 1
   for (int p = LK; p < nh; ++p, bit <<= 1, rm >>= 1) {
     const int sl = base + (t ^ bit), rr = (int)(rm & 1u);
     const bool down = (t & bit) != 0;
@@ -259,19 +374,56 @@ __device__ __forceinline__ void chip_term(const ChipConst<T>& K, Cx<T> (&y)[1 <<
       flip_either<T, LK>(y, rr, down, g, cur, S, sl);
     }
   }
+  if constexpr (CB > 0) {  // the nuclei that select the CTA
+    if constexpr (kEarly) {
+      peer_add<LK, CB>(y, pv, rank, rm, K.g + nh);
+    } else {
+      PeerVals<LK, CB> v;
+      peer_load<LK, CB>(v, smem_u32(cur), rank, rm, S, base + t);
+      peer_add<LK, CB>(y, v, rank, rm, K.g + nh);
+    }
+    rm >>= CB;
+  }
   // spin-1 nuclei: digit j, up from j + 1, down from j - 1 (FP32: a missing
   // partner reads the own slot with weight zero)
-  const int n1 = nh + K.n_one;
+  const int n0 = nh + CB, n1 = n0 + K.n_one;
   int st = bit;
 #pragma unroll 1
-  for (int p = nh; p < n1; ++p, st *= 3, rm >>= 1, dig >>= 2) {
+  for (int p = n0; p < n1; ++p, st *= 3, rm >>= 1, dig >>= 2) {
     const unsigned j = dig & 3u;
     const int rr = (int)(rm & 1u);
     const T g = K.g[p];
-    if (sizeof(T) == 4 || j < 2u)
-      flip_one<T, LK, true>(y, rr, j < 2u ? g : T(0), cur, S, base + (j < 2u ? t + st : t));
-    if (sizeof(T) == 4 || j > 0u)
-      flip_one<T, LK, false>(y, rr, j > 0u ? g : T(0), cur, S, base + (j > 0u ? t - st : t));
+    if constexpr (sizeof(T) == 4 && LK < 2) {  // both partners' loads before either product
+      const int su = base + (j < 2u ? t + st : t), sd = base + (j > 0u ? t - st : t);
+      const T gu = j < 2u ? g : T(0), gd = j > 0u ? g : T(0);
+      Cx<T> u0[KPT], u1[KPT], d0[KPT], d1[KPT];
+      Vec<T, LK>::get(cur, S, 0, su, u0);
+      Vec<T, LK>::get(cur, S, rr ? 2 : 1, su, u1);
+      Vec<T, LK>::get(cur, S, rr ? 1 : 2, sd, d0);
+      Vec<T, LK>::get(cur, S, 3, sd, d1);
+      if (rr == 0) {
+#pragma unroll
+        for (int c = 0; c < KPT; ++c) {
+          madd(y[c][2], gu, u0[c]);
+          madd(y[c][3], gu, u1[c]);
+          madd(y[c][0], gd, d0[c]);
+          madd(y[c][1], gd, d1[c]);
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < KPT; ++c) {
+          madd(y[c][1], gu, u0[c]);
+          madd(y[c][3], gu, u1[c]);
+          madd(y[c][0], gd, d0[c]);
+          madd(y[c][2], gd, d1[c]);
+        }
+      }
+    } else {
+      if (sizeof(T) == 4 || j < 2u)
+        flip_one<T, LK, true>(y, rr, j < 2u ? g : T(0), cur, S, base + (j < 2u ? t + st : t));
+      if (sizeof(T) == 4 || j > 0u)
+        flip_one<T, LK, false>(y, rr, j > 0u ? g : T(0), cur, S, base + (j > 0u ? t - st : t));
+    }
   }
   // any other spin
   if (n1 < K.n_nuc) {
@@ -345,7 +497,7 @@ __device__ __forceinline__ void chip_singlet(T* x, int xs, const Cx<T> (&y)[KPT]
 // false) only keep the barriers.  xn: the thread's entry of the row's slices,
 // stride between slices xstride (complex), between the thread's configurations
 // xs.  Not inlined: the caller's live values would spill inside the term loop.
-template <typename T, int LK>
+template <typename T, int LK, int CB>
 __device__ __noinline__ void chip_macro(int S, int base, int t, bool on, unsigned dig,
                                         const T* __restrict__ cf, int n_c, T* xn, size_t xstride,
                                         int xs, bool store_x) {
@@ -366,32 +518,38 @@ __device__ __noinline__ void chip_macro(int S, int base, int t, bool on, unsigne
       for (int e = 0; e < 4; ++e) acc[c][e] = {T(0), T(0)};
     chip_accumulate<T, KPT, false>(acc, a, cf[0], cl[0]);
   }
-  __syncthreads();
+  chip_barrier<CB>();
 #pragma unroll 1
   for (int n = 1; n < n_c; n += 2) {  // n_c is even: n odd, then n + 1 even
     if (on) {
-      chip_term<T, LK>(K, y, a, dt, b0, b1, n == 1, S, base, t, dig);
+      chip_term<T, LK, CB>(K, y, a, dt, b0, b1, n == 1, S, base, t, dig);
       chip_put<T, LK>(b1, S, base + t, y);
+    }
+    chip_arrive<CB>();
+    if (on) {
       if (store_x) chip_singlet<T, KPT>(xn + (size_t)n * xstride * 2, xs, y);
       chip_accumulate<T, KPT, true>(acc, y, cf[n], cl[n]);
     }
-    __syncthreads();
+    chip_wait<CB>();
     if (n + 1 < n_c) {
       if (on) {
-        chip_term<T, LK>(K, a, y, dt, b1, b0, false, S, base, t, dig);
+        chip_term<T, LK, CB>(K, a, y, dt, b1, b0, false, S, base, t, dig);
         chip_put<T, LK>(b0, S, base + t, a);
+      }
+      chip_arrive<CB>();
+      if (on) {
         if (store_x) chip_singlet<T, KPT>(xn + (size_t)(n + 1) * xstride * 2, xs, a);
         chip_accumulate<T, KPT, false>(acc, a, cf[n + 1], cl[n + 1]);
       }
-      __syncthreads();
+      chip_wait<CB>();
     }
   }
   if (on) chip_put<T, LK>(b0, S, base + t, acc);
 }
 
 // Two-bit digits of the spin-1 nuclei of slot t.
-__device__ __forceinline__ unsigned chip_digits(const HamDev<double>& H, int t, int lk) {
-  unsigned q = (unsigned)t >> (H.n_half - lk), dig = 0;
+__device__ __forceinline__ unsigned chip_digits(const HamDev<double>& H, int t, int lk, int cb) {
+  unsigned q = (unsigned)t >> (H.n_half - cb - lk), dig = 0;
   for (int i = 0; i < H.n_one; ++i) {
     dig |= (q % 3u) << (2 * i);
     q /= 3u;
@@ -399,11 +557,12 @@ __device__ __forceinline__ unsigned chip_digits(const HamDev<double>& H, int t, 
   return dig;
 }
 
-// Most threads of a CTA, which bounds the registers: FP32 128, FP64 255 with
+// Most threads of a CTA, which bounds the registers: FP32 96 to 128, FP64 255 with
 // several configurations per thread.
 template <typename T>
 __host__ __device__ constexpr int chip_max_threads(int lk) {
-  return sizeof(T) == 4 || lk == 0 ? 512 : 256;
+  if (sizeof(T) == 8) return lk == 0 ? 512 : 256;
+  return lk == 1 ? 640 : 512;
 }
 
 // Survival and time-trace sums of a thread's configurations.
@@ -453,10 +612,9 @@ __device__ __forceinline__ double warp_sum(double v) {
 // rows' sums.  The singlet slices of a macro-step
 // go to the CTA's scratch and come back as the thread's own entries for the
 // time integral (rp_integral.cu).
-// MT, MB: most threads of a CTA and CTAs per SM, which bound the registers (two
-// CTAs of 224 threads hold 144 registers each: at 128 the spills of four
-// configurations per thread took 15 % of the instructions and missed L1).
-template <typename T, int LK, int MT, int MB>
+// MT, MB: most threads of a CTA and CTAs per SM, which bound the registers.  CB > 0: a
+// row per cluster of 2^CB CTAs (rpc = 1), groups drawn by the cluster's rank 0.
+template <typename T, int LK, int MT, int MB, int CB>
 __global__ void __launch_bounds__(MT, MB) k_chip_items(
     const ChipArgs<T> A, const PItem* __restrict__ items, const int2* __restrict__ groups,
     int n_groups, int* __restrict__ counter, int rpc, int S, T* __restrict__ Xscratch, double* __restrict__ per_sample, double* __restrict__ trace,
@@ -473,20 +631,28 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
   // the integral's ring: buffer 1, 4 KPT slices per thread
   auto* ring = reinterpret_cast<typename SliceVal<T>::type*>(buf + (size_t)4 * KPT * S) + threadIdx.x;
   const int tid = threadIdx.x;
+  const unsigned rank = CB > 0 ? chip_rank() : 0u;
+  constexpr int cb = CB;
   T* xc = Xscratch + (size_t)blockIdx.x * A.n_c * KPT * S * 2;
   for (;;) {
-    if (tid == 0) s_group = atomicAdd(counter, 1);
-    __syncthreads();
-    const int gi = s_group;
-    if (gi >= n_groups) break;  // the same for the whole CTA
+    // rank 0 draws the group for its cluster
+    if (tid == 0 && rank == 0) s_group = atomicAdd(counter, 1);
+    chip_barrier<CB>();
+    int gi = s_group;
+    if constexpr (CB > 0) {
+      asm volatile("ld.shared::cluster.s32 %0, [%1];"
+                   : "=r"(gi)
+                   : "r"(chip_peer(smem_u32(&s_group), 0)));
+    }
+    if (gi >= n_groups) break;  // the same for the whole CTA (cluster)
     const int2 grp = groups[gi];
     const PItem I0 = items[grp.x];
     const HamDev<double>& H = A.ham[I0.sys];
     const FieldDev<double> F = A.fields[I0.field];
-    const int Sr = (int)(H.Z >> LK);
+    const int Sr = (int)(H.Z >> (LK + cb));
     const int row = tid / Sr, t = tid - row * Sr, base = row * Sr;
     const bool on = row < grp.y;
-    chip_const<T>(K, H, F, LK, tid);
+    chip_const<T>(K, H, F, LK, cb, tid);
     if (tid < 2 * rpc) sums[tid] = 0.0;
     const LayoutDev& Ly = A.lay[I0.sys];
     if (!A.deterministic)
@@ -501,11 +667,13 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
     unsigned dig = 0;
     if (on) {
       Cx<T> a[KPT][4];
-      dig = chip_digits(H, t, LK);
+      dig = chip_digits(H, t, LK, cb);
       const long long sample = items[grp.x + row].sample;
 #pragma unroll
       for (int c = 0; c < KPT; ++c) {
-        const unsigned m = ((unsigned)t << LK) | (unsigned)c;
+        const unsigned l = ((unsigned)t << LK) | (unsigned)c;
+        const int lb = H.n_half - cb;
+        const unsigned m = CB > 0 ? (((l >> lb) << (lb + cb)) | (rank << lb) | (l & ((1u << lb) - 1u))) : l;
         T d[4];
         chip_diag<T>(H, F, m, d);
 #pragma unroll
@@ -548,7 +716,7 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
     const size_t xrow = (size_t)KPT * S;
 #pragma unroll 1
     for (int km = 0; km < I0.n_macro; ++km) {
-      chip_macro<T, LK>(S, base, t, on, dig, cf, A.n_c, xc + (size_t)(base + t) * 2,
+      chip_macro<T, LK, CB>(S, base, t, on, dig, cf, A.n_c, xc + (size_t)(base + t) * 2,
                         xrow, S, integrate);
       if (integrate) {
         for (int k0 = 0; k0 < mt.x; k0 += KB) {
@@ -589,9 +757,19 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
       atomicAdd(&sums[2 * row], integral);
       atomicAdd(&sums[2 * row + 1], chip_norm<T, KPT>(a));
     }
-    __syncthreads();
-    if (tid < grp.y) {
-      const double phS = A.k_S[I0.sys] * sums[2 * tid], surv = sums[2 * tid + 1];
+    chip_barrier<CB>();
+    if (tid < grp.y && rank == 0) {
+      double si = sums[2 * tid], surv = sums[2 * tid + 1];
+      if constexpr (CB > 0) {
+        for (unsigned k = 1; k < (1u << cb); ++k) {
+          const unsigned a = chip_peer(smem_u32(&sums[2 * tid]), k);
+          double u, v;
+          asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(u), "=d"(v) : "r"(a));
+          si += u;
+          surv += v;
+        }
+      }
+      const double phS = A.k_S[I0.sys] * si;
       double* o = per_sample + items[grp.x + tid].out * 3;
       o[0] = phS;
       o[1] = 1.0 - surv - phS;  // Haberkorn: d|psi|^2/dt = -k_S <P_S> - k_T <P_T>
@@ -599,6 +777,7 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
     }
     __syncthreads();
   }
+  if constexpr (CB > 0) chip_barrier<CB>();  // no CTA leaves while a peer may read its memory
 }
 
 // ---- few configurations per SM: one thread per configuration and electron state ----
@@ -881,13 +1060,13 @@ __global__ void __launch_bounds__(chip_max_threads<T>(LK), 1) k_chip_macro(
   const FieldDev<double> F = A.fields[f];
   const int Sr = (int)(H.Z >> LK);
   const bool on = tid < Sr;
-  chip_const<T>(K, H, F, LK, tid);
+  chip_const<T>(K, H, F, LK, 0, tid);
   Cx<T>* buf = reinterpret_cast<Cx<T>*>(chip_smem + sizeof(ChipConst<T>));
   T* dt = reinterpret_cast<T*>(buf + (size_t)8 * KPT * Sr);
   unsigned dig = 0;
   if (on) {
     Cx<T> a[KPT][4];
-    dig = chip_digits(H, tid, LK);
+    dig = chip_digits(H, tid, LK, 0);
 #pragma unroll
     for (int c = 0; c < KPT; ++c) {
       const unsigned m = ((unsigned)tid << LK) | (unsigned)c;
@@ -902,7 +1081,7 @@ __global__ void __launch_bounds__(chip_max_threads<T>(LK), 1) k_chip_macro(
     chip_put<T, LK>(buf, Sr, tid, a);
   }
   __syncthreads();
-  chip_macro<T, LK>(Sr, 0, tid, on, dig,
+  chip_macro<T, LK, 0>(Sr, 0, tid, on, dig,
                     A.coef + (size_t)f * 2 * A.n_c, A.n_c,
                     X + ((size_t)r * A.n_c * Zslot + tid) * 2, (size_t)Zslot, Sr, true);
   if (on) {
@@ -979,6 +1158,34 @@ bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_
   return false;
 }
 
+// Split over clusters (FP32): the smallest cluster whose CTAs hold their share,
+// larger while the rows alone leave SMs idle.  Two configurations per thread
+// where 640 threads (96 registers) suffice, else four.
+bool chip_cluster_plan(long long Zmax, int min_half, int max_nuc, int n_items, int n_c, bool spin1_only,
+                       ChipPlan* out) {
+  if (!spin1_only) return false;
+  bool found = false;
+  for (int cb = 1; cb <= kChipMaxCb; ++cb) {
+    const long long Zl = Zmax >> cb;
+    for (int lk = 1; lk <= 2; ++lk) {
+      if (min_half - cb < lk || (Zl >> lk) > (lk == 1 ? 640 : 512) || (lk == 2 && cb < 3)) continue;
+      ChipPlan P;
+      P.cb = cb;
+      P.lk = lk;
+      P.slots = (int)(Zl >> lk);
+      P.threads = (P.slots + 31) / 32 * 32;
+      P.smem = lk == 1 ? chip_smem_bytes<float, 1>(P.slots, 1, n_c, max_nuc)
+                       : chip_smem_bytes<float, 2>(P.slots, 1, n_c, max_nuc);
+      if (P.smem > (size_t)kChipSmemMax) continue;
+      if (found && ((long long)n_items << cb) > 152) return true;
+      *out = P;
+      found = true;
+      break;
+    }
+  }
+  return found;
+}
+
 namespace {
 template <typename T, int MT>
 int split_ctas_of(const ChipPlan& P) {
@@ -993,39 +1200,72 @@ int split_ctas_of(const ChipPlan& P) {
   return n_sm * std::max(per_sm, 1);
 }
 
-template <typename T, int LK, int MT, int MB>
+// Launch configuration of a plan: `grid` CTAs, in clusters of 2^cb.
+cudaLaunchConfig_t chip_cfg(const ChipPlan& P, int grid, cudaStream_t st, cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3((unsigned)P.threads, 1, 1);
+  cfg.dynamicSmemBytes = P.smem;
+  cfg.stream = st;
+  if (P.cb > 0) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1u << P.cb;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  return cfg;
+}
+
+template <typename T, int LK, int MT, int MB, int CB>
 int chip_ctas_of(const ChipPlan& P) {
   static std::atomic<unsigned long long> attr_done;
+  const auto kf = k_chip_items<T, LK, MT, MB, CB>;
   int dev = 0, n_sm = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (smem_attr_once((const void*)k_chip_items<T, LK, MT, MB>, kChipSmemMax, attr_done) !=
-      cudaSuccess)
-    return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_chip_items<T, LK, MT, MB>, P.threads,
-                                                    P.smem) != cudaSuccess)
+  if (smem_attr_once((const void*)kf, kChipSmemMax, attr_done) != cudaSuccess) return 0;
+  if (CB > 0) {
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = chip_cfg(P, 1 << P.cb, nullptr, at);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kf, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return n << P.cb;
+  }
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, P.threads, P.smem) != cudaSuccess)
     return 0;
   return n_sm * std::max(per_sm, 1);
 }
 
-// Calls f.operator()<LK, MT, MB>() of the instance of a plan.
+// Calls f.operator()<LK, MT, MB, CB>() of the instance of a plan.
 template <typename T, typename F>
 auto chip_instance(const ChipPlan& P, F&& f) {
   constexpr int M1 = chip_max_threads<T>(1), M2 = chip_max_threads<T>(2);
-  if (P.lk == 0) return f.template operator()<0, chip_max_threads<T>(0), 1>();
-  if (P.lk == 1) return f.template operator()<1, M1, 1>();
   if constexpr (sizeof(T) == 4) {
-    if (P.threads <= 224) return f.template operator()<2, 224, 2>();
+    if (P.cb > 0) {
+      if (P.lk == 2) return f.template operator()<2, 512, 1, 3>();
+      if (P.cb == 1) return f.template operator()<1, 640, 1, 1>();
+      return P.cb == 2 ? f.template operator()<1, 640, 1, 2>() : f.template operator()<1, 640, 1, 3>();
+    }
   }
-  return f.template operator()<2, M2, 1>();
+  if (P.lk == 0) return f.template operator()<0, chip_max_threads<T>(0), 1, 0>();
+  if constexpr (sizeof(T) == 4) {
+    if (P.lk == 1 && P.threads <= 512) return f.template operator()<1, 512, 1, 0>();
+  }
+  if (P.lk == 1) return f.template operator()<1, M1, 1, 0>();
+  return f.template operator()<2, M2, 1, 0>();
 }
 
 template <typename T>
 struct ChipCtas {
   const ChipPlan& P;
-  template <int LK, int MT, int MB>
+  template <int LK, int MT, int MB, int CB>
   int operator()() const {
-    return chip_ctas_of<T, LK, MT, MB>(P);
+    return chip_ctas_of<T, LK, MT, MB, CB>(P);
   }
 };
 template <typename T>
@@ -1042,12 +1282,12 @@ struct ChipLaunch {
   double* trace;
   const ElecOp& op;
   cudaStream_t st;
-  template <int LK, int MT, int MB>
+  template <int LK, int MT, int MB, int CB>
   cudaError_t operator()() const {
-    k_chip_items<T, LK, MT, MB><<<grid, P.threads, P.smem, st>>>(
-        A, items, groups, n_groups, counter, P.rpc, P.slots, X, per_sample,
-        trace, op);
-    return cudaGetLastError();
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = chip_cfg(P, grid, st, at);
+    return cudaLaunchKernelEx(&cfg, k_chip_items<T, LK, MT, MB, CB>, A, items, groups, n_groups,
+                              counter, P.rpc, P.slots, X, per_sample, trace, op);
   }
 };
 }  // namespace
@@ -1067,7 +1307,7 @@ cudaError_t launch_chip_items(const ChipArgs<T>& A, const ChipPlan& P, const PIt
                               double* per_sample, double* trace, const ElecOp& op,
                               cudaStream_t st) {
   if (n_groups == 0 || ctas == 0) return cudaSuccess;
-  const int g = std::min(ctas, n_groups);
+  const int g = std::min(ctas, n_groups << P.cb);
   if (P.split) {
     if (P.threads <= 256)
       k_split_items<T, 256><<<g, P.threads, P.smem, st>>>(A, items, groups, n_groups, counter, P.rpc,

@@ -195,6 +195,7 @@ struct ChipArgs {
 struct ChipPlan {
   bool split = false;  // one thread per configuration and electron state
   int lk = 0;        // log2 of the configurations per thread
+  int cb = 0;        // log2 of the CTAs per row (a cluster)
   int rpc = 1;       // rows per CTA (items launch)
   int threads = 0, slots = 0;
   size_t smem = 0;
@@ -206,6 +207,9 @@ struct ChipPlan {
 template <typename T>
 bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_items, int n_c,
                bool trace, ChipPlan* out);
+// The same for systems of spin-1/2 and spin-1 nuclei beyond one CTA, in FP32.
+bool chip_cluster_plan(long long Zmax, int min_half, int max_nuc, int n_items, int n_c, bool spin1_only,
+                       ChipPlan* out);
 template <typename T>
 int chip_ctas(const ChipPlan& P);  // CTAs resident at once; before the first launch
 
