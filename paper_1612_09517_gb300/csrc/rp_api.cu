@@ -355,6 +355,17 @@ class YieldEngine {
     const bool fits = Zslot_ <= rp::small_max_configs<T>();
     chip_ = fits && !aniso_ && rp::chip_plan<T>(Zslot_, min_half_, max_nuc_, (long long)R * Zslot_,
                                                 R, n_c_, d_trace_ != nullptr, &cplan_);
+    // anisotropic systems: one thread per configuration and electron state.  The
+    // macro-step launches (kernel = 2) keep the generic kernel and, in FP32, so does
+    // kernel = 5, which agrees with them to a part of the FP32 rounding.
+    if (fits && aniso_ && ((o_.kernel == 0 && !o_.graph) || (o_.kernel == 5 && sizeof(T) == 8))) {
+      rp::ChipPlan q;
+      if (rp::aniso_plan<T>(Zslot_, min_half_, max_nuc_, R, n_c_, d_trace_ != nullptr, &q) &&
+          rp::chip_ctas<T>(q) > 0) {
+        cplan_ = q;
+        chip_ = true;
+      }
+    }
     persist_ = o_.kernel == 5 || (o_.kernel == 0 && !o_.graph &&
                                   (chip_ || rp::persistent_default(Zslot_, (int)sys_.size())));
     if (!fits || (!chip_ && (o_.deterministic == 3 || d_trace_))) persist_ = false;
@@ -381,7 +392,7 @@ class YieldEngine {
       pctas_ = std::min(pctas_, ((R + cplan_.rpc - 1) / cplan_.rpc) << cplan_.cb);
       d_counter_ = ar_.get<int>(1);
       if (!d_trace_) {
-        if (!cplan_.split) Xp_ = ar_.get<T>((size_t)pctas_ * n_c_ * ((size_t)cplan_.slots << cplan_.lk) * 2);
+        if (!cplan_.split && !cplan_.aniso) Xp_ = ar_.get<T>((size_t)pctas_ * n_c_ * ((size_t)cplan_.slots << cplan_.lk) * 2);
         plan_integral(false);
       }
       return;
@@ -469,7 +480,7 @@ class YieldEngine {
   rp::ChipArgs<T> chip_args() const {
     return rp::ChipArgs<T>{d_hamd_, d_lay_, d_kS_, d_fd_, d_rcoef_, d_L_, rp::integral_ldk(n_c_),
                            d_meta_, o_.pair_id, d_pair_, n_c_, max_nuc_, o_.deterministic, seed_,
-                           sec_rank_, sec_scale_};
+                           sec_rank_, sec_scale_, d_frame_};
   }
 
   // The weights of the time integral of every field, formed on the device: their

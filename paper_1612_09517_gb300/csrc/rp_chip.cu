@@ -1034,6 +1034,349 @@ __global__ void __launch_bounds__(MT, 1) k_split_items(
   }
 }
 
+// ---- anisotropic systems: one thread per configuration and electron state ----
+//
+// The same for tensors of any form, in rotated nuclear frames (rp_plan.cpp,
+// nuclear_frame): U = [[0, u], [w, 0]] with w real, so each electron state takes
+// one component of each partner.  A row is split over 2^CB CTAs by the outermost
+// spin-1/2 nuclei where rows are few (in FP64 the chip's 304 FP64 lanes are the
+// bound, and 32 rows on 32 SMs leave most of them idle) or long.
+template <typename T>
+struct alignas(16) AnisoConst {
+  T w[kMaxNucDev], ur[kMaxNucDev], ui[kMaxNucDev];  // 2/dE folded in, x sqrt 2 for spin 1
+  int d[kMaxNucDev], st[kMaxNucDev];
+  T J, kappa;
+  unsigned rad;
+  int lb, n_nuc;  // spin-1/2 nuclei of the CTA's own slots, all nuclei
+};
+
+template <typename T>
+struct AnisoRow {
+  T d;                   // diagonal
+  T c2r, c2i, c1r, c1i;  // couplings to states e ^ 2 and e ^ 1 of the own configuration
+};
+
+// u += (wr + i wi) q
+template <typename T>
+__device__ __forceinline__ void madd_c(Cx<T>& u, T wr, T wi, const Cx<T>& q) {
+  u.re = fma(wr, q.re, fma(-wi, q.im, u.re));
+  u.im = fma(wr, q.im, fma(wi, q.re, u.im));
+}
+
+__device__ __forceinline__ Cx<float> peer_value(unsigned a, float) {
+  Cx<float> v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.re), "=f"(v.im) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ Cx<double> peer_value(unsigned a, double) {
+  Cx<double> v;
+  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(v.re), "=d"(v.im) : "r"(a));
+  return v;
+}
+
+// y (phi_{n-2}) becomes phi_n; a = phi_{n-1} of this thread, l its local configuration.
+template <typename T, int CB>
+__device__ __forceinline__ void aniso_term(const AnisoConst<T>& K, const AnisoRow<T>& R, Cx<T>& y,
+                                           const Cx<T>& a, const Cx<T>* cur, int S, int slot, int l,
+                                           int e, unsigned rank) {
+  Cx<T> pv[CB > 0 ? CB : 1];
+#pragma unroll
+  for (int i = 0; i < CB; ++i) {  // remote values first: they take longest
+    const int flip = ((K.rad >> (K.lb + i)) & 1u) ? 1 : 2;
+    pv[i] = peer_value(chip_peer(smem_u32(cur + (e ^ flip) * S + slot), rank ^ (1u << i)), T(0));
+  }
+  Cx<T> u;
+  if (sizeof(T) == 4) u = {R.d * a.re, R.d * a.im};
+  else u = {fma(R.d, a.re, -y.re), fma(R.d, a.im, -y.im)};
+  madd_c(u, R.c2r, R.c2i, cur[(e ^ 2) * S + slot]);
+  madd_c(u, R.c1r, R.c1i, cur[(e ^ 1) * S + slot]);
+  const bool mid = e == 1 || e == 2;
+  if (K.J != T(0) && mid) madd_s(u, K.J, cur[(3 - e) * S + slot]);
+  if (K.kappa != T(0)) madd_i(u, K.kappa, mid ? cur[(3 - e) * S + slot] : a);
+  // low states (electron up) take the high ones through u (partner above) or w
+  // (below), high states the low ones through w or conj(u)
+  auto add = [&](int p, bool hi, bool down, T f, const Cx<T>& q) {
+    const bool c = hi == down;
+    const T ui = K.ui[p];
+    madd_c(u, f * (c ? K.ur[p] : K.w[p]), c ? (hi ? -f * ui : f * ui) : T(0), q);
+  };
+  unsigned rm = K.rad;
+#pragma unroll 2
+  for (int p = 0; p < K.lb; ++p, rm >>= 1) {
+    const int flip = (rm & 1u) ? 1 : 2;
+    const bool down = (l >> p) & 1;
+    add(p, (e & flip) != 0, down, T(1), cur[(e ^ flip) * S + (slot ^ (1 << p))]);
+  }
+#pragma unroll
+  for (int i = 0; i < CB; ++i, rm >>= 1) {
+    const int flip = (rm & 1u) ? 1 : 2;
+    add(K.lb + i, (e & flip) != 0, (rank >> i) & 1u, T(1), pv[i]);
+  }
+  unsigned q = (unsigned)l >> K.lb;
+#pragma unroll 1
+  for (int p = K.lb + CB; p < K.n_nuc; ++p, rm >>= 1) {
+    const unsigned dd = (unsigned)K.d[p], j = dd == 3u ? q % 3u : q % dd;
+    q = dd == 3u ? q / 3u : q / dd;
+    const int flip = (rm & 1u) ? 1 : 2, st = K.st[p];
+    const bool hi = (e & flip) != 0;
+    T fu = T(1), fd = T(1);
+    if (dd != 3u) {
+      const T I = T(0.5) * T(dd - 1), M = I - T(j);
+      fu = sqrt(I * (I + 1) - M * (M - 1));
+      fd = sqrt(I * (I + 1) - M * (M + 1));
+    }
+    if (j + 1u < dd) add(p, hi, false, fu, cur[(e ^ flip) * S + slot + st]);
+    if (j > 0u) add(p, hi, true, fd, cur[(e ^ flip) * S + slot - st]);
+  }
+  if (sizeof(T) == 4) y = {u.re - y.re, u.im - y.im};
+  else y = u;
+}
+
+template <typename T, int CB, int MT>
+__global__ void __launch_bounds__(MT, 1) k_split_aniso(
+    const ChipArgs<T> A, const PItem* __restrict__ items, const int2* __restrict__ groups,
+    int n_groups, int* __restrict__ counter, int S, double* __restrict__ per_sample,
+    double* __restrict__ trace, const ElecOp op) {
+  extern __shared__ __align__(16) unsigned char chip_smem[];
+  __shared__ int s_group;
+  __shared__ __align__(16) double sums[2];
+  __shared__ AnisoConst<T> K;
+  // two buffers [e][S], slices [n_c][S], factor [n_c][32], amplitudes
+  Cx<T>* buf = reinterpret_cast<Cx<T>*>(chip_smem);
+  Cx<T>* xs = buf + (size_t)8 * S;
+  T* sl = reinterpret_cast<T*>(xs + (trace ? 0 : (size_t)A.n_c * S));
+  double* amps = reinterpret_cast<double*>(sl + (trace ? 0 : (size_t)A.n_c * 32));
+  const int tid = threadIdx.x;
+  const unsigned rank = CB > 0 ? chip_rank() : 0u;
+  for (;;) {
+    if (tid == 0 && rank == 0) s_group = atomicAdd(counter, 1);
+    chip_barrier<CB>();
+    int gi = s_group;
+    if constexpr (CB > 0) {
+      asm volatile("ld.shared::cluster.s32 %0, [%1];"
+                   : "=r"(gi)
+                   : "r"(chip_peer(smem_u32(&s_group), 0)));
+    }
+    if (gi >= n_groups) break;  // the same for the whole cluster
+    const PItem I0 = items[groups[gi].x];
+    const HamDev<double>& H = A.ham[I0.sys];
+    const FieldDev<double> F = A.fields[I0.field];
+    const LayoutDev& Ly = A.lay[I0.sys];
+    const int Zl = (int)(H.Z >> CB), lb = H.n_half - CB;
+    const int e = tid / Zl, l = tid - e * Zl;
+    const bool on = e < 4;
+    const unsigned m = CB > 0 ? (((unsigned)l >> lb) << (lb + CB)) | (rank << lb) |
+                                    ((unsigned)l & ((1u << lb) - 1u))
+                              : (unsigned)l;
+    if (tid < H.n_nuc) {
+      const int p = tid;
+      const double c = 2.0 * F.s * (H.d[p] == 3 ? 1.41421356237309504880 : 1.0);
+      K.w[p] = (T)(c * H.U[p][4]);
+      K.ur[p] = (T)(c * H.U[p][2]);
+      K.ui[p] = (T)(c * H.U[p][3]);
+      K.d[p] = H.d[p];
+      K.st[p] = (int)(H.stride[p] >> CB);
+      // amplitudes of psi(0) in the rotated frames (Eqs. 15, 17)
+      double in[20], u[2];
+      if (A.deterministic) {
+        const int j = (int)((I0.sample / Ly.stride[p]) % Ly.d[p]);
+        for (int q = 0; q < 2 * Ly.d[p]; ++q) in[q] = q == 2 * j ? 1.0 : 0.0;
+      } else {
+        const uint32_t pair = A.pair_of ? A.pair_of[I0.sys] : A.pair_base + (uint32_t)I0.sys;
+        coherent_amp(Ly, p, pair, (unsigned long long)I0.sample, A.seed, in, u);
+      }
+      const int dn = Ly.d[p];
+      const double* D = A.frame + ((size_t)I0.sys * kMaxNucDev + p) * 200;
+      for (int i = 0; i < dn; ++i) {
+        double re = 0.0, im = 0.0;
+        for (int j = 0; j < dn; ++j) {
+          const double dr = D[2 * (i * dn + j)], di = D[2 * (i * dn + j) + 1];
+          re += dr * in[2 * j] - di * in[2 * j + 1];
+          im += dr * in[2 * j + 1] + di * in[2 * j];
+        }
+        amps[p * 20 + 2 * i] = re;
+        amps[p * 20 + 2 * i + 1] = im;
+      }
+    }
+    if (tid == 0) {
+      K.J = (T)(2.0 * F.s * H.Je);
+      K.kappa = (T)(2.0 * F.s * H.kappa);
+      unsigned rd = 0;
+      for (int p = 0; p < H.n_nuc; ++p) rd |= (unsigned)(H.rad[p] & 1) << p;
+      K.rad = rd;
+      K.lb = lb;
+      K.n_nuc = H.n_nuc;
+    }
+    if (tid < 2) sums[tid] = 0.0;
+    const T* cf = A.coef + (size_t)I0.field * 2 * A.n_c;
+    const T* cl = cf + A.n_c;
+    int2 mt = make_int2(0, 0);
+    const T* Lf = nullptr;
+    if (!trace) {
+      mt = A.meta[I0.field];
+      Lf = A.L + (size_t)I0.field * A.n_c * A.ldk;
+      if (mt.x <= 32) stage_factor<T, 32>(sl, Lf, A.ldk, (mt.y + 1) & ~1, 0, tid, blockDim.x);
+    }
+    const int n_e = (mt.y + 1) & ~1;
+    __syncthreads();
+    AnisoRow<T> R{};
+    Cx<T> a = {T(0), T(0)};
+    if (on) {
+      double b[2][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+      double pr = 1.0, pi = 0.0;
+      unsigned q = m;
+      for (int p = 0; p < H.n_nuc; ++p) {
+        const unsigned dd = (unsigned)H.d[p], j = q % dd;
+        q /= dd;
+        const double M = 0.5 * (double)(dd - 1) - (double)j;
+        for (int k = 0; k < 3; ++k) {
+          if (H.rad[p] == 0) b[0][k] += M * H.v[p][k];
+          else b[1][k] += M * H.v[p][k];
+        }
+        const double ar = amps[p * 20 + 2 * j], ai = amps[p * 20 + 2 * j + 1];
+        const double nr = pr * ar - pi * ai;
+        pi = pr * ai + pi * ar;
+        pr = nr;
+      }
+      const double sp = 0.5 * (b[0][2] + b[1][2]), sm = 0.5 * (b[0][2] - b[1][2]);
+      const double hJ = 0.5 * H.Je;
+      const double dz = e == 0 ? F.omega + hJ + sp : e == 1 ? -hJ + sm : e == 2 ? -hJ - sm
+                                                                              : -F.omega + hJ - sp;
+      R.d = (T)(2.0 * (F.s * dz - F.sh_re));
+      // S_1 . b_1 and S_2 . b_2 off the diagonal: (b_x -+ i b_y) / 2
+      R.c2r = (T)(F.s * b[0][0]);
+      R.c2i = (T)(F.s * ((e & 2) ? b[0][1] : -b[0][1]));
+      R.c1r = (T)(F.s * b[1][0]);
+      R.c1i = (T)(F.s * ((e & 1) ? b[1][1] : -b[1][1]));
+      const double s = e == 1 ? 0.70710678118654752440 : -0.70710678118654752440;
+      if (e == 1 || e == 2) a = {(T)(s * pr), (T)(s * pi)};
+    }
+    double integral = 0.0;
+    Cx<T>* b0 = buf + (size_t)(on ? e : 0) * S + l;  // this thread's entries
+    Cx<T>* b1 = b0 + (size_t)4 * S;
+    const bool keeps = !trace && on && e == 0;  // stores the slices
+    auto slice = [&](int n, const Cx<T>* b) {
+      const Cx<T> p1 = b[S + l], p2 = b[2 * S + l];
+      const T r = T(0.70710678118654752440);
+      xs[(size_t)n * S + l] = {(p1.re - p2.re) * r, (p1.im - p2.im) * r};
+    };
+#pragma unroll 1
+    for (int km = 0; km < I0.n_macro; ++km) {
+      Cx<T> y = {T(0), T(0)}, acc = {T(0), T(0)};
+      if (on) {
+        *b0 = a;
+        if (sizeof(T) == 4) madd_s(acc, cl[0], a);
+        madd_s(acc, cf[0], a);
+      }
+      chip_barrier<CB>();
+#pragma unroll 1
+      for (int n = 1; n < A.n_c; n += 2) {
+        if (on) {
+          aniso_term<T, CB>(K, R, y, a, buf, S, l, l, e, rank);
+          if (n == 1) {
+            y.re *= T(0.5);
+            y.im *= T(0.5);
+          }
+          *b1 = y;
+        }
+        chip_arrive<CB>();
+        if (on) {
+          if (keeps) slice(n - 1, buf);
+          if (sizeof(T) == 4) madd_i(acc, -cl[n], y);
+          madd_i(acc, -cf[n], y);
+        }
+        chip_wait<CB>();
+        if (n + 1 < A.n_c) {
+          if (on) {
+            aniso_term<T, CB>(K, R, a, y, buf + (size_t)4 * S, S, l, l, e, rank);
+            *b0 = a;
+          }
+          chip_arrive<CB>();
+          if (on) {
+            if (keeps) slice(n, buf + (size_t)4 * S);
+            if (sizeof(T) == 4) madd_s(acc, cl[n + 1], a);
+            madd_s(acc, cf[n + 1], a);
+          }
+          chip_wait<CB>();
+        }
+      }
+      a = acc;
+      if (!trace) {
+        if (keeps) slice(A.n_c - 1, buf + (size_t)4 * S);  // n_c is even: the last n is odd
+        __syncthreads();
+        for (int k0 = 0; k0 < mt.x; k0 += 32) {
+          if (mt.x > 32) {  // several blocks of columns: staged in turn
+            __syncthreads();
+            stage_factor<T, 32>(sl, Lf, A.ldk, n_e, k0, tid, blockDim.x);
+            __syncthreads();
+          }
+          if (on) {
+            constexpr int N = sizeof(T) == 4 ? 4 : 8;  // eight columns
+            typename ProjAcc<T>::type yr[N], yi[N];
+#pragma unroll
+            for (int k = 0; k < N; ++k) yr[k] = yi[k] = typename ProjAcc<T>::type{};
+            const T* lc = sl + 8 * e;
+#pragma unroll 2
+            for (int n = 0; n < n_e; n += 2) {
+              const Cx<T> v = xs[(size_t)n * S + l], w = xs[(size_t)(n + 1) * S + l];
+              proj_add(yr, yi, lc + n * 32, v.re, v.im);
+              proj_add(yr, yi, lc + (n + 1) * 32, w.im, -w.re);
+            }
+            integral += proj_norm8(yr, yi);
+          }
+        }
+      } else {
+        // every state of the configuration for the observables: psi(t + h) once more
+        // (no peer reads buffer 0 after the last barrier)
+        if (on) *b0 = a;
+        __syncthreads();
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        if (on && e == 0) {
+          const Cx<T> c4[4] = {buf[l], buf[S + l], buf[2 * S + l], buf[3 * S + l]};
+          trace_terms<T>(c4, op, v);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (q >= 2 && !op.on) break;
+          const double w = warp_sum(v[q]);
+          if ((tid & 31) == 0 && w != 0.0) atomicAdd(trace + 4 * (km + 1) + q, w);
+        }
+        __syncthreads();
+      }
+    }
+    if (on) {
+      atomicAdd(&sums[0], integral);
+      atomicAdd(&sums[1], (double)a.re * (double)a.re + (double)a.im * (double)a.im);
+    }
+    chip_barrier<CB>();
+    if (tid == 0 && rank == 0) {
+      double si = sums[0], surv = sums[1];
+      if constexpr (CB > 0) {
+        for (unsigned k = 1; k < (1u << CB); ++k) {
+          const unsigned p = chip_peer(smem_u32(&sums[0]), k);
+          double u, v;
+          asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(u), "=d"(v) : "r"(p));
+          si += u;
+          surv += v;
+        }
+      }
+      const double phS = A.k_S[I0.sys] * si;
+      double* o = per_sample + I0.out * 3;
+      o[0] = phS;
+      o[1] = 1.0 - surv - phS;
+      o[2] = surv;
+    }
+    __syncthreads();
+  }
+  if constexpr (CB > 0) chip_barrier<CB>();  // no CTA leaves while a peer may read its memory
+}
+
+template <typename T>
+size_t aniso_smem_bytes(int S, int n_c, int max_nuc, bool trace) {
+  return (size_t)(8 + (trace ? 0 : n_c)) * S * sizeof(Cx<T>) +
+         (trace ? 0 : (size_t)n_c * 32 * sizeof(T)) + (size_t)max_nuc * 20 * sizeof(double);
+}
+
 template <typename T>
 size_t split_smem_bytes(int S, int rpc, int n_c, int max_nuc, bool trace) {
   return (size_t)(8 + (trace ? 0 : n_c)) * S * sizeof(Cx<T>) +
@@ -1293,7 +1636,95 @@ struct ChipLaunch {
 }  // namespace
 
 template <typename T>
+bool aniso_plan(long long Zmax, int min_half, int max_nuc, int n_items, int n_c, bool trace,
+                ChipPlan* out) {
+  bool found = false;
+  for (int cb = 0; cb <= kChipMaxCb && cb <= min_half; ++cb) {
+    const long long Zl = Zmax >> cb;
+    if (4 * Zl > split_max_threads<T>()) continue;
+    ChipPlan P;
+    P.aniso = true;
+    P.cb = cb;
+    P.slots = (int)Zl;
+    P.threads = (int)((4 * Zl + 31) / 32 * 32);
+    P.smem = aniso_smem_bytes<T>(P.slots, n_c, max_nuc, trace);
+    if (P.smem > (size_t)kChipSmemMax) continue;
+    // a larger cluster only while the rows alone leave SMs idle and each CTA
+    // keeps a warp per scheduler
+    if (found && (((long long)n_items << cb) > 152 || P.threads < 128)) return true;
+    *out = P;
+    found = true;
+  }
+  return found;
+}
+
+namespace {
+template <typename T, int CB, int MT>
+int aniso_ctas_of(const ChipPlan& P) {
+  static std::atomic<unsigned long long> attr_done;
+  const auto kf = k_split_aniso<T, CB, MT>;
+  int dev = 0, n_sm = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (smem_attr_once((const void*)kf, kChipSmemMax, attr_done) != cudaSuccess) return 0;
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = chip_cfg(P, 1 << P.cb, nullptr, at);
+  const cudaError_t e = CB > 0 ? cudaOccupancyMaxActiveClusters(&n, kf, &cfg)
+                               : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kf, P.threads, P.smem);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return CB > 0 ? n << CB : n_sm * std::max(n, 1);
+}
+
+// Calls f.operator()<CB, MT>() of the instance of an anisotropic plan.
+template <typename T, typename F>
+auto aniso_instance(const ChipPlan& P, F&& f) {
+  constexpr int MX = split_max_threads<T>();
+  if (P.threads <= 256) {
+    if (P.cb == 0) return f.template operator()<0, 256>();
+    if (P.cb == 1) return f.template operator()<1, 256>();
+    return P.cb == 2 ? f.template operator()<2, 256>() : f.template operator()<3, 256>();
+  }
+  if (P.cb == 0) return f.template operator()<0, MX>();
+  if (P.cb == 1) return f.template operator()<1, MX>();
+  return P.cb == 2 ? f.template operator()<2, MX>() : f.template operator()<3, MX>();
+}
+template <typename T>
+struct AnisoCtas {
+  const ChipPlan& P;
+  template <int CB, int MT>
+  int operator()() const {
+    return aniso_ctas_of<T, CB, MT>(P);
+  }
+};
+template <typename T>
+struct AnisoLaunch {
+  const ChipArgs<T>& A;
+  const ChipPlan& P;
+  const PItem* items;
+  const int2* groups;
+  int n_groups;
+  int* counter;
+  int grid;
+  double* per_sample;
+  double* trace;
+  const ElecOp& op;
+  cudaStream_t st;
+  template <int CB, int MT>
+  cudaError_t operator()() const {
+    cudaLaunchAttribute at[1];
+    const cudaLaunchConfig_t cfg = chip_cfg(P, grid, st, at);
+    return cudaLaunchKernelEx(&cfg, k_split_aniso<T, CB, MT>, A, items, groups, n_groups, counter,
+                              P.slots, per_sample, trace, op);
+  }
+};
+}  // namespace
+
+template <typename T>
 int chip_ctas(const ChipPlan& P) {
+  if (P.aniso) return aniso_instance<T>(P, AnisoCtas<T>{P});
   if (P.split)
     return P.threads <= 256   ? split_ctas_of<T, 256>(P)
            : P.threads <= 512 ? split_ctas_of<T, 512>(P)
@@ -1308,6 +1739,9 @@ cudaError_t launch_chip_items(const ChipArgs<T>& A, const ChipPlan& P, const PIt
                               cudaStream_t st) {
   if (n_groups == 0 || ctas == 0) return cudaSuccess;
   const int g = std::min(ctas, n_groups << P.cb);
+  if (P.aniso)
+    return aniso_instance<T>(P, AnisoLaunch<T>{A, P, items, groups, n_groups, counter, g, per_sample,
+                                               trace, op, st});
   if (P.split) {
     if (P.threads <= 256)
       k_split_items<T, 256><<<g, P.threads, P.smem, st>>>(A, items, groups, n_groups, counter, P.rpc,
@@ -1351,6 +1785,7 @@ cudaError_t launch_chip_macro(const ChipArgs<T>& A, const ChipPlan& P, const int
 #define RP_CHIP_INST(T)                                                                          \
   template bool chip_plan<T>(long long, int, int, long long, int, int, bool, ChipPlan*);                    \
   template int chip_ctas<T>(const ChipPlan&);                                                    \
+  template bool aniso_plan<T>(long long, int, int, int, int, bool, ChipPlan*);                   \
   template cudaError_t launch_chip_items<T>(const ChipArgs<T>&, const ChipPlan&, const PItem*,   \
                                             const int2*, int, int*, T*, int, double*, double*,   \
                                             const ElecOp&, cudaStream_t);                        \

@@ -190,10 +190,12 @@ struct ChipArgs {
   uint64_t seed;
   const int* sec_rank;
   const double* sec_scale;
+  const double* frame;  // as SysTab::frame
 };
 
 struct ChipPlan {
   bool split = false;  // one thread per configuration and electron state
+  bool aniso = false;  // the same for anisotropic systems (ham and frame: rotated frames)
   int lk = 0;        // log2 of the configurations per thread
   int cb = 0;        // log2 of the CTAs per row (a cluster)
   int rpc = 1;       // rows per CTA (items launch)
@@ -210,6 +212,11 @@ bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_
 // The same for systems of spin-1/2 and spin-1 nuclei beyond one CTA, in FP32.
 bool chip_cluster_plan(long long Zmax, int min_half, int max_nuc, int n_items, int n_c, bool spin1_only,
                        ChipPlan* out);
+// The same for anisotropic systems (Z up to 2048 FP32, 1024 FP64, where they have the
+// spin-1/2 nuclei to split by).
+template <typename T>
+bool aniso_plan(long long Zmax, int min_half, int max_nuc, int n_items, int n_c, bool trace,
+                ChipPlan* out);
 template <typename T>
 int chip_ctas(const ChipPlan& P);  // CTAs resident at once; before the first launch
 
