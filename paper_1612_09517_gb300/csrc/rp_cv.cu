@@ -26,6 +26,7 @@
 
 #include "../../include/rp.h"
 #include "rp_kernels.cuh"
+#include "rp_mlp.cuh"
 #include "rp_plan.h"
 
 struct rp_system {
@@ -53,6 +54,15 @@ struct rp_cv {
   float* nuc = nullptr;                 // per nucleus I_k A_k / B_hyp (9) and radical
   long long adam_t = 0;
   cudaStream_t st = nullptr;
+
+  rp::MlpNet net() const {
+    rp::MlpNet N{wbf, master, {}, {}, d_in, hidden, layers};
+    for (int l = 0; l <= layers; ++l) {
+      N.w_off[l] = w_off[l];
+      N.b_off[l] = b_off[l];
+    }
+    return N;
+  }
 };
 
 namespace {
@@ -461,6 +471,32 @@ void features_dev(rp_cv* cv, int n, const double* d_B, double B_one, const long 
   cck(cudaGetLastError(), "features");
 }
 
+// Inference: the fused pass where the network fits it (hidden <= 256), else one product
+// per layer.  Training needs every layer's pre-activations and keeps the latter.
+struct Forward {
+  rp_cv* cv;
+  rp::MlpNet net;
+  bool fused;
+  __nv_bfloat16* packed = nullptr;
+  int* err = nullptr;
+  Acts A;
+
+  Forward(rp_cv* c, int n, Scratch& sc) : cv(c), net(c->net()), fused(rp::mlp_fused(net)) {
+    if (!fused) {
+      A = make_acts(cv, n, sc);
+      return;
+    }
+    packed = sc.get<__nv_bfloat16>(rp::mlp_packed_values(net));
+    err = sc.get<int>(1);
+    cck(cudaMemsetAsync(err, 0, sizeof(int), cv->st), "memset");
+    cck(rp::launch_mlp_pack(net, packed, cv->st), "weight tiles");
+  }
+  // After the stream was synchronised with h_err copied from err.
+  static void check(int h_err) {
+    if (h_err) throw CvFail{RP_ETIMEOUT, "a bounded device wait gave up (control-variate network)"};
+  }
+};
+
 }  // namespace
 
 // ------------------------------------------------------------------ C ABI
@@ -719,16 +755,24 @@ rp_status rp_cv_eval(rp_cv* cv, int n, const double* B, const long long* samples
     double* dB = sc.get<double>(std::min(n, chunk));
     long long* ds = sc.get<long long>(std::min(n, chunk));
     float* X = sc.get<float>((size_t)std::min(n, chunk) * cv->d_in);
-    Acts A = make_acts(cv, std::min(n, chunk), sc);
+    Forward F(cv, std::min(n, chunk), sc);
+    float* dg = F.fused ? sc.get<float>(std::min(n, chunk)) : F.A.a[cv->layers];
     std::vector<float> gf(std::min(n, chunk));
+    int h_err = 0;
     for (int i0 = 0; i0 < n; i0 += chunk) {
       const int m = std::min(chunk, n - i0);
       cck(cudaMemcpyAsync(dB, B + i0, m * sizeof(double), cudaMemcpyHostToDevice, st), "h2d");
       cck(cudaMemcpyAsync(ds, samples + i0, m * sizeof(long long), cudaMemcpyHostToDevice, st), "h2d");
       features_dev(cv, m, dB, 0.0, ds, 0, seed, pair_id, X, st);
-      forward(cv, m, X, A, st);
-      cck(cudaMemcpyAsync(gf.data(), A.a[cv->layers], m * sizeof(float), cudaMemcpyDeviceToHost, st), "d2h");
+      if (F.fused) {
+        cck(rp::launch_mlp(F.net, F.packed, m, X, nullptr, 0, 0.0, dg, nullptr, F.err, st), "network");
+        cck(cudaMemcpyAsync(&h_err, F.err, sizeof(int), cudaMemcpyDeviceToHost, st), "d2h");
+      } else {
+        forward(cv, m, X, F.A, st);
+      }
+      cck(cudaMemcpyAsync(gf.data(), dg, m * sizeof(float), cudaMemcpyDeviceToHost, st), "d2h");
       cck(cudaStreamSynchronize(st), "eval");
+      Forward::check(h_err);
       for (int i = 0; i < m; ++i) g[i0 + i] = gf[i];
     }
   } catch (const CvFail& e) {
@@ -747,21 +791,36 @@ rp_status rp_cv_mean(rp_cv* cv, int n_fields, const double* B, long long n_mc, u
   try {
     Scratch sc{st};
     const int chunk = 65536;
-    float* X = sc.get<float>((size_t)chunk * cv->d_in);
-    Acts A = make_acts(cv, chunk, sc);
+    const int rows = (int)std::min<long long>(chunk, n_mc);
+    float* X = sc.get<float>((size_t)rows * cv->d_in);
+    Forward F(cv, rows, sc);
+    int h_err = 0;
     double* acc = sc.get<double>(2 * (size_t)n_fields);
     cck(cudaMemsetAsync(acc, 0, 2 * n_fields * sizeof(double), st), "memset");
-    for (int f = 0; f < n_fields; ++f)
+    if (F.fused) {
+      // the directions are the same for every field: features once per chunk
+      double* dB = sc.get<double>(n_fields);
+      cck(cudaMemcpyAsync(dB, B, n_fields * sizeof(double), cudaMemcpyHostToDevice, st), "h2d");
+      for (long long s0 = 0; s0 < n_mc; s0 += chunk) {
+        const int m = (int)std::min<long long>(chunk, n_mc - s0);
+        features_dev(cv, m, nullptr, 0.0, nullptr, s0, seed, pair_id, X, st);
+        cck(rp::launch_mlp(F.net, F.packed, m, X, dB, n_fields, 1.0 / cv->B_scale, nullptr, acc,
+                           F.err, st), "network");
+      }
+      cck(cudaMemcpyAsync(&h_err, F.err, sizeof(int), cudaMemcpyDeviceToHost, st), "d2h");
+    }
+    for (int f = 0; f < n_fields && !F.fused; ++f)
       for (long long s0 = 0; s0 < n_mc; s0 += chunk) {
         const int m = (int)std::min<long long>(chunk, n_mc - s0);
         features_dev(cv, m, nullptr, B[f], nullptr, s0, seed, pair_id, X, st);
-        forward(cv, m, X, A, st);
-        k_moments<<<g1(m, 256), 256, 0, st>>>(m, A.a[cv->layers], acc + 2 * f);
+        forward(cv, m, X, F.A, st);
+        k_moments<<<g1(m, 256), 256, 0, st>>>(m, F.A.a[cv->layers], acc + 2 * f);
         cck(cudaGetLastError(), "moments");
       }
     std::vector<double> h(2 * (size_t)n_fields);
     cck(cudaMemcpyAsync(h.data(), acc, h.size() * sizeof(double), cudaMemcpyDeviceToHost, st), "d2h");
     cck(cudaStreamSynchronize(st), "mean");
+    Forward::check(h_err);
     for (int f = 0; f < n_fields; ++f) {
       const double m = h[2 * f] / (double)n_mc;
       const double v = std::max(0.0, (h[2 * f + 1] / (double)n_mc - m * m)) * n_mc / (n_mc - 1.0);

@@ -2,10 +2,9 @@
 // tcgen05.mma kind::tf32 on hi/lo-split FP32 singlet slices, accumulators in
 // tensor memory drained into FP32 partial sums in registers, FP64 contraction
 // with the time-integral weights.
-#include <stdint.h>
-
 #include "rp_device.cuh"
 #include "rp_kernels.cuh"
+#include "rp_tc.cuh"
 
 namespace rp {
 
@@ -51,41 +50,6 @@ static_assert(kGramStages % kGramGroup == 0, "stages hold whole groups");
 constexpr int kGramTcThreads = 512;  // 16 warps: 4 per tensor-memory lane quarter
 constexpr int kGramTmemCols = 512;  // two accumulator buffers, 256 columns apart
 constexpr int kGramMinSmem = 116 * 1024;  // keeps one CTA (and 512 TMEM columns) per SM
-constexpr long long kWaitLimit = 1ll << 24;
-
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
-  for (long long it = 0; it < kWaitLimit; ++it) {
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
-__device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigned bytes,
-                                          unsigned bar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-
-// tcgen05 shared-memory matrix descriptor, K-major, no swizzle: start address,
-// leading byte offset (next core matrix along K), stride byte offset (next
-// 8-row group), descriptor version 1.
-__device__ __forceinline__ uint64_t umma_desc(unsigned addr, unsigned lbo, unsigned sbo) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
 
 // Instruction descriptor of kind::tf32: D FP32, A and B TF32, both K-major.
 __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
@@ -101,12 +65,6 @@ __device__ __forceinline__ void mma_tf32(unsigned d, uint64_t a, uint64_t b, uin
       "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(unsigned bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   bar)
-               : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld4(unsigned taddr, float (&v)[4]) {
@@ -128,20 +86,6 @@ __device__ __forceinline__ void tmem_ld8(unsigned taddr, float (&v)[8]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(u[i]);
-}
-
-__device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
-  uint32_t u[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
-        "=r"(u[7]), "=r"(u[8]), "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]),
-        "=r"(u[14]), "=r"(u[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(u[i]);
 }
 
 // Nearest TF32 value of a finite float (ties away from zero): add half a unit
