@@ -2260,29 +2260,21 @@ rp_status rp_apply_h(rp_system* s, double B, int precision, int n_vec, const voi
   cudaStream_t st = (cudaStream_t)stream;
   const rp::HostSystem& hs = s->hs;
   try {
-    Arena ar(st);
+    // constants and field travel as kernel parameters: nothing to allocate or copy
     const double kbar = 0.5 * (hs.k_S + hs.k_T);
     if (precision == RP_FP64) {
       rp::FieldDev<double> F{rp::kGammaE * B, 1.0, 0.0, 0.5 * kbar};
       const rp::HamDev<double> H = make_ham<double>(hs);
-      auto* d = ar.get<rp::FieldDev<double>>(1);
-      auto* dh = ar.get<rp::HamDev<double>>(1);
-      ck(cudaMemcpyAsync(d, &F, sizeof(F), cudaMemcpyHostToDevice, st), "h2d");
-      ck(cudaMemcpyAsync(dh, &H, sizeof(H), cudaMemcpyHostToDevice, st), "h2d");
-      const rp::SysTab<double> S{dh, nullptr, nullptr, nullptr, hs.Z, 0, nullptr};
-      ck(rp::launch_step<double>(S, &H, H.aniso, 1, d, nullptr, nullptr, 0, nullptr, n_vec, (const double*)x,
+      const rp::SysTab<double> S{nullptr, nullptr, nullptr, nullptr, hs.Z, 0, nullptr};
+      ck(rp::launch_step<double>(S, &H, H.aniso, 1, nullptr, nullptr, nullptr, 0, nullptr, n_vec, (const double*)x,
                                  nullptr, (double*)y, nullptr, nullptr, nullptr, 0, 0,
-                                 rp::MODE_APPLY, 0, st), "apply kernel");
+                                 rp::MODE_APPLY, 0, st, &F), "apply kernel");
     } else {
       rp::FieldDev<float> F{(float)(rp::kGammaE * B), 1.f, 0.f, (float)(0.5 * kbar)};
       const rp::HamDev<float> H = make_ham<float>(hs);
-      auto* d = ar.get<rp::FieldDev<float>>(1);
-      auto* dh = ar.get<rp::HamDev<float>>(1);
-      ck(cudaMemcpyAsync(d, &F, sizeof(F), cudaMemcpyHostToDevice, st), "h2d");
-      ck(cudaMemcpyAsync(dh, &H, sizeof(H), cudaMemcpyHostToDevice, st), "h2d");
-      const rp::SysTab<float> S{dh, nullptr, nullptr, nullptr, hs.Z, 0, nullptr};
-      ck(rp::launch_step<float>(S, &H, H.aniso, 1, d, nullptr, nullptr, 0, nullptr, n_vec, (const float*)x, nullptr,
-                                (float*)y, nullptr, nullptr, nullptr, 0, 0, rp::MODE_APPLY, 0, st),
+      const rp::SysTab<float> S{nullptr, nullptr, nullptr, nullptr, hs.Z, 0, nullptr};
+      ck(rp::launch_step<float>(S, &H, H.aniso, 1, nullptr, nullptr, nullptr, 0, nullptr, n_vec, (const float*)x, nullptr,
+                                (float*)y, nullptr, nullptr, nullptr, 0, 0, rp::MODE_APPLY, 0, st, &F),
          "apply kernel");
     }
     ck(cudaStreamSynchronize(st), "apply kernel execution");

@@ -499,7 +499,7 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
                                           const T* __restrict__ cur, const T* __restrict__ prev,
                                           T* __restrict__ next, T* __restrict__ acc,
                                           T* __restrict__ X, const T* __restrict__ coef, int n_c,
-                                          int n, int mode, int xblk);
+                                          int n, int mode, int xblk, const FieldDev<T>& one_field);
 
 template <typename T, bool ANISO, bool MULTI, int NH = -1, int N1 = -1>
 __global__ void __launch_bounds__(kStepThreads,
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kStepThreads,
     const int* __restrict__ row_field, const int2* __restrict__ row_win, int macro_arg,
     const int* __restrict__ macro_dev, const T* __restrict__ cur, const T* __restrict__ prev,
     T* __restrict__ next, T* __restrict__ acc, T* __restrict__ X, const T* __restrict__ coef,
-    int n_c, int n, int mode, int xblk) {
+    int n_c, int n, int mode, int xblk, const FieldDev<T> one_field) {
   extern __shared__ __align__(16) unsigned char step_smem[];
   Cx<T>* tile = reinterpret_cast<Cx<T>*>(step_smem);  // planes x blockDim x 16 B
   const int r = blockIdx.y;
@@ -528,10 +528,10 @@ __global__ void __launch_bounds__(kStepThreads,
     for (int i = threadIdx.x; i < (int)(sizeof(HamDev<T>) / 16); i += blockDim.x) dst[i] = src[i];
     __syncthreads();
     step_body<T, ANISO, NH, N1>(Hs, S, tile, fields, f, r, cur, prev, next, acc, X, coef, n_c, n,
-                                mode, xblk);
+                                mode, xblk, one_field);
   } else {
     step_body<T, ANISO, NH, N1>(H1, S, tile, fields, f, r, cur, prev, next, acc, X, coef, n_c, n,
-                                mode, xblk);
+                                mode, xblk, one_field);
   }
 }
 
@@ -541,7 +541,7 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
                                           const T* __restrict__ cur, const T* __restrict__ prev,
                                           T* __restrict__ next, T* __restrict__ acc,
                                           T* __restrict__ X, const T* __restrict__ coef, int n_c,
-                                          int n, int mode, int xblk) {
+                                          int n, int mode, int xblk, const FieldDev<T>& one_field) {
   const unsigned Z = (unsigned)H.Z;
   const unsigned m = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = m < Z;
@@ -697,7 +697,7 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
       add_partner<T, ANISO>(y, c, m - st, rr, H.U[p], sqrt(I * (I + 1) - M * (M + 1)), false);
   }
 
-  term_epilogue<T, ANISO>(H, S, fields[f], a, y, b1, b2, f, r, m, row0, prev, next, acc, X, coef,
+  term_epilogue<T, ANISO>(H, S, fields ? fields[f] : one_field, a, y, b1, b2, f, r, m, row0, prev, next, acc, X, coef,
                          n_c, n, mode, xblk);
 }
 
@@ -774,7 +774,8 @@ __global__ void __launch_bounds__(kBulkTile, 2) k_cheb_step_bulk(
     const int* __restrict__ row_field, const int2* __restrict__ row_win, int macro_arg,
     const int* __restrict__ macro_dev, const float* __restrict__ cur,
     const float* __restrict__ prev, float* __restrict__ next, float* __restrict__ acc,
-    float* __restrict__ X, const float* __restrict__ coef, int n_c, int n, int mode, int xblk) {
+    float* __restrict__ X, const float* __restrict__ coef, int n_c, int n, int mode, int xblk,
+    const FieldDev<float> one_field) {
   extern __shared__ __align__(128) unsigned char bulk_smem[];
   __shared__ __align__(8) unsigned long long bar_storage[2];  // own tile, partner tiles
   const int r = blockIdx.y;
@@ -924,7 +925,7 @@ __global__ void __launch_bounds__(kBulkTile, 2) k_cheb_step_bulk(
       add_partner_q<float, ANISO>(y, q, rr, H.U[p], sqrtf(I * (I + 1.f) - M * (M + 1.f)), false);
     }
   }
-  term_epilogue<float, ANISO>(H, S, fields[f], a, y, b1, b2, f, r, m, row0, prev, next, acc, X,
+  term_epilogue<float, ANISO>(H, S, fields ? fields[f] : one_field, a, y, b1, b2, f, r, m, row0, prev, next, acc, X,
                               coef, n_c, n, mode, xblk, pre ? pv : nullptr,
                               pre ? sa : nullptr);
 }
@@ -2006,8 +2007,9 @@ cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int
                         const FieldDev<T>* fields, const int* row_field, const int2* row_win,
                         int macro, const int* macro_dev, int rows, const T* cur, const T* prev,
                         T* next, T* acc, T* X, const T* coef, int n_c, int n, int mode,
-                        int xblk, cudaStream_t st) {
+                        int xblk, cudaStream_t st, const FieldDev<T>* one_field) {
   if (rows == 0) return cudaSuccess;
+  const FieldDev<T> F1 = one_field ? *one_field : FieldDev<T>{};
   if (bulk && sizeof(T) == 4 && one && one->n_half >= kInnerBits && S.Zslot == one->Z &&
       one->Z % kBulkTile == 0) {
     const HamDev<float>& hf = *reinterpret_cast<const HamDev<float>*>(one);
@@ -2023,7 +2025,8 @@ cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int
           macro, macro_dev, reinterpret_cast<const float*>(cur),
           reinterpret_cast<const float*>(prev), reinterpret_cast<float*>(next),
           reinterpret_cast<float*>(acc), reinterpret_cast<float*>(X),
-          reinterpret_cast<const float*>(coef), n_c, n, mode, xblk);
+          reinterpret_cast<const float*>(coef), n_c, n, mode, xblk,
+          *reinterpret_cast<const FieldDev<float>*>(&F1));
       return cudaGetLastError();
     }
   }
@@ -2045,25 +2048,25 @@ cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int
   if (t1_shape) {
     k_cheb_step<T, false, false, 20, 0><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win,
                                                                macro, macro_dev, cur, prev, next,
-                                                               acc, X, coef, n_c, n, mode, xblk);
+                                                               acc, X, coef, n_c, n, mode, xblk, F1);
   } else if (one) {
     if (aniso)
       k_cheb_step<T, true, false><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
                                                          macro_dev, cur, prev, next, acc, X, coef,
-                                                         n_c, n, mode, xblk);
+                                                         n_c, n, mode, xblk, F1);
     else
       k_cheb_step<T, false, false><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
                                                           macro_dev, cur, prev, next, acc, X, coef,
-                                                          n_c, n, mode, xblk);
+                                                          n_c, n, mode, xblk, F1);
   } else {
     if (aniso)
       k_cheb_step<T, true, true><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
                                                         macro_dev, cur, prev, next, acc, X, coef,
-                                                        n_c, n, mode, xblk);
+                                                        n_c, n, mode, xblk, F1);
     else
       k_cheb_step<T, false, true><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
                                                          macro_dev, cur, prev, next, acc, X, coef,
-                                                         n_c, n, mode, xblk);
+                                                         n_c, n, mode, xblk, F1);
   }
   return cudaGetLastError();
 }
@@ -2366,7 +2369,8 @@ template cudaError_t launch_init_state<float>(const SysTab<float>&, const double
 template cudaError_t launch_step<float>(const SysTab<float>&, const HamDev<float>*, int, int,
                                         const FieldDev<float>*, const int*, const int2*, int,
                                         const int*, int, const float*, const float*, float*, float*, float*,
-                                        const float*, int, int, int, int, cudaStream_t);
+                                        const float*, int, int, int, int, cudaStream_t,
+                                        const FieldDev<float>*);
 template int small_max_configs<float>();
 template size_t persistent_smem<float>(long long, int);
 template int persistent_ctas<float>(long long, int, int);
@@ -2392,7 +2396,8 @@ template cudaError_t launch_init_state<double>(const SysTab<double>&, const doub
 template cudaError_t launch_step<double>(const SysTab<double>&, const HamDev<double>*, int, int,
                                         const FieldDev<double>*, const int*, const int2*, int,
                                         const int*, int, const double*, const double*, double*, double*, double*,
-                                        const double*, int, int, int, int, cudaStream_t);
+                                        const double*, int, int, int, int, cudaStream_t,
+                                        const FieldDev<double>*);
 template int small_max_configs<double>();
 template size_t persistent_smem<double>(long long, int);
 template int persistent_ctas<double>(long long, int, int);

@@ -120,13 +120,15 @@ cudaError_t launch_init_state(const SysTab<T>& S, const double* amps, const long
 // macro_dev != NULL: the kernels read the macro-step index from device memory
 // (graph replay; see launch_tick), else they use macro.  xblk != 0 writes the
 // singlet slices in the tensor-core Gram layout (see launch_gram_tc), else as
-// X[row][n][m] complex.
+// X[row][n][m] complex.  one_field != NULL (host): the field of every row, instead of
+// fields[row_field[r]].
 template <typename T>
 cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int bulk,
                         const FieldDev<T>* fields, const int* row_field, const int2* row_win,
                         int macro, const int* macro_dev, int rows, const T* cur, const T* prev,
                         T* next, T* acc, T* X, const T* coef, int n_c, int n, int mode,
-                        int xblk, cudaStream_t st);
+                        int xblk, cudaStream_t st,
+                        const FieldDev<T>* one_field = nullptr);
 
 // Largest Z (configurations) that launch_macro_small can hold.
 template <typename T>
