@@ -95,20 +95,18 @@ typedef struct rp_options {
   uint32_t pair_id;       /* Philox counter word 3 (radical-pair id) */
   int profile;            /* 1: time the H.psi step kernels with CUDA events */
   void* stream;           /* cudaStream_t, NULL: the legacy default stream */
-  int kernel;             /* 0: choose (5 where 128 <= Z <= 1024, or a batch of
-                             several systems fits one CTA, and graph = 0; 2
-                             where Z fits one CTA's shared memory otherwise; 4
-                             for the FP32 shapes with a compiled cluster
+  int kernel;             /* 0: choose (whole propagations on chip, as 5, where the
+                             system fits one CTA or, isotropic FP32 with spin-1/2
+                             and spin-1 nuclei, a cluster of up to 8 CTAs, and
+                             graph = 0; else 2 where Z fits one CTA's shared
+                             memory; 4 for the FP32 shapes with a compiled cluster
                              instance -- 8 spin-1/2 and 4 spin-1 nuclei,
                              isotropic, one system; else 1);
                              1: one launch per Chebyshev term (any Z);
                              2: a whole macro-step per launch with each row's
                              vectors in shared memory (Z <= 2048 FP32, 1024
-                             FP64; larger Z falls back to 1); 3: as 1, and FP32
-                             single systems with >= 8 spin-1/2 nuclei stage
-                             each block's partner configurations with bulk
-                             async copies (slower than 1 on the workloads
-                             measured so far; a candidate of rp_tune);
+                             FP64; larger Z falls back to 1);
+                             3: as 1 (kept for callers that name it);
                              4: a whole macro-step per launch on a cluster of
                              2^c CTAs per row (c <= 3) holding the row's
                              Chebyshev vectors in distributed shared memory
@@ -116,13 +114,12 @@ typedef struct rp_options {
                              2^c <= 2^(number of spin-1/2 nuclei); otherwise
                              falls back to 1);
                              5: one persistent launch over all propagations of
-                             the call: each CTA takes (field, sample) items
-                             from a device counter and runs an item's whole
-                             horizon with its vectors in shared memory (the
-                             time integral on CUDA cores in the same CTA);
-                             Z <= 2048 FP32, 1024 FP64, deterministic 0-2,
-                             rp_yields, rp_yields_batch and the converged
-                             entries; elsewhere kernel 5 selects as 0 */
+                             the call: each CTA (or cluster) takes (field,
+                             sample) items from a device counter and runs an
+                             item's whole horizon with its vectors in shared
+                             memory, the time integral included; Z <= 2048 FP32,
+                             1024 FP64, and the clusters of kernel 0; elsewhere
+                             kernel 5 selects as 0 */
   int gram;               /* time integral (Eqs. 20, 22) of each macro-step: 0 or 1
                              the low-rank factor of its weights on the CUDA cores (any
                              precision and kernel); 2 the Gram matrix of the singlet
@@ -134,7 +131,8 @@ typedef struct rp_options {
                              and time integral) in a CUDA graph and replay it; the
                              kernels then read the macro-step index from a device
                              counter.  Refill work between macro-steps stays eager.
-                             Results are identical to graph = 0. */
+                             Results are those of the same kernel with graph = 0
+                             (kernel = 0 chooses among the macro-step launches). */
 } rp_options;
 
 /* Per-call statistics (optional output of rp_yields). */

@@ -825,7 +825,8 @@ class YieldEngine {
     int lt = 0;
     while ((1 << lt) < tile) ++lt;
     std::vector<rp::TermSys<T>> sys(ns);
-    long long tab = 0, tm_max = 1;
+    const bool ring = sizeof(T) == 4 && min_half_ >= lt;
+    long long tab = 0, tm_max = 1, tiles_max = 0;
     for (int i = 0; i < ns; ++i) {
       const rp::HamDev<double>& H = hamd_[i];
       rp::TermSys<T>& Y = sys[i];
@@ -842,6 +843,11 @@ class YieldEngine {
       Y.tab = tab;
       tab += (Y.tm * nb + 3) & ~3LL;
       tm_max = std::max(tm_max, Y.tm);
+      if (ring) {
+        Y.otab = tab;
+        tab += (Y.Z / tile * nb + 3) & ~3LL;
+        tiles_max = std::max(tiles_max, Y.Z / tile);
+      }
       for (int p = 0; p < H.n_nuc; ++p) {
         Y.rad |= (unsigned)(H.rad[p] & 1) << p;
         Y.d[p] = H.d[p];
@@ -875,10 +881,13 @@ class YieldEngine {
     ck(cudaMemcpyAsync(d_sys, sys.data(), ns * sizeof(sys[0]), cudaMemcpyHostToDevice, st_), "h2d systems");
     ck(cudaMemcpyAsync(d_tf, tf.data(), nf * sizeof(tf[0]), cudaMemcpyHostToDevice, st_), "h2d fields");
     h2d += (long long)(ns * sizeof(sys[0]) + nf * sizeof(tf[0]));
-    launched(rp::launch_term_table<T>(d_hamd_, d_sys, ns, tm_max, aniso_ != 0, d_tab, st_),
+    launched(rp::launch_term_table<T>(d_hamd_, d_sys, ns, tm_max, tiles_max, aniso_ != 0, d_tab,
+                                      st_),
              "nuclear-field table");
+    if (tiles_max > 0) launches++;
     targs_ = rp::TermArgs<T>{d_sys, d_tf, d_tab, d_rcoef_, ns == 1 ? nullptr : row_sys_, nullptr, nullptr,
-                             Zslot_, plane, n_c_, tc_gram_ ? 1 : 0};
+                             Zslot_, plane, n_c_, tc_gram_ ? 1 : 0,
+                             ring ? 1 : 0};
   }
 
   // Records the launches of a macro-step of parity p (k % 2 == p) into a graph.

@@ -12,7 +12,7 @@ namespace {
 
 // ---- Exact time integral on the tensor cores (FP32 state, tcgen05 3xTF32) ----
 //
-// The same quantity as k_gram_integrate (Eqs. 20, 22): integral[r] +=
+// The same quantity as k_project of rp_integral.cu (Eqs. 20, 22): integral[r] +=
 // Re sum_nm W_nm G_nm with G_nm = sum_z conj(x_n(z)) x_m(z).  With the real
 // rows a = 2n + p (p = 0: Re x_n, p = 1: Im x_n) of the singlet slices as a
 // (2 n_c) x Z matrix A, the real Gram R = A A^T holds G (Re G_nm = R_{2n,2m} +

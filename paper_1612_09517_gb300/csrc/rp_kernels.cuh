@@ -253,7 +253,7 @@ struct alignas(16) TermField {
 // nuclear fields covers m mod tm (nuclei p < p_out) from entry tab.
 template <typename T>
 struct alignas(16) TermSys {
-  long long Z, tab, tm, pad;
+  long long Z, tab, tm, otab;  // otab: per tile, the nuclei p >= p_out (ring kernels)
   int n_half, n_nuc, p_in, p_out;
   unsigned rad;
   int pad2[3];
@@ -274,6 +274,7 @@ struct TermArgs {
   long long Zslot, plane;  // row slot and plane stride in configurations
   int n_c;
   int xblk;  // slices in the tensor-core Gram layout
+  int ring;  // k_term_ring (FP32, every n_half >= 9)
 };
 
 template <typename T>
@@ -281,7 +282,8 @@ int term_lk(bool aniso, int min_half);
 int term_tile(int lk);  // configurations per block
 template <typename T>
 cudaError_t launch_term_table(const HamDev<double>* ham, const TermSys<T>* sys, int n_sys,
-                              long long tm_max, bool aniso, T* btab, cudaStream_t st);
+                              long long tm_max, long long tiles_max, bool aniso, T* btab,
+                              cudaStream_t st);
 // One term over every active row: vectors in planes [row][e][plane], slices to X
 // (may be NULL); modes as k_cheb_step.
 template <typename T>
