@@ -638,7 +638,7 @@ class YieldEngine {
         // the whole macro-step on chip: HBM traffic is psi in, psi out and the singlet slices
         bytes = (2.0 + 0.25 * n_c_) * vbytes;
       } else {
-        for (int n = 1; n < n_c_; ++n) bytes += rp::term_vector_passes(n, n_c_) * vbytes;
+        for (int n = 1; n < n_c_; ++n) bytes += rp::term_vector_passes(sizeof(T) == 8, n, n_c_) * vbytes;
       }
       // profile events bracket the step kernels (eager) or the whole graph replay
       cudaEvent_t ev_end = o_.profile ? pev.back() : nullptr;

@@ -501,7 +501,7 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
                                           T* __restrict__ X, const T* __restrict__ coef, int n_c,
                                           int n, int mode, int xblk, const FieldDev<T>& one_field);
 
-template <typename T, bool ANISO, bool MULTI, int NH = -1, int N1 = -1>
+template <typename T, bool ANISO, int NH = -1, int N1 = -1>
 __global__ void __launch_bounds__(kStepThreads,
                                   sizeof(T) == 4 ? (ANISO ? 4 : (NH >= 0 ? 5 : 6)) : 2)
     k_cheb_step(
@@ -520,19 +520,8 @@ __global__ void __launch_bounds__(kStepThreads,
     if (macro < w.x || macro >= w.y) return;  // the whole block: one row
     f = row_field[r];
   }
-  if (MULTI) {
-    __shared__ HamDev<T> Hs;  // constants of this row's system
-    const int sidx = S.row_sys ? S.row_sys[r] : 0;
-    const int4* src = reinterpret_cast<const int4*>(S.ham + sidx);
-    int4* dst = reinterpret_cast<int4*>(&Hs);
-    for (int i = threadIdx.x; i < (int)(sizeof(HamDev<T>) / 16); i += blockDim.x) dst[i] = src[i];
-    __syncthreads();
-    step_body<T, ANISO, NH, N1>(Hs, S, tile, fields, f, r, cur, prev, next, acc, X, coef, n_c, n,
-                                mode, xblk, one_field);
-  } else {
-    step_body<T, ANISO, NH, N1>(H1, S, tile, fields, f, r, cur, prev, next, acc, X, coef, n_c, n,
-                                mode, xblk, one_field);
-  }
+  step_body<T, ANISO, NH, N1>(H1, S, tile, fields, f, r, cur, prev, next, acc, X, coef, n_c, n,
+                              mode, xblk, one_field);
 }
 
 template <typename T, bool ANISO, int NH, int N1>
@@ -2010,7 +1999,7 @@ cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int
                         int xblk, cudaStream_t st, const FieldDev<T>* one_field) {
   if (rows == 0) return cudaSuccess;
   const FieldDev<T> F1 = one_field ? *one_field : FieldDev<T>{};
-  if (bulk && sizeof(T) == 4 && one && one->n_half >= kInnerBits && S.Zslot == one->Z &&
+  if (bulk && sizeof(T) == 4 && one->n_half >= kInnerBits && S.Zslot == one->Z &&
       one->Z % kBulkTile == 0) {
     const HamDev<float>& hf = *reinterpret_cast<const HamDev<float>*>(one);
     const size_t smem = (size_t)(1 + bulk_max_partner_tiles(hf)) * kBulkTileBytes;
@@ -2035,39 +2024,23 @@ cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int
   while (b < kStepThreads && b < S.Zslot) b *= 2;
   const size_t smem = (size_t)b * 4 * sizeof(Cx<T>);
   dim3 grid(grid1(S.Zslot, b), rows);
-  HamDev<T> h1;
-  if (one) h1 = *one;
-  else std::memset(&h1, 0, sizeof(h1));
-  // compiled shape (fixed nucleus loops, 48 registers and 5 blocks per SM
-  // instead of 40 and 6): 20 spin-1/2 nuclei, isotropic -- the paper's
-  // Table I model, 3 % faster per term.  (The same for the 20-nucleus
-  // anisotropic workload needs 67 registers, 3 blocks per SM, and measured
-  // 12 % slower than the generic kernel at 4.)
-  const bool t1_shape = one && !aniso && b == kStepThreads && one->n_half == 20 &&
-                        one->n_nuc == 20;
-  if (t1_shape) {
-    k_cheb_step<T, false, false, 20, 0><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win,
-                                                               macro, macro_dev, cur, prev, next,
-                                                               acc, X, coef, n_c, n, mode, xblk, F1);
-  } else if (one) {
-    if (aniso)
-      k_cheb_step<T, true, false><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
-                                                         macro_dev, cur, prev, next, acc, X, coef,
-                                                         n_c, n, mode, xblk, F1);
-    else
-      k_cheb_step<T, false, false><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
-                                                          macro_dev, cur, prev, next, acc, X, coef,
-                                                          n_c, n, mode, xblk, F1);
-  } else {
-    if (aniso)
-      k_cheb_step<T, true, true><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
+  // compiled shape (fixed nucleus loops, 48 registers and 5 blocks per SM instead of 40
+  // and 6 in FP32): 20 spin-1/2 nuclei, isotropic -- the paper's Table I model, 3 % faster.
+  // (The same for the 20-nucleus anisotropic workload needs 67 registers, 3 blocks per SM,
+  // and measured 12 % slower than the generic kernel at 4.)
+  const bool t1_shape = !aniso && b == kStepThreads && one->n_half == 20 && one->n_nuc == 20;
+  if (t1_shape)
+    k_cheb_step<T, false, 20, 0><<<grid, b, smem, st>>>(S, *one, fields, row_field, row_win, macro,
                                                         macro_dev, cur, prev, next, acc, X, coef,
                                                         n_c, n, mode, xblk, F1);
-    else
-      k_cheb_step<T, false, true><<<grid, b, smem, st>>>(S, h1, fields, row_field, row_win, macro,
-                                                         macro_dev, cur, prev, next, acc, X, coef,
-                                                         n_c, n, mode, xblk, F1);
-  }
+  else if (aniso)
+    k_cheb_step<T, true><<<grid, b, smem, st>>>(S, *one, fields, row_field, row_win, macro,
+                                                macro_dev, cur, prev, next, acc, X, coef, n_c, n,
+                                                mode, xblk, F1);
+  else
+    k_cheb_step<T, false><<<grid, b, smem, st>>>(S, *one, fields, row_field, row_win, macro,
+                                                 macro_dev, cur, prev, next, acc, X, coef, n_c, n,
+                                                 mode, xblk, F1);
   return cudaGetLastError();
 }
 

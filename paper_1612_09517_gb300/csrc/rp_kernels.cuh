@@ -37,14 +37,26 @@ struct FieldDev {
 
 enum StepMode { MODE_APPLY = 0, MODE_FIRST = 1, MODE_MID = 2, MODE_LAST = 3 };
 
+// Terms that the accumulator takes with term n in the per-term kernels: three at a time
+// in FP32 (phi_n, phi_{n-1} and phi_{n-2} are at hand), which cuts a term from 5.25 to 3.9
+// vector passes on average; FP64 is bound by arithmetic and adds each.
+inline int term_nacc(bool fp64, int n, int mode) {
+  return mode == MODE_FIRST  ? 2
+         : fp64              ? 1
+         : mode == MODE_LAST ? (n - 2) % 3 + 1
+                             : ((n - 1) % 3 == 0 ? 3 : 0);
+}
+
 // Vector passes (multiples of one state vector of every active row) of the
 // Chebyshev term n of a macro-step in the per-term kernels: reads of
 // phi_{n-1} (and phi_{n-2}), write of phi_n (not at the last term), the
 // accumulator write (first term) or read-modify-write, the singlet slices (a
 // quarter each).
-inline double term_vector_passes(int n, int n_c) {
+inline double term_vector_passes(bool fp64, int n, int n_c) {
   if (n == 1) return 3.5;
-  return n == n_c - 1 ? 4.25 : 5.25;
+  const bool last = n == n_c - 1;
+  const double acc = term_nacc(fp64, n, last ? MODE_LAST : MODE_MID) ? 2.0 : 0.0;
+  return (last ? 2.25 : 3.25) + acc;
 }
 
 // Per-row (one propagation) metadata, device arrays of length rows.  A row is
@@ -110,18 +122,16 @@ cudaError_t launch_init_state(const SysTab<T>& S, const double* amps, const long
                               int deterministic, T* S0, T* S1, double* integral, double* survival,
                               cudaStream_t st);
 
-// One Chebyshev term over every row (see k_cheb_step).  one != NULL: every
-// row is that system (its constants travel as kernel parameters); NULL: each
-// row reads its system from S.ham.  aniso selects the anisotropic hyperfine
-// path (needed if any system of the launch has it).  bulk != 0 allows the FP32
-// variant that stages each block's partner tiles with bulk async copies
-// (taken for one system with >= 8 spin-1/2 nuclei whose tiles fit in shared
-// memory; see k_cheb_step_bulk); its bounded wait reports to S.err.
-// macro_dev != NULL: the kernels read the macro-step index from device memory
-// (graph replay; see launch_tick), else they use macro.  xblk != 0 writes the
-// singlet slices in the tensor-core Gram layout (see launch_gram_tc), else as
-// X[row][n][m] complex.  one_field != NULL (host): the field of every row, instead of
-// fields[row_field[r]].
+// One Chebyshev term over every row (see k_cheb_step), every row being the system *one
+// (its constants travel as kernel parameters).  aniso selects the anisotropic hyperfine
+// path.  bulk != 0 allows the FP32 variant that stages each block's partner tiles with
+// bulk async copies (taken for >= 8 spin-1/2 nuclei whose tiles fit in shared memory; see
+// k_cheb_step_bulk); its bounded wait reports to S.err.  macro_dev != NULL: the kernels
+// read the macro-step index from device memory (graph replay; see launch_tick), else they
+// use macro.  xblk != 0 writes the singlet slices in the tensor-core Gram layout (see
+// launch_gram_tc), else as X[row][n][m] complex.  one_field != NULL (host): the field of
+// every row, instead of fields[row_field[r]].  rp_apply_h and the allocation-free entry
+// run these kernels; the others take launch_term.
 template <typename T>
 cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int bulk,
                         const FieldDev<T>* fields, const int* row_field, const int2* row_win,

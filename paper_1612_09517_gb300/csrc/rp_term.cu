@@ -677,19 +677,21 @@ __global__ void __launch_bounds__(kTermThreads, (term_min_blocks<T, LK, ANISO>()
 // lists their partners once (addresses and weights); each thread copies its own 16 bytes
 // per component into its own shared-memory slots some entries ahead of their use
 // (cp.async, no barrier: nobody else reads them).  phi_{n-2} and the accumulator follow
-// as the list's last entries.  The tile's nuclei are unrolled and the fields of the
+// as the list's last entries.  An anisotropic partner has two entries; the second goes
+// straight to registers (a copy passes the L1 twice, which all copies would fill).  The tile's nuclei are unrolled and the fields of the
 // nuclei outside it come from a table, so a thread spends its instructions on products.
 //
 // Bounds: HBM and issue slots together.  Z = 2^20, 14 rows (7.5 GB of vectors): 355 us
 // per term in the general form, 353 with the copies alone (65 % of issue slots used, half
 // of them by integer work), 300 as it is, 5.0 TB/s of a measured 6.8.  Anisotropic, Z =
-// 2359296, 6 rows: 243, 232 and 187 ms for 3 macro-steps.
+// 2359296, 6 rows, whole call: 243, 232 and 187 ms, 177 with the second entries direct
+// (the same for every second isotropic partner: 305 us).
 constexpr int kRingThreads = kTermThreads, kRingTileBits = 9;
 constexpr int kRingParts = 2 * kMaxNucDev;
 
 template <bool ANISO>
 struct RingCfg {
-  static constexpr int RS = ANISO ? 6 : 4;  // entries (two components each) in flight
+  static constexpr int RS = 4;              // copies (two components each) in flight
   static constexpr int HE = ANISO ? 2 : 1;  // entries per partner
   static constexpr int NB = ANISO ? 6 : 2;
   static constexpr size_t smem = (size_t)kRingThreads * 16 * (4 + 2 * RS);
@@ -824,13 +826,13 @@ __global__ void __launch_bounds__(kRingThreads, ANISO ? 3 : 4) k_term_ring(
   const unsigned ring0 = (unsigned)__cvta_generic_to_shared(tile + 4 * kRingThreads + tid);
   constexpr unsigned kComp = kRingThreads * 16, kSlot = 2 * kComp;
   const unsigned rad = Y.rad;
-  const int n_pro = min(RS, (Y.n_half - kRingTileBits) * HE);
+  const int n_pro = min(RS, Y.n_half - kRingTileBits);
 #pragma unroll
   for (int q = 0; q < RS; ++q) {  // spin-1/2 nuclei next to the tile need no list
     if (q >= n_pro) break;
-    const int p = kRingTileBits + q / HE;
+    const int p = kRingTileBits + q;
     int c0, c1;
-    ring_comps<ANISO>((int)((rad >> p) & 1u), !((m0 >> p) & 1u), q % HE, c0, c1);
+    ring_comps<ANISO>((int)((rad >> p) & 1u), !((m0 >> p) & 1u), 0, c0, c1);
     const float* src = cur + row0 + (size_t)(m ^ (1u << p)) * 2;
     cp16(ring0 + q * kSlot, src + c0 * plane);
     cp16(ring0 + q * kSlot + kComp, src + c1 * plane);
@@ -1001,11 +1003,11 @@ __global__ void __launch_bounds__(kRingThreads, ANISO ? 3 : 4) k_term_ring(
     }
   }
   // partners outside the tile
-  const int np = s_np, n_ent = np * HE + 4;
+  const int np = s_np;
   unsigned slot = ring0;
   auto copy = [&](int q, unsigned at) {
-    if (q < n_ent) {
-      const longlong2 pp = s_ptr[q];
+    if (q < np + 4) {
+      const longlong2 pp = s_ptr[q < np ? q * HE : np * HE + (q - np)];
       if (pp.x) {
         cp16(at, reinterpret_cast<const float*>(pp.x) + (size_t)m * 2);
         cp16(at + kComp, reinterpret_cast<const float*>(pp.y) + (size_t)m * 2);
@@ -1040,18 +1042,22 @@ __global__ void __launch_bounds__(kRingThreads, ANISO ? 3 : 4) k_term_ring(
     const int code = __float_as_int(w.w);
     Cx<float> q[2], p[2];
     if constexpr (ANISO) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        take(q, p);
-        if (code & 2) {
-          if (code & 1) S.pair(true, 2 * h, 2 * h + 1, w.y, w.z, w.x, q, p);
-          else S.pair(true, h, h + 2, w.y, w.z, w.x, q, p);
-        } else {
-          if (code & 1) S.pair(false, 2 * h, 2 * h + 1, w.y, w.z, w.x, q, p);
-          else S.pair(false, h, h + 2, w.y, w.z, w.x, q, p);
-        }
-        refill();
-      }
+      // the second entry straight to registers, loaded one entry's work ahead
+      const longlong2 pp = s_ptr[2 * i + 1];
+      const float4 du = __ldg(reinterpret_cast<const float4*>(pp.x) + m / 2),
+                   dv = __ldg(reinterpret_cast<const float4*>(pp.y) + m / 2);
+      auto half = [&](bool up, int h) {
+        if (code & 1) S.pair(up, 2 * h, 2 * h + 1, w.y, w.z, w.x, q, p);
+        else S.pair(up, h, h + 2, w.y, w.z, w.x, q, p);
+      };
+      take(q, p);
+      if (code & 2) half(true, 0);
+      else half(false, 0);
+      refill();
+      unpack(du, q);
+      unpack(dv, p);
+      if (code & 2) half(true, 1);
+      else half(false, 1);
     } else {
       take(q, p);
       if (code & 2) {
@@ -1214,16 +1220,6 @@ __global__ void __launch_bounds__(256) k_term_outer(const HamDev<double>* __rest
     o[4] = (T)(0.5 * b[1][0]);
     o[5] = (T)(0.5 * b[1][1]);
   }
-}
-
-// Terms the accumulator takes with term n: three at a time in FP32 (phi_n, phi_{n-1} and
-// phi_{n-2} are at hand), which cuts a term from 5.25 to 3.9 vector passes on average;
-// FP64 is bound by arithmetic and adds each.
-int term_nacc(bool fp64, int n, int mode) {
-  return mode == MODE_FIRST  ? 2
-         : fp64              ? 1
-         : mode == MODE_LAST ? (n - 2) % 3 + 1
-                             : ((n - 1) % 3 == 0 ? 3 : 0);
 }
 
 template <bool ANISO>

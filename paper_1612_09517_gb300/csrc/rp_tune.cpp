@@ -3,13 +3,14 @@
 // The knobs are the ones that change how the same propagation is executed,
 // never what it computes (Eqs. 20, 22 are evaluated to the same tolerance by
 // every candidate):
-//   kernel  1 = one launch per Chebyshev term, 3 = the same with the partner
-//           tiles staged by bulk copies (where the layout allows), 2 = a whole
-//           macro-step per launch with the row in shared memory (only where
-//           Z fits), 4 = a whole macro-step per launch with the row in the
-//           distributed shared memory of a thread-block cluster (FP32
-//           isotropic systems that fit), 5 = one persistent launch over all
-//           propagations (only where Z fits one CTA; graph has no effect);
+//   kernel  1 = one launch per Chebyshev term, 2 = a whole macro-step per
+//           launch with the row in shared memory (only where Z fits), 4 = a
+//           whole macro-step per launch with the row in the distributed
+//           shared memory of a thread-block cluster (FP32 isotropic systems
+//           that fit), 5 = one persistent launch over all propagations (where
+//           Z fits one CTA, and isotropic FP32 systems of spin-1/2 and spin-1
+//           nuclei, which it takes on clusters; eager only).  Anisotropic FP32
+//           systems that fit one CTA reach their fastest launch by kernel 0;
 //   n_cheb  terms per macro-step (the planner then picks the step h that
 //           meets the tolerance: more terms, longer steps, a larger
 //           n_cheb x n_cheb time-integral Gram and more singlet slices);
@@ -149,20 +150,23 @@ rp_status rp_tune(rp_system* s, double B, int rows, const rp_options* base, rp_o
   const long long small_max = o.precision == RP_FP64 ? 1024 : 2048;
   const std::vector<int> ncs = {32, 48, 64, 88};
   std::vector<Cand> cands;
-  // kernel 3 differs from 1 only where it stages partner tiles (FP32, >= 8 spin-1/2);
-  // kernel 4 only where a row fits a thread-block cluster (FP32, isotropic)
-  const bool staged = o.precision == RP_FP32 && s->hs.n_half >= 8;
+  // kernel 4 only where a row fits a thread-block cluster (FP32, isotropic); kernel 5
+  // beyond one CTA only where clusters may take the row
   bool cluster_ok = false;
+  const bool mid = o.precision == RP_FP32 && Z > small_max && !s->hs.aniso &&
+                   s->hs.n_half + s->hs.n_one == s->hs.n_nuc;
+  const int persistent = o.precision == RP_FP32 && s->hs.aniso ? 0 : 5;
   int default_kernel = o.precision == RP_FP32
                            ? rp::default_kernel_fp32(s->hs, &cluster_ok)
                            : (Z <= small_max ? (rp::persistent_default(Z, 1) || !s->hs.aniso ? 5 : 2) : 1);
   if (default_kernel == 5 && o.graph) default_kernel = 2;  // kernel 0 with graph replay
+  if (mid && !o.graph && default_kernel != 4) default_kernel = 5;
+  if (Z <= small_max && persistent == 0 && !o.graph) default_kernel = 0;
   for (int nc : ncs)
     for (int g = 0; g <= 1; ++g) {
       cands.push_back({1, nc, g});
       if (Z <= small_max) cands.push_back({2, nc, g});
-      if (Z <= small_max && g == 0) cands.push_back({5, nc, 0});
-      if (staged) cands.push_back({3, nc, g});
+      if ((Z <= small_max || mid) && g == 0) cands.push_back({persistent, nc, 0});
       if (cluster_ok && Z > small_max) cands.push_back({4, nc, g});
     }
   const int kTrialMacro = 6;
