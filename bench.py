@@ -851,20 +851,13 @@ def main():
                           "occupy 120 of the 152 SMs"}
     else:
         achieved = step_bytes / (step_ms * 1e-3) / 1e9 if step_ms > 0 else None
-        traffic_per_row = _profile_traffic("k_cheb_step")
+        traffic_per_row = _profile_traffic("k_term_ring")
         avg_rows = row_terms / max(step_launches_timed, 1) / n_c * (n_c - 1) \
             if step_launches_timed else None
-        # the same launches at the minimum count of 4.25 vector passes per
-        # term (the accumulator read-modify-write not counted as useful)
-        passes = 3.5 + 4.25 + 5.25 * (n_c - 3)
-        achieved_min = achieved * 4.25 * (n_c - 1) / passes if achieved else None
         roofline = {
-            "bound": "hbm", "kernel": "k_cheb_step (fused H.psi + Chebyshev term)",
+            "bound": "hbm", "kernel": "k_term / k_term_ring (fused H.psi + Chebyshev term)",
             "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": (achieved / peak) if achieved else None,
-            "achieved_min_count": achieved_min,
-            "frac_min": (achieved_min / peak) if achieved_min else None,
-            "min_count_note": "4.25 vector passes per term instead of the kernel's 3.5 / 5.25 / 4.25",
             "traffic": (traffic_per_row * avg_rows) if (traffic_per_row and avg_rows) else None,
             "peak_source": peak_src,
             "algorithmic_bytes_per_launch": step_bytes / max(step_launches_timed, 1),

@@ -493,8 +493,9 @@ rp_status rp_trace_propagations(const rp_system* sys, int deterministic, long lo
 /* Launch-configuration autotuner (the paper has no counterpart: its method
  * ran serially on CPUs).  For one system, precision and concurrency it times
  * the candidates
- *   kernel in {1, 2 (only if Z fits in shared memory), 3 (only FP32 with
- *   >= 8 spin-1/2 nuclei, where it stages partner tiles)},
+ *   kernel in {1, 2 (only if Z fits in shared memory), 4 (FP32, isotropic, on a
+ *   cluster), 5 (where it applies, see rp_options; 0 stands for it for
+ *   anisotropic FP32 systems)},
  *   n_cheb in {32, 48, 64, 88},  graph in {0, 1}
  * on `rows` coherent-state samples at field B (mT) over six macro-steps
  * through rp_yields (one untimed run, the faster of two timed runs by the
