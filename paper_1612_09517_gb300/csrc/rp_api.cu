@@ -13,6 +13,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <string>
 #include <vector>
@@ -527,14 +528,21 @@ class YieldEngine {
        "h2d items");
     h2d += (long long)(h.size() * sizeof(rp::PItem));
     ck(cudaMemsetAsync(d_counter_, 0, sizeof(int), st_), "cudaMemsetAsync");
+    const cudaStream_t ls = side_launch_ ? side_launch_ : st_;
     if (o_.profile) {
       cudaEvent_t e0, e1;
       ck(cudaEventCreate(&e0), "cudaEventCreate");
       pev.push_back(e0);
       ck(cudaEventCreate(&e1), "cudaEventCreate");
       pev.push_back(e1);
-      ck(cudaEventRecord(e0, st_), "cudaEventRecord");
+      ck(cudaEventRecord(e0, ls), "cudaEventRecord");
     }
+    // everything the kernel reads was made on st_; only the kernel runs on the side
+    auto fork = [&]() {
+      if (!side_launch_) return;
+      ck(cudaEventRecord(side_fork_, st_), "cudaEventRecord");
+      ck(cudaStreamWaitEvent(side_launch_, side_fork_, 0), "cudaStreamWaitEvent");
+    };
     if (chip_) {
       // groups of items of one field (the rows of a CTA)
       std::vector<int2> groups;
@@ -549,21 +557,24 @@ class YieldEngine {
       ck(cudaMemcpyAsync(d_groups, groups.data(), groups.size() * sizeof(int2), cudaMemcpyHostToDevice, st_),
          "h2d groups");
       h2d += (long long)(groups.size() * sizeof(int2));
+      fork();
       launched(rp::launch_chip_items<T>(chip_args(), cplan_, d_items, d_groups, (int)groups.size(),
-                                        d_counter_, Xp_, pctas_, d_ps, d_trace_, trace_op_, st_),
+                                        d_counter_, Xp_, pctas_, d_ps, d_trace_, trace_op_, ls),
                "on-chip kernel");
-    } else
+    } else {
+      fork();
       launched(rp::launch_persistent_small<T>(S_, aniso_, d_fdev_, d_coef_, d_L_, d_meta_, d_items, (int)n,
                                             d_counter_, n_c_, o_.deterministic, seed_, Xp_, pctas_,
-                                            d_ps, st_),
+                                            d_ps, ls),
              "persistent kernel");
+    }
     step_launches += 1;
     if (o_.profile) {
-      ck(cudaEventRecord(pev.back(), st_), "cudaEventRecord");
+      ck(cudaEventRecord(pev.back(), ls), "cudaEventRecord");
       pev_bytes.push_back(step_bytes_all);
       pev_launches.push_back(1);
     }
-    ck(cudaStreamSynchronize(st_), "kernel execution");
+    if (!side_launch_) ck(cudaStreamSynchronize(st_), "kernel execution");
   }
 
   void run(const std::vector<Item>& items, double* d_ps) {
@@ -716,6 +727,16 @@ class YieldEngine {
   }
 
   void set_seed(uint64_t seed) { seed_ = seed; }
+
+  // One launch over all items (after alloc_rows).
+  bool persistent() const { return persist_; }
+  // The persistent kernel runs on `side` after the work queued on the engine's stream,
+  // and run() returns without waiting for it; `fork` is the caller's event for that.
+  // The caller synchronises `side` before the engine's arena goes.
+  void launch_on(cudaStream_t side, cudaEvent_t fork) {
+    side_launch_ = side;
+    side_fork_ = fork;
+  }
 
   // J_z-sector tables of deterministic = 3 (device arrays; before alloc_rows).
   void set_sectors(const int* rank, const double* scale) {
@@ -940,6 +961,8 @@ class YieldEngine {
   bool overlap_ = false;
   bool persist_ = false;
   bool chip_ = false;
+  cudaStream_t side_launch_ = nullptr;
+  cudaEvent_t side_fork_ = nullptr;
   bool term_ = false;
   int term_lk_ = 0;
   rp::TermArgs<T> targs_{};
@@ -1614,6 +1637,36 @@ rp_status run_converged_cv(rp_system* sys, int n_fields, const double* fields, d
   return RP_OK;
 }
 
+// Streams beside the caller's for kernels that may run at the same time, made on first
+// use, at most kMax; the destructor waits for them.
+struct SideStreams {
+  static constexpr int kMax = 8;
+  std::vector<cudaStream_t> s;
+  size_t at = 0;
+  cudaEvent_t fork = nullptr;
+
+  cudaStream_t next() {
+    if (!fork) ck(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming), "cudaEventCreate");
+    if (s.size() < (size_t)kMax) {
+      cudaStream_t n = nullptr;
+      ck(cudaStreamCreateWithFlags(&n, cudaStreamNonBlocking), "cudaStreamCreate");
+      s.push_back(n);
+      return n;
+    }
+    return s[at++ % s.size()];
+  }
+  void sync() {
+    for (cudaStream_t x : s) ck(cudaStreamSynchronize(x), "kernel execution");
+  }
+  ~SideStreams() {
+    for (cudaStream_t x : s) {
+      cudaStreamSynchronize(x);
+      cudaStreamDestroy(x);
+    }
+    if (fork) cudaEventDestroy(fork);
+  }
+};
+
 // Several radical pairs in one pass (see rp_yields_batch in rp.h): systems are
 // grouped by size so that a row slot is at most twice a system's Z; every
 // group runs all its (system, field, sample) items on one pool of rows.
@@ -1653,6 +1706,38 @@ rp_status run_batch(int n_sys, rp_system* const* systems, const int* n_fields,
   int R_max = 0;
   Arena outer(st);
   double* d_ps = outer.get<double>((size_t)std::max<long long>(n_samples, 1) * 3);
+  // Groups that run as one persistent launch do so beside each other: a group's rows
+  // rarely fill the chip (16 rows of Z = 1152 take 16 of 152 SMs for 8 ms), and the
+  // kernels share nothing but the per-sample output.  Each group keeps its scratch until
+  // its kernel is done.  Twelve pairs, Z 96 to 13824, 16 rows each: 69 ms one after the
+  // other, 28 ms like this.
+  struct Pending {
+    std::unique_ptr<Arena> ar;
+    std::unique_ptr<YieldEngine<T>> eng;  // goes before its arena
+  };
+  std::vector<Pending> live;
+  SideStreams sides;  // goes first: waits for the kernels of `live`
+  auto finish = [&]() {
+    sides.sync();
+    if (!live.empty()) ck(cudaStreamSynchronize(st), "group");
+    for (Pending& p : live) {
+      YieldEngine<T>& eng = *p.eng;
+      launches += eng.launches;
+      graphs += eng.graph_launches;
+      step_launches += eng.step_launches;
+      row_terms += eng.row_terms;
+      h2d += eng.h2d;
+      d2h += eng.d2h;
+      step_bytes += eng.step_bytes_all;
+      for (size_t i = 0; i + 1 < eng.pev.size(); i += 2) {
+        float t = 0.f;
+        ck(cudaEventElapsedTime(&t, eng.pev[i], eng.pev[i + 1]), "cudaEventElapsedTime");
+        step_ms += t;
+        step_timed += eng.pev_launches[i / 2];
+      }
+    }
+    live.clear();
+  };
   ck(cudaEventRecord(ev.a, st), "cudaEventRecord");
   for (size_t g0 = 0; g0 < order.size();) {
     size_t g1 = g0;
@@ -1677,36 +1762,35 @@ rp_status run_batch(int n_sys, rp_system* const* systems, const int* n_fields,
     }
     const std::vector<Item> items = make_items(gplans, first, count, out0, o.sample_offset, SampleMode{},
                                                &sys_of_field);
-    {
-      Arena ar(st);
-      YieldEngine<T> eng(group, o, n_c, st, ar, &pairs);
-      eng.set_seed(seed);
-      eng.set_fields(gplans, &sys_of_field);
+    auto prepare = [&]() {
+      Pending p;
+      p.ar = std::make_unique<Arena>(st);
+      p.eng = std::make_unique<YieldEngine<T>>(group, o, n_c, st, *p.ar, &pairs);
+      p.eng->set_seed(seed);
+      p.eng->set_fields(gplans, &sys_of_field);
       long long Zmax = 1;
       for (auto* h : group) Zmax = std::max<long long>(Zmax, h->Z);
       rp::HostSystem probe;
       probe.Z = Zmax;
       const int R = choose_rows<T>(probe, o, n_c, (long long)items.size());
       R_max = std::max(R_max, R);
-      eng.alloc_rows(R);
-      eng.run(items, d_ps);
-      ck(cudaStreamSynchronize(st), "group");
-      launches += eng.launches;
-      graphs += eng.graph_launches;
-      step_launches += eng.step_launches;
-      row_terms += eng.row_terms;
-      h2d += eng.h2d;
-      d2h += eng.d2h;
-      step_bytes += eng.step_bytes_all;
-      for (size_t i = 0; i + 1 < eng.pev.size(); i += 2) {
-        float t = 0.f;
-        ck(cudaEventElapsedTime(&t, eng.pev[i], eng.pev[i + 1]), "cudaEventElapsedTime");
-        step_ms += t;
-        step_timed += eng.pev_launches[i / 2];
-      }
+      p.eng->alloc_rows(R);
+      const bool side = p.eng->persistent() && !o.profile && lg(order.front()) != lg(order.back());
+      if (side) p.eng->launch_on(sides.next(), sides.fork);
+      p.eng->run(items, d_ps);
+      live.push_back(std::move(p));
+      if (!side) finish();
+    };
+    try {
+      prepare();
+    } catch (const CudaFail& e) {
+      if (e.st != RP_ENOMEM || live.empty()) throw;
+      finish();  // give back the scratch of the groups in flight, then once more
+      prepare();
     }
     g0 = g1;
   }
+  finish();
   // per-(system, field) statistics on the device
   std::vector<long long> offcnt(2 * (size_t)n_pairs);
   {
