@@ -172,9 +172,10 @@ int default_kernel_fp32(const HostSystem& hs, bool* cluster_ok) {
   return macro_cluster_default(hf) ? 4 : 1;
 }
 
-// kernel = 0 runs the persistent launch (kernel 5) for systems that fit one
-// CTA with 128 <= Z <= 1024, and for batches of several such systems up to
-// the size limit (measured faster than the on-chip macro-step launches).
+// Where the on-chip kernels of rp_chip.cu do not take a system that fits one CTA,
+// kernel = 0 runs the generic persistent launch for 128 <= Z <= 1024, and for batches of
+// several such systems up to the size limit (measured faster than the on-chip
+// macro-step launches).
 bool persistent_default(long long Zslot, int n_systems) {
   return Zslot >= 128 && (Zslot <= 1024 || n_systems > 1);
 }

@@ -678,14 +678,16 @@ __global__ void __launch_bounds__(kTermThreads, (term_min_blocks<T, LK, ANISO>()
 // per component into its own shared-memory slots some entries ahead of their use
 // (cp.async, no barrier: nobody else reads them).  phi_{n-2} and the accumulator follow
 // as the list's last entries.  An anisotropic partner has two entries; the second goes
-// straight to registers (a copy passes the L1 twice, which all copies would fill).  The tile's nuclei are unrolled and the fields of the
-// nuclei outside it come from a table, so a thread spends its instructions on products.
+// straight to registers (a copy passes the L1 twice, which all copies would fill).  The
+// tile's nuclei are unrolled and the fields of the nuclei outside it come from a table,
+// so a thread spends its instructions on products.
 //
-// Bounds: HBM and issue slots together.  Z = 2^20, 14 rows (7.5 GB of vectors): 355 us
-// per term in the general form, 353 with the copies alone (65 % of issue slots used, half
-// of them by integer work), 300 as it is, 5.0 TB/s of a measured 6.8.  Anisotropic, Z =
-// 2359296, 6 rows, whole call: 243, 232 and 187 ms, 177 with the second entries direct
-// (the same for every second isotropic partner: 305 us).
+// Bounds: HBM (isotropic), issue slots and L1 (anisotropic).  Z = 2^20, 14 rows (1.9 GB
+// of vectors): 355 us per term in the general form, 353 with the copies alone (65 % of
+// issue slots used, half of them by integer work), 300 as it is: at 3.9 vector passes
+// 6.1 TB/s of a measured 6.8.  Anisotropic, Z = 2359296, 6 rows, whole call: 243, 232
+// and 187 ms, 177 with the second entries direct (the same for every second isotropic
+// partner: 305 us).
 constexpr int kRingThreads = kTermThreads, kRingTileBits = 9;
 constexpr int kRingParts = 2 * kMaxNucDev;
 
