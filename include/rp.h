@@ -73,7 +73,8 @@ typedef struct rp_options {
   int n_cheb;             /* Chebyshev terms per macro-step, multiple of 4 in [8, 88]
                              (0: 88) */
   double tol;             /* truncation bound per macro-step (0: 1e-15 FP64, 1e-9 FP32) */
-  int max_rows;           /* concurrent propagations (0: from free device memory) */
+  int max_rows;           /* concurrent propagations (0: from free device memory; the
+                             cluster kernel, path 4, one per cluster that runs at once) */
   int deterministic;      /* 1: trace over the Z basis states |S, M> (Eq. 14)
                              instead of M coherent-state samples; M is ignored.
                              2: M basis states |S, M> drawn uniformly at random

@@ -420,6 +420,11 @@ class YieldEngine {
       cluster_ = (kq == 4 ? rp::macro_cluster_plan(hf, nullptr)
                                  : rp::macro_cluster_default(hf)) &&
                  rp::macro_cluster_max_active(hf) > 0;
+      // rows: one per cluster that runs at once, the others follow as rows finish (items
+      // come longest first).  More rows only leave clusters idle in the last wave of
+      // every macro-step: 64 propagations of Z = 20736 on 15 clusters at once, 79.1 ms in
+      // 64 rows, 73.1 in 45, 69.8 in 30, 68.8 in 15; 192 propagations 206.8 and 188.8 ms.
+      if (cluster_ && o_.max_rows <= 0) R_ = R = std::min(R, rp::macro_cluster_max_active(hf));
     }
     // the per-term kernels keep the state vectors in planes (rp_term.cu)
     term_ = !small_ && !cluster_;
