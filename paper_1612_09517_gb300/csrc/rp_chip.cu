@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
     const int row = tid / Sr, t = tid - row * Sr, base = row * Sr;
     const bool on = row < grp.y;
     chip_const<T>(K, H, F, LK, cb, tid);
-    if (tid < 2 * rpc) sums[tid] = 0.0;
+    for (int q = tid; q < 2 * rpc; q += blockDim.x) sums[q] = 0.0;
     const LayoutDev& Ly = A.lay[I0.sys];
     if (!A.deterministic)
       for (int q = tid; q < grp.y * Ly.n_nuc; q += blockDim.x) {
@@ -856,7 +856,7 @@ __global__ void __launch_bounds__(MT, 1) k_split_items(
     const int row = tid / (4 * Z), e = (tid - row * 4 * Z) / Z, m = tid % Z;
     const int slot = row * Z + m;  // 4 Z is a multiple of Z
     const bool on = row < grp.y;
-    if (tid < 2 * rpc) sums[tid] = 0.0;
+    for (int q = tid; q < 2 * rpc; q += blockDim.x) sums[q] = 0.0;
     const LayoutDev& Ly = A.lay[I0.sys];
     if (!A.deterministic)
       for (int q = tid; q < grp.y * Ly.n_nuc; q += blockDim.x) {
