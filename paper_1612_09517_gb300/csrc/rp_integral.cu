@@ -286,6 +286,58 @@ __global__ void __launch_bounds__(kProjThreads) k_project(
   if (tid == 0) atomicAdd(integral + r, tot);
 }
 
+// The same in FP64 for rows of at most 96 configurations.  A warp's FP64 instruction holds
+// its scheduler for 64 cycles however many of its lanes work, so a row of 16 configurations
+// on one warp leaves three of the four schedulers idle.  Here a warp takes eight columns of
+// every configuration, 32 at a time.  64 rows, one macro-step, in us (k_project, this):
+// Z = 16 154 and 53, 64 158 and 101, 96 159 and 148, 125 163 and 204; the Gram matrix of the
+// slices took 81 at Z = 16.
+constexpr int kFewConfigs = 96;
+constexpr int kFewCols = 32;  // eight per warp
+
+__global__ void __launch_bounds__(kProjThreads) k_project_few(
+    const SysTab<double> S, const double* __restrict__ X, const double* __restrict__ L, int ldk,
+    const int2* __restrict__ meta, const int* __restrict__ row_field,
+    const int2* __restrict__ row_win, int macro_arg, const int* __restrict__ macro_dev, int n_c,
+    double* __restrict__ integral) {
+  extern __shared__ __align__(16) unsigned char proj_smem[];
+  __shared__ double red[kProjThreads];
+  double* sl = reinterpret_cast<double*>(proj_smem);  // [n_c][kFewCols]
+  const int r = blockIdx.x, tid = threadIdx.x;
+  const int macro = macro_dev ? *macro_dev : macro_arg;
+  {
+    const int2 w = row_win[r];
+    if (macro < w.x || macro >= w.y) return;
+  }
+  const int Z = (int)S.ham[S.row_sys ? S.row_sys[r] : 0].Z;
+  const size_t Zs = (size_t)S.Zslot;
+  const int f = row_field[r];
+  const int2 mt = meta[f];
+  const int n_e = (mt.y + 1) & ~1;  // n_c is even
+  const double2* Xr = reinterpret_cast<const double2*>(X) + (size_t)r * n_c * Zs;
+  const double* l = sl + 8 * (tid >> 5);
+  double sum = 0.0;
+  for (int k0 = 0; k0 < mt.x; k0 += kFewCols) {
+    __syncthreads();
+    stage_factor<double, kFewCols>(sl, L + (size_t)f * n_c * ldk, ldk, n_e, k0, tid, kProjThreads);
+    __syncthreads();
+    for (int z = tid & 31; z < Z; z += 32) {
+      double yr[8], yi[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) yr[k] = yi[k] = 0.0;
+#pragma unroll 2
+      for (int n = 0; n < n_e; n += 2) {
+        const double2 u = Xr[n * Zs + z], v = Xr[(n + 1) * Zs + z];
+        proj_add(yr, yi, l + n * kFewCols, u.x, u.y);
+        proj_add(yr, yi, l + (n + 1) * kFewCols, v.y, -v.x);
+      }
+      sum += proj_norm8(yr, yi);
+    }
+  }
+  const double tot = block_sum<kProjThreads>(sum, red);
+  if (tid == 0) atomicAdd(integral + r, tot);
+}
+
 }  // namespace
 
 int integral_ldk(int n_c) { return (n_c + 7) & ~7; }
@@ -322,6 +374,13 @@ cudaError_t launch_project(const SysTab<T>& S, const T* X, const T* L, const int
                            const int* macro_dev, int rows, int n_c, double* integral,
                            cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
+  if constexpr (sizeof(T) == 8) {
+    if (S.Zslot <= kFewConfigs) {
+      k_project_few<<<rows, kProjThreads, (size_t)n_c * kFewCols * sizeof(double), st>>>(
+          S, X, L, integral_ldk(n_c), meta, row_field, row_win, macro, macro_dev, n_c, integral);
+      return cudaGetLastError();
+    }
+  }
   // a CTA takes up to 8 tiles of configurations (its L costs one tile's loads),
   // fewer where the rows alone would not give every SM several CTAs
   const long long tile = (long long)kProjThreads * ProjCfg<T>::kCfg;

@@ -495,42 +495,56 @@ __device__ __forceinline__ void term_epilogue(const HamDev<T>& H, const SysTab<T
 // every per-nucleus constant a fixed offset.
 template <typename T, bool ANISO, int NH = -1, int N1 = -1>
 __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S, Cx<T>* tile,
-                                          const FieldDev<T>* __restrict__ fields, int f, int r,
+                                          const FieldDev<T>& F, int f, int r,
                                           const T* __restrict__ cur, const T* __restrict__ prev,
                                           T* __restrict__ next, T* __restrict__ acc,
                                           T* __restrict__ X, const T* __restrict__ coef, int n_c,
-                                          int n, int mode, int xblk, const FieldDev<T>& one_field);
+                                          int n, int mode, int xblk);
 
-template <typename T, bool ANISO, int NH = -1, int N1 = -1>
+// Field of a step launch: by value for H psi (APPLY), else the table of every field.  A
+// call whose thousands of launches are all latency (rp_yields_static, Z = 16, 64 rows,
+// FP32) takes 36 ms with one kernel that chooses at run time, 26 like this.
+template <typename T, bool APPLY>
+struct StepField {
+  FieldDev<T> one;
+};
+template <typename T>
+struct StepField<T, false> {
+  const FieldDev<T>* all;
+};
+
+template <typename T, bool ANISO, bool APPLY, int NH = -1, int N1 = -1>
 __global__ void __launch_bounds__(kStepThreads,
                                   sizeof(T) == 4 ? (ANISO ? 4 : (NH >= 0 ? 5 : 6)) : 2)
     k_cheb_step(
-    const SysTab<T> S, const HamDev<T> H1, const FieldDev<T>* __restrict__ fields,
+    const SysTab<T> S, const HamDev<T> H1, const StepField<T, APPLY> fields,
     const int* __restrict__ row_field, const int2* __restrict__ row_win, int macro_arg,
     const int* __restrict__ macro_dev, const T* __restrict__ cur, const T* __restrict__ prev,
     T* __restrict__ next, T* __restrict__ acc, T* __restrict__ X, const T* __restrict__ coef,
-    int n_c, int n, int mode, int xblk, const FieldDev<T> one_field) {
+    int n_c, int n, int mode, int xblk) {
   extern __shared__ __align__(16) unsigned char step_smem[];
   Cx<T>* tile = reinterpret_cast<Cx<T>*>(step_smem);  // planes x blockDim x 16 B
   const int r = blockIdx.y;
-  int f = 0;
-  if (mode != MODE_APPLY) {
+  if constexpr (APPLY) {
+    step_body<T, ANISO, NH, N1>(H1, S, tile, fields.one, 0, r, cur, prev, next, acc, X, coef, n_c,
+                                n, MODE_APPLY, xblk);
+  } else {
     const int macro = macro_dev ? *macro_dev : macro_arg;
     const int2 w = row_win[r];
     if (macro < w.x || macro >= w.y) return;  // the whole block: one row
-    f = row_field[r];
+    const int f = row_field[r];
+    step_body<T, ANISO, NH, N1>(H1, S, tile, fields.all[f], f, r, cur, prev, next, acc, X, coef,
+                                n_c, n, mode, xblk);
   }
-  step_body<T, ANISO, NH, N1>(H1, S, tile, fields, f, r, cur, prev, next, acc, X, coef, n_c, n,
-                              mode, xblk, one_field);
 }
 
 template <typename T, bool ANISO, int NH, int N1>
 __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S, Cx<T>* tile,
-                                          const FieldDev<T>* __restrict__ fields, int f, int r,
+                                          const FieldDev<T>& F, int f, int r,
                                           const T* __restrict__ cur, const T* __restrict__ prev,
                                           T* __restrict__ next, T* __restrict__ acc,
                                           T* __restrict__ X, const T* __restrict__ coef, int n_c,
-                                          int n, int mode, int xblk, const FieldDev<T>& one_field) {
+                                          int n, int mode, int xblk) {
   const unsigned Z = (unsigned)H.Z;
   const unsigned m = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = m < Z;
@@ -686,8 +700,8 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
       add_partner<T, ANISO>(y, c, m - st, rr, H.U[p], sqrt(I * (I + 1) - M * (M + 1)), false);
   }
 
-  term_epilogue<T, ANISO>(H, S, fields ? fields[f] : one_field, a, y, b1, b2, f, r, m, row0, prev, next, acc, X, coef,
-                         n_c, n, mode, xblk);
+  term_epilogue<T, ANISO>(H, S, F, a, y, b1, b2, f, r, m, row0, prev, next, acc, X, coef, n_c, n,
+                          mode, xblk);
 }
 
 // ---- FP32 term with the block's partner tiles staged by bulk async copies ----
@@ -2024,23 +2038,26 @@ cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int
   while (b < kStepThreads && b < S.Zslot) b *= 2;
   const size_t smem = (size_t)b * 4 * sizeof(Cx<T>);
   dim3 grid(grid1(S.Zslot, b), rows);
-  // compiled shape (fixed nucleus loops, 48 registers and 5 blocks per SM instead of 40
-  // and 6 in FP32): 20 spin-1/2 nuclei, isotropic -- the paper's Table I model, 3 % faster.
+  // H psi: compiled shape (fixed nucleus loops, 48 registers and 5 blocks per SM instead of
+  // 40 and 6 in FP32): 20 spin-1/2 nuclei, isotropic -- the paper's Table I model, 3 % faster.
   // (The same for the 20-nucleus anisotropic workload needs 67 registers, 3 blocks per SM,
   // and measured 12 % slower than the generic kernel at 4.)
-  const bool t1_shape = !aniso && b == kStepThreads && one->n_half == 20 && one->n_nuc == 20;
-  if (t1_shape)
-    k_cheb_step<T, false, 20, 0><<<grid, b, smem, st>>>(S, *one, fields, row_field, row_win, macro,
-                                                        macro_dev, cur, prev, next, acc, X, coef,
-                                                        n_c, n, mode, xblk, F1);
-  else if (aniso)
-    k_cheb_step<T, true><<<grid, b, smem, st>>>(S, *one, fields, row_field, row_win, macro,
-                                                macro_dev, cur, prev, next, acc, X, coef, n_c, n,
-                                                mode, xblk, F1);
-  else
-    k_cheb_step<T, false><<<grid, b, smem, st>>>(S, *one, fields, row_field, row_win, macro,
-                                                 macro_dev, cur, prev, next, acc, X, coef, n_c, n,
-                                                 mode, xblk, F1);
+  const StepField<T, false> all{fields};
+  const StepField<T, true> field{F1};
+  auto go = [&](auto kf, const auto& F) {
+    kf<<<grid, b, smem, st>>>(S, *one, F, row_field, row_win, macro, macro_dev, cur, prev, next,
+                              acc, X, coef, n_c, n, mode, xblk);
+  };
+  if (mode != MODE_APPLY) {
+    if (aniso) go(k_cheb_step<T, true, false>, all);
+    else go(k_cheb_step<T, false, false>, all);
+  } else if (aniso) {
+    go(k_cheb_step<T, true, true>, field);
+  } else if (b == kStepThreads && one->n_half == 20 && one->n_nuc == 20) {
+    go(k_cheb_step<T, false, true, 20, 0>, field);
+  } else {
+    go(k_cheb_step<T, false, true>, field);
+  }
   return cudaGetLastError();
 }
 
