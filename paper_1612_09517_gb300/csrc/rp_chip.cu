@@ -606,6 +606,70 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sums over a block in a fixed order, so that equal calls give equal bits (atomics on
+// shared memory add in the order in which the warps arrive).
+
+// sums[2 row], sums[2 row + 1] of the rows of a block, a row's `per_row` threads side by
+// side: thread i left its integral at p[i * step] and its norm at p[i * step + norm].  A
+// warp per row, once per item.
+__device__ __forceinline__ void row_sums(const double* p, int step, int norm, int rows,
+                                         int per_row, double* sums, int tid) {
+  const int lane = tid & 31, warps = (int)blockDim.x >> 5;
+#pragma unroll 1
+  for (int row = tid >> 5; row < rows; row += warps) {
+    double a = 0.0, b = 0.0;
+#pragma unroll 1
+    for (int i = lane; i < per_row; i += 32) {
+      const double* q = p + (row * per_row + i) * step;
+      a += q[0];
+      b += q[norm];
+    }
+    a = warp_sum(a);
+    b = warp_sum(b);
+    if (lane == 0) {
+      sums[2 * row] = a;
+      sums[2 * row + 1] = b;
+    }
+  }
+}
+
+// Scratch of trace_add: sums of the warps, then of the block (read by rank 0 of a cluster).
+struct alignas(16) TraceSums {
+  double warp[32][4], block[4];
+};
+
+// at[q] += the block's (cluster's) sum of v[q]: one addition per macro-step.  Every thread
+// of the block calls it; the barriers of the next macro-step keep its scratch.
+template <int CB>
+__device__ __forceinline__ void trace_add(TraceSums& W, const double (&v)[4], int nq, double* at,
+                                          int tid, unsigned rank) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (q >= nq) break;
+    const double w = warp_sum(v[q]);
+    if ((tid & 31) == 0) W.warp[tid >> 5][q] = w;
+  }
+  __syncthreads();
+  double s = 0.0;
+  if (tid < nq) {
+#pragma unroll 1
+    for (int k = 0; k < ((int)blockDim.x >> 5); ++k) s += W.warp[k][tid];
+  }
+  if constexpr (CB > 0) {
+    if (tid < nq) W.block[tid] = s;
+    chip_barrier<CB>();
+    if (tid < nq && rank == 0)
+      for (unsigned k = 1; k < (1u << CB); ++k) {
+        double u;
+        asm volatile("ld.shared::cluster.f64 %0, [%1];"
+                     : "=d"(u)
+                     : "r"(chip_peer(smem_u32(&W.block[tid]), k)));
+        s += u;
+      }
+  }
+  if (tid < nq && rank == 0) atomicAdd(at + tid, s);
+}
+
 // One launch over all items: CTAs take groups of up to rpc items of one field
 // from a device counter and run their whole horizon.  Shared memory: two
 // buffers of S slots (the second doubles as the integral's ring), the factor L,
@@ -622,6 +686,7 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
   constexpr int KPT = 1 << LK, KB = ProjCfg<T>::kB;
   extern __shared__ __align__(16) unsigned char chip_smem[];
   __shared__ int s_group;
+  __shared__ TraceSums s_trace;
   ChipConst<T>& K = *reinterpret_cast<ChipConst<T>*>(chip_smem);
   Cx<T>* buf = reinterpret_cast<Cx<T>*>(chip_smem + sizeof(ChipConst<T>));
   T* dt = reinterpret_cast<T*>(buf + (size_t)8 * KPT * S);  // diagonals [KPT][S][4]
@@ -653,7 +718,6 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
     const int row = tid / Sr, t = tid - row * Sr, base = row * Sr;
     const bool on = row < grp.y;
     chip_const<T>(K, H, F, LK, cb, tid);
-    for (int q = tid; q < 2 * rpc; q += blockDim.x) sums[q] = 0.0;
     const LayoutDev& Ly = A.lay[I0.sys];
     if (!A.deterministic)
       for (int q = tid; q < grp.y * Ly.n_nuc; q += blockDim.x) {
@@ -743,20 +807,21 @@ __global__ void __launch_bounds__(MT, MB) k_chip_items(
 #pragma unroll
           for (int c = 0; c < KPT; ++c) trace_terms<T>(a[c], op, v);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (q >= 2 && !op.on) break;
-          const double w = warp_sum(v[q]);
-          if ((tid & 31) == 0 && w != 0.0) atomicAdd(trace + 4 * (km + 1) + q, w);
-        }
+        trace_add<CB>(s_trace, v, op.on ? 4 : 2, trace + 4 * (km + 1), tid, rank);
       }
     }
+    // integral and norm to the thread's own entries of the ring, which it is done with
+    constexpr int kStep = (int)(sizeof(typename SliceVal<T>::type) / sizeof(double));
     if (on) {
       Cx<T> a[KPT][4];
       chip_get<T, LK>(buf, S, base + t, a);
-      atomicAdd(&sums[2 * row], integral);
-      atomicAdd(&sums[2 * row + 1], chip_norm<T, KPT>(a));
+      double* own = reinterpret_cast<double*>(ring);
+      own[0] = integral;
+      own[kStep * S] = chip_norm<T, KPT>(a);
     }
+    __syncthreads();
+    row_sums(reinterpret_cast<const double*>(buf + (size_t)4 * KPT * S), kStep, kStep * S, grp.y, Sr,
+             sums, tid);
     chip_barrier<CB>();
     if (tid < grp.y && rank == 0) {
       double si = sums[2 * tid], surv = sums[2 * tid + 1];
@@ -836,6 +901,7 @@ __global__ void __launch_bounds__(MT, 1) k_split_items(
     double* __restrict__ trace, const ElecOp op) {
   extern __shared__ __align__(16) unsigned char chip_smem[];
   __shared__ int s_group;
+  __shared__ TraceSums s_trace;
   // two buffers [e][S], slices [n_c][S], factor [n_c][32], sums, amplitudes
   Cx<T>* buf = reinterpret_cast<Cx<T>*>(chip_smem);
   Cx<T>* xs = buf + (size_t)8 * S;
@@ -856,7 +922,6 @@ __global__ void __launch_bounds__(MT, 1) k_split_items(
     const int row = tid / (4 * Z), e = (tid - row * 4 * Z) / Z, m = tid % Z;
     const int slot = row * Z + m;  // 4 Z is a multiple of Z
     const bool on = row < grp.y;
-    for (int q = tid; q < 2 * rpc; q += blockDim.x) sums[q] = 0.0;
     const LayoutDev& Ly = A.lay[I0.sys];
     if (!A.deterministic)
       for (int q = tid; q < grp.y * Ly.n_nuc; q += blockDim.x) {
@@ -1010,18 +1075,17 @@ __global__ void __launch_bounds__(MT, 1) k_split_items(
           const Cx<T> c4[4] = {buf[slot], buf[S + slot], buf[2 * S + slot], buf[3 * S + slot]};
           trace_terms<T>(c4, op, v);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (q >= 2 && !op.on) break;
-          const double w = warp_sum(v[q]);
-          if ((tid & 31) == 0 && w != 0.0) atomicAdd(trace + 4 * (km + 1) + q, w);
-        }
+        trace_add<0>(s_trace, v, op.on ? 4 : 2, trace + 4 * (km + 1), tid, 0u);
       }
     }
+    double* part = reinterpret_cast<double*>(buf);  // psi is in registers
+    __syncthreads();
     if (on) {
-      atomicAdd(&sums[2 * row], integral);
-      atomicAdd(&sums[2 * row + 1], (double)a.re * (double)a.re + (double)a.im * (double)a.im);
+      part[2 * tid] = integral;
+      part[2 * tid + 1] = (double)a.re * (double)a.re + (double)a.im * (double)a.im;
     }
+    __syncthreads();
+    row_sums(part, 2, 1, grp.y, 4 * Z, sums, tid);
     __syncthreads();
     if (tid < grp.y) {
       const double phS = A.k_S[I0.sys] * sums[2 * tid], surv = sums[2 * tid + 1];
@@ -1133,12 +1197,13 @@ __device__ __forceinline__ void aniso_term(const AnisoConst<T>& K, const AnisoRo
 }
 
 template <typename T, int CB, int MT>
-__global__ void __launch_bounds__(MT, 1) k_split_aniso(
+__global__ void __launch_bounds__(MT, CB == 0 && MT == 256 ? 2 : 1) k_split_aniso(
     const ChipArgs<T> A, const PItem* __restrict__ items, const int2* __restrict__ groups,
     int n_groups, int* __restrict__ counter, int S, double* __restrict__ per_sample,
     double* __restrict__ trace, const ElecOp op) {
   extern __shared__ __align__(16) unsigned char chip_smem[];
   __shared__ int s_group;
+  __shared__ TraceSums s_trace;
   __shared__ __align__(16) double sums[2];
   __shared__ AnisoConst<T> K;
   // two buffers [e][S], slices [n_c][S], factor [n_c][32], amplitudes
@@ -1207,7 +1272,6 @@ __global__ void __launch_bounds__(MT, 1) k_split_aniso(
       K.lb = lb;
       K.n_nuc = H.n_nuc;
     }
-    if (tid < 2) sums[tid] = 0.0;
     const T* cf = A.coef + (size_t)I0.field * 2 * A.n_c;
     const T* cl = cf + A.n_c;
     int2 mt = make_int2(0, 0);
@@ -1335,19 +1399,18 @@ __global__ void __launch_bounds__(MT, 1) k_split_aniso(
           const Cx<T> c4[4] = {buf[l], buf[S + l], buf[2 * S + l], buf[3 * S + l]};
           trace_terms<T>(c4, op, v);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (q >= 2 && !op.on) break;
-          const double w = warp_sum(v[q]);
-          if ((tid & 31) == 0 && w != 0.0) atomicAdd(trace + 4 * (km + 1) + q, w);
-        }
+        trace_add<CB>(s_trace, v, op.on ? 4 : 2, trace + 4 * (km + 1), tid, rank);
         __syncthreads();
       }
     }
+    double* part = reinterpret_cast<double*>(buf);  // psi is in registers
+    __syncthreads();
     if (on) {
-      atomicAdd(&sums[0], integral);
-      atomicAdd(&sums[1], (double)a.re * (double)a.re + (double)a.im * (double)a.im);
+      part[2 * tid] = integral;
+      part[2 * tid + 1] = (double)a.re * (double)a.re + (double)a.im * (double)a.im;
     }
+    __syncthreads();
+    row_sums(part, 2, 1, 1, 4 * Zl, sums, tid);
     chip_barrier<CB>();
     if (tid == 0 && rank == 0) {
       double si = sums[0], surv = sums[1];

@@ -382,10 +382,13 @@ cudaError_t launch_project(const SysTab<T>& S, const T* X, const T* L, const int
     }
   }
   // a CTA takes up to 8 tiles of configurations (its L costs one tile's loads),
-  // fewer where the rows alone would not give every SM several CTAs
+  // fewer where the rows alone would not give every SM several CTAs.  A row of up to
+  // 1024 configurations is one CTA's: its sum then runs in a fixed order, and equal calls
+  // give equal bits
   const long long tile = (long long)kProjThreads * ProjCfg<T>::kCfg;
   const long long tiles = (S.Zslot + tile - 1) / tile;
-  const long long per = std::min<long long>(8, std::max<long long>(1, tiles * rows / (152 * 12)));
+  const long long per = S.Zslot <= 1024 ? tiles
+                                        : std::min<long long>(8, std::max<long long>(1, tiles * rows / (152 * 12)));
   dim3 grid((unsigned)((tiles + per - 1) / per), rows);
   const size_t smem = proj_smem_bytes<T>(n_c);
   static std::atomic<unsigned long long> attr_done;
