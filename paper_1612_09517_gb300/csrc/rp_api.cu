@@ -1782,7 +1782,10 @@ rp_status run_batch(int n_sys, rp_system* const* systems, const int* n_fields,
       R_max = std::max(R_max, R);
       p.eng->alloc_rows(R);
       const bool side = p.eng->persistent() && !o.profile && lg(order.front()) != lg(order.back());
-      if (side) p.eng->launch_on(sides.next(), sides.fork);
+      if (side) {
+        const cudaStream_t s = sides.next();  // makes the event on its first call
+        p.eng->launch_on(s, sides.fork);
+      }
       p.eng->run(items, d_ps);
       live.push_back(std::move(p));
       if (!side) finish();
