@@ -74,7 +74,11 @@ typedef struct rp_options {
                              (0: 88) */
   double tol;             /* truncation bound per macro-step (0: 1e-15 FP64, 1e-9 FP32) */
   int max_rows;           /* concurrent propagations (0: from free device memory; the
-                             cluster kernel, path 4, one per cluster that runs at once) */
+                             cluster kernel, path 4, one per cluster that runs at once).
+                             It bounds the rows kept in device memory: yields that run as
+                             one launch (kernel 5; kernel 0 where 128 <= Z <= 1024, and
+                             batches of systems that fit one CTA) keep none and take all
+                             the CTAs that run at once */
   int deterministic;      /* 1: trace over the Z basis states |S, M> (Eq. 14)
                              instead of M coherent-state samples; M is ignored.
                              2: M basis states |S, M> drawn uniformly at random

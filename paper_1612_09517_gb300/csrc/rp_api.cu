@@ -179,6 +179,14 @@ int default_kernel_fp32(const HostSystem& hs, bool* cluster_ok) {
 bool persistent_default(long long Zslot, int n_systems) {
   return Zslot >= 128 && (Zslot <= 1024 || n_systems > 1);
 }
+
+// Calls that always run as one launch over all items.  Such a launch keeps no rows in
+// device memory, so max_rows does not bound it (Z = 864, 32 propagations, max_rows = 1:
+// 2.8 ms, 38.9 with one block at a time).
+bool one_launch(long long Zslot, long long Zmax_chip, int n_systems, const rp_options& o) {
+  return Zslot <= Zmax_chip && o.deterministic != 3 &&
+         (o.kernel == 5 || (o.kernel == 0 && !o.graph && persistent_default(Zslot, n_systems)));
+}
 }  // namespace rp
 
 namespace {
@@ -346,7 +354,8 @@ class YieldEngine {
 
   long long zslot() const { return Zslot_; }
 
-  void alloc_rows(int R) {
+  // in_flight: propagations of the largest round to come, where there are several (0: R)
+  void alloc_rows(int R, long long in_flight = 0) {
     R_ = R;
     // Isotropic systems that fit one CTA run their whole horizon on chip in one
     // launch over all items (kernel = 5, and kernel = 0 without graph replay,
@@ -391,7 +400,9 @@ class YieldEngine {
     if (persist_ && chip_) {
       pctas_ = rp::chip_ctas<T>(cplan_);
       if (pctas_ <= 0) throw CudaFail{RP_ECUDA, "on-chip kernel: no device"};
-      pctas_ = std::min(pctas_, ((R + cplan_.rpc - 1) / cplan_.rpc) << cplan_.cb);
+      const bool all = !d_trace_ && rp::one_launch(Zslot_, rp::small_max_configs<T>(), (int)sys_.size(), o_);
+      const long long rows = all ? std::max<long long>(R, in_flight) : R;
+      pctas_ = (int)std::min<long long>(pctas_, ((rows + cplan_.rpc - 1) / cplan_.rpc) << cplan_.cb);
       d_counter_ = ar_.get<int>(1);
       if (!d_trace_) {
         if (!cplan_.split && !cplan_.aniso) Xp_ = ar_.get<T>((size_t)pctas_ * n_c_ * ((size_t)cplan_.slots << cplan_.lk) * 2);
@@ -1009,8 +1020,10 @@ class YieldEngine {
 
 // Rows to allocate: the caller's cap, else 45 % of free device memory.
 template <typename T>
-int choose_rows(const rp::HostSystem& hs, const rp_options& o, int n_c, long long items) {
-  long long cap = o.max_rows > 0 ? o.max_rows : 0;
+int choose_rows(const rp::HostSystem& hs, const rp_options& o, int n_c, long long items,
+                bool trace = false, int n_systems = 1) {
+  const bool all = !trace && rp::one_launch(hs.Z, rp::small_max_configs<T>(), n_systems, o);
+  long long cap = o.max_rows > 0 && !all ? o.max_rows : 0;
   if (cap == 0) {
     size_t fr = 0, tot = 0;
     ck(cudaMemGetInfo(&fr, &tot), "cudaMemGetInfo");
@@ -1205,7 +1218,7 @@ rp_status run_time_trace(rp_system* sys, double B, int M, uint64_t seed, double 
   std::vector<long long> first(1, 0), count(1, Mr), out0(1, 0);
   const std::vector<Item> items = make_items(plans, first, count, out0, o.sample_offset,
                                              SampleMode{o.deterministic, seed, o.pair_id, hs.Z});
-  const int R = choose_rows<T>(hs, o, n_c, (long long)items.size());
+  const int R = choose_rows<T>(hs, o, n_c, (long long)items.size(), true);
   std::vector<double> h_tr(4 * (size_t)n_times, 0.0);
   rp::ElecOp op{};
   if (A_e) {
@@ -1293,7 +1306,7 @@ rp_status run_converged(rp_system* sys, int n_fields, const double* fields, doub
     ck(cudaEventRecord(ev.a, st), "cudaEventRecord");
     eng.set_fields(plans);
     R = choose_rows<T>(hs, o, n_c, std::max<long long>((long long)n_fields * M_min, 256));
-    eng.alloc_rows(R);
+    eng.alloc_rows(R, (long long)n_fields * M_max);
     for (int round = 0; round < 8; ++round) {
       std::vector<long long> first(n_fields), count(n_fields), out0(n_fields);
       long long n = 0;
@@ -1415,7 +1428,7 @@ rp_status run_converged_cv(rp_system* sys, int n_fields, const double* fields, d
     ck(cudaEventRecord(ev.a, st), "cudaEventRecord");
     eng.set_fields(plans);
     R = choose_rows<T>(hs, o, n_c, std::max<long long>((long long)n_fields * M_min, 256));
-    eng.alloc_rows(R);
+    eng.alloc_rows(R, (long long)n_fields * M_max);
     // run counts[f] new samples of field f starting at first[f]; per-sample results appended
     auto run_round = [&](const std::vector<long long>& first, const std::vector<long long>& count,
                          std::vector<std::vector<double>>& dst) {
@@ -1778,7 +1791,7 @@ rp_status run_batch(int n_sys, rp_system* const* systems, const int* n_fields,
       for (auto* h : group) Zmax = std::max<long long>(Zmax, h->Z);
       rp::HostSystem probe;
       probe.Z = Zmax;
-      const int R = choose_rows<T>(probe, o, n_c, (long long)items.size());
+      const int R = choose_rows<T>(probe, o, n_c, (long long)items.size(), false, (int)group.size());
       R_max = std::max(R_max, R);
       p.eng->alloc_rows(R);
       const bool side = p.eng->persistent() && !o.profile && lg(order.front()) != lg(order.back());
