@@ -524,14 +524,18 @@ class YieldEngine {
     if (n > 2000000000LL) throw CudaFail{RP_EINVAL, "too many propagations for one launch"};
     std::vector<rp::PItem> h((size_t)n);
     std::vector<double> cost((size_t)n);
+    // HBM: the singlet slices out and back in per macro-step; the kernels with one thread
+    // per configuration and electron state keep them on chip, a time trace has none
+    const bool slices = !d_trace_ && !(chip_ && (cplan_.split || cplan_.aniso));
+    double bytes = 0.0;
     for (long long i = 0; i < n; ++i) {
       const Item& it = items[(size_t)i];
       h[(size_t)i] = rp::PItem{it.field, it.sys, it.n_macro, 0, it.sample, it.out};
       cost[(size_t)i] = (double)it.n_macro * (double)sys_[it.sys]->Z;
       row_terms += (long long)it.n_macro * n_c_;
-      // HBM: the singlet slices out and back in per macro-step
-      step_bytes_all += 2.0 * n_c_ * (double)sys_[it.sys]->Z * 2.0 * sizeof(T) * it.n_macro;
+      if (slices) bytes += 2.0 * n_c_ * (double)sys_[it.sys]->Z * 2.0 * sizeof(T) * it.n_macro;
     }
+    step_bytes_all += bytes;
     // longest items first (the CTAs take them in this order), so the launch
     // does not end on one long item started last
     std::vector<size_t> ord((size_t)n);
@@ -588,7 +592,7 @@ class YieldEngine {
     step_launches += 1;
     if (o_.profile) {
       ck(cudaEventRecord(pev.back(), ls), "cudaEventRecord");
-      pev_bytes.push_back(step_bytes_all);
+      pev_bytes.push_back(bytes);
       pev_launches.push_back(1);
     }
     if (!side_launch_) ck(cudaStreamSynchronize(st_), "kernel execution");
