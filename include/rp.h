@@ -158,7 +158,8 @@ typedef struct rp_stats {
   long long graph_launches;     /* macro-steps replayed from a CUDA graph (graph = 1);
                                    their kernels are counted in kernel_launches */
   int kernel_path;              /* kernel path of the Chebyshev terms (rp_options.kernel
-                                   values 1-5; rp_yields and rp_yields_converged) */
+                                   values 1, 2, 4 and 5; rp_yields and
+                                   rp_yields_converged) */
   double cv_ms;                 /* rp_yields_cv: host wall time of the control-variate
                                    work (training, mu = E[g], evaluation, estimates) */
 } rp_stats;

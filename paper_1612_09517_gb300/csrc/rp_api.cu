@@ -744,7 +744,7 @@ class YieldEngine {
     ck(cudaMemcpyAsync(&h_err, d_err_, sizeof(int), cudaMemcpyDeviceToHost, st_), "d2h error word");
     d2h += (long long)sizeof(int);
     ck(cudaStreamSynchronize(st_), "kernel execution");
-    if (h_err) throw CudaFail{RP_ETIMEOUT, "a bounded device wait gave up (bulk tile copies)"};
+    if (h_err) throw CudaFail{RP_ETIMEOUT, "a bounded device wait gave up (tensor-core time integral)"};
   }
 
   void set_seed(uint64_t seed) { seed_ = seed; }
@@ -765,11 +765,11 @@ class YieldEngine {
     sec_scale_ = scale;
   }
 
-  // Kernel path taken (rp_stats.kernel_path): 5 persistent, 4 cluster, 2 one
-  // CTA per row, 3 staged per-term, 1 per-term.
+  // Kernel path taken (rp_stats.kernel_path): 5 one launch over all items, 4 clusters, 2
+  // one CTA per row, 1 one launch per term.
   int kernel_path() const {
     if (persist_) return Zslot_ <= rp::small_max_configs<T>() ? 5 : 4;
-    return cluster_ ? 4 : (small_ ? 2 : (o_.kernel == 3 ? 3 : 1));
+    return cluster_ ? 4 : (small_ ? 2 : 1);
   }
   // Rows propagated at once: CTAs of the persistent launch, else allocated rows.
   int rows_used() const { return persist_ ? pctas_ >> cplan_.cb : R_; }
