@@ -1,24 +1,31 @@
 // Forward pass of the control-variate network on the tensor cores.
 //
-// The weights are BF16 numbers; an FP32 activation is the exact sum of three (8 + 8 +
-// 8 mantissa bits), so a layer is three tcgen05.mma kind::f16 products per weight tile
-// with FP32 accumulators: every product is exact, as in an FP32 multiply-add of the
-// same numbers.  The tensor core's FP32 sums are not rounded to nearest, and the error
-// grows with the number of MMAs into one accumulator: after 32 inputs (2 MMAs of each
-// part, the low parts first) the accumulator is drained into FP32 sums in registers while the other buffer fills.
+// The tensor core's FP32 sums are truncated, not rounded to nearest, and a truncated sum is
+// too small in magnitude: every layer's result shrinks, which no averaging over samples
+// removes.  So the large products are summed without any rounding.  The activations of a
+// row and the weights of an output are each cut at 2^-8 of their largest magnitude,
+//   a = a1 + a2 + a3,  w = w1 + w2,
+// a1 and w1 whole multiples (at most 128 in magnitude) of a power of two of the row or
+// output.  A sum of up to 256 products a1 w1 then has at most 23 bits: exact in FP32 in any
+// order.  It has an accumulator of its own.  a2, a3 (BF16) and w2 hold what is left, and
+// the products with them, 2^-8 of the sum and smaller, go to a second accumulator, where
+// truncation is far below the FP32 rounding of the result.  w1 + w2 is the BF16 weight
+// exactly, a1 + a2 + a3 the FP32 activation to 2^-26 of the row's largest.  Errors of g,
+// E[g] and its variance against 64 bits, 4096 samples, 3 x 256, means over six networks:
+// 2.2e-7 (rms), 2.2e-8 and 2.8e-8; the layer-by-layer pass in rounded FP32 has 6.4e-7,
+// 1.6e-8 and 3.3e-8; one accumulator drained every 32 inputs had 2.9e-7, 7.7e-8, 3.1e-7.
+// (Numbers below 2^-119 or from 2^126 on are not cut: a1 or w1 is zero.)
 //
 // One CTA takes 128 feature rows through all layers: activations never leave the chip.
 // 512 threads hold the sums of one row and a quarter of the outputs each, apply bias
 // and SiLU and write the split activations as the next layer's A operand (256 threads
 // with half a row each spilled: with the issuing warp they have 168 registers); one
-// thread of another warp streams weight tiles (16 inputs x all outputs, one bulk copy each, four in
-// flight) and issues the MMAs.  All waits are bounded.
+// thread of another warp streams weight tiles (w1 and w2 of 16 inputs x all outputs in
+// turn, one bulk copy each, four in flight) and issues the MMAs.  All waits are bounded.
 //
-// Bounds: within a CTA the layers of a tile are a chain (products, drain, SiLU, next
-// operand); the tensor cores are busy about a quarter of the time.  65536 rows x 8
-// fields, 46 inputs, 3 x 256: 9.3 ms as FP32 CUDA-core products with a pass over memory
-// per layer and activation, 2.1 ms here.  Draining every 64 inputs instead of 32 takes
-// 1.9 ms, but the variance of g is then off by 1.1e-6 (5e-7 as it is, 6e-7 in FP32).
+// Bounds: within a CTA the layers of a tile are a chain (products, SiLU, next operand).
+// 65536 rows x 8 fields, 46 inputs, 3 x 256: 9.3 ms as FP32 CUDA-core products with a pass
+// over memory per layer and activation, 2.2 ms with the drained accumulator, 2.1 here.
 #include <algorithm>
 #include <atomic>
 
@@ -34,9 +41,8 @@ constexpr int kRows = 128;
 constexpr int kWorkers = 512;           // four threads per row
 constexpr int kMlpThreads = kWorkers + 32;
 constexpr int kTileK = 16, kTiles = 4;  // inputs per weight tile, tiles in flight
-constexpr int kGroup = 2;               // weight tiles per accumulator
 
-// outputs padded to the tile of an instance, inputs of the first layer to whole tiles
+// Outputs padded to the tile of an instance, inputs of the first layer to whole tiles
 inline int pad_hidden(int h) { return h <= 64 ? 64 : h <= 128 ? 128 : 256; }
 __host__ __device__ inline int pad_in(int d) { return (d + kTileK - 1) / kTileK * kTileK; }
 
@@ -61,19 +67,35 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
   return v;
 }
-__device__ __forceinline__ void mbar_arrive(unsigned bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void worker_sync() {
   asm volatile("bar.sync 1, %0;" ::"n"(kWorkers) : "memory");
 }
 
-// Weight tile t of the stream: [input / 8][output / 8][8 outputs][8 inputs]; after the
-// tiles the biases of the hidden layers and the output layer's weights, FP32, HP each.
+// The power of two that cuts numbers of magnitude up to `top`: multiples of it reach 128 at
+// `top`.  Zero where nothing is cut: tops whose powers leave the range of FP32.
+struct Cut {
+  float grid, inv;
+};
+__device__ __forceinline__ Cut cut_of(float top) {
+  const int e = (int)(__float_as_uint(top) >> 23) - 126;  // 2^(e-1) <= top < 2^e
+  if (e < -118 || e > 126) return {0.f, 0.f};
+  return {__uint_as_float((unsigned)(e + 120) << 23), __uint_as_float((unsigned)(134 - e) << 23)};
+}
+// v less its multiple of the grid (to nearest), which goes to `high`; both exact.
+__device__ __forceinline__ float cut_high(const Cut& c, float v, float& high) {
+  const float q = fmaf(v, c.inv, 12582912.f) - 12582912.f;  // 1.5 2^23: rounds to an integer
+  high = q * c.grid;
+  return fmaf(-q, c.grid, v);
+}
+
+// Tile t of the stream: [part][input / 8][output / 8][8 outputs][8 inputs], part 0 w1 and 1
+// w2; after the tiles the biases of the hidden layers and the output layer's weights, FP32,
+// HP each.  A warp per output of a hidden layer, then a thread per value of the rest.
 __global__ void k_mlp_pack(const MlpNet N, int HP, __nv_bfloat16* __restrict__ out, long long total) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) {
-    const int j = (int)(i - total), l = j / HP, o = j % HP;
+  const int rows = N.layers * HP, warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (warp >= rows) {
+    const int j = (warp - rows) * 32 + lane, l = j / HP, o = j % HP;
     if (l > N.layers) return;
     float v = 0.f;
     if (o < N.hidden)
@@ -81,17 +103,28 @@ __global__ void k_mlp_pack(const MlpNet N, int HP, __nv_bfloat16* __restrict__ o
     reinterpret_cast<float*>(out + total)[j] = v;
     return;
   }
-  const int tile = HP * kTileK, t = (int)(i / tile), w = (int)(i % tile);
-  const int t0 = pad_in(N.d_in) / kTileK, th = HP / kTileK;
-  const int l = t < t0 ? 0 : 1 + (t - t0) / th, c = t < t0 ? t : (t - t0) % th;
-  const int k = c * kTileK + w / (HP * 8) * 8 + w % 8, o = w % (HP * 8) / 8;
-  const int in = l == 0 ? N.d_in : N.hidden;
-  out[i] = k < in && o < N.hidden ? N.wbf[N.w_off[l] + (long long)o * in + k] : __float2bfloat16(0.f);
+  const int l = warp / HP, o = warp % HP;
+  const int in = l == 0 ? N.d_in : N.hidden, pad = l == 0 ? pad_in(N.d_in) : HP;
+  const int t0 = l == 0 ? 0 : (pad_in(N.d_in) + (l - 1) * HP) / kTileK;  // first tile of the layer
+  const __nv_bfloat16* w = N.wbf + N.w_off[l] + (long long)o * in;
+  const bool on = o < N.hidden;
+  float top = 0.f;
+  for (int k = lane; on && k < in; k += 32) top = fmaxf(top, fabsf(__bfloat162float(w[k])));
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, s));
+  const Cut c = cut_of(top);
+  for (int k = lane; k < pad; k += 32) {
+    float high, low = 0.f;
+    low = cut_high(c, on && k < in ? __bfloat162float(w[k]) : 0.f, high);
+    __nv_bfloat16* d = out + (size_t)(2 * (t0 + k / kTileK)) * HP * kTileK +
+                       (k % kTileK) / 8 * (HP * 8) + o * 8 + k % 8;
+    d[0] = __float2bfloat16(high);
+    d[(size_t)HP * kTileK] = __float2bfloat16(low);
+  }
 }
 
-// Eight activations of a row to the A operand (parts `part` bytes apart): v = hi + mid +
-// lo exactly, barring underflow of the low parts.
-__device__ __forceinline__ void put8(unsigned char* A, unsigned part, int row, int k8,
+// Eight activations of a row to the three parts of the A operand (`part` bytes apart).
+__device__ __forceinline__ void put8(unsigned char* A, unsigned part, int row, int k8, const Cut& c,
                                      float (&v)[8]) {
   unsigned char* d = A + (unsigned)k8 * (kRows * 16) + (unsigned)row * 16;
 #pragma unroll
@@ -99,10 +132,17 @@ __device__ __forceinline__ void put8(unsigned char* A, unsigned part, int row, i
     unsigned w[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+      float x = v[2 * i], y = v[2 * i + 1];
+      if (q == 0) {
+        v[2 * i] = cut_high(c, x, x);
+        v[2 * i + 1] = cut_high(c, y, y);
+      }
+      const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
       w[i] = *reinterpret_cast<const unsigned*>(&h);
-      v[2 * i] -= __low2float(h);
-      v[2 * i + 1] -= __high2float(h);
+      if (q > 0) {
+        v[2 * i] = x - __low2float(h);
+        v[2 * i + 1] = y - __high2float(h);
+      }
     }
     *reinterpret_cast<uint4*>(d + q * part) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -115,23 +155,22 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
     double* __restrict__ acc, int* __restrict__ err, unsigned part) {
   constexpr int CPT = HP / 4;  // outputs per thread
   constexpr unsigned kTileBytes = HP * kTileK * 2;
-  extern __shared__ __align__(1024) unsigned char mlp_smem[];
-  // full[tile], empty[tile], ready[accumulator], drained[accumulator]
-  __shared__ __align__(8) unsigned long long bars[2 * kTiles + 4];
+  extern __shared__ __align__(128) unsigned char mlp_smem[];
+  // full[tile], empty[tile], then: a layer's products are done
+  __shared__ __align__(8) unsigned long long bars[2 * kTiles + 1];
   __shared__ unsigned tmem_slot;
-  __shared__ float part_g[3][kRows];
+  // largest magnitudes of the quarters of a row; at the end their shares of g
+  __shared__ float quarters[4][kRows];
+  __shared__ double moments[4][2];
   unsigned char* A = mlp_smem;  // three parts of [input / 8][row][8 inputs]
   const unsigned a_base = smem_u32(mlp_smem), w_base = a_base + 3 * part;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   auto full = [&](int i) { return smem_u32(&bars[i]); };
   auto empty = [&](int i) { return smem_u32(&bars[kTiles + i]); };
-  auto ready = [&](int i) { return smem_u32(&bars[2 * kTiles + i]); };
-  auto drained = [&](int i) { return smem_u32(&bars[2 * kTiles + 2 + i]); };
+  const unsigned ready = smem_u32(&bars[2 * kTiles]);
   if (tid == 0) {
-    for (int i = 0; i < 2 * kTiles + 4; ++i)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bars[i])),
-                   "r"(i >= 2 * kTiles + 2 ? kWorkers : 1)
-                   : "memory");
+    for (int i = 0; i < 2 * kTiles + 1; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bars[i])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -150,11 +189,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
   const int units = blocks * nf;
   const int mine = ((int)blockIdx.x < units) ? (units - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int K0 = pad_in(N.d_in);
-  const int per_unit = K0 / kTileK + (N.layers - 1) * (HP / kTileK);
+  const int per_unit = 2 * (K0 / kTileK + (N.layers - 1) * (HP / kTileK));
   const float* aux = reinterpret_cast<const float*>(packed + (size_t)per_unit * (HP * kTileK));
   const long long total = (long long)mine * per_unit;  // weight tiles this CTA takes
   long long loaded = 0, used = 0;                      // of the copying thread
-  int groups = 0;                                      // accumulators filled so far
+  unsigned phase = 0;                                  // of `ready`
   int failed = 0;
   auto load_next = [&]() {
     bulk_load(w_base + (unsigned)(loaded % kTiles) * kTileBytes,
@@ -166,6 +205,13 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
     while (loaded < total && loaded < kTiles) load_next();
 
   const int row = (warp & 3) * 32 + lane, quarter = (warp >> 2) & 3;  // of a worker
+  // the cut of a worker's row from the largest magnitude of its quarter
+  auto row_cut = [&](float top) {
+    quarters[quarter][row] = top;
+    worker_sync();
+    return cut_of(fmaxf(fmaxf(quarters[0][row], quarters[1][row]),
+                        fmaxf(quarters[2][row], quarters[3][row])));
+  };
   for (int iu = 0; iu < mine; ++iu) {
     const int u = (int)blockIdx.x + iu * (int)gridDim.x;
     const int f = u % nf, i0 = u / nf * kRows;
@@ -174,15 +220,20 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
       // features as the first A operand, zero beyond d_in and beyond the rows
       const float* xi = x + (size_t)(i0 + row) * N.d_in;
       const float xb = fields ? (float)(fields[f] * inv_scale) : 0.f;
+      auto feature = [&](int k) {
+        if (!valid || k >= N.d_in) return 0.f;
+        return fields && k == N.d_in - 1 ? xb : xi[k];
+      };
+      float top = 0.f;
+      for (int k8 = quarter; k8 < K0 / 8; k8 += 4)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) top = fmaxf(top, fabsf(feature(8 * k8 + j)));
+      const Cut c = row_cut(top);
       for (int k8 = quarter; k8 < K0 / 8; k8 += 4) {
         float v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int k = 8 * k8 + j;
-          v[j] = 0.f;
-          if (valid && k < N.d_in) v[j] = fields && k == N.d_in - 1 ? xb : xi[k];
-        }
-        put8(A, part, row, k8, v);
+        for (int j = 0; j < 8; ++j) v[j] = feature(8 * k8 + j);
+        put8(A, part, row, k8, c, v);
       }
     }
     for (int l = 0; l < N.layers; ++l) {
@@ -190,108 +241,113 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       if (__syncthreads_or(failed)) goto done;  // all threads
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int nt = (l == 0 ? K0 : HP) / kTileK, ng = (nt + kGroup - 1) / kGroup;
+      const int nt = (l == 0 ? K0 : HP) / kTileK;
       if (warp == kWorkers / 32) {
         if (lane == 0) {
           const uint32_t id = idesc_bf16(kRows, HP);
-          for (int g = 0; g < ng; ++g) {
-            const int b = (groups + g) & 1, use = (groups + g) >> 1;  // earlier uses of it
-            const int t0 = g * kGroup, t1 = min(nt, t0 + kGroup);
-            if (use > 0 && !wait(drained(b), (unsigned)(use - 1) & 1u)) failed = 1;
-            for (int t = t0; t < t1 && !failed; ++t) {
-              const long long w = used + (t - t0);
-              if (!wait(full((int)(w % kTiles)), (unsigned)(w / kTiles) & 1u)) failed = 1;
+          // the slot that tile p was in, once the MMAs that read it are done
+          auto refill = [&](long long before) {
+            while (!failed && loaded < total && loaded - kTiles < before) {
+              const long long p = loaded - kTiles;
+              if (wait(empty((int)(p % kTiles)), (unsigned)(p / kTiles) & 1u)) load_next();
+              else failed = 1;
             }
-            if (failed) break;
+          };
+          for (int t = 0; t < 2 * nt && !failed; ++t) {
+            const int s = (int)(used % kTiles), low = t & 1;
+            if (!wait(full(s), (unsigned)(used / kTiles) & 1u)) {
+              failed = 1;
+              break;
+            }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            // the low parts first: only sums with the high part round at full size
+            const uint64_t b = umma_desc(w_base + (unsigned)s * kTileBytes, HP * 16, 128);
+            // a1 w1 to the first accumulator, all other products to the second
 #pragma unroll
-            for (int q = 2; q >= 0; --q)
-              for (int t = t0; t < t1; ++t) {
-                const int s = (int)((used + (t - t0)) % kTiles);
-                mma_bf16(tmem + (unsigned)(b * HP),
-                         umma_desc(a_base + (unsigned)q * part + (unsigned)t * (2 * kRows * 16),
-                                   kRows * 16, 128),
-                         umma_desc(w_base + (unsigned)s * kTileBytes, HP * 16, 128), id,
-                         t == t0 && q == 2 ? 0u : 1u);
-              }
-            for (int t = t0; t < t1; ++t) mma_commit(empty((int)((used + (t - t0)) % kTiles)));
-            mma_commit(ready(b));
-            // tiles of the previous group are free once its MMAs are done
-            for (long long p = loaded - kTiles; p < used && loaded < total; ++p) {
-              if (!wait(empty((int)(p % kTiles)), (unsigned)(p / kTiles) & 1u)) {
-                failed = 1;
-                break;
-              }
-              load_next();
+            for (int q = 2; q >= 0; --q) {
+              const bool exact = q == 0 && !low;
+              mma_bf16(tmem + (exact ? 0u : (unsigned)HP),
+                       umma_desc(a_base + (unsigned)q * part + (unsigned)(t >> 1) * (2 * kRows * 16),
+                                 kRows * 16, 128),
+                       b, id, t == 0 && (exact || q == 2) ? 0u : 1u);
             }
-            used += t1 - t0;
+            mma_commit(empty(s));
+            ++used;
+            refill(used - 1);
+          }
+          if (!failed) {
+            mma_commit(ready);
+            refill(used);
           }
         }
-        groups += ng;
         failed = __shfl_sync(0xffffffffu, failed, 0);
         continue;
       }
-      float z[CPT];
-      for (int g = 0; g < ng; ++g) {
-        const int b = (groups + g) & 1;
-        if (!failed && !wait(ready(b), (unsigned)((groups + g) >> 1) & 1u)) failed = 1;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const unsigned col = tmem + (((unsigned)(warp & 3) * 32u) << 16) + (unsigned)(b * HP + quarter * CPT);
-#pragma unroll
-        for (int i = 0; i < CPT; i += 16) {
-          float v[16];
-          tmem_ld16(col + (unsigned)i, v);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) z[i + j] = g == 0 ? v[j] : z[i + j] + v[j];
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        mbar_arrive(drained(b));
-      }
-      groups += ng;
-      // bias, SiLU, then the next layer's operand (every MMA of this layer is done) or
+      if (!failed && !wait(ready, phase)) failed = 1;
+      phase ^= 1u;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // sums, bias, SiLU, then the next layer's operand (every MMA of this layer is done) or
       // the output layer's products
       // (outputs beyond hidden have zero weights and bias: SiLU gives zero)
       const bool last = l == N.layers - 1;
       const float4* bias = reinterpret_cast<const float4*>(aux + l * HP + quarter * CPT);
       const float4* wo = reinterpret_cast<const float4*>(aux + N.layers * HP + quarter * CPT);
-      float g = 0.f;
+      const unsigned col = tmem + (((unsigned)(warp & 3) * 32u) << 16) + (unsigned)(quarter * CPT);
+      float z[CPT], top = 0.f;
 #pragma unroll
-      for (int i = 0; i < CPT; i += 8) {
-        const float4 b0 = __ldg(bias + i / 4), b1 = __ldg(bias + i / 4 + 1);
-        float v[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+      for (int i = 0; i < CPT; i += 16) {
+        float v[16], w[16];
+        tmem_ld16(col + (unsigned)i, v);
+        tmem_ld16(col + (unsigned)(HP + i), w);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float a = z[i + j] + v[j];
-          v[j] = a / (1.f + __expf(-a));
-        }
-        if (!last) {
-          put8(A, part, row, (quarter * CPT + i) / 8, v);
-        } else {
-          const float4 w0 = __ldg(wo + i / 4), w1 = __ldg(wo + i / 4 + 1);
-          const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+        for (int j = 0; j < 16; j += 4) {
+          const float4 b = __ldg(bias + (i + j) / 4);
+          const float bb[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-          for (int j = 0; j < 8; ++j) g = fmaf(v[j], w[j], g);
-        }
-      }
-      if (last) {
-        if (quarter > 0) part_g[quarter - 1][row] = g;
-        worker_sync();
-        if (quarter == 0) {
-          g += part_g[0][row] + part_g[1][row] + part_g[2][row] + __ldg(N.params + N.b_off[N.layers]);
-          if (!fields) {
-            if (valid) out[i0 + row] = g;
-          } else {
-            const double v = valid ? (double)g : 0.0;
-            const double s1 = warp_sum(v), s2 = warp_sum(v * v);
-            if (lane == 0) {
-              atomicAdd(acc + 2 * f, s1);
-              atomicAdd(acc + 2 * f + 1, s2);
-            }
+          for (int k = 0; k < 4; ++k) {
+            const float a = (v[j + k] + w[j + k]) + bb[k];
+            z[i + j + k] = a / (1.f + __expf(-a));
+            top = fmaxf(top, fabsf(z[i + j + k]));
           }
         }
-        worker_sync();  // part_g is free again
       }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      if (!last) {
+        const Cut c = row_cut(top);
+#pragma unroll
+        for (int i = 0; i < CPT; i += 8) {
+          float v[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = z[i + j];
+          put8(A, part, row, (quarter * CPT + i) / 8, c, v);
+        }
+        continue;
+      }
+      float g = 0.f;
+#pragma unroll
+      for (int i = 0; i < CPT; i += 4) {
+        const float4 w = __ldg(wo + i / 4);
+        g = fmaf(z[i + 3], w.w, fmaf(z[i + 2], w.z, fmaf(z[i + 1], w.y, fmaf(z[i], w.x, g))));
+      }
+      quarters[quarter][row] = g;
+      worker_sync();
+      if (quarter == 0) {
+        g = quarters[0][row] + quarters[1][row] + quarters[2][row] + quarters[3][row] +
+            __ldg(N.params + N.b_off[N.layers]);
+        if (!fields) {
+          if (valid) out[i0 + row] = g;
+        } else {
+          const double v = valid ? (double)g : 0.0;
+          const double s1 = warp_sum(v), s2 = warp_sum(v * v);
+          if (lane == 0) {
+            moments[warp][0] = s1;
+            moments[warp][1] = s2;
+          }
+        }
+      }
+      worker_sync();  // `quarters` is free again, the moments are there
+      if (fields && tid < 2)
+        atomicAdd(acc + 2 * f + tid,
+                  (moments[0][tid] + moments[1][tid]) + (moments[2][tid] + moments[3][tid]));
     }
   }
 done:
@@ -338,15 +394,16 @@ bool mlp_fused(const MlpNet& net) {
 }
 static long long mlp_tile_values(const MlpNet& net) {
   const int HP = pad_hidden(net.hidden);
-  return (long long)HP * (pad_in(net.d_in) + (net.layers - 1) * HP);
+  return 2ll * HP * (pad_in(net.d_in) + (net.layers - 1) * HP);
 }
 size_t mlp_packed_values(const MlpNet& net) {  // FP32 values count twice
   return (size_t)mlp_tile_values(net) + 2 * (size_t)(net.layers + 1) * pad_hidden(net.hidden);
 }
 cudaError_t launch_mlp_pack(const MlpNet& net, __nv_bfloat16* packed, cudaStream_t st) {
   const int HP = pad_hidden(net.hidden);
-  const long long total = mlp_tile_values(net), threads = total + (net.layers + 1) * HP;
-  k_mlp_pack<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(net, HP, packed, total);
+  const long long total = mlp_tile_values(net);
+  const int warps = net.layers * HP + ((net.layers + 1) * HP + 31) / 32;
+  k_mlp_pack<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(net, HP, packed, total);
   return cudaGetLastError();
 }
 cudaError_t launch_mlp(const MlpNet& net, const __nv_bfloat16* packed, int n, const float* x,
