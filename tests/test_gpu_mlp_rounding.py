@@ -40,6 +40,33 @@ def _forward64(p, x, d_in, hidden, layers):
     return a[:, 0].cpu().numpy()
 
 
+@pytest.mark.parametrize("ratio", [50.0, 1e4])
+@pytest.mark.parametrize("hidden,layers", [(256, 3), (64, 1)])
+def test_inputs_of_different_magnitude(hidden, layers, ratio):
+    """The field feature is `ratio` times the others, its weights as much smaller."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    torch.cuda.set_device(0)
+    from paper_1612_09517_gb300 import rp
+    rp.use_torch_allocator()
+    s = wl.config2().system
+    sy = rp.System(s)
+    e = []
+    for seed in range(4):
+        fused = rp.ControlVariate(sy, hidden=hidden, layers=layers, init_seed=seed + 1)
+        wide = rp.ControlVariate(sy, hidden=WIDE, layers=layers)
+        p = fused.get_params()
+        p[:hidden * fused.d_in].reshape(hidden, -1)[:, -1] /= ratio
+        fused.set_params(p)
+        wide.set_params(_pad(p, fused.d_in, hidden, layers))
+        x = mlp.features(11, 0, np.arange(N), s, 10.0 * ratio, 10.0).astype(np.float32).astype(np.float64)
+        ref = _forward64(p, x, fused.d_in, hidden, layers)
+        e.append([np.sqrt(np.mean((cv.eval(np.full(N, 10.0 * ratio), np.arange(N), 11) - ref) ** 2))
+                  for cv in (fused, wide)])
+    rms_f, rms_w = np.mean(e, axis=0)
+    assert rms_f <= rms_w
+
+
 @pytest.mark.parametrize("hidden,layers", [(256, 3), (256, 1), (200, 2), (128, 3), (64, 2)])
 def test_no_more_rounding_than_fp32(hidden, layers):
     if not torch.cuda.is_available():
