@@ -17,7 +17,12 @@
 // E[g] and its variance against 64 bits, 4096 samples, 3 x 256, means over six networks:
 // 2.2e-7 (rms), 2.2e-8 and 2.8e-8; the layer-by-layer pass in rounded FP32 has 6.4e-7,
 // 1.6e-8 and 3.3e-8; one accumulator drained every 32 inputs had 2.9e-7, 7.7e-8, 3.1e-7.
-// (Numbers below 2^-119 or from 2^126 on are not cut: a1 or w1 is zero.)
+// (Rows and outputs whose largest is below 2^-119 or from 2^126 on are not cut: a1 is then
+// the upper eight bits of a, w1 zero.)
+//
+// A row with an infinity or NaN among its activations would turn every product of the split
+// into NaN, where an infinity passes an FP32 multiply-add.  The tensor cores get zeros for
+// its finite values, and the sums of the infinite and NaN ones are formed beside them.
 //
 // One CTA takes 128 feature rows through all layers: activations never leave the chip.
 // 512 threads hold the sums of one row and a quarter of the outputs each, apply bias
@@ -63,6 +68,18 @@ __device__ __forceinline__ void mma_bf16(unsigned d, uint64_t a, uint64_t b, uin
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// Eight columns of each accumulator.
+__device__ __forceinline__ void tmem_ld8x2(unsigned a, unsigned b, float (&v)[8], float (&w)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+        "=f"(v[7]), "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3]), "=f"(w[4]), "=f"(w[5]),
+        "=f"(w[6]), "=f"(w[7])
+      : "r"(a), "r"(b)
+      : "memory");
+}
 __device__ __forceinline__ bool wait(unsigned bar, unsigned parity) {
   return mbar_wait<(1ll << 20)>(bar, parity);
 }
@@ -80,8 +97,10 @@ __device__ __forceinline__ void worker_sync() {
 struct Cut {
   float grid, inv;
 };
-__device__ __forceinline__ Cut cut_of(float top) {
-  const int e = (int)(__float_as_uint(top) >> 23) - 126;  // 2^(e-1) <= top < 2^e
+// top: the bits of the magnitude, which compare as integers, NaN above infinity
+__device__ __forceinline__ unsigned mag(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ Cut cut_of(unsigned top) {
+  const int e = (int)(top >> 23) - 126;  // 2^(e-1) <= top < 2^e
   if (e < -118 || e > 126) return {0.f, 0.f};
   return {__uint_as_float((unsigned)(e + 120) << 23), __uint_as_float((unsigned)(134 - e) << 23)};
 }
@@ -106,7 +125,7 @@ __global__ void __launch_bounds__(4 * kMaxIn) k_mlp_scale(const MlpNet N, float*
     const __nv_bfloat16* w = N.wbf + N.w_off[l] + k;
 #pragma unroll 8
     for (int o = threadIdx.x / kMaxIn; o < N.hidden; o += 4)
-      m = max(m, __float_as_uint(fabsf(__bfloat162float(w[(long long)o * in]))));
+      m = max(m, mag(__bfloat162float(w[(long long)o * in])));
   }
   atomicMax(&top[k], m);
   atomicMax(&all, m);
@@ -139,11 +158,11 @@ __global__ void k_mlp_pack(const MlpNet N, int HP, const float* __restrict__ sca
   const __nv_bfloat16* w = N.wbf + N.w_off[l] + (long long)o * in;
   const bool on = o < N.hidden;
   const float* sc = scale + l * kMaxIn;
-  float top = 0.f;
+  unsigned top = 0u;
   for (int k = lane; on && k < in; k += 32)
-    top = fmaxf(top, fabsf(__bfloat162float(w[k])) / sc[k]);  // powers of two: exact
+    top = max(top, mag(__bfloat162float(w[k]) / sc[k]));  // powers of two: exact
 #pragma unroll
-  for (int s = 16; s > 0; s >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, s));
+  for (int s = 16; s > 0; s >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, s));
   const Cut c = cut_of(top);
   for (int k = lane; k < pad; k += 32) {
     float high, low = 0.f;
@@ -155,10 +174,38 @@ __global__ void k_mlp_pack(const MlpNet N, int HP, const float* __restrict__ sca
   }
 }
 
+// Eight activations of a row that is not cut: eight bits each (truncated: rounding could
+// reach infinity), or what is not finite of a row that holds such values (`odd`).
+__device__ __noinline__ void put8_uncut(unsigned char* d, unsigned part, bool odd, float4 lo, float4 hi) {
+  const float v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  __nv_bfloat16 h[3][8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const unsigned b = __float_as_uint(v[i]);
+    float r = v[i];
+    if (odd) {
+      const bool finite = (b & 0x7f800000u) != 0x7f800000u;
+      h[0][i] = __ushort_as_bfloat16(finite ? 0 : (b & 0x7fffffu) ? 0x7fff : (unsigned short)(b >> 16));
+      r = 0.f;
+    } else {
+      h[0][i] = __ushort_as_bfloat16((unsigned short)(b >> 16));
+      r -= __bfloat162float(h[0][i]);
+    }
+    h[1][i] = __float2bfloat16(r);
+    h[2][i] = __float2bfloat16(r - __bfloat162float(h[1][i]));
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) *reinterpret_cast<uint4*>(d + q * part) = *reinterpret_cast<const uint4*>(h[q]);
+}
+
 // Eight activations of a row to the three parts of the A operand (`part` bytes apart).
 __device__ __forceinline__ void put8(unsigned char* A, unsigned part, int row, int k8, const Cut& c,
-                                     float (&v)[8]) {
+                                     bool odd, float (&v)[8]) {
   unsigned char* d = A + (unsigned)k8 * (kRows * 16) + (unsigned)row * 16;
+  if (c.inv == 0.f) {
+    put8_uncut(d, part, odd, make_float4(v[0], v[1], v[2], v[3]), make_float4(v[4], v[5], v[6], v[7]));
+    return;
+  }
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     unsigned w[4];
@@ -192,7 +239,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
   __shared__ __align__(8) unsigned long long bars[2 * kTiles + 1];
   __shared__ unsigned tmem_slot;
   // largest magnitudes of the quarters of a row; at the end their shares of g
-  __shared__ float quarters[4][kRows];
+  __shared__ __align__(4) unsigned quarters[4][kRows];
   __shared__ double moments[4][2];
   unsigned char* A = mlp_smem;  // three parts of [input / 8][row][8 inputs]
   const unsigned a_base = smem_u32(mlp_smem), w_base = a_base + 3 * part;
@@ -239,11 +286,13 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
 
   const int row = (warp & 3) * 32 + lane, quarter = (warp >> 2) & 3;  // of a worker
   // the cut of a worker's row from the largest magnitude of its quarter
-  auto row_cut = [&](float top) {
+  bool odd = false;  // the row holds infinities or NaN
+  auto row_cut = [&](unsigned top) {
     quarters[quarter][row] = top;
     worker_sync();
-    return cut_of(fmaxf(fmaxf(quarters[0][row], quarters[1][row]),
-                        fmaxf(quarters[2][row], quarters[3][row])));
+    top = max(max(quarters[0][row], quarters[1][row]), max(quarters[2][row], quarters[3][row]));
+    odd = top >= 0x7f800000u;
+    return cut_of(top);
   };
   for (int iu = 0; iu < mine; ++iu) {
     const int u = (int)blockIdx.x + iu * (int)gridDim.x;
@@ -264,16 +313,17 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
           if (valid && k < N.d_in) v[j] = (fields && k == N.d_in - 1 ? xb : xi[k]) * mm[j];
         }
       };
-      float v[8], top = 0.f;
+      float v[8];
+      unsigned top = 0u;
       for (int k8 = quarter; k8 < K0 / 8; k8 += 4) {
         features(k8, v);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) top = fmaxf(top, fabsf(v[j]));
+        for (int j = 0; j < 8; ++j) top = max(top, mag(v[j]));
       }
       const Cut c = row_cut(top);
       for (int k8 = quarter; k8 < K0 / 8; k8 += 4) {
         features(k8, v);
-        put8(A, part, row, k8, c, v);
+        put8(A, part, row, k8, c, odd, v);
       }
     }
     for (int l = 0; l < N.layers; ++l) {
@@ -333,22 +383,48 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
       const float4* wo = reinterpret_cast<const float4*>(aux + N.layers * HP + quarter * CPT);
       const float4* next = reinterpret_cast<const float4*>(scales + (l + 1) * kMaxIn + quarter * CPT);
       const unsigned col = tmem + (((unsigned)(warp & 3) * 32u) << 16) + (unsigned)(quarter * CPT);
-      float z[CPT], top = 0.f;
+      // sums of an odd row: its values that are not finite lie in the first part of the
+      // operand, the other two have room for the sums of this thread's outputs
+      auto odd_sums = [&](int o) {  // of outputs o .. o + 3
+        return reinterpret_cast<float4*>(A + (unsigned)(1 + ((o >> 2) & 1)) * part +
+                                         (unsigned)(o / 8) * (kRows * 16) + (unsigned)row * 16);
+      };
+      if (odd) {
+        const int in = l == 0 ? N.d_in : N.hidden;
+#pragma unroll 1
+        for (int o = quarter * CPT; o < (quarter + 1) * CPT; ++o) {
+          float sum = 0.f;
+          const __nv_bfloat16* w = N.wbf + N.w_off[l] + (long long)o * in;
+#pragma unroll 1
+          for (int k = 0; o < N.hidden && k < in; ++k) {
+            const float a = __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(
+                A + (unsigned)(k / 8) * (kRows * 16) + (unsigned)row * 16 + (unsigned)(k % 8) * 2));
+            if (a != 0.f) sum = fmaf(a, __bfloat162float(w[k]), sum);
+          }
+          reinterpret_cast<float*>(odd_sums(o))[o & 3] = sum;
+        }
+      }
+      float z[CPT];
+      unsigned top = 0u;
 #pragma unroll
-      for (int i = 0; i < CPT; i += 16) {
-        float v[16], w[16];
-        tmem_ld16(col + (unsigned)i, v);
-        tmem_ld16(col + (unsigned)(HP + i), w);
+      for (int i = 0; i < CPT; i += 8) {
+        float v[8], w[8];
+        tmem_ld8x2(col + (unsigned)i, col + (unsigned)(HP + i), v, w);
 #pragma unroll
-        for (int j = 0; j < 16; j += 4) {
+        for (int j = 0; j < 8; j += 4) {
           const float4 b = __ldg(bias + (i + j) / 4);
           const float4 m = last ? make_float4(1.f, 1.f, 1.f, 1.f) : __ldg(next + (i + j) / 4);
           const float bb[4] = {b.x, b.y, b.z, b.w}, mm[4] = {m.x, m.y, m.z, m.w};
+          if (odd) {
+            const float4 q = *odd_sums(quarter * CPT + i + j);
+            v[j] = q.x, v[j + 1] = q.y, v[j + 2] = q.z, v[j + 3] = q.w;
+            w[j] = w[j + 1] = w[j + 2] = w[j + 3] = 0.f;
+          }
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const float a = (v[j + k] + w[j + k]) + bb[k];
             z[i + j + k] = a / (1.f + __expf(-a)) * mm[k];
-            top = fmaxf(top, fabsf(z[i + j + k]));
+            top = max(top, mag(z[i + j + k]));
           }
         }
       }
@@ -360,7 +436,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
           float v[8];
 #pragma unroll
           for (int j = 0; j < 8; ++j) v[j] = z[i + j];
-          put8(A, part, row, (quarter * CPT + i) / 8, c, v);
+          put8(A, part, row, (quarter * CPT + i) / 8, c, odd, v);
         }
         continue;
       }
@@ -370,10 +446,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
         const float4 w = __ldg(wo + i / 4);
         g = fmaf(z[i + 3], w.w, fmaf(z[i + 2], w.z, fmaf(z[i + 1], w.y, fmaf(z[i], w.x, g))));
       }
-      quarters[quarter][row] = g;
+      quarters[quarter][row] = __float_as_uint(g);
       worker_sync();
       if (quarter == 0) {
-        g = quarters[0][row] + quarters[1][row] + quarters[2][row] + quarters[3][row] +
+        g = __uint_as_float(quarters[0][row]) + __uint_as_float(quarters[1][row]) +
+            __uint_as_float(quarters[2][row]) + __uint_as_float(quarters[3][row]) +
             __ldg(N.params + N.b_off[N.layers]);
         if (!fields) {
           if (valid) out[i0 + row] = g;
