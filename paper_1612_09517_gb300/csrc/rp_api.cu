@@ -461,9 +461,17 @@ class YieldEngine {
     // cluster macro-steps leave SMs idle (clusters fill whole GPC pairs of 8):
     // the time integral of macro-step k runs on a second stream, reading its own
     // copy of the singlet slices, while macro-step k + 1 propagates
+    // (where there is room for that copy)
     overlap_ = cluster_ && !o_.graph && !d_trace_;
     if (overlap_) {
-      X2_ = ar_.get<T>((size_t)R * x_row);
+      try {
+        X2_ = ar_.get<T>((size_t)R * x_row);
+      } catch (const CudaFail& e) {
+        if (e.st != RP_ENOMEM) throw;
+        overlap_ = false;
+      }
+    }
+    if (overlap_) {
       if (tc_gram_) ck(cudaMemsetAsync(X2_, 0, (size_t)R * x_row * sizeof(T), st_), "cudaMemsetAsync");
       if (!side_st_) ck(cudaStreamCreateWithFlags(&side_st_, cudaStreamNonBlocking), "cudaStreamCreate");
       for (int i = 0; i < 2; ++i) {
