@@ -2390,19 +2390,13 @@ rp_status rp_apply_h(rp_system* s, double B, int precision, int n_vec, const voi
     // constants and field travel as kernel parameters: nothing to allocate or copy
     const double kbar = 0.5 * (hs.k_S + hs.k_T);
     if (precision == RP_FP64) {
-      rp::FieldDev<double> F{rp::kGammaE * B, 1.0, 0.0, 0.5 * kbar};
+      const rp::FieldDev<double> F{rp::kGammaE * B, 1.0, 0.0, 0.5 * kbar};
       const rp::HamDev<double> H = make_ham<double>(hs);
-      const rp::SysTab<double> S{nullptr, nullptr, nullptr, nullptr, hs.Z, 0, nullptr};
-      ck(rp::launch_step<double>(S, &H, H.aniso, 1, nullptr, nullptr, nullptr, 0, nullptr, n_vec, (const double*)x,
-                                 nullptr, (double*)y, nullptr, nullptr, nullptr, 0, 0,
-                                 rp::MODE_APPLY, 0, st, &F), "apply kernel");
+      ck(rp::launch_apply<double>(H, H.aniso, F, n_vec, (const double*)x, (double*)y, st), "apply kernel");
     } else {
-      rp::FieldDev<float> F{(float)(rp::kGammaE * B), 1.f, 0.f, (float)(0.5 * kbar)};
+      const rp::FieldDev<float> F{(float)(rp::kGammaE * B), 1.f, 0.f, (float)(0.5 * kbar)};
       const rp::HamDev<float> H = make_ham<float>(hs);
-      const rp::SysTab<float> S{nullptr, nullptr, nullptr, nullptr, hs.Z, 0, nullptr};
-      ck(rp::launch_step<float>(S, &H, H.aniso, 1, nullptr, nullptr, nullptr, 0, nullptr, n_vec, (const float*)x, nullptr,
-                                (float*)y, nullptr, nullptr, nullptr, 0, 0, rp::MODE_APPLY, 0, st, &F),
-         "apply kernel");
+      ck(rp::launch_apply<float>(H, H.aniso, F, n_vec, (const float*)x, (float*)y, st), "apply kernel");
     }
     ck(cudaStreamSynchronize(st), "apply kernel execution");
   } catch (const CudaFail& e) {

@@ -137,13 +137,6 @@ __device__ __forceinline__ void store_singlet(T* x, const Cx<T> (&v)[4]) {
   x[1] = (v[1].im - v[2].im) * r;
 }
 
-template <typename T>
-__device__ __forceinline__ void store_singlet_blk(T* x, const Cx<T> (&v)[4]) {
-  const T r = T(0.70710678118654752440);
-  x[0] = (v[1].re - v[2].re) * r;
-  x[4] = (v[1].im - v[2].im) * r;
-}
-
 // y += Mx q on the electron of radical rr, Mx a 2x2 complex matrix (re/im arrays).
 template <typename T>
 __device__ __forceinline__ void apply_e2x2(Cx<T> (&y)[4], const Cx<T> (&q)[4], int rr,
@@ -419,8 +412,7 @@ __device__ __forceinline__ void term_epilogue(const HamDev<T>& H, const SysTab<T
                                               const T* __restrict__ prev, T* __restrict__ next,
                                               T* __restrict__ acc, T* __restrict__ X,
                                               const T* __restrict__ coef, int n_c, int n,
-                                              int mode, int xblk, const Cx<T>* pre_pv = nullptr,
-                                              const Cx<T>* pre_acc = nullptr) {
+                                              int mode) {
   Cx<T> z[4];
   finish_z<T, ANISO>(H, F, a, y, b1, b2, z);
   const size_t off = row0 + (size_t)m * 8;
@@ -447,22 +439,12 @@ __device__ __forceinline__ void term_epilogue(const HamDev<T>& H, const SysTab<T
       cmac(s[e], c1r, c1i, z[e]);
     }
     store4(acc + off, s);
-    if (xblk) {
-      store_singlet_blk(xblk_addr(X, r, 0, m, S.Zslot, n_c), a);
-      store_singlet_blk(xblk_addr(X, r, 1, m, S.Zslot, n_c), z);
-    } else {
-      store_singlet(xr + (size_t)m * 2, a);
-      store_singlet(xr + (Zs + m) * 2, z);
-    }
+    store_singlet(xr + (size_t)m * 2, a);
+    store_singlet(xr + (Zs + m) * 2, z);
     return;
   }
   Cx<T> pv[4];
-  if (pre_pv) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) pv[e] = pre_pv[e];
-  } else {
-    load4(prev + off, pv);
-  }
+  load4(prev + off, pv);
   Cx<T> ph[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
@@ -471,12 +453,7 @@ __device__ __forceinline__ void term_epilogue(const HamDev<T>& H, const SysTab<T
   }
   if (mode == MODE_MID) store4(next + off, ph);
   Cx<T> s[4];
-  if (pre_acc) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) s[e] = pre_acc[e];
-  } else {
-    load4_rw(acc + off, s);
-  }
+  load4_rw(acc + off, s);
   const T cr = cf[2 * n], ci = cf[2 * n + 1];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
@@ -484,8 +461,7 @@ __device__ __forceinline__ void term_epilogue(const HamDev<T>& H, const SysTab<T
     cmac(s[e], cr, ci, ph[e]);
   }
   store4(acc + off, s);
-  if (xblk) store_singlet_blk(xblk_addr(X, r, n, m, S.Zslot, n_c), ph);
-  else store_singlet(xr + ((size_t)n * Zs + m) * 2, ph);
+  store_singlet(xr + ((size_t)n * Zs + m) * 2, ph);
 }
 
 // Body of one Chebyshev term; H is either the kernel-parameter copy (one
@@ -499,7 +475,7 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
                                           const T* __restrict__ cur, const T* __restrict__ prev,
                                           T* __restrict__ next, T* __restrict__ acc,
                                           T* __restrict__ X, const T* __restrict__ coef, int n_c,
-                                          int n, int mode, int xblk);
+                                          int n, int mode);
 
 // Field of a step launch: by value for H psi (APPLY), else the table of every field.  A
 // call whose thousands of launches are all latency (rp_yields_static, Z = 16, 64 rows,
@@ -518,23 +494,22 @@ __global__ void __launch_bounds__(kStepThreads,
                                   sizeof(T) == 4 ? (ANISO ? 4 : (NH >= 0 ? 5 : 6)) : 2)
     k_cheb_step(
     const SysTab<T> S, const HamDev<T> H1, const StepField<T, APPLY> fields,
-    const int* __restrict__ row_field, const int2* __restrict__ row_win, int macro_arg,
-    const int* __restrict__ macro_dev, const T* __restrict__ cur, const T* __restrict__ prev,
+    const int* __restrict__ row_field, const int2* __restrict__ row_win, int macro,
+    const T* __restrict__ cur, const T* __restrict__ prev,
     T* __restrict__ next, T* __restrict__ acc, T* __restrict__ X, const T* __restrict__ coef,
-    int n_c, int n, int mode, int xblk) {
+    int n_c, int n, int mode) {
   extern __shared__ __align__(16) unsigned char step_smem[];
   Cx<T>* tile = reinterpret_cast<Cx<T>*>(step_smem);  // planes x blockDim x 16 B
   const int r = blockIdx.y;
   if constexpr (APPLY) {
     step_body<T, ANISO, NH, N1>(H1, S, tile, fields.one, 0, r, cur, prev, next, acc, X, coef, n_c,
-                                n, MODE_APPLY, xblk);
+                                n, MODE_APPLY);
   } else {
-    const int macro = macro_dev ? *macro_dev : macro_arg;
     const int2 w = row_win[r];
     if (macro < w.x || macro >= w.y) return;  // the whole block: one row
     const int f = row_field[r];
     step_body<T, ANISO, NH, N1>(H1, S, tile, fields.all[f], f, r, cur, prev, next, acc, X, coef,
-                                n_c, n, mode, xblk);
+                                n_c, n, mode);
   }
 }
 
@@ -544,7 +519,7 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
                                           const T* __restrict__ cur, const T* __restrict__ prev,
                                           T* __restrict__ next, T* __restrict__ acc,
                                           T* __restrict__ X, const T* __restrict__ coef, int n_c,
-                                          int n, int mode, int xblk) {
+                                          int n, int mode) {
   const unsigned Z = (unsigned)H.Z;
   const unsigned m = blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = m < Z;
@@ -583,16 +558,7 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
     }
   }
   __syncthreads();
-  if (!valid) {  // no barrier below
-    // the tensor-core integral reads whole 16-configuration chunks: keep the
-    // padding past Z at zero (a refilled row may hold a larger system's slices)
-    if (xblk && mode != MODE_APPLY && m < ((Z + kXChunk - 1) / kXChunk) * kXChunk) {
-      const Cx<T> zero[4] = {{T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}, {T(0), T(0)}};
-      store_singlet_blk(xblk_addr(X, r, n, m, S.Zslot, n_c), zero);
-      if (mode == MODE_FIRST) store_singlet_blk(xblk_addr(X, r, 0, m, S.Zslot, n_c), zero);
-    }
-    return;
-  }
+  if (!valid) return;  // no barrier below
 
   Cx<T> y[4];
 #pragma unroll
@@ -701,10 +667,10 @@ __device__ __forceinline__ void step_body(const HamDev<T>& H, const SysTab<T>& S
   }
 
   term_epilogue<T, ANISO>(H, S, F, a, y, b1, b2, f, r, m, row0, prev, next, acc, X, coef, n_c, n,
-                          mode, xblk);
+                          mode);
 }
 
-// ---- FP32 term with the block's partner tiles staged by bulk async copies ----
+// ---- FP32 H psi with the block's partner tiles staged by bulk async copies ----
 //
 // When every nucleus outside the innermost kInnerBits spin-1/2 positions has a
 // stride that is a multiple of the block (n_half >= kInnerBits and 256
@@ -773,26 +739,14 @@ __device__ __forceinline__ int bulk_partner_tiles(const HamDev<float>& H, unsign
 
 template <bool ANISO>
 __global__ void __launch_bounds__(kBulkTile, 2) k_cheb_step_bulk(
-    const SysTab<float> S, const HamDev<float> H, const FieldDev<float>* __restrict__ fields,
-    const int* __restrict__ row_field, const int2* __restrict__ row_win, int macro_arg,
-    const int* __restrict__ macro_dev, const float* __restrict__ cur,
-    const float* __restrict__ prev, float* __restrict__ next, float* __restrict__ acc,
-    float* __restrict__ X, const float* __restrict__ coef, int n_c, int n, int mode, int xblk,
-    const FieldDev<float> one_field) {
+    const HamDev<float> H, const FieldDev<float> F, const float* __restrict__ cur,
+    float* __restrict__ next) {
   extern __shared__ __align__(128) unsigned char bulk_smem[];
   __shared__ __align__(8) unsigned long long bar_storage[2];  // own tile, partner tiles
-  const int r = blockIdx.y;
-  int f = 0;
-  if (mode != MODE_APPLY) {
-    const int macro = macro_dev ? *macro_dev : macro_arg;
-    const int2 w = row_win[r];
-    if (macro < w.x || macro >= w.y) return;  // the whole block: one row
-    f = row_field[r];
-  }
   float* tiles = reinterpret_cast<float*>(bulk_smem);
   const unsigned bar_own = smem_u32(&bar_storage[0]), bar_part = smem_u32(&bar_storage[1]);
   const unsigned c0 = blockIdx.x * kBulkTile;
-  const size_t row0 = (size_t)r * S.Zslot * 8;
+  const size_t row0 = (size_t)blockIdx.y * H.Z * 8;
   const float* c = cur + row0;
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_own) : "memory");
@@ -817,19 +771,10 @@ __global__ void __launch_bounds__(kBulkTile, 2) k_cheb_step_bulk(
   }
   const unsigned t = threadIdx.x;
   const unsigned m = c0 + t;
-  const size_t off = row0 + (size_t)m * 8;
-  // the streams this thread reads anyway, in flight during the tile copies
-  Cx<float> pv[4], sa[4];
-  const bool pre = mode == MODE_MID || mode == MODE_LAST;
-  if (pre) {
-    load4(prev + off, pv);
-    load4_rw(acc + off, sa);
-  }
   __shared__ float4 wtp[ANISO ? kMaxNucDev * 2 * 4 : 1];
   if (ANISO) fill_wtab_packed(wtp, H, H.n_half);
   __syncthreads();  // the barriers are initialised before anyone polls them
-  if (!bulk_wait(bar_own) ) {
-    if (S.err) atomicOr(S.err, 1);
+  if (!bulk_wait(bar_own)) {
     bulk_wait(bar_own);  // let copies still in flight land before the block exits
     bulk_wait(bar_part);
     return;
@@ -861,7 +806,6 @@ __global__ void __launch_bounds__(kBulkTile, 2) k_cheb_step_bulk(
     }
   }
   if (!bulk_wait(bar_part)) {
-    if (S.err) atomicOr(S.err, 1);
     bulk_wait(bar_part);
     return;
   }
@@ -928,9 +872,9 @@ __global__ void __launch_bounds__(kBulkTile, 2) k_cheb_step_bulk(
       add_partner_q<float, ANISO>(y, q, rr, H.U[p], sqrtf(I * (I + 1.f) - M * (M + 1.f)), false);
     }
   }
-  term_epilogue<float, ANISO>(H, S, fields ? fields[f] : one_field, a, y, b1, b2, f, r, m, row0, prev, next, acc, X,
-                              coef, n_c, n, mode, xblk, pre ? pv : nullptr,
-                              pre ? sa : nullptr);
+  Cx<float> z[4];
+  finish_z<float, ANISO>(H, F, a, y, b1, b2, z);
+  store4(next + row0 + (size_t)m * 8, z);
 }
 
 // Largest number of partner tiles over the tiles of a system (host side).
@@ -1998,66 +1942,63 @@ cudaError_t launch_init_state(const SysTab<T>& S, const double* amps, const long
   return cudaGetLastError();
 }
 
-// The FP32 bulk kernel is only launched from launch_step<float>; the cast
-// lets launch_step<double> compile the (never taken) branch.
+namespace {
+// Block and grid of the step kernel: power-of-two blocks, so that m XOR 2^p stays inside the
+// block for 2^p < b.
 template <typename T>
-SysTab<float> S_as_float(const SysTab<T>& S) {
-  return *reinterpret_cast<const SysTab<float>*>(&S);
+struct StepShape {
+  int b = 32;
+  dim3 grid;
+  size_t smem;
+  StepShape(long long Zslot, int rows) {
+    while (b < kStepThreads && b < Zslot) b *= 2;
+    grid = dim3(grid1(Zslot, b), rows);
+    smem = (size_t)b * 4 * sizeof(Cx<T>);
+  }
+};
+}  // namespace
+
+template <typename T>
+cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>& one, int aniso,
+                        const FieldDev<T>* fields, const int* row_field, const int2* row_win,
+                        int macro, int rows, const T* cur, const T* prev, T* next, T* acc, T* X,
+                        const T* coef, int n_c, int n, int mode, cudaStream_t st) {
+  if (rows == 0) return cudaSuccess;
+  const StepShape<T> q(S.Zslot, rows);
+  const auto kf = aniso ? k_cheb_step<T, true, false> : k_cheb_step<T, false, false>;
+  kf<<<q.grid, q.b, q.smem, st>>>(S, one, StepField<T, false>{fields}, row_field, row_win, macro,
+                                  cur, prev, next, acc, X, coef, n_c, n, mode);
+  return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int bulk,
-                        const FieldDev<T>* fields, const int* row_field, const int2* row_win,
-                        int macro, const int* macro_dev, int rows, const T* cur, const T* prev,
-                        T* next, T* acc, T* X, const T* coef, int n_c, int n, int mode,
-                        int xblk, cudaStream_t st, const FieldDev<T>* one_field) {
+cudaError_t launch_apply(const HamDev<T>& one, int aniso, const FieldDev<T>& field, int rows,
+                         const T* x, T* y, cudaStream_t st) {
   if (rows == 0) return cudaSuccess;
-  const FieldDev<T> F1 = one_field ? *one_field : FieldDev<T>{};
-  if (bulk && sizeof(T) == 4 && one->n_half >= kInnerBits && S.Zslot == one->Z &&
-      one->Z % kBulkTile == 0) {
-    const HamDev<float>& hf = *reinterpret_cast<const HamDev<float>*>(one);
-    const size_t smem = (size_t)(1 + bulk_max_partner_tiles(hf)) * kBulkTileBytes;
-    if (smem <= (size_t)kBulkMaxSmem) {
+  if constexpr (sizeof(T) == 4) {
+    const size_t smem = (size_t)(1 + bulk_max_partner_tiles(one)) * kBulkTileBytes;
+    if (one.n_half >= kInnerBits && one.Z % kBulkTile == 0 && smem <= (size_t)kBulkMaxSmem) {
       static std::atomic<unsigned long long> attr_done[2];
       auto kf = aniso ? k_cheb_step_bulk<true> : k_cheb_step_bulk<false>;
       const cudaError_t e = smem_attr_once((const void*)kf, kBulkMaxSmem, attr_done[aniso ? 1 : 0]);
       if (e != cudaSuccess) return e;
-      dim3 grid((unsigned)(one->Z / kBulkTile), rows);
-      kf<<<grid, kBulkTile, smem, st>>>(
-          S_as_float(S), hf, reinterpret_cast<const FieldDev<float>*>(fields), row_field, row_win,
-          macro, macro_dev, reinterpret_cast<const float*>(cur),
-          reinterpret_cast<const float*>(prev), reinterpret_cast<float*>(next),
-          reinterpret_cast<float*>(acc), reinterpret_cast<float*>(X),
-          reinterpret_cast<const float*>(coef), n_c, n, mode, xblk,
-          *reinterpret_cast<const FieldDev<float>*>(&F1));
+      kf<<<dim3((unsigned)(one.Z / kBulkTile), rows), kBulkTile, smem, st>>>(one, field, x, y);
       return cudaGetLastError();
     }
   }
-  // power-of-two blocks so that m XOR 2^p stays inside the block for 2^p < b
-  int b = 32;
-  while (b < kStepThreads && b < S.Zslot) b *= 2;
-  const size_t smem = (size_t)b * 4 * sizeof(Cx<T>);
-  dim3 grid(grid1(S.Zslot, b), rows);
-  // H psi: compiled shape (fixed nucleus loops, 48 registers and 5 blocks per SM instead of
-  // 40 and 6 in FP32): 20 spin-1/2 nuclei, isotropic -- the paper's Table I model, 3 % faster.
-  // (The same for the 20-nucleus anisotropic workload needs 67 registers, 3 blocks per SM,
-  // and measured 12 % slower than the generic kernel at 4.)
-  const StepField<T, false> all{fields};
-  const StepField<T, true> field{F1};
-  auto go = [&](auto kf, const auto& F) {
-    kf<<<grid, b, smem, st>>>(S, *one, F, row_field, row_win, macro, macro_dev, cur, prev, next,
-                              acc, X, coef, n_c, n, mode, xblk);
-  };
-  if (mode != MODE_APPLY) {
-    if (aniso) go(k_cheb_step<T, true, false>, all);
-    else go(k_cheb_step<T, false, false>, all);
-  } else if (aniso) {
-    go(k_cheb_step<T, true, true>, field);
-  } else if (b == kStepThreads && one->n_half == 20 && one->n_nuc == 20) {
-    go(k_cheb_step<T, false, true, 20, 0>, field);
-  } else {
-    go(k_cheb_step<T, false, true>, field);
-  }
+  const StepShape<T> q(one.Z, rows);
+  SysTab<T> S{};
+  S.Zslot = one.Z;
+  // compiled shape (fixed nucleus loops, 48 registers and 5 blocks per SM instead of 40 and 6
+  // in FP32): 20 spin-1/2 nuclei, isotropic -- the paper's Table I model, 3 % faster.  (The
+  // same for the 20-nucleus anisotropic workload needs 67 registers, 3 blocks per SM, and
+  // measured 12 % slower than the generic kernel at 4.)
+  const bool t1_shape = q.b == kStepThreads && one.n_half == 20 && one.n_nuc == 20;
+  const auto kf = aniso      ? k_cheb_step<T, true, true>
+                  : t1_shape ? k_cheb_step<T, false, true, 20, 0>
+                             : k_cheb_step<T, false, true>;
+  kf<<<q.grid, q.b, q.smem, st>>>(S, one, StepField<T, true>{field}, nullptr, nullptr, 0, x,
+                                  nullptr, y, nullptr, nullptr, nullptr, 0, 0, MODE_APPLY);
   return cudaGetLastError();
 }
 
@@ -2356,11 +2297,12 @@ template cudaError_t launch_coherent_amps<float>(const SysTab<float>&, const lon
 template cudaError_t launch_init_state<float>(const SysTab<float>&, const double*, const long long*,
                                               const int*, const int2*, int, int, float*, float*, double*,
                                               double*, cudaStream_t);
-template cudaError_t launch_step<float>(const SysTab<float>&, const HamDev<float>*, int, int,
-                                        const FieldDev<float>*, const int*, const int2*, int,
-                                        const int*, int, const float*, const float*, float*, float*, float*,
-                                        const float*, int, int, int, int, cudaStream_t,
-                                        const FieldDev<float>*);
+template cudaError_t launch_step<float>(const SysTab<float>&, const HamDev<float>&, int,
+                                        const FieldDev<float>*, const int*, const int2*, int, int,
+                                        const float*, const float*, float*, float*, float*, const float*,
+                                        int, int, int, cudaStream_t);
+template cudaError_t launch_apply<float>(const HamDev<float>&, int, const FieldDev<float>&, int,
+                                         const float*, float*, cudaStream_t);
 template int small_max_configs<float>();
 template size_t persistent_smem<float>(long long, int);
 template int persistent_ctas<float>(long long, int, int);
@@ -2383,11 +2325,12 @@ template cudaError_t launch_coherent_amps<double>(const SysTab<double>&, const l
 template cudaError_t launch_init_state<double>(const SysTab<double>&, const double*, const long long*,
                                               const int*, const int2*, int, int, double*, double*, double*,
                                               double*, cudaStream_t);
-template cudaError_t launch_step<double>(const SysTab<double>&, const HamDev<double>*, int, int,
-                                        const FieldDev<double>*, const int*, const int2*, int,
-                                        const int*, int, const double*, const double*, double*, double*, double*,
-                                        const double*, int, int, int, int, cudaStream_t,
-                                        const FieldDev<double>*);
+template cudaError_t launch_step<double>(const SysTab<double>&, const HamDev<double>&, int,
+                                        const FieldDev<double>*, const int*, const int2*, int, int,
+                                        const double*, const double*, double*, double*, double*, const double*,
+                                        int, int, int, cudaStream_t);
+template cudaError_t launch_apply<double>(const HamDev<double>&, int, const FieldDev<double>&, int,
+                                         const double*, double*, cudaStream_t);
 template int small_max_configs<double>();
 template size_t persistent_smem<double>(long long, int);
 template int persistent_ctas<double>(long long, int, int);

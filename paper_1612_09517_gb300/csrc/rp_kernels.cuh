@@ -122,23 +122,22 @@ cudaError_t launch_init_state(const SysTab<T>& S, const double* amps, const long
                               int deterministic, T* S0, T* S1, double* integral, double* survival,
                               cudaStream_t st);
 
-// One Chebyshev term over every row (see k_cheb_step), every row being the system *one
+// One Chebyshev term over every row (see k_cheb_step), every row being the system `one`
 // (its constants travel as kernel parameters).  aniso selects the anisotropic hyperfine
-// path.  bulk != 0 allows the FP32 variant that stages each block's partner tiles with
-// bulk async copies (taken for >= 8 spin-1/2 nuclei whose tiles fit in shared memory; see
-// k_cheb_step_bulk); its bounded wait reports to S.err.  macro_dev != NULL: the kernels
-// read the macro-step index from device memory (graph replay; see launch_tick), else they
-// use macro.  xblk != 0 writes the singlet slices in the tensor-core Gram layout (see
-// launch_gram_tc), else as X[row][n][m] complex.  one_field != NULL (host): the field of
-// every row, instead of fields[row_field[r]].  rp_apply_h and the allocation-free entry
-// run these kernels; the others take launch_term.
+// path; singlet slices go to X[row][n][m] complex.  The allocation-free entry runs it; the
+// others take launch_term.
 template <typename T>
-cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>* one, int aniso, int bulk,
+cudaError_t launch_step(const SysTab<T>& S, const HamDev<T>& one, int aniso,
                         const FieldDev<T>* fields, const int* row_field, const int2* row_win,
-                        int macro, const int* macro_dev, int rows, const T* cur, const T* prev,
-                        T* next, T* acc, T* X, const T* coef, int n_c, int n, int mode,
-                        int xblk, cudaStream_t st,
-                        const FieldDev<T>* one_field = nullptr);
+                        int macro, int rows, const T* cur, const T* prev, T* next, T* acc, T* X,
+                        const T* coef, int n_c, int n, int mode, cudaStream_t st);
+
+// y = (H - i K) x for `rows` state vectors (rp_apply_h).  FP32 systems with >= 8 spin-1/2
+// nuclei whose partner tiles fit in shared memory stage them by bulk copies
+// (k_cheb_step_bulk), the others run k_cheb_step.
+template <typename T>
+cudaError_t launch_apply(const HamDev<T>& one, int aniso, const FieldDev<T>& field, int rows,
+                         const T* x, T* y, cudaStream_t st);
 
 // Largest Z (configurations) that launch_macro_small can hold.
 template <typename T>
@@ -214,6 +213,9 @@ struct ChipPlan {
   int threads = 0, slots = 0;
   size_t smem = 0;
 };
+
+// SMs of GB300: the rules of the launch plans are for this chip (grids ask the device).
+constexpr int kChipSms = 152;
 
 // Launch shape for systems of at most Zmax configurations, at least min_half
 // spin-1/2 and at most max_nuc nuclei each, `load` configurations in all over
@@ -351,8 +353,8 @@ cudaError_t launch_project(const SysTab<T>& S, const T* X, const T* L, const int
                            const int* macro_dev, int rows, int n_c, double* integral,
                            cudaStream_t st);
 
-// The same time integral on the tensor cores (FP32 singlet slices written by
-// launch_step with xblk = 1; tcgen05.mma kind::tf32 with a hi/lo split of
+// The same time integral on the tensor cores (FP32 singlet slices that
+// launch_term and launch_macro_cluster write with xblk = 1; tcgen05.mma kind::tf32 with a hi/lo split of
 // every value, FP64 contraction with W).  Row r covers the configurations of
 // its system ham[row_sys[r]] (row_sys NULL: system 0); Zs is the slot stride.
 // n_sm sizes the grid; err receives

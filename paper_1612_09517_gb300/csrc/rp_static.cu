@@ -301,11 +301,10 @@ rp_status run_static(const rp::HostSystem& hs, int n_fields, const double* field
       for (int r = 0; r < rows; ++r) act += (k < h_win[r].y) ? 1 : 0;
       for (int n = 1; n < n_c; ++n) {
         const int mode = (n == 1) ? rp::MODE_FIRST : (n == n_c - 1 ? rp::MODE_LAST : rp::MODE_MID);
-        L1(rp::launch_step<T>(SYS, &H, H.aniso, 0, d_fdev, d_field, d_win, (int)k, nullptr, rows,
-                              phi[(n - 1) % 3],
-                              n >= 2 ? phi[(n - 2) % 3] : nullptr,
+        L1(rp::launch_step<T>(SYS, H, H.aniso, d_fdev, d_field, d_win, (int)k, rows,
+                              phi[(n - 1) % 3], n >= 2 ? phi[(n - 2) % 3] : nullptr,
                               mode == rp::MODE_LAST ? nullptr : phi[n % 3], Q, X, d_coef, n_c, n,
-                              mode, 0, st),
+                              mode, st),
            "step kernel");
         steps++;
       }

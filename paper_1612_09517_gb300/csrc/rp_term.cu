@@ -37,17 +37,11 @@ constexpr int kTermThreads = 256;
 // KPT complex values at p (16- or 32-byte aligned for KPT > 1).
 template <typename T, int KPT>
 __device__ __forceinline__ void gload(const T* p, Cx<T> (&q)[KPT]) {
-  if constexpr (sizeof(T) * KPT == 16) {  // 32 bytes
-    if constexpr (sizeof(T) == 4) {
-      asm("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-          : "=f"(q[0].re), "=f"(q[0].im), "=f"(q[1].re), "=f"(q[1].im), "=f"(q[2].re),
-            "=f"(q[2].im), "=f"(q[3].re), "=f"(q[3].im)
-          : "l"(p));
-    } else {
-      asm("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
-          : "=d"(q[0].re), "=d"(q[0].im), "=d"(q[1].re), "=d"(q[1].im)
-          : "l"(p));
-    }
+  static_assert(KPT <= 2, "one or two configurations per thread");
+  if constexpr (sizeof(T) * KPT == 16) {  // two FP64 values
+    asm("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
+        : "=d"(q[0].re), "=d"(q[0].im), "=d"(q[1].re), "=d"(q[1].im)
+        : "l"(p));
   } else if constexpr (sizeof(T) * KPT == 8) {  // 16 bytes
     if constexpr (sizeof(T) == 4) {
       const float4 v = *reinterpret_cast<const float4*>(p);
@@ -65,16 +59,9 @@ __device__ __forceinline__ void gload(const T* p, Cx<T> (&q)[KPT]) {
 template <typename T, int KPT>
 __device__ __forceinline__ void gstore(T* p, const Cx<T> (&q)[KPT]) {
   if constexpr (sizeof(T) * KPT == 16) {
-    if constexpr (sizeof(T) == 4) {
-      asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(q[0].re),
-                   "f"(q[0].im), "f"(q[1].re), "f"(q[1].im), "f"(q[2].re), "f"(q[2].im),
-                   "f"(q[3].re), "f"(q[3].im)
-                   : "memory");
-    } else {
-      asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(q[0].re), "d"(q[0].im),
-                   "d"(q[1].re), "d"(q[1].im)
-                   : "memory");
-    }
+    asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(q[0].re), "d"(q[0].im),
+                 "d"(q[1].re), "d"(q[1].im)
+                 : "memory");
   } else if constexpr (sizeof(T) * KPT == 8) {
     if constexpr (sizeof(T) == 4)
       *reinterpret_cast<float4*>(p) = make_float4(q[0].re, q[0].im, q[1].re, q[1].im);
