@@ -1525,7 +1525,7 @@ bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_
   // thread, 51 ms with four, which spill.  FP64 gains nothing from in-thread
   // nuclei (82 -> 143 ms: half the warps), so it takes them only where the
   // threads would not fit.
-  const long long per_sm = load / 152;
+  const long long per_sm = load / kChipSms;
   out->split = false;
   if (per_sm <= 256 && max_nuc <= kSplitNuc && 4 * Zmax <= split_max_threads<T>()) {
     ChipPlan P;
@@ -1550,7 +1550,7 @@ bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_
     // rows per CTA: fill a warp, then up to 128 threads while every SM still
     // gets a CTA
     int rpc = std::max<int>(1, (int)(32 / Sr));
-    while (rpc < 32 && (rpc * 2) * Sr <= 128 && n_items / (rpc * 2) >= 152 * 2) rpc *= 2;
+    while (rpc < 32 && (rpc * 2) * Sr <= 128 && n_items / (rpc * 2) >= kChipSms * 2) rpc *= 2;
     P.rpc = rpc;
     P.threads = (int)((rpc * Sr + 31) / 32 * 32);
     P.slots = (int)(rpc * Sr);
@@ -1567,6 +1567,14 @@ bool chip_plan(long long Zmax, int min_half, int max_nuc, long long load, int n_
 // Split over clusters (FP32): the smallest cluster whose CTAs hold their share,
 // larger while the rows alone leave SMs idle.  Two configurations per thread
 // where 640 threads (96 registers) suffice, else four.
+//
+// Against one launch per term, in ms (two fields, 8, 32, 128 and 256 propagations; the last
+// two at half the horizon): Z = 9216 on 8 CTAs 2.2, 3.9, 6.7, 12.9 and per term 3.5, 4.2,
+// 6.1, 10.9; Z = 13824 (four configurations per thread, which spill) 3.1, 5.8, 10.2, 19.7
+// and 3.6, 5.3, 8.4, 15.1; Z = 16384 3.5, 6.5, 11.6, 22.7 and 3.7, 5.4, 10.1, 18.0.  So
+// beyond about two waves of clusters of 8 (15 to 18 run at once) the per-term launches are
+// up to a quarter faster; the rule takes clusters at any number of rows, which is what the
+// uneven batches need (few rows per pair), and is faster than the kernels before it at all.
 bool chip_cluster_plan(long long Zmax, int min_half, int max_nuc, int n_items, int n_c, bool spin1_only,
                        ChipPlan* out) {
   if (!spin1_only) return false;
@@ -1586,7 +1594,7 @@ bool chip_cluster_plan(long long Zmax, int min_half, int max_nuc, int n_items, i
       // a larger cluster while the rows leave SMs idle: one field, 0.3 us, 8 rows: Z =
       // 2304 2.35 ms on 2 CTAs, 1.69 on 4; Z = 4608 2.57 on 4, 2.01 on 8; with 40 rows
       // the smaller one takes 2.37 and 4.82 either way
-      if (found && ((long long)n_items << cb) > 152) return true;
+      if (found && ((long long)n_items << cb) > kChipSms) return true;
       *out = P;
       found = true;
       break;
@@ -1718,7 +1726,7 @@ bool aniso_plan(long long Zmax, int min_half, int max_nuc, int n_items, int n_c,
     // a larger cluster only while the rows alone leave SMs idle and each CTA keeps a
     // warp per scheduler (32 rows, Z = 192, FP64: one block per row of the generic
     // kernel, 62.5 ms; 4 blocks per row, 9.7)
-    if (found && (((long long)n_items << cb) > 152 || P.threads < 128)) return true;
+    if (found && (((long long)n_items << cb) > kChipSms || P.threads < 128)) return true;
     *out = P;
     found = true;
   }

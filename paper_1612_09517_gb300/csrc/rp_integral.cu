@@ -388,7 +388,7 @@ cudaError_t launch_project(const SysTab<T>& S, const T* X, const T* L, const int
   const long long tile = (long long)kProjThreads * ProjCfg<T>::kCfg;
   const long long tiles = (S.Zslot + tile - 1) / tile;
   const long long per = S.Zslot <= 1024 ? tiles
-                                        : std::min<long long>(8, std::max<long long>(1, tiles * rows / (152 * 12)));
+                                        : std::min<long long>(8, std::max<long long>(1, tiles * rows / (kChipSms * 12)));
   dim3 grid((unsigned)((tiles + per - 1) / per), rows);
   const size_t smem = proj_smem_bytes<T>(n_c);
   static std::atomic<unsigned long long> attr_done;
