@@ -182,7 +182,7 @@ bool persistent_default(long long Zslot, int n_systems) {
 
 // Calls that always run as one launch over all items.  Such a launch keeps no rows in
 // device memory, so max_rows does not bound it (Z = 864, 32 propagations, max_rows = 1:
-// 2.8 ms, 38.9 with one block at a time).
+// 2.5 ms, 38.9 with one block at a time).
 bool one_launch(long long Zslot, long long Zmax_chip, int n_systems, const rp_options& o) {
   return Zslot <= Zmax_chip && o.deterministic != 3 &&
          (o.kernel == 5 || (o.kernel == 0 && !o.graph && persistent_default(Zslot, n_systems)));

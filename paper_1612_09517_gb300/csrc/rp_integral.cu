@@ -228,9 +228,11 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_integral(
 // plans in FP32, two in FP64) through a ring of asynchronous copies.  FP32 works
 // on pairs (y_k, y_{k+1}) by fma.rn.f32x2.  The squares of one configuration
 // are summed in T and added in FP64.
+// CLUSTER: the CTAs of a row form a thread-block cluster and its first one adds their sums
+// in order.
 constexpr int kProjThreads = 128;
 
-template <typename T>
+template <typename T, bool CLUSTER>
 __global__ void __launch_bounds__(kProjThreads) k_project(
     const SysTab<T> S, const T* __restrict__ X, const T* __restrict__ L, int ldk,
     const int2* __restrict__ meta, const int* __restrict__ row_field,
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project(
   const long long Zs = S.Zslot;
   const long long z0 = (long long)blockIdx.x * z_per_cta;
   const long long z1 = min(Z, z0 + z_per_cta);
-  if (z0 >= z1) return;
+  if (!CLUSTER && z0 >= z1) return;
   const int f = row_field[r];
   const int2 mt = meta[f];
   const int n_e = (mt.y + 1) & ~1;  // n_c is even
@@ -283,7 +285,26 @@ __global__ void __launch_bounds__(kProjThreads) k_project(
     }
   }
   const double tot = block_sum<kProjThreads>(sum, red);
-  if (tid == 0) atomicAdd(integral + r, tot);
+  if constexpr (CLUSTER) {
+    __shared__ double part;
+    if (tid == 0) part = tot;
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    if (blockIdx.x == 0 && tid == 0) {  // the cluster's rank 0
+      double s = integral[r];
+      for (unsigned k = 0; k < gridDim.x; ++k) {
+        unsigned a;
+        double v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(&part)), "r"(k));
+        asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+        s += v;
+      }
+      integral[r] = s;
+    }
+    // no CTA leaves while the first one may read its sum
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  } else if (tid == 0) {
+    atomicAdd(integral + r, tot);
+  }
 }
 
 // The same in FP64 for rows of at most 96 configurations.  A warp's FP64 instruction holds
@@ -381,23 +402,39 @@ cudaError_t launch_project(const SysTab<T>& S, const T* X, const T* L, const int
       return cudaGetLastError();
     }
   }
-  // a CTA takes up to 8 tiles of configurations (its L costs one tile's loads),
-  // fewer where the rows alone would not give every SM several CTAs.  A row of up to
-  // 1024 configurations is one CTA's: its sum then runs in a fixed order, and equal calls
-  // give equal bits
   const long long tile = (long long)kProjThreads * ProjCfg<T>::kCfg;
   const long long tiles = (S.Zslot + tile - 1) / tile;
-  const long long per = S.Zslot <= 1024 ? tiles
-                                        : std::min<long long>(8, std::max<long long>(1, tiles * rows / (kChipSms * 12)));
-  dim3 grid((unsigned)((tiles + per - 1) / per), rows);
   const size_t smem = proj_smem_bytes<T>(n_c);
-  static std::atomic<unsigned long long> attr_done;
-  const cudaError_t e = smem_attr_once((const void*)k_project<T>, (int)proj_smem_bytes<T>(88), attr_done);
-  if (e != cudaSuccess) return e;
-  k_project<T><<<grid, kProjThreads, smem, st>>>(S, X, L, integral_ldk(n_c), meta, row_field,
-                                                 row_win, macro, macro_dev, n_c, per * tile,
-                                                 integral);
-  return cudaGetLastError();
+  static std::atomic<unsigned long long> attr_done[2];
+  auto go = [&](auto kf, unsigned ctas, unsigned cluster, long long per, int k) {
+    const cudaError_t e = smem_attr_once((const void*)kf, (int)proj_smem_bytes<T>(88), attr_done[k]);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas, (unsigned)rows, 1);
+    cfg.blockDim = dim3(kProjThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kf, S, X, L, integral_ldk(n_c), meta, row_field, row_win, macro,
+                              macro_dev, n_c, per * tile, integral);
+  };
+  // A row of up to 1024 configurations is one cluster's, a tile per CTA: its sum runs in a
+  // fixed order, and equal calls give equal bits.  (One CTA per row does so too: whole
+  // calls of kernel = 2, Z = 864, FP64, 32 rows, 62 ms against 39.)
+  if (S.Zslot <= 1024) {
+    unsigned c = 1;
+    while (c < tiles) c *= 2;
+    return c == 1 ? go(k_project<T, false>, 1u, 1u, 1, 0) : go(k_project<T, true>, c, c, 1, 1);
+  }
+  // a CTA takes up to 8 tiles of configurations (its L costs one tile's loads),
+  // fewer where the rows alone would not give every SM several CTAs
+  const long long per = std::min<long long>(8, std::max<long long>(1, tiles * rows / (kChipSms * 12)));
+  return go(k_project<T, false>, (unsigned)((tiles + per - 1) / per), 1u, per, 0);
 }
 
 #define RP_INTEGRAL_INST(T)                                                                       \
