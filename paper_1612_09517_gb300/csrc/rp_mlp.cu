@@ -29,7 +29,7 @@
 // and SiLU and write the split activations as the next layer's A operand (256 threads
 // with half a row each spilled: with the issuing warp they have 168 registers); one
 // thread of another warp streams weight tiles (w1 and w2 of 16 inputs x all outputs in
-// turn, one bulk copy each, four in flight) and issues the MMAs.  All waits are bounded.
+// turn, one bulk copy each, 32 KB in flight) and issues the MMAs.  All waits are bounded.
 //
 // Bounds: within a CTA the layers of a tile are a chain (products, SiLU, next operand).
 // 65536 rows x 8 fields, 46 inputs, 3 x 256: 9.3 ms as FP32 CUDA-core products with a pass
@@ -49,7 +49,8 @@ namespace {
 constexpr int kRows = 128;
 constexpr int kWorkers = 512;           // four threads per row
 constexpr int kMlpThreads = kWorkers + 32;
-constexpr int kTileK = 16, kTiles = 4;  // inputs per weight tile, tiles in flight
+constexpr int kTileK = 16;  // inputs per weight tile
+constexpr int kRing = 32 * 1024;  // bytes of weight tiles in flight
 
 // Outputs padded to the tile of an instance, inputs of the first layer to whole tiles
 inline int pad_hidden(int h) { return h <= 64 ? 64 : h <= 128 ? 128 : 256; }
@@ -111,62 +112,69 @@ __device__ __forceinline__ float cut_high(const Cut& c, float v, float& high) {
   return fmaf(-q, c.grid, v);
 }
 
-// scale[l][k] (256 per layer): the power of two of input k's largest weight, relative to that
-// of the layer and at least 2^-60.  A block of 1024 threads per layer.
-constexpr int kMaxIn = 256;
-__global__ void __launch_bounds__(4 * kMaxIn) k_mlp_scale(const MlpNet N, float* __restrict__ scale) {
-  __shared__ unsigned top[kMaxIn], all;
-  const int l = blockIdx.x, k = threadIdx.x % kMaxIn, in = l == 0 ? N.d_in : N.hidden;
-  if (threadIdx.x < kMaxIn) top[k] = 0u;
-  if (threadIdx.x == 0) all = 0u;
-  __syncthreads();
-  unsigned m = 0u;  // magnitudes compare as integers
-  if (k < in) {
-    const __nv_bfloat16* w = N.wbf + N.w_off[l] + k;
-#pragma unroll 8
-    for (int o = threadIdx.x / kMaxIn; o < N.hidden; o += 4)
-      m = max(m, mag(__bfloat162float(w[(long long)o * in])));
-  }
-  atomicMax(&top[k], m);
-  atomicMax(&all, m);
-  __syncthreads();
-  if (threadIdx.x < kMaxIn) {
-    const int e = max((int)(top[k] >> 23) - (int)(all >> 23), -60);
-    scale[l * kMaxIn + k] = __uint_as_float((unsigned)(127 + e) << 23);
-  }
-}
-
-// Tile t of the stream: [part][input / 8][output / 8][8 outputs][8 inputs], part 0 w1 and 1
-// w2; after the tiles the biases of the hidden layers and the output layer's weights, FP32,
-// HP each, then the scales of k_mlp_scale.  A warp per output of a hidden layer, then a thread per value of the rest.
-__global__ void k_mlp_pack(const MlpNet N, int HP, const float* __restrict__ scale,
-                           __nv_bfloat16* __restrict__ out, long long total) {
-  const int rows = N.layers * HP, warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (warp >= rows) {
-    const int j = (warp - rows) * 32 + lane, l = j / HP, o = j % HP;
-    if (l > N.layers) return;
-    float v = 0.f;
-    if (o < N.hidden)
-      v = l < N.layers ? N.params[N.b_off[l] + o] : __bfloat162float(N.wbf[N.w_off[l] + o]);
-    reinterpret_cast<float*>(out + total)[j] = v;
-    return;
-  }
-  const int l = warp / HP, o = warp % HP;
+// The packed weights: tiles in the order of the stream, tile t as [part][input / 8]
+// [output / 8][8 outputs][8 inputs], part 0 w1 and 1 w2; then, in FP32, the biases of the
+// hidden layers and the output layer's weights, HP each, and the scales, 256 per layer.
+// Input k of layer l has the power of two of its largest weight, relative to that of the
+// layer and at least 2^-60.  Each block finds the scales of its layer and takes 32 of its
+// outputs, one per warp.
+constexpr int kMaxIn = 256, kPackThreads = 1024;
+__global__ void __launch_bounds__(kPackThreads) k_mlp_pack(const MlpNet N, int HP,
+                                                           __nv_bfloat16* __restrict__ out,
+                                                           long long total) {
+  __shared__ unsigned tops[kMaxIn], all;
+  __shared__ float sc[kMaxIn];
+  const int tid = threadIdx.x, lane = tid & 31, per = HP / 32;
+  const int l = (int)blockIdx.x / per, o = (int)blockIdx.x % per * 32 + (tid >> 5);
   const int in = l == 0 ? N.d_in : N.hidden, pad = l == 0 ? pad_in(N.d_in) : HP;
+  float* aux = reinterpret_cast<float*>(out + total);
+  if (tid < kMaxIn) tops[tid] = 0u;
+  if (tid == 0) all = 0u;
+  __syncthreads();
+  {
+    const int k = tid % kMaxIn;
+    unsigned m = 0u;  // magnitudes compare as integers
+    if (k < in) {
+      const __nv_bfloat16* w = N.wbf + N.w_off[l] + k;
+#pragma unroll 16
+      for (int q = tid / kMaxIn; q < N.hidden; q += kPackThreads / kMaxIn)
+        m = max(m, mag(__bfloat162float(w[(long long)q * in])));
+      atomicMax(&tops[k], m);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) atomicMax(&all, m);
+  }
+  __syncthreads();
+  if (tid < kMaxIn) {
+    const int e = max((int)(tops[tid] >> 23) - (int)(all >> 23), -60);
+    sc[tid] = __uint_as_float((unsigned)(127 + e) << 23);
+    if (blockIdx.x % per == 0) aux[(N.layers + 1) * HP + l * kMaxIn + tid] = sc[tid];
+  }
+  // biases, and the output layer's weights from the blocks of the last hidden layer
+  if (lane == 0) {
+    const bool on = o < N.hidden;
+    aux[l * HP + o] = on ? N.params[N.b_off[l] + o] : 0.f;
+    if (l == N.layers - 1) aux[N.layers * HP + o] = on ? __bfloat162float(N.wbf[N.w_off[N.layers] + o]) : 0.f;
+  }
+  __syncthreads();
   const int t0 = l == 0 ? 0 : (pad_in(N.d_in) + (l - 1) * HP) / kTileK;  // first tile of the layer
   const __nv_bfloat16* w = N.wbf + N.w_off[l] + (long long)o * in;
   const bool on = o < N.hidden;
-  const float* sc = scale + l * kMaxIn;
+  float v[kMaxIn / 32];
   unsigned top = 0u;
-  for (int k = lane; on && k < in; k += 32)
-    top = max(top, mag(__bfloat162float(w[k]) / sc[k]));  // powers of two: exact
 #pragma unroll
-  for (int s = 16; s > 0; s >>= 1) top = max(top, __shfl_xor_sync(0xffffffffu, top, s));
-  const Cut c = cut_of(top);
-  for (int k = lane; k < pad; k += 32) {
-    float high, low = 0.f;
-    low = cut_high(c, on && k < in ? __bfloat162float(w[k]) / sc[k] : 0.f, high);
+  for (int i = 0; i < kMaxIn / 32; ++i) {
+    const int k = i * 32 + lane;
+    v[i] = on && k < in ? __bfloat162float(w[k]) / sc[k] : 0.f;  // powers of two: exact
+    top = max(top, mag(v[i]));
+  }
+  const Cut c = cut_of(__reduce_max_sync(0xffffffffu, top));
+#pragma unroll
+  for (int i = 0; i < kMaxIn / 32; ++i) {
+    const int k = i * 32 + lane;
+    if (k >= pad) break;
+    float high;
+    const float low = cut_high(c, v[i], high);
     __nv_bfloat16* d = out + (size_t)(2 * (t0 + k / kTileK)) * HP * kTileK +
                        (k % kTileK) / 8 * (HP * 8) + o * 8 + k % 8;
     d[0] = __float2bfloat16(high);
@@ -234,6 +242,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(
     double* __restrict__ acc, int* __restrict__ err, unsigned part) {
   constexpr int CPT = HP / 4;  // outputs per thread
   constexpr unsigned kTileBytes = HP * kTileK * 2;
+  constexpr int kTiles = kRing / (int)kTileBytes;  // 4 to 16
   extern __shared__ __align__(128) unsigned char mlp_smem[];
   // full[tile], empty[tile], then: a layer's products are done
   __shared__ __align__(8) unsigned long long bars[2 * kTiles + 1];
@@ -494,8 +503,8 @@ cudaError_t launch_mlp_of(const MlpNet& net, const __nv_bfloat16* packed, int n,
   const int ka = std::max(HP, pad_in(net.d_in));
   const unsigned part = (unsigned)ka * kRows * 2;
   // at least 116 KB: one CTA per SM, which owns the tensor memory it asks for
-  const int smem = std::max((int)(3 * part + kTiles * HP * kTileK * 2), 116 * 1024);
-  cudaError_t e = smem_attr_once((const void*)kf, 3 * 2 * kRows * 256 + kTiles * 256 * kTileK * 2, attr_done);
+  const int smem = std::max((int)(3 * part) + kRing, 116 * 1024);
+  cudaError_t e = smem_attr_once((const void*)kf, 3 * 2 * kRows * 256 + kRing, attr_done);
   if (e != cudaSuccess) return e;
   int dev = 0, n_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -521,11 +530,7 @@ size_t mlp_packed_values(const MlpNet& net) {  // FP32 values count twice
 }
 cudaError_t launch_mlp_pack(const MlpNet& net, __nv_bfloat16* packed, cudaStream_t st) {
   const int HP = pad_hidden(net.hidden);
-  const long long total = mlp_tile_values(net);
-  const int warps = net.layers * HP + ((net.layers + 1) * HP + 31) / 32;
-  float* scale = reinterpret_cast<float*>(packed + total) + (size_t)(net.layers + 1) * HP;
-  k_mlp_scale<<<net.layers, 4 * kMaxIn, 0, st>>>(net, scale);
-  k_mlp_pack<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(net, HP, scale, packed, total);
+  k_mlp_pack<<<net.layers * HP / 32, kPackThreads, 0, st>>>(net, HP, packed, mlp_tile_values(net));
   return cudaGetLastError();
 }
 cudaError_t launch_mlp(const MlpNet& net, const __nv_bfloat16* packed, int n, const float* x,
